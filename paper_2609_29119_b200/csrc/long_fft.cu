@@ -16,86 +16,17 @@
 //                                memory, then the inverse B-point DFT over q2, times conj W_Lp^{j2 q1}, written
 //                                transposed to Tinv[j2][q1].
 //            pass C':            inverse A-point DFT over q1, scaled, unpacked to x[2j], x[2j+1].
-// When Lp is small (A == 1) the row kernels read / write the signal directly and passes C, C' vanish.
+// When Lp is small (A == 1) one kernel per direction does it all (short_fft.cu).
 //
 // Weighted-bin scratch: P planes of Lp+1 bins per signal; band b writes plane b mod P, where P is the
 // largest number of bands covering one bin, so two bands of one plane never share a bin and the sum
 // over the bands covering bin k reads planes (lo + i) mod P, i < n, at index k: coalesced, no atomics.
 #include <algorithm>
 
-#include "engine.cuh"
-#include "internal.hpp"
+#include "long_common.cuh"
 #include "static_fft.cuh"
 
 namespace cqt {
-
-extern __shared__ float2 smem_long[];
-
-struct LongArgs {
-    const FftPlan *ffts;
-    const float2 *tw;
-    int fft_A, fft_B;
-    int A, B, Lp;
-    int tw_lp, log_lp_c, n_lp;   // two-level table of W_Lp and its entry count
-    int tw_n, log_n_c, n_n;      // two-level table of W_N
-    int tw_cols, tw_rows;
-    int valid_len;
-    int aligned;           // signal rows allow float2 access
-    long long x_stride;
-    const float *x_in;
-    float *x_out;
-    float2 *T;
-    long long t_pitch;
-    float2 *X;             // half spectrum rows (forward)
-    long long x_pitch;
-    // inverse: overlap-add + retangle in the prologue of the row pass
-    int log_b, log_own;    // log2 B, log2 (2 TWr)
-    const float2 *Y;
-    long long y_pitch;     // per signal
-    long long y_plane;     // per plane
-    int planes;
-    const int32_t *cover;
-    float scale;
-    uint32_t cols_magic, rows_magic;
-    int *dbg;
-    // sliced source (forward column pass of the streaming form): row r is slice r / channels of channel r % channels,
-    // its sample i is slice_win[i] * ring[channel][(slice_first + (r / channels) * hop + i) mod ring_len], zero
-    // before the start of the stream
-    const float *ring;
-    const float *slice_win;
-    long long ring_len, slice_first, hop;
-    int channels;
-};
-
-__device__ __forceinline__ float2 load_packed(const float *row, int j, int valid_len, int aligned) {
-    const int i = 2 * j;
-    if (i + 1 < valid_len) {
-        if (aligned) return __ldcs(reinterpret_cast<const float2 *>(row + i));   // read once: streaming
-        return make_float2(__ldcs(row + i), __ldcs(row + i + 1));
-    }
-    if (i < valid_len) return make_float2(__ldcs(row + i), 0.f);
-    return make_float2(0.f, 0.f);
-}
-
-__device__ __forceinline__ void store_packed(float *row, int j, float2 v, int valid_len, int aligned) {
-    const int i = 2 * j;
-    if (i + 1 < valid_len) {
-        if (aligned) __stcs(reinterpret_cast<float2 *>(row + i), v);
-        else { __stcs(row + i, v.x); __stcs(row + i + 1, v.y); }
-    } else if (i < valid_len) {
-        __stcs(row + i, v.x);
-    }
-}
-
-// copies the full twiddle table of a power-of-two plan into shared memory
-__device__ __forceinline__ void stage_full(float2 *dst, const float2 *__restrict__ tw_base, const FftPlan &fp, int tid, int nthr) {
-    const float2 *src = tw_base + fp.tw_full_off;
-    for (int i = tid; i < fp.M; i += nthr) dst[i] = __ldg(src + i);
-}
-
-__device__ __forceinline__ void stage_table(float2 *dst, const float2 *__restrict__ src, int n, int tid, int nthr) {
-    for (int i = tid; i < n; i += nthr) dst[i] = __ldg(src + i);
-}
 
 // Every pass exists once as a template over a compile-time Shape (radices, columns, pitch) and is instantiated
 // for the common shapes plus the run-time planned fallback.
@@ -189,37 +120,28 @@ template <class SH>
 __device__ __forceinline__ void rows_fwd_body(const LongArgs &a, const FftPlan &fp, float2 *buf, const float2 *tws,
                                               const float2 *wn, int t, int ch, int tid, int nthr) {
     const int A = a.A, B = a.B, TW = a.tw_rows;
-    const bool direct = (A == 1);
-    const int ncols = direct ? 1 : 2 * TW;
-    const int pitch = SH::is_static ? SH::PITCH : (direct ? 1 : ncols + 1);   // odd: conflict-free transposing accesses
-    if (direct) {
-        const float *row = a.x_in + (long long)ch * a.x_stride;
-        const Tile tile{buf, pitch, ncols, a.rows_magic, B * pitch, a.dbg};
-        auto load = [&](int j, int) -> float2 { return load_packed(row, j, a.valid_len, a.aligned); };
-        fft_fused_keep<-1, BlockSync, true, false, true>(tile, fp, tws, load, tid, nthr);
+    const int ncols = 2 * TW;
+    const int pitch = SH::is_static ? SH::PITCH : ncols + 1;   // odd: conflict-free transposing accesses
+    const float2 *T = a.T + (long long)ch * a.t_pitch;
+    auto load = [&](int j2, int r) -> float2 {
+        const int i = row_of(t, r, TW, A) * B + j2;
+        return CQT_CHK(a.dbg, 202, i, a.Lp) ? __ldg(T + i) : make_float2(0.f, 0.f);
+    };
+    if constexpr (SH::is_static) {
+        auto nostore = [](int, int, float2) {};
+        tile_fft_static<SH, -1, false, true>(buf, tws, load, nostore, tid, nthr);
     } else {
-        const float2 *T = a.T + (long long)ch * a.t_pitch;
-        auto load = [&](int j2, int r) -> float2 {
-            const int i = row_of(t, r, TW, A) * B + j2;
-            return CQT_CHK(a.dbg, 202, i, a.Lp) ? __ldg(T + i) : make_float2(0.f, 0.f);
-        };
-        if constexpr (SH::is_static) {
-            auto nostore = [](int, int, float2) {};
-            tile_fft_static<SH, -1, false, true>(buf, tws, load, nostore, tid, nthr);
-        } else {
-            const Tile tile{buf, pitch, ncols, a.rows_magic, B * pitch, a.dbg};
-            fft_fused_keep<-1, BlockSync, true, false, true>(tile, fp, tws, load, tid, nthr);
-        }
+        const Tile tile{buf, pitch, ncols, a.rows_magic, B * pitch, a.dbg};
+        fft_fused_keep<-1, BlockSync, true, false, true>(tile, fp, tws, load, tid, nthr);
     }
     float2 *X = a.X + (long long)ch * a.x_pitch;
     // epilogue: each thread keeps one row (column r) and walks k2; for rows other than k1 = 0 the partner
     // Z_{Lp-k} sits in the mirror row's column at k2' = B-1-k2, whose position is the digit-wise complement B-1-pos(k2);
     // row 0 pairs with itself at k2' = (B - k2) mod B, row A/2 with itself at B-1-k2
-    const int nown = direct ? 1 : 2 * TW;
-    const int r = direct ? 0 : (tid & (nown - 1));
-    const int kstart = direct ? tid : (tid >> a.log_own), kstep = direct ? nthr : (nthr >> a.log_own);
-    const int k1 = direct ? 0 : row_of(t, r, TW, A);
-    const int rp = (direct || k1 == 0 || 2 * k1 == A) ? r : (r < TW ? r + TW : r - TW);
+    const int r = tid & (ncols - 1);
+    const int kstart = tid >> a.log_own, kstep = nthr >> a.log_own;
+    const int k1 = row_of(t, r, TW, A);
+    const int rp = (k1 == 0 || 2 * k1 == A) ? r : (r < TW ? r + TW : r - TW);
     for (int k2 = kstart; k2 < B; k2 += kstep) {
         const uint32_t pos = SH::pos(fp, (uint32_t)k2);
         uint32_t posp;
@@ -248,9 +170,7 @@ __global__ void __launch_bounds__(512, 2) rfft_rows_fwd_kernel(LongArgs a) {
     pdl_launch_dependents();
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int ch = blockIdx.y, t = blockIdx.x;
-    const bool direct = (a.A == 1);
-    const int ncols = direct ? 1 : 2 * a.tw_rows;
-    const int pitch = direct ? 1 : ncols + 1;
+    const int pitch = 2 * a.tw_rows + 1;
     const FftPlan &fp = a.ffts[a.fft_B];
     float2 *buf = smem_long;
     float2 *tws = buf + (size_t)a.B * pitch;
@@ -261,76 +181,6 @@ __global__ void __launch_bounds__(512, 2) rfft_rows_fwd_kernel(LongArgs a) {
     rows_fwd_body<SH>(a, fp, buf, tws, wn, t, ch, tid, nthr);
 }
 
-// ---------------------------------------------------------------- inverse: overlap-add + retangle
-// sum over the bands covering bin k, in band order
-// Sum over the bands covering bin k, in band order.  The cover word is (plane of the first covering band << 8) | number
-// of covering bands; band i of the range sits in plane (first + i) mod planes.  The first kUnroll plane values are loaded
-// unconditionally-predicated before any is used, so that their latencies overlap; absent terms add +0.
-constexpr int kGatherUnroll = 3;
-struct GatherLoads {
-    float2 v[kGatherUnroll];
-    int n, off, plane_len, wrap;
-};
-__device__ __forceinline__ GatherLoads gather_issue(const LongArgs &a, const float2 *__restrict__ Y, int k, int32_t cv) {
-    GatherLoads g;
-    g.n = cv & 255;
-    g.plane_len = (int)a.y_plane;
-    g.wrap = a.planes * g.plane_len;
-    g.off = (cv >> 8) * g.plane_len + k;
-    if (!CQT_CHK(a.dbg, 206, g.n, a.planes + 1)) g.n = 0;
-#pragma unroll
-    for (int i = 0; i < kGatherUnroll; ++i) {
-        g.v[i] = i < g.n ? __ldg(Y + g.off) : make_float2(0.f, 0.f);
-        g.off += g.plane_len;
-        if (g.off >= g.wrap) g.off -= g.wrap;
-    }
-    return g;
-}
-__device__ __forceinline__ float2 gather_finish(const float2 *__restrict__ Y, GatherLoads &g) {
-    float2 acc = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < kGatherUnroll; ++i) { acc.x += g.v[i].x; acc.y += g.v[i].y; }
-    for (int i = kGatherUnroll; i < g.n; ++i) {
-        const float2 v = __ldg(Y + g.off);
-        acc.x += v.x;
-        acc.y += v.y;
-        g.off += g.plane_len;
-        if (g.off >= g.wrap) g.off -= g.wrap;
-    }
-    return acc;
-}
-
-// One pair (q, m = Lp - q) of packed bins: both half-spectrum bins are summed once (bands in fixed order) and both
-// packed bins follow from the same two values (Eq. retangle with w_{Lp-q} = -conj w_q):
-//   Z_q      = s [ (X_q + conj X_m) + i conj(w) (X_q - conj X_m) ]
-//   Z_{Lp-q} = s [ (X_m + conj X_q) - i w (X_m - conj X_q) ],   w = exp(-2 pi i q / N), s = 1/(2 Lp)
-// wn: two-level table of W_N (shared memory).
-__device__ __forceinline__ void retangle_finish(const LongArgs &a, const float2 *__restrict__ Y, const float2 *wn, int q,
-                                                GatherLoads &gq, GatherLoads &gm, float2 &zq, float2 &zm) {
-    float2 xq = gather_finish(Y, gq);
-    float2 xm = gather_finish(Y, gm);
-    if (q == 0) { xq.y = 0.f; xm.y = 0.f; }   // bins 0 and N/2 are made real
-    const float2 w = twiddle_s(wn, a.log_n_c, (uint32_t)q);
-    {
-        const float2 ev = make_float2(xq.x + xm.x, xq.y - xm.y);   // X_q + conj X_m
-        const float2 od = make_float2(xq.x - xm.x, xq.y + xm.y);   // X_q - conj X_m
-        const float2 rot = cmul(make_float2(w.y, w.x), od);        // i conj(w) = (w.y, w.x)
-        zq = make_float2(a.scale * (ev.x + rot.x), a.scale * (ev.y + rot.y));
-    }
-    {
-        const float2 ev = make_float2(xm.x + xq.x, xm.y - xq.y);   // X_m + conj X_q
-        const float2 od = make_float2(xm.x - xq.x, xm.y + xq.y);   // X_m - conj X_q
-        const float2 rot = cmul(make_float2(w.y, -w.x), od);       // -i w = (w.y, -w.x)
-        zm = make_float2(a.scale * (ev.x + rot.x), a.scale * (ev.y + rot.y));
-    }
-}
-__device__ __forceinline__ void retangle_pair(const LongArgs &a, const float2 *__restrict__ Y, const float2 *wn, int q, int m,
-                                              float2 &zq, float2 &zm) {
-    const int32_t cvq = __ldg(a.cover + q), cvm = __ldg(a.cover + m);
-    GatherLoads gq = gather_issue(a, Y, q, cvq), gm = gather_issue(a, Y, m, cvm);
-    retangle_finish(a, Y, wn, q, gq, gm, zq, zm);
-}
-
 // ---------------------------------------------------------------- inverse, pass R' (overlap-add + retangle + B-point pass)
 // The tile holds TW rows q1 and their mirror rows A - q1 (the same rows as the forward row pass, see row_of), so
 // the two packed bins of every pair (q, Lp - q) lie in one tile: the prologue sums each half-spectrum bin once and
@@ -339,68 +189,57 @@ template <class SH>
 __device__ __forceinline__ void rows_inv_body(const LongArgs &a, const FftPlan &fp, float2 *buf, const float2 *tws,
                                               const float2 *wl, const float2 *wn, int t, int ch, int tid, int nthr) {
     const int A = a.A, B = a.B, TW = a.tw_rows, Lp = a.Lp;
-    const bool direct = (A == 1);
-    const int ncols = direct ? 1 : 2 * TW;
-    const int pitch = SH::is_static ? SH::PITCH : (direct ? 1 : ncols + 1);
+    const int ncols = 2 * TW;
+    const int pitch = SH::is_static ? SH::PITCH : ncols + 1;
     const float2 *Y = a.Y + (long long)ch * a.y_pitch;
     __syncthreads();   // the table of W_N is staged
-    if (direct) {
-        for (int q = tid; q <= (Lp >> 1); q += nthr) {
-            const int m = Lp - q;
+    // Four pairs per thread and round: all cover words are fetched first, then the plane values of two pairs
+    // at a time, so that the dependent loads of one pair overlap those of the others.
+    const int log_tw = 31 - __clz(TW);
+    constexpr int kPairs = 4;
+    for (int base = 0; base < TW * B; base += kPairs * nthr) {
+        int q[kPairs], r[kPairs], q2[kPairs];
+        int32_t cq[kPairs], cm[kPairs];
+        bool ok[kPairs], self[kPairs];
+#pragma unroll
+        for (int u = 0; u < kPairs; ++u) {
+            const int idx = base + u * nthr + tid;
+            r[u] = idx & (TW - 1);
+            q2[u] = idx >> log_tw;
+            const int k1 = TW * t + 1 + r[u];
+            self[u] = 2 * k1 == A;           // row A/2 is its own mirror: the pairs (q2, B-1-q2) of one column
+            ok[u] = idx < TW * B && !(self[u] && q2[u] >= (B >> 1));
+            q[u] = ok[u] ? k1 + A * q2[u] : 1;
+            if (!CQT_CHK(a.dbg, 210, Lp - q[u], Lp) || !CQT_CHK(a.dbg, 211, q[u], Lp)) { ok[u] = false; q[u] = 1; }
+            cq[u] = __ldg(a.cover + q[u]);
+            cm[u] = __ldg(a.cover + (Lp - q[u]));
+        }
+#pragma unroll
+        for (int u = 0; u < kPairs; u += 2) {
+            GatherLoads g0q = gather_issue(a, Y, q[u], cq[u]), g0m = gather_issue(a, Y, Lp - q[u], cm[u]);
+            GatherLoads g1q = gather_issue(a, Y, q[u + 1], cq[u + 1]), g1m = gather_issue(a, Y, Lp - q[u + 1], cm[u + 1]);
+            float2 zq, zm;
+            retangle_finish(a, Y, wn, q[u], g0q, g0m, zq, zm);
+            if (ok[u]) {
+                buf[q2[u] * pitch + r[u]] = zq;
+                buf[(B - 1 - q2[u]) * pitch + (self[u] ? r[u] : r[u] + TW)] = zm;
+            }
+            retangle_finish(a, Y, wn, q[u + 1], g1q, g1m, zq, zm);
+            if (ok[u + 1]) {
+                buf[q2[u + 1] * pitch + r[u + 1]] = zq;
+                buf[(B - 1 - q2[u + 1]) * pitch + (self[u + 1] ? r[u + 1] : r[u + 1] + TW)] = zm;
+            }
+        }
+    }
+    if (2 * TW * (t + 1) == A) {
+        // the last tile's spare column holds row 0, which pairs with itself: bins A q2 and A (B - q2)
+        const int rz = 2 * TW - 1;
+        for (int q2 = tid; q2 <= (B >> 1); q2 += nthr) {
+            const int q = A * q2, m = Lp - q;
             float2 zq, zm;
             retangle_pair(a, Y, wn, q, m, zq, zm);
-            buf[q] = zq;
-            if (q != 0 && m != q) buf[m] = zm;
-        }
-    } else {
-        // Four pairs per thread and round: all cover words are fetched first, then the plane values of two pairs
-        // at a time, so that the dependent loads of one pair overlap those of the others.
-        const int log_tw = 31 - __clz(TW);
-        constexpr int kPairs = 4;
-        for (int base = 0; base < TW * B; base += kPairs * nthr) {
-            int q[kPairs], r[kPairs], q2[kPairs];
-            int32_t cq[kPairs], cm[kPairs];
-            bool ok[kPairs], self[kPairs];
-#pragma unroll
-            for (int u = 0; u < kPairs; ++u) {
-                const int idx = base + u * nthr + tid;
-                r[u] = idx & (TW - 1);
-                q2[u] = idx >> log_tw;
-                const int k1 = TW * t + 1 + r[u];
-                self[u] = 2 * k1 == A;           // row A/2 is its own mirror: the pairs (q2, B-1-q2) of one column
-                ok[u] = idx < TW * B && !(self[u] && q2[u] >= (B >> 1));
-                q[u] = ok[u] ? k1 + A * q2[u] : 1;
-                if (!CQT_CHK(a.dbg, 210, Lp - q[u], Lp) || !CQT_CHK(a.dbg, 211, q[u], Lp)) { ok[u] = false; q[u] = 1; }
-                cq[u] = __ldg(a.cover + q[u]);
-                cm[u] = __ldg(a.cover + (Lp - q[u]));
-            }
-#pragma unroll
-            for (int u = 0; u < kPairs; u += 2) {
-                GatherLoads g0q = gather_issue(a, Y, q[u], cq[u]), g0m = gather_issue(a, Y, Lp - q[u], cm[u]);
-                GatherLoads g1q = gather_issue(a, Y, q[u + 1], cq[u + 1]), g1m = gather_issue(a, Y, Lp - q[u + 1], cm[u + 1]);
-                float2 zq, zm;
-                retangle_finish(a, Y, wn, q[u], g0q, g0m, zq, zm);
-                if (ok[u]) {
-                    buf[q2[u] * pitch + r[u]] = zq;
-                    buf[(B - 1 - q2[u]) * pitch + (self[u] ? r[u] : r[u] + TW)] = zm;
-                }
-                retangle_finish(a, Y, wn, q[u + 1], g1q, g1m, zq, zm);
-                if (ok[u + 1]) {
-                    buf[q2[u + 1] * pitch + r[u + 1]] = zq;
-                    buf[(B - 1 - q2[u + 1]) * pitch + (self[u + 1] ? r[u + 1] : r[u + 1] + TW)] = zm;
-                }
-            }
-        }
-        if (2 * TW * (t + 1) == A) {
-            // the last tile's spare column holds row 0, which pairs with itself: bins A q2 and A (B - q2)
-            const int rz = 2 * TW - 1;
-            for (int q2 = tid; q2 <= (B >> 1); q2 += nthr) {
-                const int q = A * q2, m = Lp - q;
-                float2 zq, zm;
-                retangle_pair(a, Y, wn, q, m, zq, zm);
-                buf[q2 * pitch + rz] = zq;
-                if (q2 != 0 && m != q) buf[(B - q2) * pitch + rz] = zm;
-            }
+            buf[q2 * pitch + rz] = zq;
+            if (q2 != 0 && m != q) buf[(B - q2) * pitch + rz] = zm;
         }
     }
     __syncthreads();
@@ -412,21 +251,16 @@ __device__ __forceinline__ void rows_inv_body(const LongArgs &a, const FftPlan &
         const Tile tile{buf, pitch, ncols, a.rows_magic, B * pitch, a.dbg};
         fft_fused_keep<+1, BlockSync, true, true, true>(tile, fp, tws, load, tid, nthr);
     }
-    if (direct) {
-        float *row = a.x_out + (long long)ch * a.x_stride;
-        for (int j = tid; j < B; j += nthr) store_packed(row, j, buf[SH::pos(fp, (uint32_t)j)], a.valid_len, a.aligned);
-    } else {
-        float2 *T = a.T + (long long)ch * a.t_pitch;
-        // The inverse keeps its intermediate transposed, Tinv[j2][q1]: consecutive threads take consecutive columns r, so
-        // the shared-memory reads (odd pitch) are conflict-free and the 8-byte stores of a warp fall in runs of TW rows;
-        // reading the digit-reversed positions of consecutive j2 instead would hit one bank 16 times.
-        for (int e = tid; e < ncols * B; e += nthr) {
-            const int j2 = e >> a.log_own, r = e - (j2 << a.log_own);
-            const int q1 = row_of(t, r, TW, A);
-            const float2 v = buf[SH::pos(fp, (uint32_t)j2) * (uint32_t)pitch + r];
-            const float2 w = cconj(twiddle_s(wl, a.log_lp_c, (uint32_t)j2 * (uint32_t)q1));
-            if (CQT_CHK(a.dbg, 207, j2 * A + q1, a.Lp)) T[j2 * A + q1] = cmul(v, w);
-        }
+    float2 *T = a.T + (long long)ch * a.t_pitch;
+    // The inverse keeps its intermediate transposed, Tinv[j2][q1]: consecutive threads take consecutive columns r, so
+    // the shared-memory reads (odd pitch) are conflict-free and the 8-byte stores of a warp fall in runs of TW rows;
+    // reading the digit-reversed positions of consecutive j2 instead would hit one bank 16 times.
+    for (int e = tid; e < ncols * B; e += nthr) {
+        const int j2 = e >> a.log_own, r = e - (j2 << a.log_own);
+        const int q1 = row_of(t, r, TW, A);
+        const float2 v = buf[SH::pos(fp, (uint32_t)j2) * (uint32_t)pitch + r];
+        const float2 w = cconj(twiddle_s(wl, a.log_lp_c, (uint32_t)j2 * (uint32_t)q1));
+        if (CQT_CHK(a.dbg, 207, j2 * A + q1, a.Lp)) T[j2 * A + q1] = cmul(v, w);
     }
 }
 
@@ -435,9 +269,7 @@ __global__ void __launch_bounds__(512, 2) irfft_rows_kernel(LongArgs a) {
     pdl_launch_dependents();
     const int tid = threadIdx.x, nthr = blockDim.x;
     const int ch = blockIdx.y, t = blockIdx.x;
-    const bool direct = (a.A == 1);
-    const int ncols = direct ? 1 : 2 * a.tw_rows;
-    const int pitch = direct ? 1 : ncols + 1;
+    const int pitch = 2 * a.tw_rows + 1;
     const FftPlan &fp = a.ffts[a.fft_B];
     float2 *buf = smem_long;
     float2 *tws = buf + (size_t)a.B * pitch;
@@ -445,7 +277,7 @@ __global__ void __launch_bounds__(512, 2) irfft_rows_kernel(LongArgs a) {
     float2 *wl = wn + a.n_n;
     stage_full(tws, a.tw, fp, tid, nthr);
     stage_table(wn, a.tw + a.tw_n, a.n_n, tid, nthr);
-    if (!direct) stage_table(wl, a.tw + a.tw_lp, a.n_lp, tid, nthr);
+    stage_table(wl, a.tw + a.tw_lp, a.n_lp, tid, nthr);
     pdl_wait();   // the tables above belong to the plan; what follows reads the predecessor's output
     rows_inv_body<SH>(a, fp, buf, tws, wl, wn, t, ch, tid, nthr);
 }
@@ -486,55 +318,17 @@ __global__ void __launch_bounds__(512, 2) irfft_cols_kernel(LongArgs a) {
     cols_inv_body<SH>(a, fp, buf, tws, j2_0, ch, tid, nthr);
 }
 
-// ---------------------------------------------------------------- host side
-static uint32_t magic_of(uint32_t d) { return d <= 1 ? 0u : (uint32_t)(((1ull << 32) + d - 1) / d); }
-
-static LongArgs base_args(const cqt_plan &p, int64_t valid_len, int64_t x_stride, const void *xptr) {
-    LongArgs a{};
-    a.ffts = p.d.ffts;
-    a.tw = p.d.tw;
-    a.fft_A = p.lf.fft_A;
-    a.fft_B = p.lf.fft_B;
-    a.A = (int)p.lf.A;
-    a.B = (int)p.lf.B;
-    a.Lp = (int)p.lf.Lp;
-    a.tw_lp = p.lf.tw_lp;
-    a.log_lp_c = p.lf.log_lp_c;
-    a.n_lp = p.lf.n_lp;
-    a.tw_n = p.lf.tw_n;
-    a.log_n_c = p.lf.log_n_c;
-    a.n_n = p.lf.n_n;
-    a.tw_cols = p.lf.tw_cols;
-    a.tw_rows = p.lf.tw_rows;
-    a.valid_len = (int)valid_len;
-    a.x_stride = x_stride;
-    a.aligned = ((reinterpret_cast<uintptr_t>(xptr) & 7) == 0 && (x_stride & 1) == 0) ? 1 : 0;
-    a.t_pitch = p.lf.Lp;
-    a.x_pitch = p.lf.x_pitch;
-    a.y_pitch = p.y_pitch;
-    a.y_plane = p.y_plane;
-    a.planes = p.y_planes;
-    a.cover = p.d.cover;
-    a.cols_magic = magic_of(a.tw_cols);
-    a.dbg = p.d.dbg;
-    a.log_b = 0;
-    while ((1ll << a.log_b) < p.lf.B) ++a.log_b;
-    a.log_own = 0;
-    while ((1 << a.log_own) < 2 * p.lf.tw_rows) ++a.log_own;
-    return a;
-}
-
 static size_t plan_tw(const cqt_plan &p, int fft) { return (size_t)p.ffts[fft].M; }
 
 static size_t rows_fwd_smem(const cqt_plan &p) {
     const LongFft &lf = p.lf;
-    const size_t data = lf.A == 1 ? (size_t)lf.B : (size_t)lf.B * (2 * lf.tw_rows + 1);
+    const size_t data = (size_t)lf.B * (2 * lf.tw_rows + 1);
     return (data + plan_tw(p, lf.fft_B) + lf.n_n) * 8;
 }
 static size_t rows_inv_smem(const cqt_plan &p) {
     const LongFft &lf = p.lf;
-    const size_t data = lf.A == 1 ? (size_t)lf.B : (size_t)lf.B * (2 * lf.tw_rows + 1);
-    return (data + plan_tw(p, lf.fft_B) + lf.n_n + (lf.A == 1 ? 0 : lf.n_lp)) * 8;
+    const size_t data = (size_t)lf.B * (2 * lf.tw_rows + 1);
+    return (data + plan_tw(p, lf.fft_B) + lf.n_n + lf.n_lp) * 8;
 }
 static size_t cols_smem(const cqt_plan &p) {
     const LongFft &lf = p.lf;
@@ -570,11 +364,11 @@ static const void *cols_fwd_sliced_fn(const cqt_plan &p) {
     return PickKernel<ColsFwdSlicedK, Sh_8_8_8_16_16, Sh_16_16_1_16_16, Sh_16_8_1_16_16>::get(p.ffts[p.lf.fft_A], p.lf.tw_cols);
 }
 static const void *rows_fwd_fn(const cqt_plan &p) {
-    const int ncols = p.lf.A == 1 ? 1 : 2 * p.lf.tw_rows;
+    const int ncols = 2 * p.lf.tw_rows;
     return PickKernel<RowsFwdK, Sh_8_8_8_16_17, Sh_16_16_1_16_17, Sh_16_8_1_16_17, Sh_16_8_8_8_9>::get(p.ffts[p.lf.fft_B], ncols);
 }
 static const void *rows_inv_fn(const cqt_plan &p) {
-    const int ncols = p.lf.A == 1 ? 1 : 2 * p.lf.tw_rows;
+    const int ncols = 2 * p.lf.tw_rows;
     return PickKernel<RowsInvK, Sh_8_8_8_16_17, Sh_16_16_1_16_17, Sh_16_8_1_16_17, Sh_16_8_8_8_9>::get(p.ffts[p.lf.fft_B], ncols);
 }
 static const void *cols_inv_fn(const cqt_plan &p) {
@@ -618,9 +412,7 @@ cudaError_t launch_rfft_forward(const cqt_plan &p, const float *x, int64_t x_str
         dim3 grid2((unsigned)(lf.A / (2 * lf.tw_rows)), (unsigned)batch);
         launch_long(rows_fwd_fn(p), grid2, threads_for((size_t)lf.B * (2 * lf.tw_rows), p.ffts[lf.fft_B]), rows_fwd_smem(p), a, st);
     } else {
-        a.rows_magic = 0;
-        dim3 grid2(1, (unsigned)batch);
-        launch_long(rows_fwd_fn(p), grid2, threads_for((size_t)lf.B, p.ffts[lf.fft_B]), rows_fwd_smem(p), a, st);
+        launch_short_rfft_forward(p, a, batch, st);
     }
     note_launch(p, "rfft_rows_fwd", st);
     return cudaGetLastError();
@@ -648,28 +440,23 @@ cudaError_t launch_rfft_inverse(const cqt_plan &p, const float2 *Y, float2 *T, f
         launch_long(cols_inv_fn(p), grid2, threads_for((size_t)lf.A * lf.tw_cols, p.ffts[lf.fft_A]), cols_smem(p), a, st);
         note_launch(p, "irfft_cols", st);
     } else {
-        a.rows_magic = 0;
-        dim3 grid(1, (unsigned)batch);
-        launch_long(rows_inv_fn(p), grid, threads_for((size_t)lf.B, p.ffts[lf.fft_B]), rows_inv_smem(p), a, st);
+        launch_short_rfft_inverse(p, a, batch, st);
         note_launch(p, "irfft_rows", st);
     }
     return cudaGetLastError();
 }
 
 cudaError_t configure_long_fft_kernels(const cqt_plan &p) {
-    cudaError_t e;
-    e = allow_dynamic_smem(rows_fwd_fn(p), rows_fwd_smem(p), p);
+    if (p.lf.A == 1) return configure_short_fft_kernels(p);
+    cudaError_t e = allow_dynamic_smem(rows_fwd_fn(p), rows_fwd_smem(p), p);
     if (e != cudaSuccess) return e;
     e = allow_dynamic_smem(rows_inv_fn(p), rows_inv_smem(p), p);
     if (e != cudaSuccess) return e;
-    if (p.lf.A > 1) {
-        e = allow_dynamic_smem(cols_fwd_fn(p), cols_smem(p), p);
-        if (e != cudaSuccess) return e;
-        e = allow_dynamic_smem(cols_fwd_sliced_fn(p), cols_smem(p), p);
-        if (e != cudaSuccess) return e;
-        e = allow_dynamic_smem(cols_inv_fn(p), cols_smem(p), p);
-    }
-    return e;
+    e = allow_dynamic_smem(cols_fwd_fn(p), cols_smem(p), p);
+    if (e != cudaSuccess) return e;
+    e = allow_dynamic_smem(cols_fwd_sliced_fn(p), cols_smem(p), p);
+    if (e != cudaSuccess) return e;
+    return allow_dynamic_smem(cols_inv_fn(p), cols_smem(p), p);
 }
 
 }  // namespace cqt

@@ -1,0 +1,48 @@
+"""The launch forms that depend on sizes: the one-pass FFT of short signals at each of its lengths and with more signals
+than CTAs, the band launches on both sides of the batch where they change; against the fp64 oracle, first and last row."""
+import numpy as np
+import pytest
+
+import workloads as wl
+from helpers import band_rel_errors, library_plan, oracle_layout, small_workload, split_bands
+from oracle import nsgt_oracle as orc
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5
+
+
+def check_rows(w, batch):
+    lay, plan = oracle_layout(w), library_plan(w)
+    x = torch.randn(batch, w.valid_len, generator=torch.Generator().manual_seed(w.N + batch)).cuda()
+    c = plan.analyse(x, valid_len=w.valid_len)
+    y = plan.synthesise_adjoint(x, valid_len=w.valid_len)
+    xr = plan.synthesise(y, valid_len=w.valid_len)
+    rows = sorted({0, batch - 1})
+    xs = orc.pad_signal(x[rows].cpu().numpy(), w.N)
+    assert band_rel_errors(lay, c[rows].cpu().numpy(), orc.analyse(lay, xs)).max() <= TOL
+    assert band_rel_errors(lay, y[rows].cpu().numpy(), orc.synthesise_adjoint(lay, xs)).max() <= TOL
+    want = orc.synthesise(lay, split_bands(lay, y[rows].cpu().numpy().astype(np.complex128)))[..., :w.valid_len]
+    got = xr[rows].cpu().numpy()
+    assert (np.linalg.norm(got - want, axis=-1) / np.linalg.norm(want, axis=-1)).max() <= TOL
+    plan.close()
+
+
+@pytest.mark.parametrize("batch", [1, 2501])
+@pytest.mark.parametrize("log_n", range(6, 14))
+def test_one_pass_fft_lengths(log_n, batch):
+    n = 1 << log_n
+    check_rows(small_workload(f"short{n}", N=n, valid_len=n - 3, fs=float(n), fmin=max(3.0, n / 64.0), fmax=n / 2.0,
+                              bins_per_octave=4, m_policy=wl.M_SMOOTH, channels=batch), batch)
+
+
+# 24 bands per octave from short to long on either side of the few-items form; lengths with large prime factors (direct
+# sums and chirp-z); a band long enough for 1024 threads
+@pytest.mark.parametrize("batch", [1, 5, 9, 70])
+@pytest.mark.parametrize("kw", [dict(N=1 << 15, valid_len=30001, bins_per_octave=24, m_policy=wl.M_SMOOTH),
+                                dict(N=1 << 14, valid_len=1 << 14, bins_per_octave=6, m_policy=wl.M_MULT4),
+                                dict(N=1 << 15, valid_len=1 << 15, bins_per_octave=12, fmax=11025.0, m_policy=wl.M_POW2)],
+                         ids=lambda k: f"n{k['N']}_b{k['bins_per_octave']}_p{k['m_policy']}")
+def test_band_launch_forms(kw, batch):
+    check_rows(small_workload("forms", **{"fs": 44100.0, "fmin": 60.0, "fmax": 22050.0, "channels": batch, **kw}), batch)
