@@ -181,6 +181,7 @@ void free_device(cqt_plan *p) {
     cudaFree(p->d.tab_analysis_adj); cudaFree(p->d.tab_synthesis_adj);
     cudaFree(p->d.cover); cudaFree(p->d.dbg); cudaFree(p->d.zero_seg);
     for (auto &c : p->cls) cudaFree(c.d_items);
+    cudaFree(p->merged.d_items);
     for (auto &g : p->two_pass) cudaFree(g.d_recs);
     for (cudaEvent_t e : p->ev) cudaEventDestroy(e);
     for (int i = 0; i < cqt_plan::kHelpers; ++i) {
@@ -377,6 +378,13 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         }
         return bestA;
     };
+    // shared memory per item: padded buffer + two-level twiddle table (two buffers for generic radices,
+    // the length-L buffer and that plan's table for chirp-z)
+    auto band_elems = [&](int32_t b) -> int64_t {
+        const FftPlan &bf = p->ffts[(size_t)p->bands[(size_t)b].fft];
+        return bf.generic == 2 ? bf.blu_L + p->ffts[(size_t)bf.blu_fft].tw_count
+                               : (bf.generic ? 2 * (int64_t)bf.M + bf.st[0].radix : bf.M + 16 + bf.tw_count);
+    };
     for (int i : order) {
         const int64_t M = L.bands[i].M;
         int c = 0;
@@ -399,11 +407,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
                 bfz.blu_fft = fl;
                 bfz.generic = 2;
             }
-            // shared memory per item: padded buffer + two-level twiddle table (two buffers for generic radices,
-            // the length-L buffer and that plan's table for chirp-z)
-            const FftPlan &bf = p->ffts[p->bands[i].fft];
-            const int64_t elems = bf.generic == 2 ? bf.blu_L + p->ffts[bf.blu_fft].tw_count
-                                                  : (bf.generic ? 2 * M + bf.st[0].radix : M + 16 + bf.tw_count);
+            const int64_t elems = band_elems(i);
             if (elems > smem_cap_elems) {   // the cap is per work item; the classes with several items per CTA are far below it
                 A2 = split_two_pass(M);
                 if (!A2) { delete p; return CQT_ERR_UNSUPPORTED; }
@@ -412,7 +416,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
                 p->cls[c].work.push_back(i);
                 p->cls[c].max_elems = (int)std::max<int64_t>(p->cls[c].max_elems, elems);
                 p->cls[c].n_bands++;
-                if (bf.generic) p->cls[c].has_generic = true;
+                if (p->ffts[p->bands[i].fft].generic) p->cls[c].has_generic = true;
             }
         }
         if (!single) {
@@ -441,6 +445,29 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     }
     // a middle class whose longest band has at most one butterfly per thread at half the threads runs narrower CTAs
     if (p->cls[2].n_bands && L.bands[(size_t)p->cls[2].work[0]].M <= 2304) { p->cls[2].threads = 128; p->cls[2].min_blocks = 8; }
+    // the same bands for the one-launch form: about one radix-8 butterfly per thread and stage, so that an item's chain
+    // of dependent instructions is as short as its stages allow
+    {
+        MergedBands &mg = p->merged;
+        auto lg_threads = [&](int32_t b) {
+            const FftPlan &bf = p->ffts[(size_t)p->bands[(size_t)b].fft];
+            const int64_t points = bf.generic == 2 ? bf.blu_L : bf.M;
+            int lg = 5;
+            while (lg < 10 && (3ll << lg) < points / 4) ++lg;   // 1.5 * threads < points / 8
+            return lg;
+        };
+        for (int c = kNumClasses - 1; c >= 1; --c) {
+            mg.work.insert(mg.work.end(), p->cls[c].work.begin(), p->cls[c].work.end());
+            mg.has_generic = mg.has_generic || p->cls[c].has_generic;
+        }
+        std::stable_sort(mg.work.begin(), mg.work.end(), [&](int32_t x, int32_t y) { return lg_threads(x) > lg_threads(y); });
+        for (size_t i = 0; i < mg.work.size(); ++i) {
+            const int lg = lg_threads(mg.work[i]);
+            if (mg.segs.empty() || mg.segs.back().lg_nthr != lg) mg.segs.push_back({(int)i, 0, lg, 0});
+            mg.segs.back().n_bands++;
+            mg.segs.back().elems = std::max(mg.segs.back().elems, (int)band_elems(mg.work[i]));
+        }
+    }
     // estimates for the per-call assignment of classes to streams (band.cu): total work, and the time one CTA
     // needs for the longest item (microseconds per element by class, from measured kernel times)
     {
@@ -499,16 +526,18 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     p->n_zero_seg = (int)zero_seg.size();
     if (p->n_zero_seg) chk(upload(p->d.zero_seg, zero_seg));
     chk(upload(p->d.dbg, std::vector<int>(8, 0)));
-    for (auto &c : p->cls) {
+    auto upload_items = [&](BandItem *&dst, const std::vector<int32_t> &work) {
         // record and radix plan of every band of the class, in launch order: what a work item fetches first
-        std::vector<BandItem> items(c.work.size());
+        std::vector<BandItem> items(work.size());
         for (size_t i = 0; i < items.size(); ++i) {
-            const int b = c.work[i];
+            const int b = work[i];
             items[i].br = p->bands[(size_t)b];
             items[i].fp = p->ffts[(size_t)p->bands[(size_t)b].fft];
         }
-        chk(upload(c.d_items, items));
-    }
+        chk(upload(dst, items));
+    };
+    for (auto &c : p->cls) upload_items(c.d_items, c.work);
+    upload_items(p->merged.d_items, p->merged.work);
     cudaDeviceProp prop;
     chk(cudaGetDeviceProperties(&prop, p->device));
     p->sm_count = prop.multiProcessorCount;

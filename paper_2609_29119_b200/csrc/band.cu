@@ -55,6 +55,98 @@ static cudaError_t launch_class(const cqt_plan &p, int cls, const char *name, Ba
     return e;
 }
 
+const void *band_analysis_merged_kernel(bool generic);    // band_analysis.cu
+const void *band_synthesis_merged_kernel(bool generic);   // band_synthesis.cu
+
+// Shape of the few-items form for a batch: the bands longer than class 0's in one launch (two when some of them take
+// 1024 threads each: those then do not set the CTA size of the others), class 0 in one.
+struct FewLaunch {
+    struct Part {
+        BandSegments sg{};
+        int threads = 0, grid = 0;
+        size_t smem = 0;
+    };
+    Part part[2];
+    int short_threads = 0, short_grid = 0;
+};
+
+// Segments [first, last) in CTAs filled to 1 / share; returns the SMs the launch occupies, and whether CTAs hold more
+// than one item.
+static long long few_part(const cqt_plan &p, int64_t batch, int first, int last, int share, FewLaunch::Part &t, bool &spread) {
+    t = FewLaunch::Part{};
+    if (first == last) return 0;
+    const MergedBands &mg = p.merged;
+    t.threads = std::max(128, 1 << mg.segs[first].lg_nthr);
+    t.sg.n = last - first;
+    long long grid = 0;
+    for (int i = first; i < last; ++i) {
+        const MergedBands::Segment &s = mg.segs[i];
+        const int full = std::min(t.threads >> s.lg_nthr, kMaxGroups), per = std::max(1, full / share);
+        spread = spread || per > 1;
+        t.sg.s[i - first] = BandSegment{(int)grid, s.first_band, s.n_bands, s.lg_nthr, per, s.elems};
+        t.smem = std::max(t.smem, (size_t)per * s.elems * sizeof(float2));
+        grid += ((long long)s.n_bands * batch + per - 1) / per;
+        if (grid > (1 << 20)) return grid;
+    }
+    t.grid = (int)grid;
+    const long long cta_smem = (long long)t.smem + kMaxGroups * (long long)sizeof(BandItem) + 1024;
+    const long long per_sm = std::min<long long>(1024 / t.threads, (p.max_smem_optin + 1024) / cta_smem);
+    return per_sm > 0 ? (grid + per_sm - 1) / per_sm : 1 << 20;
+}
+
+// The few-items form is taken where every CTA of the longer bands is resident at once.  A call that small is a chain of
+// latencies, and side by side on streams each class adds a launch, an event and two cross-stream waits to it.
+static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
+    const int n = (int)p.merged.segs.size();
+    const int split = n && p.merged.segs[0].lg_nthr == 10 ? 1 : 0;
+    if (n - split > kMaxSegments) return false;
+    for (int share = 1;; share *= 2) {   // emptier CTAs while there are SMs to spread over
+        FewLaunch t;
+        bool spread = false;
+        long long sms = few_part(p, batch, 0, split, share, t.part[0], spread);
+        sms += few_part(p, batch, split, n, share, t.part[1], spread);
+        if (sms > p.sm_count) {
+            if (share == 1) return false;
+            break;
+        }
+        f = t;
+        if (!spread) break;
+    }
+    const long long items = (long long)p.cls[0].n_bands * batch;
+    if (items > 16ll * p.sm_count) return false;
+    f.short_threads = items > 4ll * p.sm_count ? 256 : 64;
+    f.short_grid = (int)((items * 32 + f.short_threads - 1) / f.short_threads);
+    return true;
+}
+
+template <bool ANALYSIS>
+static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cudaStream_t st) {
+    static const char *names[2][3] = {{"bands_to_spectrum/1024_threads", "bands_to_spectrum/merged", "bands_to_spectrum/class0"},
+                                      {"bands_from_spectrum/1024_threads", "bands_from_spectrum/merged", "bands_from_spectrum/class0"}};
+    cudaError_t e = cudaSuccess;
+    const int launches = (f.part[0].grid > 0) + (f.part[1].grid > 0) + (f.short_grid > 0);
+    a.chain = launches > 1 ? kChainHead : kAlone;
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+        FewLaunch::Part &t = f.part[i];
+        if (!t.grid) continue;
+        a.items = p.merged.d_items;
+        void *args[] = {&a, &t.sg};
+        const void *fn = ANALYSIS ? band_analysis_merged_kernel(p.merged.has_generic) : band_synthesis_merged_kernel(p.merged.has_generic);
+        e = launch_kernel(fn, dim3((unsigned)t.grid), dim3((unsigned)t.threads), args, t.smem, st);
+        note_launch(p, names[ANALYSIS][i], st);
+        a.chain = kChainMember;
+    }
+    if (f.short_grid && e == cudaSuccess) {
+        const BandClass &c = p.cls[0];
+        a.items = c.d_items;
+        void *args[] = {&a};
+        e = launch_kernel(class_kernel<ANALYSIS>(c, 32), dim3((unsigned)f.short_grid), dim3((unsigned)f.short_threads), args,
+                          (size_t)c.max_elems * (f.short_threads / 32) * sizeof(float2), st);
+        note_launch(p, names[ANALYSIS][2], st);
+    }
+    return e;
+}
+
 // The classes of one call are independent (disjoint outputs), and most of them alone leave SMs idle, so they run
 // side by side on the caller's stream and the plan's helper streams (one stream per class when all five classes
 // have bands): fork after the caller's stream, join back into it.
@@ -108,10 +200,20 @@ struct ForkJoin {
     }
 };
 
+static bool has_two_pass(const cqt_plan &p) { return !p.two_pass[0].bands.empty() || !p.two_pass[1].bands.empty(); }
+
 cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, float2 *c,
                                        float2 *scratch, int64_t batch, cudaStream_t st) {
+    FewLaunch f;
+    if (!has_two_pass(p) && few_shape(p, batch, f)) {
+        BandArgs a = make_args(p, p.cls[0], table, batch);
+        a.spec = X;
+        a.spec_pitch = p.lf.x_pitch;
+        a.coef = c;
+        return launch_few<true>(p, a, f, st);
+    }
     ForkJoin fj(p, st, batch);
-    if (!p.two_pass[0].bands.empty() || !p.two_pass[1].bands.empty()) {
+    if (has_two_pass(p)) {
         cudaError_t e = launch_two_pass_from_spectrum(p, table, X, c, scratch, batch, fj.two_pass_stream());
         if (e != cudaSuccess) { fj.join(); return e; }
     }
@@ -145,8 +247,16 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
+    FewLaunch f;
+    if (!has_two_pass(p) && few_shape(p, batch, f)) {
+        BandArgs a = make_args(p, p.cls[0], table, batch);
+        a.coef = const_cast<float2 *>(c);
+        a.Y = Y;
+        a.fold = fold_sidebands ? 1 : 0;
+        return launch_few<false>(p, a, f, st);
+    }
     ForkJoin fj(p, st, batch);
-    if (!p.two_pass[0].bands.empty() || !p.two_pass[1].bands.empty()) {
+    if (has_two_pass(p)) {
         cudaError_t e = launch_two_pass_to_spectrum(p, table, fold_sidebands, c, Y, scratch, batch, fj.two_pass_stream());
         if (e != cudaSuccess) { fj.join(); return e; }
     }
@@ -166,6 +276,10 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
 }
 
 cudaError_t configure_band_kernels(const cqt_plan &p) {
+    for (const void *fn : {band_analysis_merged_kernel(p.merged.has_generic), band_synthesis_merged_kernel(p.merged.has_generic)}) {
+        cudaError_t e = allow_dynamic_smem(fn, 0, p);
+        if (e != cudaSuccess) return e;
+    }
     for (int i = 0; i < kNumClasses; ++i) {
         if (p.cls[i].n_bands == 0) continue;
         for (int lanes : {p.cls[i].lanes_few, p.cls[i].lanes_many}) {

@@ -3,21 +3,11 @@
 
 namespace cqt {
 
-template <int THREADS, int MINB, int LANES, int MAXR, bool GEN>
-__global__ void __launch_bounds__(THREADS, MINB) bands_from_spectrum_kernel(BandArgs a) {
-    pdl_launch_dependents();
-    using G = Group<LANES>;
-    using Sync = GroupSync<LANES>;
-    const int item = G::item();
-    if (item >= a.n_work * a.batch) return;   // whole group exits together
-    const int tid = G::tid(), nthr = G::nthr();
-    __shared__ BandItem item_s[LANES ? THREADS / (LANES ? LANES : 1) : 1];
-    BandItem &it = item_s[G::slot()];
-    fetch_item<Sync>(a.items[item / a.batch], it, tid, nthr);   // records in launch order of the class
+// One work item (band record and radix plan `it`, signal ch) on nthr threads with `buf` as their shared memory.
+template <class Sync, int MAXR, bool GEN>
+__device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem &it, int ch, float2 *buf, int tid, int nthr) {
     const BandRec br = it.br;
-    const int ch = item % a.batch;
     const FftPlan &fp = it.fp;
-    float2 *buf = smem_band + (size_t)G::slot() * a.max_elems;
     const float2 *X = a.spec + (long long)ch * a.spec_pitch;
     const float *tab = a.table + br.tab_off;
     const int M = br.M, half = a.N >> 1;
@@ -41,7 +31,7 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_from_spectrum_kernel(Band
     float2 *out = a.coef + (long long)ch * a.coeff_count + br.coeff_off;
     // GEN: the class holds lengths with prime factors above 5 (only the multiple-of-4 length policy makes them);
     // the other instantiations leave the chirp-z and direct-sum code out
-    if (GEN && fp.generic) pdl_wait();
+    if (GEN && fp.generic) chain_begin(a);
     if (GEN && fp.generic == 2) {
         auto store_c = [&](int n, int, float2 v) { out[n] = v; };
         chirp_z_transform<+1, Sync>(buf, fp, a.ffts, a.tw, load, store_c, a.dbg, tid, nthr);
@@ -50,14 +40,14 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_from_spectrum_kernel(Band
     if (GEN && fp.generic) {
         float2 *alt = buf + M;
         for (int m = tid; m < M; m += nthr) buf[m] = load(m, 0);
-        Sync::sync();
+        Sync::sync(nthr);
         fft_dif<+1, Sync, false>(buf, alt, 1, 1, 0u, fp, a.tw, tid, nthr);
         for (int n = tid; n < M; n += nthr) out[n] = buf[dif_pos(fp, n)];
         return;
     }
     float2 *tws = buf + M + 16;
     if (fp.nstages > 1) stage_twiddles(tws, a.tw, fp, tid, nthr);
-    pdl_wait();   // record, plan and twiddle table belong to the plan; what follows touches the predecessor's output
+    chain_begin(a);   // record, plan and twiddle table belong to the plan; what follows touches the predecessor's output
     const Tile t{buf, 1, 1, 0u, M + 16, a.dbg};
     // coefficients are written once and not read again by this call: streaming stores keep the L2 for the spectrum
     auto store = [&](int n, int, float2 v) { if (CQT_CHK(a.dbg, 303, n, M)) __stcs(out + n, v); };
@@ -78,6 +68,39 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_from_spectrum_kernel(Band
         return;
     }
     fft_fused<+1, Sync, false, true, false, true, false, false, MAXR>(t, fp, tws, load, store, tid, nthr);
+}
+
+// One class: groups of LANES lanes (or the whole CTA) per item.
+template <int THREADS, int MINB, int LANES, int MAXR, bool GEN>
+__global__ void __launch_bounds__(THREADS, MINB) bands_from_spectrum_kernel(BandArgs a) {
+    chain_enter(a);
+    using G = Group<LANES>;
+    using Sync = GroupSync<LANES>;
+    const int item = G::item();
+    if (item >= a.n_work * a.batch) return;   // whole group exits together
+    const int tid = G::tid(), nthr = G::nthr();
+    __shared__ BandItem item_s[LANES ? THREADS / (LANES ? LANES : 1) : 1];
+    BandItem &it = item_s[G::slot()];
+    fetch_item<Sync>(a.items[item / a.batch], it, tid, nthr);   // records in launch order of the class
+    analysis_item<Sync, MAXR, GEN>(a, it, item % a.batch, smem_band + (size_t)G::slot() * a.max_elems, tid, nthr);
+    chain_end(a);
+}
+
+// Every band of 128 < M that fits a CTA in one launch (see BandSegments).
+template <bool GEN>
+__global__ void __launch_bounds__(1024, 1) all_bands_from_spectrum_kernel(BandArgs a, BandSegments sg) {
+    chain_enter(a);
+    MergedItem m;
+    if (!merged_item(a, sg, m)) return;
+    __shared__ BandItem item_s[kMaxGroups];
+    BandItem &it = item_s[m.slot];
+    fetch_item<NamedSync>(a.items[m.band], it, m.tid, m.nthr);
+    analysis_item<NamedSync, 16, GEN>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
+    chain_end(a);
+}
+
+const void *band_analysis_merged_kernel(bool generic) {
+    return generic ? (const void *)all_bands_from_spectrum_kernel<true> : (const void *)all_bands_from_spectrum_kernel<false>;
 }
 
 const void *band_analysis_kernel(const BandClass &c, int lanes) {

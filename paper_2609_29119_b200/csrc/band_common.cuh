@@ -32,8 +32,58 @@ struct BandArgs {
     float2 *Y;               // synthesis form: weighted-bin rows
     long long y_pitch;
     long long table_len;
+    int chain;               // kAlone, kChainHead, kChainMember
     int *dbg;
 };
+
+// Band kernels of one call write disjoint outputs and need nothing of one another, only the kernel before the first
+// of them.  In a chain on one stream the head lets its successor start only once all of its own CTAs have seen that
+// kernel finish, so a member needs no wait before it reads; it waits for its predecessor at its end instead, so that
+// "the last member has finished" means all have.  No event and no second stream is involved.
+enum { kAlone = 0, kChainHead = 1, kChainMember = 2 };
+__device__ __forceinline__ void chain_enter(const BandArgs &a) {
+    if (a.chain != kChainHead) pdl_launch_dependents();
+}
+__device__ __forceinline__ void chain_begin(const BandArgs &a) {
+    if (a.chain != kChainMember) pdl_wait();
+    if (a.chain == kChainHead) pdl_launch_dependents();
+}
+__device__ __forceinline__ void chain_end(const BandArgs &a) {
+    if (a.chain == kChainMember) pdl_wait();
+}
+
+// One launch for all bands of a call with few work items (band.cu decides).  The bands are ordered by the number of
+// threads an item of theirs gets, a power of two; a segment is a run of bands with the same number, walked by CTAs
+// cta0 .. of the grid with per_cta items each (fewer than blockDim / nthr when there are SMs to spread over: the
+// remaining threads exit).
+constexpr int kMaxSegments = 6;    // 32 ... 1024 threads per item
+constexpr int kMaxGroups = 16;     // items per CTA (one named barrier each)
+struct BandSegment {
+    int cta0, first_band, n_work, lg_nthr, per_cta, elems;   // elems: shared-memory elements of one item
+};
+struct BandSegments {
+    int n;
+    BandSegment s[kMaxSegments];
+};
+struct MergedItem {
+    int band, ch, slot, tid, nthr, smem_off;
+};
+__device__ __forceinline__ bool merged_item(const BandArgs &a, const BandSegments &sg, MergedItem &m) {
+    BandSegment s = sg.s[0];
+#pragma unroll
+    for (int i = 1; i < kMaxSegments; ++i)
+        if (i < sg.n && (int)blockIdx.x >= sg.s[i].cta0) s = sg.s[i];
+    m.slot = (int)threadIdx.x >> s.lg_nthr;
+    const int item = ((int)blockIdx.x - s.cta0) * s.per_cta + m.slot;
+    if (m.slot >= s.per_cta || item >= s.n_work * a.batch) return false;   // whole groups leave together
+    m.nthr = 1 << s.lg_nthr;
+    m.tid = (int)threadIdx.x & (m.nthr - 1);
+    const int b = item / a.batch;
+    m.band = s.first_band + b;
+    m.ch = item - b * a.batch;
+    m.smem_off = m.slot * s.elems;
+    return true;
+}
 
 // THREADS / MINB: launch bounds of the class (64 registers per thread when THREADS * MINB = 1024 ... 2048)
 // LANES: 0 = the whole CTA works on one item; 32, 16, 8 = that many consecutive lanes per item (THREADS / LANES items
@@ -59,7 +109,7 @@ template <class Sync>
 __device__ __forceinline__ void fetch_item(const BandItem &g, BandItem &s, int tid, int nthr) {
     constexpr int kWords = (int)(sizeof(BandItem) / sizeof(int));
     for (int i = tid; i < kWords; i += nthr) reinterpret_cast<int *>(&s)[i] = __ldg(reinterpret_cast<const int *>(&g) + i);
-    Sync::sync();
+    Sync::sync(nthr);
 }
 
 // Chirp-z (Bluestein) evaluation of an M-point DFT of sign SIGN whose length has a large prime factor:
@@ -89,7 +139,7 @@ __device__ __forceinline__ void chirp_z_transform(float2 *buf, const FftPlan &fp
         if (SIGN > 0) f.y = -f.y;
         buf[p] = cmul(buf[p], f);
     }
-    Sync::sync();
+    Sync::sync(nthr);
     fft_dit_inverse<Sync>(tl, fl, twl, tid, nthr);
     for (int k = tid; k < M; k += nthr) {
         float2 w = __ldg(chirp + k);

@@ -24,21 +24,11 @@ struct RegularStore {
     }
 };
 
-template <int THREADS, int MINB, int LANES, int MAXR, bool GEN>
-__global__ void __launch_bounds__(THREADS, MINB) bands_to_spectrum_kernel(BandArgs a) {
-    pdl_launch_dependents();
-    using G = Group<LANES>;
-    using Sync = GroupSync<LANES>;
-    const int item = G::item();
-    if (item >= a.n_work * a.batch) return;
-    const int tid = G::tid(), nthr = G::nthr();
-    __shared__ BandItem item_s[LANES ? THREADS / (LANES ? LANES : 1) : 1];
-    BandItem &it = item_s[G::slot()];
-    fetch_item<Sync>(a.items[item / a.batch], it, tid, nthr);   // records in launch order of the class
+// One work item (band record and radix plan `it`, signal ch) on nthr threads with `buf` as their shared memory.
+template <class Sync, int MAXR, bool GEN>
+__device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem &it, int ch, float2 *buf, int tid, int nthr) {
     const BandRec br = it.br;
-    const int ch = item % a.batch;
     const FftPlan &fp = it.fp;
-    float2 *buf = smem_band + (size_t)G::slot() * a.max_elems;
     const int M = br.M;
     const float2 *in = a.coef + (long long)ch * a.coeff_count + br.coeff_off;
     // adjoint of analysis, sidebands: U[m] + conj U[-m] is the DFT of 2 Re c
@@ -67,7 +57,7 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_to_spectrum_kernel(BandAr
     };
     // GEN: the class holds lengths with prime factors above 5 (only the multiple-of-4 length policy makes them);
     // the other instantiations leave the chirp-z and direct-sum code out
-    if (GEN && fp.generic) pdl_wait();
+    if (GEN && fp.generic) chain_begin(a);
     if (GEN && fp.generic == 2) {
         chirp_z_transform<-1, Sync>(buf, fp, a.ffts, a.tw, load, store, a.dbg, tid, nthr);
         return;
@@ -75,14 +65,14 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_to_spectrum_kernel(BandAr
     if (GEN && fp.generic) {
         float2 *alt = buf + M;
         for (int n = tid; n < M; n += nthr) buf[n] = load(n, 0);
-        Sync::sync();
+        Sync::sync(nthr);
         fft_dif<-1, Sync, false>(buf, alt, 1, 1, 0u, fp, a.tw, tid, nthr);
         for (int m = tid; m < M; m += nthr) store(m, 0, buf[dif_pos(fp, m)]);
         return;
     }
     float2 *tws = buf + M + 16;
     if (fp.nstages > 1) stage_twiddles(tws, a.tw, fp, tid, nthr);
-    pdl_wait();   // record, plan and twiddle table belong to the plan; what follows touches the predecessor's output
+    chain_begin(a);   // record, plan and twiddle table belong to the plan; what follows touches the predecessor's output
     const Tile t{buf, 1, 1, 0u, M + 16, a.dbg};
     if (br.side == 0) {
         // regular band: all bins in range, plane row and table share the support index j = d - d0
@@ -95,6 +85,39 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_to_spectrum_kernel(BandAr
         return;
     }
     fft_fused<-1, Sync, false, true, false, true, false, false, MAXR>(t, fp, tws, load, store, tid, nthr);
+}
+
+// One class: groups of LANES lanes (or the whole CTA) per item.
+template <int THREADS, int MINB, int LANES, int MAXR, bool GEN>
+__global__ void __launch_bounds__(THREADS, MINB) bands_to_spectrum_kernel(BandArgs a) {
+    chain_enter(a);
+    using G = Group<LANES>;
+    using Sync = GroupSync<LANES>;
+    const int item = G::item();
+    if (item >= a.n_work * a.batch) return;   // whole group exits together
+    const int tid = G::tid(), nthr = G::nthr();
+    __shared__ BandItem item_s[LANES ? THREADS / (LANES ? LANES : 1) : 1];
+    BandItem &it = item_s[G::slot()];
+    fetch_item<Sync>(a.items[item / a.batch], it, tid, nthr);   // records in launch order of the class
+    synthesis_item<Sync, MAXR, GEN>(a, it, item % a.batch, smem_band + (size_t)G::slot() * a.max_elems, tid, nthr);
+    chain_end(a);
+}
+
+// Every band of 128 < M that fits a CTA in one launch (see BandSegments).
+template <bool GEN>
+__global__ void __launch_bounds__(1024, 1) all_bands_to_spectrum_kernel(BandArgs a, BandSegments sg) {
+    chain_enter(a);
+    MergedItem m;
+    if (!merged_item(a, sg, m)) return;
+    __shared__ BandItem item_s[kMaxGroups];
+    BandItem &it = item_s[m.slot];
+    fetch_item<NamedSync>(a.items[m.band], it, m.tid, m.nthr);
+    synthesis_item<NamedSync, 16, GEN>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
+    chain_end(a);
+}
+
+const void *band_synthesis_merged_kernel(bool generic) {
+    return generic ? (const void *)all_bands_to_spectrum_kernel<true> : (const void *)all_bands_to_spectrum_kernel<false>;
 }
 
 const void *band_synthesis_kernel(const BandClass &c, int lanes) {

@@ -20,17 +20,26 @@ namespace cqt {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// sync(nthr): barrier of the nthr threads that work on one item
 struct BlockSync {
-    static __device__ __forceinline__ void sync() { __syncthreads(); }
+    static __device__ __forceinline__ void sync(int) { __syncthreads(); }
 };
 struct WarpSync {
-    static __device__ __forceinline__ void sync() { __syncwarp(); }
+    static __device__ __forceinline__ void sync(int) { __syncwarp(); }
+};
+// nthr consecutive threads of the CTA, a power of two >= 32 known at run time: a named barrier per group (at most 16
+// groups of 64 or more threads), the warp barrier for groups of one warp.  A CTA is all groups of one size.
+struct NamedSync {
+    static __device__ __forceinline__ void sync(int nthr) {
+        if (nthr == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(threadIdx.x >> (31 - __clz(nthr))), "r"(nthr) : "memory");
+    }
 };
 // LANES consecutive lanes of a warp (a power of two below 32) working on one item: the groups of a warp may be in
 // different places of the code (items with different radix plans), so each synchronises with its own lane mask
 template <int LANES>
 struct LaneGroupSync {
-    static __device__ __forceinline__ void sync() {
+    static __device__ __forceinline__ void sync(int) {
         __syncwarp(((1u << LANES) - 1u) << ((threadIdx.x & 31u) & ~(unsigned)(LANES - 1)));
     }
 };
@@ -118,7 +127,7 @@ __device__ void dif_stage_generic(float2 *buf, float2 *alt, float2 *wp, int pitc
         if (SIGN > 0) t.y = -t.y;
         wp[x] = t;
     }
-    Sync::sync();
+    Sync::sync(nthr);
     for (int w = tid; w < M * ncols; w += nthr) {
         const int e = w / ncols, col = w - e * ncols;
         const int kq = e / s, np = e - kq * s;
@@ -138,7 +147,7 @@ __device__ void dif_stage_generic(float2 *buf, float2 *alt, float2 *wp, int pitc
         if (SIGN > 0) t.y = -t.y;
         alt[(size_t)e * pitch + col] = cmul(make_float2(ax, ay), t);
     }
-    Sync::sync();
+    Sync::sync(nthr);
     for (int w = tid; w < M * ncols; w += nthr) {
         const int e = w / ncols, col = w - e * ncols;
         buf[(size_t)e * pitch + col] = alt[(size_t)e * pitch + col];
@@ -177,7 +186,7 @@ __device__ void fft_dif(float2 *buf, float2 *alt, int pitch, int ncols, uint32_t
             }
         }
 #undef CQT_STAGE
-        Sync::sync();
+        Sync::sync(nthr);
         n_cur = s;
         tmul *= r;
     }
@@ -312,7 +321,7 @@ __device__ __forceinline__ void first_stage(const Tile &t, const FftPlan &fp, co
             }
             if (SIGN < 0) Codelet<R>::run(re, im); else Codelet<R>::run(im, re);
         }
-        if (base == 0) Sync::sync();
+        if (base == 0) Sync::sync(nthr);
         if (active) {
             if (DIRECT) apply_twiddle_direct<R, SIGN>(tw, b, re, im);
             else apply_twiddle_powers<R, SIGN>(tw, logC, b, re, im);
@@ -514,7 +523,7 @@ __device__ void fft_dit_inverse(const Tile &t, const FftPlan &fp, const float2 *
             case 16: dit_stage<16>(t, fp, tw, j, n_cur, tmul, tid, nthr); break;
             default: break;
         }
-        Sync::sync();
+        Sync::sync(nthr);
     }
 }
 
@@ -532,7 +541,7 @@ template <int SIGN, class Sync, bool POW2, bool PAD, bool COLFAST_IN, bool REV, 
 __device__ __forceinline__ void fft_fused(const Tile &t, const FftPlan &fp, const float2 *tw, Load load, Store store, int tid, int nthr) {
     const int d = fp.nstages;
     if (d == 1) {
-        Sync::sync();   // tables staged by the caller become visible to the functors
+        Sync::sync(nthr);   // tables staged by the caller become visible to the functors
 #define X(RR) case RR: if constexpr (POW2 || RR <= MAXR) only_stage<RR, SIGN>(t, load, store, tid, nthr); break;
         if (POW2) { switch (fp.st[0].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
         else { switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
@@ -543,7 +552,7 @@ __device__ __forceinline__ void fft_fused(const Tile &t, const FftPlan &fp, cons
     if (POW2) { switch (fp.st[0].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
     else { switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
 #undef X
-    Sync::sync();
+    Sync::sync(nthr);
     int n_cur = fp.st[0].stride, tmul = fp.st[0].radix;
 #pragma unroll 1
     for (int j = 1; j < d - 1; ++j) {
@@ -551,7 +560,7 @@ __device__ __forceinline__ void fft_fused(const Tile &t, const FftPlan &fp, cons
         if (POW2) { switch (fp.st[j].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
         else { switch (fp.st[j].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
 #undef X
-        Sync::sync();
+        Sync::sync(nthr);
         n_cur = fp.st[j].stride;
         tmul *= fp.st[j].radix;
     }
@@ -572,14 +581,14 @@ __device__ __forceinline__ void fft_fused_keep(const Tile &t, const FftPlan &fp,
         if (POW2) { switch (fp.st[0].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
         else { switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
 #undef X
-        Sync::sync();
+        Sync::sync(nthr);
         return;
     }
 #define X(RR) case RR: first_stage<RR, SIGN, false, COLFAST_IN, DIRECT, Sync>(t, fp, tw, load, tid, nthr); break;
     if (POW2) { switch (fp.st[0].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
     else { switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
 #undef X
-    Sync::sync();
+    Sync::sync(nthr);
     int n_cur = fp.st[0].stride, tmul = fp.st[0].radix;
 #pragma unroll 1
     for (int j = 1; j < d; ++j) {
@@ -587,7 +596,7 @@ __device__ __forceinline__ void fft_fused_keep(const Tile &t, const FftPlan &fp,
         if (POW2) { switch (fp.st[j].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
         else { switch (fp.st[j].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
 #undef X
-        Sync::sync();
+        Sync::sync(nthr);
         n_cur = fp.st[j].stride;
         tmul *= fp.st[j].radix;
     }

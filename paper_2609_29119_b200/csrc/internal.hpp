@@ -28,6 +28,16 @@ struct BandClass {
     std::vector<int32_t> work;
 };
 
+// The single-CTA bands longer than class 0's ordered for one launch of all of them (calls with few work items): bands of one
+// segment get the same number of threads per item, a power of two.
+struct MergedBands {
+    struct Segment { int first_band, n_bands, lg_nthr, elems; };   // elems: shared-memory elements (float2) of one item
+    std::vector<Segment> segs;       // most threads first
+    std::vector<int32_t> work;       // band indices in launch order
+    BandItem *d_items = nullptr;
+    bool has_generic = false;
+};
+
 struct LongFft {
     int64_t Lp = 0, A = 1, B = 0;
     int fft_A = -1, fft_B = -1;   // FftPlan indices
@@ -77,6 +87,7 @@ struct cqt_plan {
     int n_zero_seg = 0;                // zero-fill segments (layouts with nested supports only)
     cqt::LongFft lf;
     cqt::BandClass cls[cqt::kNumClasses];
+    cqt::MergedBands merged;
     cqt::TwoPassGroup two_pass[2];     // [0]: both factors <= 256, [1]: larger factors
     int64_t two_pass_pitch = 0;        // scratch elements per signal for the two-pass bands
     cqt::DevicePlan d;
