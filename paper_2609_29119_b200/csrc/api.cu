@@ -133,33 +133,24 @@ void host_fft_pow2(std::vector<std::complex<double>> &v) {   // in-place radix-2
     }
 }
 
-int64_t host_dif_pos(const FftPlan &fp, int64_t k) {
-    int64_t pos = 0, rem = k;
-    for (int j = 0; j < fp.nstages; ++j) { pos = pos * fp.st[j].radix + rem % fp.st[j].radix; rem /= fp.st[j].radix; }
-    return pos;
-}
-
-// chirp exp(-i pi n^2 / M) and the filter spectrum DFT_L(conj chirp, wrapped) / L in the DIF output order of `fl`
-void make_chirp_tables(int64_t M, const FftPlan &fl, std::vector<float2> &tw, FftPlan &fp) {
-    const int64_t L = fl.M;
-    fp.blu_L = (int32_t)L;
-    fp.blu_chirp_off = (int32_t)tw.size();
-    std::vector<std::complex<double>> b(L, 0.0);
-    for (int64_t n = 0; n < M; ++n) {
-        const double ang = -kPi * (double)((n * n) % (2 * M)) / (double)M;
-        tw.push_back(make_float2((float)std::cos(ang), (float)std::sin(ang)));
-        const std::complex<double> c = std::polar(1.0, -ang);   // conj chirp
-        b[n] = c;
-        if (n) b[L - n] = c;
+// tables of a band on the chirp-z kernel (see ChirpRec): sub-transforms of m points, convolution length L
+void make_chirp_tables(int64_t m, int64_t L, std::vector<float2> &tw, ChirpRec &cr) {
+    cr.pre_off = (int32_t)tw.size();
+    for (int64_t k0 = 0; k0 < 4; ++k0)
+        for (int64_t n = 0; n < m; ++n) {
+            // n k0 / (2 m) + n^2 / m in units of 1 / (2 m), periodic with 4 m
+            const double ang = -kPi * (double)((n * k0 + 2 * n * n) % (4 * m)) / (double)(2 * m);
+            tw.push_back(make_float2((float)std::cos(ang), (float)std::sin(ang)));
+        }
+    std::vector<std::complex<double>> b((size_t)L, 0.0);
+    for (int64_t n = 0; n < m; ++n) {
+        const std::complex<double> c = std::polar(1.0, kPi * (double)((n * n) % (2 * m)) / (double)m);   // conj chirp
+        b[(size_t)n] = c;
+        if (n) b[(size_t)(L - n)] = c;
     }
     host_fft_pow2(b);
-    fp.blu_filter_off = (int32_t)tw.size();
-    std::vector<float2> perm(L);
-    for (int64_t k = 0; k < L; ++k) {
-        const std::complex<double> v = b[k] / (double)L;
-        perm[host_dif_pos(fl, k)] = make_float2((float)v.real(), (float)v.imag());
-    }
-    tw.insert(tw.end(), perm.begin(), perm.end());
+    cr.filter_off = (int32_t)tw.size();
+    for (const std::complex<double> &v : b) tw.push_back(make_float2((float)(v.real() / (double)L), (float)(v.imag() / (double)L)));
 }
 
 template <class T>
@@ -182,6 +173,7 @@ void free_device(cqt_plan *p) {
     cudaFree(p->d.cover); cudaFree(p->d.dbg); cudaFree(p->d.zero_seg);
     for (auto &c : p->cls) cudaFree(c.d_items);
     cudaFree(p->merged.d_items);
+    cudaFree(p->chirp.d_recs);
     for (auto &g : p->two_pass) cudaFree(g.d_recs);
     for (cudaEvent_t e : p->ev) cudaEventDestroy(e);
     for (int i = 0; i < cqt_plan::kHelpers; ++i) {
@@ -378,13 +370,18 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         }
         return bestA;
     };
-    // shared memory per item: padded buffer + two-level twiddle table (two buffers for generic radices,
-    // the length-L buffer and that plan's table for chirp-z)
+    // shared memory per item: padded buffer + two-level twiddle table (two buffers for a direct-sum stage)
     auto band_elems = [&](int32_t b) -> int64_t {
         const FftPlan &bf = p->ffts[(size_t)p->bands[(size_t)b].fft];
-        return bf.generic == 2 ? bf.blu_L + p->ffts[(size_t)bf.blu_fft].tw_count
-                               : (bf.generic ? 2 * (int64_t)bf.M + bf.st[0].radix : bf.M + 16 + bf.tw_count);
+        return bf.generic ? 2 * (int64_t)bf.M + bf.st[0].radix : bf.M + 16 + bf.tw_count;
     };
+    auto smooth = [](int64_t m) {
+        for (int f : {2, 3, 5})
+            while (m % f == 0) m /= f;
+        return m == 1;
+    };
+    p->band_class.assign(L.bands.size(), -1);
+    std::vector<int> chirp_bands[kChirpLengths];
     for (int i : order) {
         const int64_t M = L.bands[i].M;
         int c = 0;
@@ -392,21 +389,17 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         bool single = M <= two_pass_min;
         int64_t A2 = 0;
         if (!single) { A2 = split_two_pass(M); single = A2 == 0; }
+        p->band_class[(size_t)i] = (int8_t)c;
+        if (c > 0 && !smooth(M)) {
+            const int li = M % 4 == 0 ? chirp_length_index(M / 4) : -1;
+            if (li < 0) { delete p; return CQT_ERR_UNSUPPORTED; }
+            chirp_bands[li].push_back(i);
+            continue;
+        }
         if (single) {
             // short bands: fewer registers, more CTAs per SM
             p->bands[i].fft = plan_for(M, kPlanBand, p->cls[c].max_radix);
             if (p->bands[i].fft < 0) { delete p; return CQT_ERR_UNSUPPORTED; }
-            // a length with a large prime factor is evaluated as a chirp-z transform (two power-of-two transforms
-            // of length L >= 2M - 1 in shared memory) instead of direct sums
-            if (p->ffts[p->bands[i].fft].generic == 1 && p->ffts[p->bands[i].fft].st[0].radix >= 32 && M <= 8192) {
-                int64_t Lz = 64;
-                while (Lz < 2 * M - 1) Lz *= 2;
-                const int fl = plan_for(Lz, kPlanPow2, 16);
-                FftPlan &bfz = p->ffts[p->bands[i].fft];
-                make_chirp_tables(M, p->ffts[fl], tw, bfz);
-                bfz.blu_fft = fl;
-                bfz.generic = 2;
-            }
             const int64_t elems = band_elems(i);
             if (elems > smem_cap_elems) {   // the cap is per work item; the classes with several items per CTA are far below it
                 A2 = split_two_pass(M);
@@ -420,6 +413,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
             }
         }
         if (!single) {
+            p->band_class[(size_t)i] = -1;
             TwoPassBand tb{};
             tb.band = i;
             tb.A = (int32_t)A2;
@@ -443,6 +437,24 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
             }
         }
     }
+    // every length L that occurs: one full twiddle table; bands of equal length share their tables
+    for (int li = 0; li < kChirpLengths; ++li) {
+        p->chirp.n_bands[li] = (int)chirp_bands[li].size();
+        std::map<int64_t, ChirpRec> of_length;
+        for (int b : chirp_bands[li]) {
+            const int64_t M = L.bands[(size_t)b].M;
+            if (!of_length.count(M)) {
+                ChirpRec cr{};
+                const int f = plan_for(chirp_length(li), kPlanPow2, 16);
+                make_chirp_tables(M / 4, chirp_length(li), tw, cr);
+                cr.tw_full_off = p->ffts[(size_t)f].tw_full_off;
+                of_length[M] = cr;
+            }
+            ChirpRec cr = of_length[M];
+            cr.br = p->bands[(size_t)b];
+            p->chirp.recs.push_back(cr);
+        }
+    }
     // a middle class whose longest band has at most one butterfly per thread at half the threads runs narrower CTAs
     if (p->cls[2].n_bands && L.bands[(size_t)p->cls[2].work[0]].M <= 2304) { p->cls[2].threads = 128; p->cls[2].min_blocks = 8; }
     // the same bands for the one-launch form: about one radix-8 butterfly per thread and stage, so that an item's chain
@@ -451,15 +463,11 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         MergedBands &mg = p->merged;
         auto lg_threads = [&](int32_t b) {
             const FftPlan &bf = p->ffts[(size_t)p->bands[(size_t)b].fft];
-            const int64_t points = bf.generic == 2 ? bf.blu_L : bf.M;
             int lg = 5;
-            while (lg < 10 && (3ll << lg) < points / 4) ++lg;   // 1.5 * threads < points / 8
+            while (lg < 10 && (3ll << lg) < bf.M / 4) ++lg;   // 1.5 * threads < points / 8
             return lg;
         };
-        for (int c = kNumClasses - 1; c >= 1; --c) {
-            mg.work.insert(mg.work.end(), p->cls[c].work.begin(), p->cls[c].work.end());
-            mg.has_generic = mg.has_generic || p->cls[c].has_generic;
-        }
+        for (int c = kNumClasses - 1; c >= 1; --c) mg.work.insert(mg.work.end(), p->cls[c].work.begin(), p->cls[c].work.end());
         std::stable_sort(mg.work.begin(), mg.work.end(), [&](int32_t x, int32_t y) { return lg_threads(x) > lg_threads(y); });
         for (size_t i = 0; i < mg.work.size(); ++i) {
             const int lg = lg_threads(mg.work[i]);
@@ -472,8 +480,6 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     // needs for the longest item (microseconds per element by class, from measured kernel times)
     {
         const double us_per_elem[kNumClasses] = {0.04, 0.015, 0.004, 0.0016, 0.0016};
-        // classes holding lengths with a prime factor above 5 (direct sums, chirp-z with two longer transforms)
-        const double generic_factor[kNumClasses] = {1.3, 1.3, 2.0, 3.5, 3.5};
         for (int c = 0; c < kNumClasses; ++c) {
             BandClass &bc = p->cls[c];
             int64_t longest = 0;
@@ -482,7 +488,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
                 bc.stage_work += (double)M * (p->ffts[(size_t)p->bands[(size_t)b].fft].nstages + 1);
                 longest = std::max(longest, M);
             }
-            bc.latency_us = bc.n_bands ? (5.0 + us_per_elem[c] * (double)longest) * (bc.has_generic ? generic_factor[c] : 1.0) : 0.0;
+            bc.latency_us = bc.n_bands ? 5.0 + us_per_elem[c] * (double)longest : 0.0;
         }
     }
     if (p->device < 0) { *out = p; return CQT_OK; }
@@ -538,6 +544,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     };
     for (auto &c : p->cls) upload_items(c.d_items, c.work);
     upload_items(p->merged.d_items, p->merged.work);
+    chk(upload(p->chirp.d_recs, p->chirp.recs));
     cudaDeviceProp prop;
     chk(cudaGetDeviceProperties(&prop, p->device));
     p->sm_count = prop.multiProcessorCount;
@@ -552,6 +559,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     }
     chk(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
     if (e == cudaSuccess) chk(configure_band_kernels(*p));
+    if (e == cudaSuccess) chk(configure_chirp_kernels(*p));
     if (e == cudaSuccess) chk(configure_long_fft_kernels(*p));
     for (auto &g : p->two_pass) chk(upload(g.d_recs, g.bands));
     if (e == cudaSuccess) chk(configure_two_pass_kernels(*p));
@@ -579,10 +587,7 @@ cqt_status cqt_plan_band_info(const cqt_plan *p, int64_t band, cqt_band_info *ou
     const HostBand &hb = p->lay.bands[band];
     out->centre_hz = hb.centre_hz; out->centre_bin = hb.kc; out->support = hb.S; out->first_offset = hb.d0;
     out->M = hb.M; out->coeff_offset = hb.coeff_off; out->table_offset = hb.tab_off; out->is_sideband = hb.side;
-    out->launch_class = -1;   // two-pass bands belong to no single-CTA class
-    for (int c = 0; c < kNumClasses; ++c)
-        for (int32_t b : p->cls[c].work)
-            if (b == band) out->launch_class = c;
+    out->launch_class = p->band_class[(size_t)band];   // -1: two-pass bands belong to no single-CTA class
     return CQT_OK;
 }
 

@@ -8,7 +8,6 @@ namespace cqt {
 static BandArgs make_args(const cqt_plan &p, const BandClass &c, const float *table, int64_t batch) {
     BandArgs a{};
     a.items = c.d_items;
-    a.ffts = p.d.ffts;
     a.tw = p.d.tw;
     a.table = table;
     a.n_work = c.n_bands;
@@ -55,8 +54,8 @@ static cudaError_t launch_class(const cqt_plan &p, int cls, const char *name, Ba
     return e;
 }
 
-const void *band_analysis_merged_kernel(bool generic);    // band_analysis.cu
-const void *band_synthesis_merged_kernel(bool generic);   // band_synthesis.cu
+const void *band_analysis_merged_kernel();    // band_analysis.cu
+const void *band_synthesis_merged_kernel();   // band_synthesis.cu
 
 // Shape of the few-items form for a batch: the bands longer than class 0's in one launch (two when some of them take
 // 1024 threads each: those then do not set the CTA size of the others), class 0 in one.
@@ -67,6 +66,7 @@ struct FewLaunch {
         size_t smem = 0;
     };
     Part part[2];
+    bool chirp = false;                 // bands on the chirp-z kernel
     int short_threads = 0, short_grid = 0;
 };
 
@@ -103,7 +103,9 @@ static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
     for (int share = 1;; share *= 2) {   // emptier CTAs while there are SMs to spread over
         FewLaunch t;
         bool spread = false;
-        long long sms = few_part(p, batch, 0, split, share, t.part[0], spread);
+        t.chirp = !p.chirp.recs.empty();
+        long long sms = t.chirp ? (chirp_grid(p, batch, nullptr) + 1) / 2 : 0;   // two CTAs of it share an SM
+        sms += few_part(p, batch, 0, split, share, t.part[0], spread);
         sms += few_part(p, batch, split, n, share, t.part[1], spread);
         if (sms > p.sm_count) {
             if (share == 1) return false;
@@ -124,14 +126,18 @@ static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cuda
     static const char *names[2][3] = {{"bands_to_spectrum/1024_threads", "bands_to_spectrum/merged", "bands_to_spectrum/class0"},
                                       {"bands_from_spectrum/1024_threads", "bands_from_spectrum/merged", "bands_from_spectrum/class0"}};
     cudaError_t e = cudaSuccess;
-    const int launches = (f.part[0].grid > 0) + (f.part[1].grid > 0) + (f.short_grid > 0);
+    const int launches = f.chirp + (f.part[0].grid > 0) + (f.part[1].grid > 0) + (f.short_grid > 0);
     a.chain = launches > 1 ? kChainHead : kAlone;
+    if (f.chirp) {
+        e = launch_chirp(p, ANALYSIS, a, st);
+        a.chain = kChainMember;
+    }
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
         FewLaunch::Part &t = f.part[i];
         if (!t.grid) continue;
         a.items = p.merged.d_items;
         void *args[] = {&a, &t.sg};
-        const void *fn = ANALYSIS ? band_analysis_merged_kernel(p.merged.has_generic) : band_synthesis_merged_kernel(p.merged.has_generic);
+        const void *fn = ANALYSIS ? band_analysis_merged_kernel() : band_synthesis_merged_kernel();
         e = launch_kernel(fn, dim3((unsigned)t.grid), dim3((unsigned)t.threads), args, t.smem, st);
         note_launch(p, names[ANALYSIS][i], st);
         a.chain = kChainMember;
@@ -217,6 +223,14 @@ cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, co
         cudaError_t e = launch_two_pass_from_spectrum(p, table, X, c, scratch, batch, fj.two_pass_stream());
         if (e != cudaSuccess) { fj.join(); return e; }
     }
+    if (!p.chirp.recs.empty()) {
+        BandArgs a = make_args(p, p.cls[0], table, batch);
+        a.spec = X;
+        a.spec_pitch = p.lf.x_pitch;
+        a.coef = c;
+        cudaError_t e = launch_chirp(p, true, a, fj.two_pass_stream());
+        if (e != cudaSuccess) { fj.join(); return e; }
+    }
     static const char *names[kNumClasses] = {"bands_from_spectrum/class0", "bands_from_spectrum/class1",
                                               "bands_from_spectrum/class2", "bands_from_spectrum/class3",
                                               "bands_from_spectrum/class4"};
@@ -260,6 +274,14 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
         cudaError_t e = launch_two_pass_to_spectrum(p, table, fold_sidebands, c, Y, scratch, batch, fj.two_pass_stream());
         if (e != cudaSuccess) { fj.join(); return e; }
     }
+    if (!p.chirp.recs.empty()) {
+        BandArgs a = make_args(p, p.cls[0], table, batch);
+        a.coef = const_cast<float2 *>(c);
+        a.Y = Y;
+        a.fold = fold_sidebands ? 1 : 0;
+        cudaError_t e = launch_chirp(p, false, a, fj.two_pass_stream());
+        if (e != cudaSuccess) { fj.join(); return e; }
+    }
     static const char *names[kNumClasses] = {"bands_to_spectrum/class0", "bands_to_spectrum/class1",
                                               "bands_to_spectrum/class2", "bands_to_spectrum/class3",
                                               "bands_to_spectrum/class4"};
@@ -276,7 +298,7 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
 }
 
 cudaError_t configure_band_kernels(const cqt_plan &p) {
-    for (const void *fn : {band_analysis_merged_kernel(p.merged.has_generic), band_synthesis_merged_kernel(p.merged.has_generic)}) {
+    for (const void *fn : {band_analysis_merged_kernel(), band_synthesis_merged_kernel()}) {
         cudaError_t e = allow_dynamic_smem(fn, 0, p);
         if (e != cudaSuccess) return e;
     }

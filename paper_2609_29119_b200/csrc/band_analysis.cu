@@ -29,15 +29,10 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
         return make_float2(g * xv.x, mirrored ? -(g * xv.y) : g * xv.y);
     };
     float2 *out = a.coef + (long long)ch * a.coeff_count + br.coeff_off;
-    // GEN: the class holds lengths with prime factors above 5 (only the multiple-of-4 length policy makes them);
-    // the other instantiations leave the chirp-z and direct-sum code out
-    if (GEN && fp.generic) chain_begin(a);
-    if (GEN && fp.generic == 2) {
-        auto store_c = [&](int n, int, float2 v) { out[n] = v; };
-        chirp_z_transform<+1, Sync>(buf, fp, a.ffts, a.tw, load, store_c, a.dbg, tid, nthr);
-        return;
-    }
+    // GEN: the class holds lengths with prime factors above 5 (only the multiple-of-4 length policy makes them, and the
+    // longer ones run on the chirp-z kernel); the other instantiations leave the direct-sum code out
     if (GEN && fp.generic) {
+        chain_begin(a);
         float2 *alt = buf + M;
         for (int m = tid; m < M; m += nthr) buf[m] = load(m, 0);
         Sync::sync(nthr);
@@ -87,7 +82,6 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_from_spectrum_kernel(Band
 }
 
 // Every band of 128 < M that fits a CTA in one launch (see BandSegments).
-template <bool GEN>
 __global__ void __launch_bounds__(1024, 1) all_bands_from_spectrum_kernel(BandArgs a, BandSegments sg) {
     chain_enter(a);
     MergedItem m;
@@ -95,18 +89,16 @@ __global__ void __launch_bounds__(1024, 1) all_bands_from_spectrum_kernel(BandAr
     __shared__ BandItem item_s[kMaxGroups];
     BandItem &it = item_s[m.slot];
     fetch_item<NamedSync>(a.items[m.band], it, m.tid, m.nthr);
-    analysis_item<NamedSync, 16, GEN>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
+    analysis_item<NamedSync, 16, false>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
     chain_end(a);
 }
 
-const void *band_analysis_merged_kernel(bool generic) {
-    return generic ? (const void *)all_bands_from_spectrum_kernel<true> : (const void *)all_bands_from_spectrum_kernel<false>;
-}
+const void *band_analysis_merged_kernel() { return (const void *)all_bands_from_spectrum_kernel; }
 
 const void *band_analysis_kernel(const BandClass &c, int lanes) {
 #define X(T, B, W, R)                                                                          \
     if (c.threads == T && c.min_blocks == B && lanes == W && c.max_radix <= R)  \
-        return c.has_generic ? (const void *)bands_from_spectrum_kernel<T, B, W, R, true> : (const void *)bands_from_spectrum_kernel<T, B, W, R, false>;
+        return W && c.has_generic ? (const void *)bands_from_spectrum_kernel<T, B, W, R, (W > 0)> : (const void *)bands_from_spectrum_kernel<T, B, W, R, false>;
     CQT_KERNEL_TABLE(X)
 #undef X
     return nullptr;

@@ -17,7 +17,6 @@ namespace cqt {
 
 struct BandArgs {
     const BandItem *items;   // per band of the class, in launch order (longest first): record + radix plan
-    const FftPlan *ffts;
     const float2 *tw;
     const float *table;
     int n_work;
@@ -112,41 +111,47 @@ __device__ __forceinline__ void fetch_item(const BandItem &g, BandItem &s, int t
     Sync::sync(nthr);
 }
 
-// Chirp-z (Bluestein) evaluation of an M-point DFT of sign SIGN whose length has a large prime factor:
-//   X[k] = c[k] sum_n (x[n] c[n]) conj(c[k-n]),  c[n] = exp(SIGN i pi n^2 / M),
-// the convolution through two power-of-two transforms of length L >= 2M - 1 in shared memory: forward DIF
-// (natural -> digit-reversed), product with the precomputed filter spectrum (stored in that order, 1/L included),
-// the DIF network backwards (digit-reversed -> natural).  load(n) yields x[n]; store(k, ., X[k]).
-template <int SIGN, class Sync, class Load, class Store>
-__device__ __forceinline__ void chirp_z_transform(float2 *buf, const FftPlan &fp, const FftPlan *ffts, const float2 *tw,
-                                                  Load load, Store store, int *dbg, int tid, int nthr) {
-    const FftPlan &fl = ffts[fp.blu_fft];
-    const int M = fp.M, L = fp.blu_L;
-    float2 *twl = buf + L;
-    stage_twiddles(twl, tw, fl, tid, nthr);
-    const float2 *chirp = tw + fp.blu_chirp_off;   // exp(-i pi n^2 / M)
-    const float2 *filt = tw + fp.blu_filter_off;
-    const Tile tl{buf, 1, 1, 0u, L, dbg};
-    auto loadc = [&](int n, int) -> float2 {
-        if (n >= M) return make_float2(0.f, 0.f);
-        float2 w = __ldg(chirp + n);
-        if (SIGN > 0) w.y = -w.y;
-        return cmul(load(n, 0), w);
-    };
-    fft_fused_keep<-1, Sync, true, false, false>(tl, fl, twl, loadc, tid, nthr);
-    for (int p = tid; p < L; p += nthr) {
-        float2 f = __ldg(filt + p);
-        if (SIGN > 0) f.y = -f.y;
-        buf[p] = cmul(buf[p], f);
-    }
-    Sync::sync(nthr);
-    fft_dit_inverse<Sync>(tl, fl, twl, tid, nthr);
-    for (int k = tid; k < M; k += nthr) {
-        float2 w = __ldg(chirp + k);
-        if (SIGN > 0) w.y = -w.y;
-        store(k, 0, cmul(buf[k], w));
-    }
+// Analysis form, any band: slot m of the transform's input, i.e. tab[d] X[kc + d] with d = m or m - M, zero outside the
+// support; bins outside 0..N/2 are the conjugates of their mirror bins.
+__device__ __forceinline__ float2 slot_value(const BandRec &br, const float *__restrict__ tab,
+                                             const float2 *__restrict__ X, int N, int m) {
+    const int last_pos = br.d0 + br.S - 1, first_neg = br.M + br.d0;
+    int d;
+    if (m <= last_pos) d = m;
+    else if (m >= first_neg) d = m - br.M;
+    else return make_float2(0.f, 0.f);
+    const float g = __ldg(tab + (d - br.d0));
+    const int k = br.kc + d;
+    float2 xv;
+    if (k < 0) xv = cconj(__ldg(X + (-k)));
+    else if (k > (N >> 1)) xv = cconj(__ldg(X + (N - k)));
+    else xv = __ldg(X + k);
+    return make_float2(g * xv.x, g * xv.y);
 }
+
+// Synthesis form, any band: output u of slot m, times the window table, to bin kc + d of the band's plane Y (only bins
+// 0..N/2 are kept).
+__device__ __forceinline__ void slot_store(const BandRec &br, const float *__restrict__ tab, float2 *__restrict__ Y, int N, int m, float2 u,
+                                           int *dbg = nullptr, long long limit = 1ll << 40) {
+    const int last_pos = br.d0 + br.S - 1, first_neg = br.M + br.d0;
+    int d;
+    if (m <= last_pos) d = m;
+    else if (m >= first_neg) d = m - br.M;
+    else return;
+    const int k = br.kc + d;
+    if (k < 0 || k > (N >> 1)) return;
+    const float h = __ldg(tab + (d - br.d0));
+    if (CQT_CHK(dbg, 404, k, limit)) Y[k] = make_float2(h * u.x, h * u.y);
+}
+
+// band_chirp.cu: bands of more than 128 coefficients whose length has a prime factor above 5
+constexpr int kChirpThreads = 256;
+struct ChirpSegment {
+    int cta0, n_cta, first_band, n_bands;
+};
+int chirp_grid(const cqt_plan &p, int64_t batch, ChirpSegment *seg);
+size_t chirp_smem(const cqt_plan &p);
+cudaError_t launch_chirp(const cqt_plan &p, bool analysis, const BandArgs &b, cudaStream_t st);
 
 // Kernel instantiations: (threads per CTA, CTAs per SM the registers must allow, lanes per item or 0 for the whole CTA, largest radix
 // compiled in), each with and without the prime-factor paths (GEN): code a class never runs is left out, which also

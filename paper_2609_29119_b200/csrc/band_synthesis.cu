@@ -55,14 +55,10 @@ __device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem
         const float h = __ldg(tab + (d - br.d0));
         if (CQT_CHK(a.dbg, 306, (long long)br.y_off + k, a.y_pitch)) Y[k] = make_float2(h * u.x, h * u.y);
     };
-    // GEN: the class holds lengths with prime factors above 5 (only the multiple-of-4 length policy makes them);
-    // the other instantiations leave the chirp-z and direct-sum code out
-    if (GEN && fp.generic) chain_begin(a);
-    if (GEN && fp.generic == 2) {
-        chirp_z_transform<-1, Sync>(buf, fp, a.ffts, a.tw, load, store, a.dbg, tid, nthr);
-        return;
-    }
+    // GEN: the class holds lengths with prime factors above 5 (only the multiple-of-4 length policy makes them, and the
+    // longer ones run on the chirp-z kernel); the other instantiations leave the direct-sum code out
     if (GEN && fp.generic) {
+        chain_begin(a);
         float2 *alt = buf + M;
         for (int n = tid; n < M; n += nthr) buf[n] = load(n, 0);
         Sync::sync(nthr);
@@ -104,7 +100,6 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_to_spectrum_kernel(BandAr
 }
 
 // Every band of 128 < M that fits a CTA in one launch (see BandSegments).
-template <bool GEN>
 __global__ void __launch_bounds__(1024, 1) all_bands_to_spectrum_kernel(BandArgs a, BandSegments sg) {
     chain_enter(a);
     MergedItem m;
@@ -112,18 +107,16 @@ __global__ void __launch_bounds__(1024, 1) all_bands_to_spectrum_kernel(BandArgs
     __shared__ BandItem item_s[kMaxGroups];
     BandItem &it = item_s[m.slot];
     fetch_item<NamedSync>(a.items[m.band], it, m.tid, m.nthr);
-    synthesis_item<NamedSync, 16, GEN>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
+    synthesis_item<NamedSync, 16, false>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
     chain_end(a);
 }
 
-const void *band_synthesis_merged_kernel(bool generic) {
-    return generic ? (const void *)all_bands_to_spectrum_kernel<true> : (const void *)all_bands_to_spectrum_kernel<false>;
-}
+const void *band_synthesis_merged_kernel() { return (const void *)all_bands_to_spectrum_kernel; }
 
 const void *band_synthesis_kernel(const BandClass &c, int lanes) {
 #define X(T, B, W, R)                                                                          \
     if (c.threads == T && c.min_blocks == B && lanes == W && c.max_radix <= R)  \
-        return c.has_generic ? (const void *)bands_to_spectrum_kernel<T, B, W, R, true> : (const void *)bands_to_spectrum_kernel<T, B, W, R, false>;
+        return W && c.has_generic ? (const void *)bands_to_spectrum_kernel<T, B, W, R, (W > 0)> : (const void *)bands_to_spectrum_kernel<T, B, W, R, false>;
     CQT_KERNEL_TABLE(X)
 #undef X
     return nullptr;

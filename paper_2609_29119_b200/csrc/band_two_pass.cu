@@ -11,8 +11,7 @@
 #include <algorithm>
 #include <cstdlib>
 
-#include "engine.cuh"
-#include "internal.hpp"
+#include "band_common.cuh"
 
 namespace cqt {
 
@@ -40,22 +39,6 @@ struct TwoPassArgs {
     long long scratch_pitch;
     int *dbg;
 };
-
-__device__ __forceinline__ float2 slot_value(const BandRec &br, const float *__restrict__ tab,
-                                             const float2 *__restrict__ X, int N, int m) {
-    const int last_pos = br.d0 + br.S - 1, first_neg = br.M + br.d0;
-    int d;
-    if (m <= last_pos) d = m;
-    else if (m >= first_neg) d = m - br.M;
-    else return make_float2(0.f, 0.f);
-    const float g = __ldg(tab + (d - br.d0));
-    const int k = br.kc + d;
-    float2 xv;
-    if (k < 0) xv = cconj(__ldg(X + (-k)));
-    else if (k > (N >> 1)) xv = cconj(__ldg(X + (N - k)));
-    else xv = __ldg(X + k);
-    return make_float2(g * xv.x, g * xv.y);
-}
 
 __device__ __forceinline__ void copy_table(float2 *dst, const float2 *__restrict__ src, int n, int tid, int nthr) {
     for (int i = tid; i < n; i += nthr) dst[i] = __ldg(src + i);
@@ -140,18 +123,8 @@ __global__ void __launch_bounds__(THREADS, MINB) band2p_rows_kernel(TwoPassArgs 
     } else {
         const float *tab = a.table + br.tab_off;
         float2 *Y = a.Y + (long long)ch * a.y_pitch + br.y_off;
-        const int M = br.M, last_pos = br.d0 + br.S - 1, first_neg = M + br.d0, half = a.N >> 1;
         auto store = [&](int q, int r, float2 u) {
-            if (r >= nrows) return;
-            const long long m = (long long)(r0 + r) + (long long)rec.A * q;
-            int d;
-            if (m <= last_pos) d = (int)m;
-            else if (m >= first_neg) d = (int)(m - M);
-            else return;
-            const int k = br.kc + d;
-            if (k < 0 || k > half) return;
-            const float h = __ldg(tab + (d - br.d0));
-            if (CQT_CHK(a.dbg, 404, (long long)br.y_off + k, a.y_pitch)) Y[k] = make_float2(h * u.x, h * u.y);
+            if (r < nrows) slot_store(br, tab, Y, a.N, (r0 + r) + rec.A * q, u, a.dbg, (long long)a.y_pitch - br.y_off);
         };
         fft_fused<-1, BlockSync, false, false, false, false, true, true>(t, fp, twf, load, store, tid, nthr);
     }

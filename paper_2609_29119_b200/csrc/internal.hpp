@@ -19,7 +19,7 @@ struct BandClass {
     int lanes_few = 0, lanes_many = 0;   // > 0: several (band, signal) items per CTA, that many lanes each, in a call
                                          // with few / many items; 0: one item per CTA
     int max_radix = 16;      // largest butterfly radix in the class's plans
-    bool has_generic = false; // some band of the class has a prime factor above 5 (direct-sum stage or chirp-z)
+    bool has_generic = false; // some band has a length with a prime factor above 5 (direct-sum stage)
     int max_elems = 0;       // shared-memory elements (float2) per item
     int n_bands = 0;         // bands in the class
     double stage_work = 0.0; // element-stages of the class's transforms per signal (stream assignment)
@@ -35,7 +35,12 @@ struct MergedBands {
     std::vector<Segment> segs;       // most threads first
     std::vector<int32_t> work;       // band indices in launch order
     BandItem *d_items = nullptr;
-    bool has_generic = false;
+};
+
+struct ChirpBands {
+    int n_bands[kChirpLengths] = {};   // per length L of the sub-transforms, longest first
+    std::vector<ChirpRec> recs;        // in that order
+    ChirpRec *d_recs = nullptr;
 };
 
 struct LongFft {
@@ -88,6 +93,8 @@ struct cqt_plan {
     cqt::LongFft lf;
     cqt::BandClass cls[cqt::kNumClasses];
     cqt::MergedBands merged;
+    cqt::ChirpBands chirp;
+    std::vector<int8_t> band_class;    // length class of every band, -1: two-pass kernels
     cqt::TwoPassGroup two_pass[2];     // [0]: both factors <= 256, [1]: larger factors
     int64_t two_pass_pitch = 0;        // scratch elements per signal for the two-pass bands
     cqt::DevicePlan d;
@@ -182,6 +189,11 @@ cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, co
 cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool fold_sidebands, const float2 *c,
                                      float2 *Y, float2 *scratch, int64_t batch, cudaStream_t st);
 cudaError_t configure_band_kernels(const cqt_plan &p);
+
+// band_chirp.cu
+int chirp_length_index(int64_t m);     // which L serves m-point sub-transforms, -1: none
+int chirp_length(int index);
+cudaError_t configure_chirp_kernels(const cqt_plan &p);
 
 // band_two_pass.cu
 cudaError_t launch_two_pass_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, float2 *c,

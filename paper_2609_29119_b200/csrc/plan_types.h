@@ -29,16 +29,11 @@ struct FftPlan {
     int32_t nstages;
     int32_t logC;
     int32_t tw_off;                 // into the plan's twiddle array (float2 elements)
-    int32_t generic;                // 1: stage 0 is a generic (direct-sum) radix; 2: chirp-z (Bluestein) transform, see blu_*
+    int32_t generic;                // 1: stage 0 is a generic (direct-sum) radix
     int32_t tw_count;               // entries of the two-level table (C + ceil(M / C))
     int32_t pad_delta;              // 1 if single-column buffers skip one element per s_0 positions (bank spread)
     int32_t tw_full_off;            // power-of-two plans: offset of the full table exp(-2 pi i y / M), y < M; else -1
     StageRec st[kMaxStages];        // per-stage constants, one 32-byte record each (two 16-byte loads in the kernels)
-    // chirp-z evaluation of a length with a large prime factor: two power-of-two transforms of length blu_L
-    int32_t blu_L;                  // power of two >= 2 M - 1
-    int32_t blu_fft;                // FftPlan index of the length-blu_L plan
-    int32_t blu_chirp_off;          // exp(-i pi n^2 / M), n < M, in the twiddle array
-    int32_t blu_filter_off;         // DFT of the conjugate chirp / blu_L, in the digit-reversed order of that plan
 };
 
 // One band of the layout as the kernels see it.
@@ -61,6 +56,16 @@ struct BandItem {
     BandRec br;
     FftPlan fp;
 };
+
+// A band on the chirp-z kernel (M = 4 m, m with a prime factor above 5): offsets into the twiddle array.
+struct ChirpRec {
+    BandRec br;
+    int32_t pre_off;       // exp(-i pi (n k0 / (2 m) + n^2 / m)), four runs (k0) of m entries
+    int32_t filter_off;    // DFT_L of the conjugate chirp (wrapped) / L
+    int32_t tw_full_off;   // full table of W_L
+    int32_t pad_;
+};
+constexpr int kChirpLengths = 7;   // L = 8192 ... 128
 
 // A band transformed in two passes (M = A * B) through a scratch row.
 struct TwoPassRec {

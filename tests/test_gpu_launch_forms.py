@@ -46,3 +46,32 @@ def test_one_pass_fft_lengths(log_n, batch):
                          ids=lambda k: f"n{k['N']}_b{k['bins_per_octave']}_p{k['m_policy']}")
 def test_band_launch_forms(kw, batch):
     check_rows(small_workload("forms", **{"fs": 44100.0, "fmin": 60.0, "fmax": 22050.0, "channels": batch, **kw}), batch)
+
+
+@pytest.mark.parametrize("m", [33, 64 - 3, 127, 257, 509, 1021, 2039, 2053, 3191])
+def test_lengths_with_a_large_prime_factor(m):
+    """Regular bands of 4 m coefficients, m prime or not 5-smooth, up to both sides of each convolution length: against
+    numpy's FFT of the windowed, slot-placed spectrum; the round trip covers the synthesis form."""
+    from paper_2609_29119_b200 import Plan, M_MULT4
+    N, M = 1 << 15, 4 * m
+    centre = [N / 4.0 - 0.1 * M, N / 4.0 + 0.1 * M]
+    plan = Plan.from_bands(float(N), N, centre, [M - 1.5] * 2, m_policy=M_MULT4)
+    rng = np.random.default_rng(m)
+    x = rng.standard_normal((3, N)).astype(np.float32)
+    xd = torch.from_numpy(x).cuda()
+    c = plan.analyse(xd)
+    g, _ = plan.tables()
+    X = np.fft.rfft(x.astype(np.float64))
+    for bi in plan.bands():
+        if bi.is_sideband:
+            continue
+        assert bi.M == M
+        d = np.arange(bi.first_offset, bi.first_offset + bi.support)
+        slots = np.zeros((3, M), dtype=np.complex128)
+        slots[:, d % M] = g[bi.table_offset:bi.table_offset + bi.support] * X[:, bi.centre_bin + d]
+        want = np.fft.ifft(slots)
+        got = c[:, bi.coeff_offset:bi.coeff_offset + M].cpu().numpy()
+        assert (np.linalg.norm(got - want, axis=1) / np.linalg.norm(want, axis=1)).max() <= TOL
+    y = plan.synthesise(c).cpu().numpy().astype(np.float64)
+    assert (np.sum((y - x) ** 2, axis=1) / np.sum(x.astype(np.float64) ** 2, axis=1)).max() <= 1e-12
+    plan.close()
