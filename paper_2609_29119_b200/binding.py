@@ -1,4 +1,5 @@
-"""ctypes binding with the same names as include/cqt.h.
+"""Binding with the same names as include/cqt.h: ctypes for plans and queries, a native module (csrc/torch_ext.cpp) for
+the calls that programs make per batch.
 
 Argument marshalling only: every step of the transform runs in the CUDA kernels of
 libcqt_b200.so.  torch is used for device memory and streams.  There is no CPU fallback:
@@ -15,6 +16,10 @@ M_MULT4, M_SMOOTH, M_POW2 = 0, 1, 2
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB: Optional[C.CDLL] = None
+
+
+# transforms by the numbers of csrc/torch_ext.cpp
+ANALYSE, SYNTHESISE_ADJOINT, SYNTHESISE, ANALYSE_ADJOINT, ANALYSE_STATIC_WS = range(5)
 
 
 class CqtError(RuntimeError):
@@ -109,6 +114,25 @@ def load_library() -> C.CDLL:
     return _LIB
 
 
+_EXT = None
+
+
+def native():
+    """The native module of the per-batch calls (loaded on first use: it needs torch)."""
+    global _EXT
+    if _EXT is None:
+        import torch  # noqa: F401  (its libraries first)
+        load_library()
+        try:
+            from . import _cqt_torch
+        except ImportError as e:
+            raise RuntimeError("paper_2609_29119_b200/_cqt_torch.so is missing or does not match this torch: build it with "
+                               "`python -m paper_2609_29119_b200.build`") from e
+        _cqt_torch.set_error(CqtError)
+        _EXT = _cqt_torch
+    return _EXT
+
+
 def status_string(status: int) -> str:
     return load_library().cqt_status_string(status).decode()
 
@@ -182,6 +206,7 @@ class Plan:
 
     def _adopt(self, h, device) -> None:
         self.handle = h
+        self._h = h.value
         self.device = device
         self.N = int(self.lib.cqt_plan_signal_length(h))
         self.num_bands = int(self.lib.cqt_plan_num_bands(h))
@@ -193,6 +218,7 @@ class Plan:
         if getattr(self, "handle", None):
             self.lib.cqt_plan_destroy(self.handle)
             self.handle = None
+            self._h = 0
 
     def __del__(self):
         try:
@@ -246,50 +272,22 @@ class Plan:
         return [(names[i].decode(), float(ms[i])) for i in range(m)]
 
     # ---- transforms (x: [batch, >= valid_len] float32 cuda; c: [batch, coeff_count] complex64 cuda)
-    def _sig(self, x, valid_len):
-        import torch
-        assert x.is_cuda and x.dtype == torch.float32 and x.dim() == 2 and x.stride(1) == 1
-        return x.shape[0], (x.shape[1] if valid_len is None else valid_len), x.stride(0)
-
-    def analyse(self, x, valid_len=None, out=None, ws=None, stream=None, _fn="cqt_analyse"):
-        import torch
-        batch, vl, stride = self._sig(x, valid_len)
-        if out is None:
-            out = torch.empty((batch, self.coeff_count), dtype=torch.complex64, device=x.device)
-        ws = self.workspace(batch) if ws is None else ws
-        _check(getattr(self.lib, _fn)(self.handle, x.data_ptr(), stride, batch, vl, out.data_ptr(), ws.data_ptr(),
-                                      ws.numel(), _stream_ptr(stream)), _fn)
-        return out
+    def analyse(self, x, valid_len=None, out=None, ws=None, stream=None):
+        return native().transform(self, ANALYSE, x, valid_len, out, ws, stream)
 
     def analyse_static_ws(self, x, valid_len=None, out=None, stream=None):
         """cqt_analyse_static_ws: analysis for callers that cannot allocate; scratch is the library's own
         fixed 16 MiB array (shared by all calls, so overlapping calls race), limited batch."""
-        import torch
-        batch, vl, stride = self._sig(x, valid_len)
-        if out is None:
-            out = torch.empty((batch, self.coeff_count), dtype=torch.complex64, device=x.device)
-        _check(self.lib.cqt_analyse_static_ws(self.handle, x.data_ptr(), stride, batch, vl, out.data_ptr(),
-                                              _stream_ptr(stream)), "cqt_analyse_static_ws")
-        return out
+        return native().transform(self, ANALYSE_STATIC_WS, x, valid_len, out, None, stream)
 
-    def synthesise(self, c, valid_len=None, out=None, ws=None, stream=None, _fn="cqt_synthesise"):
-        import torch
-        assert c.is_cuda and c.dtype == torch.complex64 and c.dim() == 2 and c.is_contiguous()
-        assert c.shape[1] == self.coeff_count
-        batch = c.shape[0]
-        vl = self.N if valid_len is None else valid_len
-        if out is None:
-            out = torch.empty((batch, vl), dtype=torch.float32, device=c.device)
-        ws = self.workspace(batch) if ws is None else ws
-        _check(getattr(self.lib, _fn)(self.handle, c.data_ptr(), batch, vl, out.data_ptr(), out.stride(0), ws.data_ptr(),
-                                      ws.numel(), _stream_ptr(stream)), _fn)
-        return out
+    def synthesise(self, c, valid_len=None, out=None, ws=None, stream=None):
+        return native().transform(self, SYNTHESISE, c, valid_len, out, ws, stream)
 
     def analyse_adjoint(self, c_bar, valid_len=None, out=None, ws=None, stream=None):
-        return self.synthesise(c_bar, valid_len, out, ws, stream, _fn="cqt_analyse_adjoint")
+        return native().transform(self, ANALYSE_ADJOINT, c_bar, valid_len, out, ws, stream)
 
     def synthesise_adjoint(self, x_bar, valid_len=None, out=None, ws=None, stream=None):
-        return self.analyse(x_bar, valid_len, out, ws, stream, _fn="cqt_synthesise_adjoint")
+        return native().transform(self, SYNTHESISE_ADJOINT, x_bar, valid_len, out, ws, stream)
 
 
 class SliCQ:
@@ -300,11 +298,13 @@ class SliCQ:
         h = C.c_void_p()
         _check(self.lib.slicq_create(plan.handle, channels, transition, max_slices_in_flight, C.byref(h)), "slicq_create")
         self.handle = h
+        self._h = h.value
 
     def close(self):
         if getattr(self, "handle", None):
             self.lib.slicq_destroy(self.handle)
             self.handle = None
+            self._h = 0
 
     def __del__(self):
         try:
@@ -316,11 +316,7 @@ class SliCQ:
         return int(self.lib.slicq_device_bytes(self.handle))
 
     def push(self, x, stream=None) -> int:
-        done = C.c_int64()
-        n = x.shape[1]
-        _check(self.lib.slicq_push(self.handle, x.data_ptr() if n else None, x.stride(0) if n else 0, n,
-                                   _stream_ptr(stream), C.byref(done)), "slicq_push")
-        return int(done.value)
+        return native().slicq_push(self._h, x, stream)
 
     def coeffs(self, slice_index: int):
         """complex64 view [channels, coeff_count] of one analysed slice (valid until it is pulled)."""
@@ -330,10 +326,7 @@ class SliCQ:
         return _DevicePtrTensor(p.value, (self.channels, self.plan.coeff_count), self.plan.device)
 
     def pull(self, y, stream=None) -> int:
-        wrote = C.c_int64()
-        _check(self.lib.slicq_pull(self.handle, y.data_ptr(), y.stride(0), y.shape[1], _stream_ptr(stream),
-                                   C.byref(wrote)), "slicq_pull")
-        return int(wrote.value)
+        return native().slicq_pull(self._h, y, stream)
 
     def flush(self, stream=None) -> None:
         _check(self.lib.slicq_flush(self.handle, _stream_ptr(stream)), "slicq_flush")

@@ -10,6 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libcqt_b200.so")
+EXT = os.path.join(HERE, "_cqt_torch.so")        # Python side of the transform calls, linked to LIB and torch
 SOURCES = ["layout.cpp", "api.cu", "band.cu", "band_analysis.cu", "band_synthesis.cu", "band_two_pass.cu", "band_chirp.cu", "long_fft.cu", "short_fft.cu", "slicq.cu", "static_ws.cu"]
 HEADERS = ["layout.hpp", "plan_types.h", "internal.hpp", "engine.cuh", "band_common.cuh", "long_common.cuh",
            "static_fft.cuh", "codelets_gen.cuh",
@@ -77,6 +78,21 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
         if res.returncode:
             sys.stderr.write(res.stdout + res.stderr)
             raise RuntimeError("link failed")
+    ext_src = os.path.join(CSRC, "torch_ext.cpp")
+    if force or _stale(EXT, [ext_src, hdrs[-1]]):
+        import sysconfig
+        from torch.utils import cpp_extension as ce
+        import torch
+        libs = ce.library_paths()
+        cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+               ext_src, "-o", EXT, "-I" + sysconfig.get_paths()["include"],
+               "-I" + os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include") if os.path.isabs(nvcc) else "-I/usr/local/cuda/include"]
+        cmd += ["-I" + p for p in ce.include_paths()] + ["-L" + p for p in libs] + ["-Wl,-rpath," + p for p in libs]
+        cmd += ["-L" + HERE, "-Wl,-rpath,$ORIGIN", "-lcqt_b200", "-ltorch_python", "-ltorch_cpu", "-ltorch", "-lc10", "-lc10_cuda"]
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode:
+            sys.stderr.write(res.stdout + res.stderr)
+            raise RuntimeError("the torch extension failed to build")
     return LIB
 
 
