@@ -315,9 +315,6 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     lf.n_lp = (int)tw.size() - lf.tw_lp;
     lf.tw_n = append_twiddles(tw, N, lf.log_n_c);
     lf.n_n = (int)tw.size() - lf.tw_n;
-    // tile widths chosen so that two CTAs of the row kernels (three of the column kernels) share an SM
-    lf.tw_rows = lf.A == 1 ? 1 : (int)std::min<int64_t>(lf.B <= 512 ? 8 : 4, lf.A / 2);
-    lf.tw_cols = lf.A == 1 ? 1 : (int)std::min<int64_t>(lf.A <= 512 ? 16 : 8, lf.B);
     lf.x_pitch = (lf.Lp + 1 + 7) / 8 * 8;
 
     // ---- band records
@@ -510,7 +507,13 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         }
     }
     std::vector<int32_t> cover(N / 2 + 1);
-    for (int64_t k = 0; k <= N / 2; ++k) cover[k] = ((L.cover_lo[k] % p->y_planes) << 8) | L.cover_n[k];
+    for (int64_t k = 0; k <= N / 2; ++k) {
+        cover[k] = ((L.cover_lo[k] % p->y_planes) << 8) | L.cover_n[k];
+        if (p->y_planes <= 3) {   // a bit mask of the planes instead (cover_is_mask)
+            cover[k] = 0;
+            for (int i = 0; i < L.cover_n[k]; ++i) cover[k] |= 1 << ((L.cover_lo[k] + i) % p->y_planes);
+        }
+    }
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
     chk(upload(p->d.bands, p->bands));
@@ -560,7 +563,8 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     chk(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
     if (e == cudaSuccess) chk(configure_band_kernels(*p));
     if (e == cudaSuccess) chk(configure_chirp_kernels(*p));
-    if (e == cudaSuccess) chk(configure_long_fft_kernels(*p));
+    if (e == cudaSuccess) chk(p->lf.A == 1 ? configure_short_fft_kernels(*p) : configure_long_forward_kernels(*p));
+    if (e == cudaSuccess && p->lf.A > 1) chk(configure_long_inverse_kernels(*p));
     for (auto &g : p->two_pass) chk(upload(g.d_recs, g.bands));
     if (e == cudaSuccess) chk(configure_two_pass_kernels(*p));
     cudaSetDevice(cur);

@@ -25,7 +25,7 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
         const bool mirrored = k < 0 || k > half;
         const int km = k < 0 ? -k : (k > half ? a.N - k : k);
         if (!CQT_CHK(a.dbg, 302, km, half + 1)) return make_float2(0.f, 0.f);
-        const float2 xv = __ldg(X + km);
+        const float2 xv = ld_data(X + km);
         return make_float2(g * xv.x, mirrored ? -(g * xv.y) : g * xv.y);
     };
     float2 *out = a.coef + (long long)ch * a.coeff_count + br.coeff_off;
@@ -56,7 +56,7 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
             const int j = lo ? m - br.d0 : m - shift_neg;
             if (!CQT_CHK(a.dbg, 309, j, br.S)) return make_float2(0.f, 0.f);
             const float g = __ldg(tab + j);
-            const float2 xv = __ldg(Xs + j);
+            const float2 xv = ld_data(Xs + j);
             return make_float2(g * xv.x, g * xv.y);
         };
         fft_fused<+1, Sync, false, true, false, true, false, false, MAXR>(t, fp, tws, load_regular, store, tid, nthr);

@@ -123,9 +123,9 @@ __device__ __forceinline__ float2 slot_value(const BandRec &br, const float *__r
     const float g = __ldg(tab + (d - br.d0));
     const int k = br.kc + d;
     float2 xv;
-    if (k < 0) xv = cconj(__ldg(X + (-k)));
-    else if (k > (N >> 1)) xv = cconj(__ldg(X + (N - k)));
-    else xv = __ldg(X + k);
+    if (k < 0) xv = cconj(ld_data(X + (-k)));
+    else if (k > (N >> 1)) xv = cconj(ld_data(X + (N - k)));
+    else xv = ld_data(X + k);
     return make_float2(g * xv.x, g * xv.y);
 }
 

@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(THREADS, MINB) band2p_cols_kernel(TwoPassArgs 
         if (c >= ncols) return make_float2(0.f, 0.f);
         const int idx = r * rec.B + c0 + c;
         if (ANALYSIS) return slot_value(br, tab, X, a.N, idx);
-        float2 v = __ldg(cin + idx);
+        float2 v = ld_data(cin + idx);
         if (fold) v = make_float2(2.f * v.x, 0.f);
         return v;
     };
@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(THREADS, MINB) band2p_rows_kernel(TwoPassArgs 
     auto load = [&](int p, int r) -> float2 {
         if (r >= nrows) return make_float2(0.f, 0.f);
         const long long i = (long long)(r0 + r) * rec.B + p;
-        return CQT_CHK(a.dbg, 402, i, br.M) ? __ldg(T + i) : make_float2(0.f, 0.f);
+        return CQT_CHK(a.dbg, 402, i, br.M) ? ld_data(T + i) : make_float2(0.f, 0.f);
     };
     if (ANALYSIS) {
         float2 *out = a.coef + (long long)ch * a.coeff_count + br.coeff_off;

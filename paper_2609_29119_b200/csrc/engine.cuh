@@ -20,6 +20,14 @@ namespace cqt {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// A value that an earlier kernel of the chain wrote.  Not __ldg: a non-coherent load counts as invariant, and the compiler
+// may move it above pdl_wait.  Volatile statements keep their order.
+__device__ __forceinline__ float2 ld_data(const float2 *p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 // sync(nthr): barrier of the nthr threads that work on one item
 struct BlockSync {
     static __device__ __forceinline__ void sync(int) { __syncthreads(); }

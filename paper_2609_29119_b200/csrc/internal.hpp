@@ -49,8 +49,6 @@ struct LongFft {
     int tw_lp = 0, tw_n = 0;      // two-level tables of W_Lp and W_N inside the twiddle array
     int log_lp_c = 0, log_n_c = 0;
     int n_lp = 0, n_n = 0;        // entry counts of those tables
-    int tw_rows = 1;              // rows per mirrored half handled by one CTA of the row kernels (forward and inverse)
-    int tw_cols = 1;              // columns per CTA of the column kernels
     int64_t x_pitch = 0;          // elements per signal of the half-spectrum buffer (Lp + 1 rounded up)
 };
 
@@ -72,7 +70,7 @@ struct DevicePlan {
     float *tab_synthesis = nullptr;    // h
     float *tab_analysis_adj = nullptr; // N g / (2 M)
     float *tab_synthesis_adj = nullptr;// h w_k / N
-    int32_t *cover = nullptr;          // per bin: (plane of the first covering band << 8) | number of covering bands
+    int32_t *cover = nullptr;          // per bin: the planes that hold it (plane_sum in long_common.cuh)
     int *dbg = nullptr;                // 8 status words of the debug-bounds build
     int2 *zero_seg = nullptr;          // (offset into one signal's weighted-bin scratch, length): bins synthesis zero-fills
 };
@@ -120,7 +118,7 @@ enum { TAB_ANALYSIS = 0, TAB_SYNTHESIS = 1, TAB_ANALYSIS_ADJ = 2, TAB_SYNTHESIS_
 // api.cu: called after every kernel launch (and once at the start of a call with name == nullptr)
 void note_launch(const cqt_plan &p, const char *name, cudaStream_t st);
 
-// long_fft.cu
+// long_fft_forward.cu, long_fft_inverse.cu
 // Input of the forward long FFT taken from a ring buffer of a stream instead of signal rows (sliced transform, slice
 // cut fused into the load): row r = slice r / channels of channel r % channels; sample i of that slice is
 // win[i] * ring[channel * ring_len + (first + (r / channels) * hop + i) mod ring_len], zero before the stream's start.
@@ -148,7 +146,9 @@ inline cudaError_t allow_dynamic_smem(const void *fn, size_t need, const cqt_pla
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
-cudaError_t configure_long_fft_kernels(const cqt_plan &p);
+cudaError_t configure_long_forward_kernels(const cqt_plan &p);
+cudaError_t configure_long_inverse_kernels(const cqt_plan &p);
+cudaError_t configure_short_fft_kernels(const cqt_plan &p);
 
 // Launch with the programmatic-serialization attribute (see pdl_wait in engine.cuh).
 inline cudaError_t launch_kernel(const void *fn, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t st) {

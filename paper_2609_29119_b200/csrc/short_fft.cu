@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(S::T, S::T >= 512 ? 2 : 4) short_rfft_forward_
     pdl_launch_dependents();
     const int tid = threadIdx.x;
     float2 *buf = smem_short, *twf = buf + S::BUF, *wn = twf + S::Lp;
-    stage_full(twf, a.tw, a.ffts[a.fft_B], tid, S::T);
+    stage_table(twf, a.tw + a.tw_full_B, S::Lp, tid, S::T);
     stage_table(wn, a.tw + a.tw_n, a.n_n, tid, S::T);
     pdl_wait();
     constexpr int NB = S::Lp / S::RL;
@@ -127,13 +127,18 @@ __global__ void __launch_bounds__(S::T, S::T >= 512 ? 2 : 4) short_rfft_forward_
     }
 }
 
-template <class S>
+template <class S, bool MASK>
 __global__ void __launch_bounds__(S::T, S::T >= 512 ? 2 : 4) short_rfft_inverse_kernel(LongArgs a, int batch) {
     pdl_launch_dependents();
     const int tid = threadIdx.x;
     float2 *buf = smem_short, *twf = buf + S::BUF, *wn = twf + S::Lp, *nat = wn + a.n_n;
-    stage_full(twf, a.tw, a.ffts[a.fft_B], tid, S::T);
-    stage_table(wn, a.tw + a.tw_n, a.n_n, tid, S::T);
+    stage_table(twf, a.tw + a.tw_full_B, S::Lp, tid, S::T);
+    constexpr float s = 0.5f / (float)S::Lp;
+    for (int i = tid; i < a.n_n; i += S::T) {   // the low part of the table of W_N times s
+        float2 w = __ldg(a.tw + a.tw_n + i);
+        if (i < (1 << a.log_n_c)) { w.x *= s; w.y *= s; }
+        wn[i] = w;
+    }
     // bin pairs (q, Lp - q): q = tid + u T for q <= Lp/2
     constexpr int NP = S::Lp / 2 / S::T > 0 ? S::Lp / 2 / S::T : 1;
     int32_t cq[NP], cm[NP];
@@ -149,29 +154,21 @@ __global__ void __launch_bounds__(S::T, S::T >= 512 ? 2 : 4) short_rfft_inverse_
     for (int ch = blockIdx.x; ch < batch; ch += gridDim.x) {
         const float2 *Y = a.Y + (long long)ch * a.y_pitch;
 #pragma unroll
-        for (int u = 0; u < NP; u += 2) {
-            constexpr int W = NP > 1 ? 2 : 1;
-            GatherLoads gq[W], gm[W];
-#pragma unroll
-            for (int v = 0; v < W; ++v) {
-                const int q = min(tid + (u + v) * S::T, S::Lp / 2);
-                gq[v] = gather_issue(a, Y, q, cq[u + v]);
-                gm[v] = gather_issue(a, Y, S::Lp - q, cm[u + v]);
-            }
-#pragma unroll
-            for (int v = 0; v < W; ++v) {
-                const int q = tid + (u + v) * S::T, m = S::Lp - q;
-                if (q > S::Lp / 2) break;
-                float2 zq, zm;
-                retangle_finish(a, Y, wn, q, gq[v], gm[v], zq, zm);
-                nat[q] = zq;
-                if (q != 0 && m != q) nat[m] = zm;
-            }
+        for (int u = 0; u < NP; ++u) {
+            const int q = tid + u * S::T, m = S::Lp - q;
+            if (q > S::Lp / 2) break;
+            float2 xq = plane_sum<MASK>(a, Y, q, cq[u]), xm = plane_sum<MASK>(a, Y, m, cm[u]), zq, zm;
+            if (q == 0) { xq.y = 0.f; xm.y = 0.f; }   // bins 0 and N/2 are made real
+            retangle(xq, xm, twiddle_s(wn, a.log_n_c, (uint32_t)q), s, zq, zm);
+            nat[q] = zq;
+            if (q != 0 && m != q) nat[m] = zm;
         }
         if (tid == 0 && NP * S::T <= S::Lp / 2) {   // the pair of the middle bin with itself
+            constexpr int q = S::Lp / 2;
+            const float2 xq = plane_sum<MASK>(a, Y, q, __ldg(a.cover + q));
             float2 zq, zm;
-            retangle_pair(a, Y, wn, S::Lp / 2, S::Lp / 2, zq, zm);
-            nat[S::Lp / 2] = zq;
+            retangle(xq, xq, twiddle_s(wn, a.log_n_c, (uint32_t)q), s, zq, zm);
+            nat[q] = zq;
         }
         __syncthreads();
         float re[S::RL], im[S::RL];
@@ -207,7 +204,7 @@ static ShortKernel short_kernel(const cqt_plan &p, bool forward) {
     ShortKernel k;
 #define X(S)                                                                                                             \
     if (p.lf.Lp == S::Lp && fp.st[0].radix == S::R0 && fp.st[1].radix == S::R1) {                                         \
-        k.fn = forward ? (const void *)short_rfft_forward_kernel<S> : (const void *)short_rfft_inverse_kernel<S>;         \
+        k.fn = forward ? (const void *)short_rfft_forward_kernel<S> : (cover_is_mask(p) ? (const void *)short_rfft_inverse_kernel<S, true> : (const void *)short_rfft_inverse_kernel<S, false>);         \
         k.threads = S::T;                                                                                                 \
         k.smem = sizeof(float2) * ((size_t)S::BUF + S::Lp + p.lf.n_n + (forward ? 0 : S::Lp));                            \
     }

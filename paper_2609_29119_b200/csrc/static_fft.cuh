@@ -1,176 +1,92 @@
-// Three-stage tile transform with every stride, radix and column count known at compile time (the common
-// shapes of the long FFT passes: 512 = 8 x 8 x 8 points on 16 or 18 interleaved columns).  Same data flow as the
-// run-time planned engine (first stage from a load functor, middle stage in shared memory, last stage to a
-// store functor or back to shared memory); with constant strides the index arithmetic folds into immediates.
+// Tile transforms with every radix, stride and column count known at compile time: LEN = R0 R1 R2 points (R2 = 1: two
+// stages) on NC interleaved columns in shared memory, T threads with 16 elements each.  In-place decimation in
+// frequency: stage 0 has butterflies over positions b + q LEN/R0, the last stage leaves frequency
+// k0 + R0 k1 (+ R0 R1 q) in butterfly b = k0 R1 + k1, element q.  The kernels fuse their loads into stage 0 and their
+// stores into the last stage, both on registers.
 #pragma once
 #include "engine.cuh"
 
 namespace cqt {
 
-template <int R0, int R1, int R2, int NC, int PITCH, int SIGN, bool COLFAST_IN, bool KEEP, class Load, class Store>
-__device__ __forceinline__ void tile_fft3(float2 *buf, const float2 *twf, Load load, Store store, int tid, int nthr) {
-    constexpr int M = R0 * R1 * R2;
-    constexpr int S0 = R1 * R2;
-    // ---- stage 0: operands from the functor, butterflies over positions b + q S0
-    {
-        constexpr int total = S0 * NC;
-        for (int base = 0; base < total; base += nthr) {
-            const int w = base + tid;
-            const bool active = w < total;
-            const int b = COLFAST_IN ? w / NC : w % S0;
-            const int col = COLFAST_IN ? w % NC : w / S0;
-            float re[R0], im[R0];
-            if (active) {
-#pragma unroll
-                for (int q = 0; q < R0; ++q) {
-                    const float2 v = load(b + q * S0, col);
-                    re[q] = v.x; im[q] = v.y;
-                }
-                if (SIGN < 0) Codelet<R0>::run(re, im); else Codelet<R0>::run(im, re);
-            }
-            if (base == 0) __syncthreads();   // staged tables become visible
-            if (active) {
-                apply_twiddle_direct<R0, SIGN>(twf, (uint32_t)b, re, im);
-                float2 *p = buf + b * PITCH + col;
-#pragma unroll
-                for (int q = 0; q < R0; ++q) p[q * S0 * PITCH] = make_float2(re[q], im[q]);
-            }
-        }
-    }
-    __syncthreads();
-    // ---- stage 1: sub-transforms of length S0, stride R2
-    {
-        constexpr int total = (M / R1) * NC;
-        for (int w = tid; w < total; w += nthr) {
-            const int b = w / NC, col = w % NC;
-            const int blk = b / R2, np = b % R2;
-            float2 *p = buf + (blk * S0 + np) * PITCH + col;
-            float re[R1], im[R1];
-#pragma unroll
-            for (int q = 0; q < R1; ++q) {
-                const float2 v = p[q * R2 * PITCH];
-                re[q] = v.x; im[q] = v.y;
-            }
-            if (SIGN < 0) Codelet<R1>::run(re, im); else Codelet<R1>::run(im, re);
-            apply_twiddle_direct<R1, SIGN>(twf, (uint32_t)(np * R0), re, im);
-#pragma unroll
-            for (int q = 0; q < R1; ++q) p[q * R2 * PITCH] = make_float2(re[q], im[q]);
-        }
-    }
-    __syncthreads();
-    // ---- stage 2: stride 1; butterfly b = k0 R1 + k1 holds frequencies k0 + R0 k1 + R0 R1 q
-    {
-        constexpr int total = (M / R2) * NC;
-        for (int w = tid; w < total; w += nthr) {
-            const int b = w / NC, col = w % NC;
-            float2 *p = buf + (b * R2) * PITCH + col;
-            float re[R2], im[R2];
-#pragma unroll
-            for (int q = 0; q < R2; ++q) {
-                const float2 v = p[q * PITCH];
-                re[q] = v.x; im[q] = v.y;
-            }
-            if (SIGN < 0) Codelet<R2>::run(re, im); else Codelet<R2>::run(im, re);
-            if (KEEP) {
-#pragma unroll
-                for (int q = 0; q < R2; ++q) p[q * PITCH] = make_float2(re[q], im[q]);
-            } else {
-                const int klow = b / R1 + R0 * (b % R1);
-#pragma unroll
-                for (int q = 0; q < R2; ++q) store(klow + q * (R0 * R1), col, make_float2(re[q], im[q]));
-            }
-        }
-    }
-    if (KEEP) __syncthreads();
-}
+enum { kPlain = 0, kOddPitch = 1, kSwizzle = 2 };   // shared-memory layouts of a tile
 
-// Two-stage variant: M = R0 * R1.
-template <int R0, int R1, int NC, int PITCH, int SIGN, bool COLFAST_IN, bool KEEP, class Load, class Store>
-__device__ __forceinline__ void tile_fft2(float2 *buf, const float2 *twf, Load load, Store store, int tid, int nthr) {
-    constexpr int M = R0 * R1;
-    constexpr int S0 = R1;
-    {
-        constexpr int total = S0 * NC;
-        for (int base = 0; base < total; base += nthr) {
-            const int w = base + tid;
-            const bool active = w < total;
-            const int b = COLFAST_IN ? w / NC : w % S0;
-            const int col = COLFAST_IN ? w % NC : w / S0;
-            float re[R0], im[R0];
-            if (active) {
-#pragma unroll
-                for (int q = 0; q < R0; ++q) {
-                    const float2 v = load(b + q * S0, col);
-                    re[q] = v.x; im[q] = v.y;
-                }
-                if (SIGN < 0) Codelet<R0>::run(re, im); else Codelet<R0>::run(im, re);
-            }
-            if (base == 0) __syncthreads();   // staged tables become visible
-            if (active) {
-                apply_twiddle_direct<R0, SIGN>(twf, (uint32_t)b, re, im);
-                float2 *p = buf + b * PITCH + col;
-#pragma unroll
-                for (int q = 0; q < R0; ++q) p[q * S0 * PITCH] = make_float2(re[q], im[q]);
-            }
-        }
+template <int LEN_, int R0_, int R1_, int R2_, int NC_, int LAYOUT_>
+struct TileShape {
+    static constexpr int LEN = LEN_, R0 = R0_, R1 = R1_, R2 = R2_, NC = NC_, LAYOUT = LAYOUT_;
+    static constexpr int S0 = LEN / R0, RL = R2 > 1 ? R2 : R1, NL = LEN / RL;   // NL: butterflies of the last stage
+    static constexpr int T = LEN * NC / 16;
+    // kOddPitch: consecutive positions of one column lie in different banks; kSwizzle: half-tiles (8 + 8 or 4 + 4
+    // columns) of consecutive positions do
+    static constexpr int PITCH = LAYOUT == kOddPitch ? NC + 1 : NC;
+    static constexpr int ELEMS = LEN * PITCH;
+    static_assert(R0 * R1 * R2 == LEN, "radices");
+    static __device__ __forceinline__ int at(int p, int col) {
+        if constexpr (LAYOUT == kSwizzle) return p * NC + (col ^ (NC == 16 ? (p & 1) << 3 : ((p >> 1) & 1) << 2));
+        else return p * PITCH + col;
     }
-    __syncthreads();
-    {
-        constexpr int total = (M / R1) * NC;   // butterfly b = k0 holds frequencies k0 + R0 q
-        for (int w = tid; w < total; w += nthr) {
-            const int b = w / NC, col = w % NC;
-            float2 *p = buf + (b * R1) * PITCH + col;
-            float re[R1], im[R1];
-#pragma unroll
-            for (int q = 0; q < R1; ++q) {
-                const float2 v = p[q * PITCH];
-                re[q] = v.x; im[q] = v.y;
-            }
-            if (SIGN < 0) Codelet<R1>::run(re, im); else Codelet<R1>::run(im, re);
-            if (KEEP) {
-#pragma unroll
-                for (int q = 0; q < R1; ++q) p[q * PITCH] = make_float2(re[q], im[q]);
-            } else {
-#pragma unroll
-                for (int q = 0; q < R1; ++q) store(b + q * R0, col, make_float2(re[q], im[q]));
-            }
-        }
+    // position of frequency k
+    static __device__ __forceinline__ int position(int k) {
+        if constexpr (R2 > 1) return ((k % R0) * R1 + (k / R0) % R1) * R2 + k / (R0 * R1);
+        else return (k % R0) * R1 + k / R0;
     }
-    if (KEEP) __syncthreads();
-}
-
-// Compile-time shape of a tile transform: R0 = 0 means "use the run-time planned engine", R2 = 1 two stages.
-template <int R0_, int R1_, int R2_, int NC_, int PITCH_>
-struct Shape {
-    static constexpr int R0 = R0_, R1 = R1_, R2 = R2_, NC = NC_, PITCH = PITCH_;
-    static constexpr bool is_static = R0_ > 0;
-    static __host__ __device__ __forceinline__ bool matches(const FftPlan &fp, int ncols) {
-        if constexpr (R0_ == 0) return true;
-        else if constexpr (R2_ == 1) return ncols == NC_ && fp.nstages == 2 && fp.st[0].radix == R0_ && fp.st[1].radix == R1_;
-        else return ncols == NC_ && fp.nstages == 3 && fp.st[0].radix == R0_ && fp.st[1].radix == R1_ && fp.st[2].radix == R2_;
-    }
-    // position of frequency k after a KEEP transform
-    static __device__ __forceinline__ uint32_t pos(const FftPlan &fp, uint32_t k) {
-        if constexpr (R0_ == 0) return dif_pos_pow2(fp, k);
-        else if constexpr (R2_ == 1) return (k % R0_) * R1_ + k / R0_;
-        else return ((k % R0_) * R1_ + (k / R0_) % R1_) * R2_ + k / (R0_ * R1_);
-    }
+    // lowest frequency of butterfly b of the last stage
+    static __device__ __forceinline__ int low(int b) { return R2 > 1 ? b / R1 + R0 * (b % R1) : b; }
 };
 
-template <class SH, int SIGN, bool COLFAST_IN, bool KEEP, class Load, class Store>
-__device__ __forceinline__ void tile_fft_static(float2 *buf, const float2 *twf, Load load, Store store, int tid, int nthr) {
-    if constexpr (SH::R2 == 1) tile_fft2<SH::R0, SH::R1, SH::NC, SH::PITCH, SIGN, COLFAST_IN, KEEP>(buf, twf, load, store, tid, nthr);
-    else tile_fft3<SH::R0, SH::R1, (SH::R2 > 1 ? SH::R2 : 2), SH::NC, SH::PITCH, SIGN, COLFAST_IN, KEEP>(buf, twf, load, store, tid, nthr);
+template <int R, int SIGN>
+__device__ __forceinline__ void dft(float (&re)[R], float (&im)[R]) {
+    if (SIGN < 0) Codelet<R>::run(re, im); else Codelet<R>::run(im, re);
 }
 
-// position of frequency k after tile_fft3 with KEEP: k = k0 + R0 k1 + R0 R1 k2 sits at (k0 R1 + k1) R2 + k2
-template <int R0, int R1, int R2>
-__device__ __forceinline__ int tile_fft3_pos(int k) {
-    return ((k % R0) * R1 + (k / R0) % R1) * R2 + k / (R0 * R1);
+// end of stage 0 for one butterfly: twiddles, store.  twf: full table of W_LEN
+template <class S, int SIGN>
+__device__ __forceinline__ void finish_first(float2 *buf, const float2 *twf, int b, int col, float (&re)[S::R0], float (&im)[S::R0]) {
+    dft<S::R0, SIGN>(re, im);
+    apply_twiddle_direct<S::R0, SIGN>(twf, (uint32_t)b, re, im);
+#pragma unroll
+    for (int q = 0; q < S::R0; ++q) buf[S::at(b + q * S::S0, col)] = make_float2(re[q], im[q]);
 }
 
-__device__ __forceinline__ bool plan_is(const FftPlan &fp, int r0, int r1, int r2) {
-    return fp.nstages == 3 && fp.st[0].radix == r0 && fp.st[1].radix == r1 && fp.st[2].radix == r2;
+// the stage between first and last, in shared memory
+template <class S, int SIGN>
+__device__ __forceinline__ void tile_middle(float2 *buf, const float2 *twf, int tid) {
+    if constexpr (S::R2 > 1) {
+        constexpr int R1 = S::R1, R2 = S::R2, units = S::LEN / R1 * S::NC / S::T;
+        static_assert(units * S::T * R1 == S::LEN * S::NC, "whole rounds");
+#pragma unroll
+        for (int u = 0; u < units; ++u) {
+            const int w = tid + u * S::T, col = w % S::NC, b = w / S::NC, np = b % R2, p = (b / R2) * S::S0 + np;
+            float re[R1], im[R1];
+#pragma unroll
+            for (int q = 0; q < R1; ++q) {
+                const float2 v = buf[S::at(p + q * R2, col)];
+                re[q] = v.x; im[q] = v.y;
+            }
+            dft<R1, SIGN>(re, im);
+            apply_twiddle_direct<R1, SIGN>(twf, (uint32_t)(np * S::R0), re, im);
+#pragma unroll
+            for (int q = 0; q < R1; ++q) buf[S::at(p + q * R2, col)] = make_float2(re[q], im[q]);
+        }
+        __syncthreads();
+    }
+}
+
+// butterfly b of the last stage of column col into registers
+template <class S, int SIGN>
+__device__ __forceinline__ void last_butterfly(const float2 *buf, int b, int col, float (&re)[S::RL], float (&im)[S::RL]) {
+#pragma unroll
+    for (int q = 0; q < S::RL; ++q) {
+        const float2 v = buf[S::at(b * S::RL + q, col)];
+        re[q] = v.x; im[q] = v.y;
+    }
+    dft<S::RL, SIGN>(re, im);
+}
+
+// log2 of the low part of a two-level table of n = 2^m entries (see append_twiddles in api.cu)
+__host__ __device__ constexpr int low_bits(int64_t n) {
+    int l = 0;
+    while ((1ll << (2 * l)) < n) ++l;
+    return l;
 }
 
 }  // namespace cqt
