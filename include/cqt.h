@@ -219,7 +219,7 @@ cqt_status cqt_analyse_static_ws(const cqt_plan *plan, const float *x, int64_t x
  *   x^ = F_N^{-1} sum_lambda diag(h_lambda) E_lambda^T F_M c_lambda, imaginary parts at DC and
  *   Nyquist dropped, negative frequencies by conjugate symmetry.  S T = I on real signals.
  * Per band: M-point DFT in shared memory, dual-window multiply, weighted bins written in bin
- * order to scratch; the first pass of the packed inverse FFT sums, per bin and in fixed band
+ * order to scratch; the first pass of the packed inverse FFT sums, per bin and in a fixed
  * order (no atomics, bitwise reproducible), the bands that cover it and applies Eq. retangle.
  */
 cqt_status cqt_synthesise(const cqt_plan *plan, const cqt_c64 *c, int64_t batch, int64_t valid_len,

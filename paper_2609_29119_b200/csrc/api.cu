@@ -317,6 +317,28 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     lf.n_n = (int)tw.size() - lf.tw_n;
     lf.x_pitch = (lf.Lp + 1 + 7) / 8 * 8;
 
+    // Plane of every band in the weighted-bin scratch: bands of one plane share no bin.  Range starts ascend, so the lowest
+    // plane that is free never exceeds the largest cover, and bins that few bands cover use the lowest planes only.
+    std::vector<int> plane_of(L.bands.size());
+    std::vector<int32_t> cover(N / 2 + 1, 0);
+    {
+        std::vector<int64_t> end((size_t)p->y_planes, -1);
+        for (size_t i = 0; i < L.bands.size(); ++i) {
+            const HostBand &hb = L.bands[i];
+            const int64_t s = hb.kc + hb.d0 + hb.j_lo - hb.zl, e = s + hb.zl + hb.n_in - 1 + hb.zr;
+            int pl = (int)(i % (size_t)p->y_planes);
+            if (cover_is_mask(*p)) {
+                pl = 0;
+                while (pl + 1 < p->y_planes && end[(size_t)pl] >= s) ++pl;
+                end[(size_t)pl] = e;
+                for (int64_t k = s; k <= e; ++k) cover[(size_t)k] |= 1 << pl;
+            }
+            plane_of[i] = pl;
+        }
+        if (!cover_is_mask(*p))
+            for (int64_t k = 0; k <= N / 2; ++k) cover[(size_t)k] = ((L.cover_lo[k] % p->y_planes) << 8) | L.cover_n[k];
+    }
+
     // ---- band records
     p->bands.resize(L.bands.size());
     for (size_t i = 0; i < L.bands.size(); ++i) {
@@ -324,7 +346,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         BandRec &br = p->bands[i];
         br.kc = (int32_t)hb.kc; br.d0 = (int32_t)hb.d0; br.S = (int32_t)hb.S; br.M = (int32_t)hb.M;
         br.tab_off = (int32_t)hb.tab_off; br.coeff_off = (int32_t)hb.coeff_off;
-        br.y_off = (int32_t)((int64_t)(i % p->y_planes) * p->y_plane);
+        br.y_off = (int32_t)((int64_t)plane_of[i] * p->y_plane);
         br.side = hb.side;
         br.fft = -1;
     }
@@ -504,14 +526,6 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
             tS[hb.tab_off + j] = (float)h;
             tTA[hb.tab_off + j] = (float)((double)N * g / (2.0 * (double)hb.M));
             tSA[hb.tab_off + j] = (float)(h * wk / (double)N);
-        }
-    }
-    std::vector<int32_t> cover(N / 2 + 1);
-    for (int64_t k = 0; k <= N / 2; ++k) {
-        cover[k] = ((L.cover_lo[k] % p->y_planes) << 8) | L.cover_n[k];
-        if (p->y_planes <= 3) {   // a bit mask of the planes instead (cover_is_mask)
-            cover[k] = 0;
-            for (int i = 0; i < L.cover_n[k]; ++i) cover[k] |= 1 << ((L.cover_lo[k] + i) % p->y_planes);
         }
     }
     cudaError_t e = cudaSuccess;

@@ -112,6 +112,9 @@ struct cqt_plan {
 
 namespace cqt {
 
+// the per-bin cover words of the plan are bit masks of planes (plane_sum in long_common.cuh)
+inline bool cover_is_mask(const cqt_plan &p) { return p.y_planes <= 31; }
+
 // table selectors of the band kernels
 enum { TAB_ANALYSIS = 0, TAB_SYNTHESIS = 1, TAB_ANALYSIS_ADJ = 2, TAB_SYNTHESIS_ADJ = 3 };
 
@@ -119,14 +122,18 @@ enum { TAB_ANALYSIS = 0, TAB_SYNTHESIS = 1, TAB_ANALYSIS_ADJ = 2, TAB_SYNTHESIS_
 void note_launch(const cqt_plan &p, const char *name, cudaStream_t st);
 
 // long_fft_forward.cu, long_fft_inverse.cu
-// Input of the forward long FFT taken from a ring buffer of a stream instead of signal rows (sliced transform, slice
-// cut fused into the load): row r = slice r / channels of channel r % channels; sample i of that slice is
-// win[i] * ring[channel * ring_len + (first + (r / channels) * hop + i) mod ring_len], zero before the stream's start.
+// Input of the forward long FFT taken from a stream instead of signal rows (sliced transform, slice cut fused into the
+// load): row r = slice r / channels of channel r % channels; sample i of that slice is win[i] * stream sample
+// first + (r / channels) * hop + i, zero before the stream's start.  Stream samples from index new_first on are in the
+// caller's buffer (fresh, zeros if null), older ones in the ring (sample n at n mod ring_len).  The last slice of the
+// call also stores its fresh samples of index >= keep_from in the ring, where later slices find them.
 struct SliceSource {
-    const float *ring;
+    float *ring;
     const float *win;
     long long ring_len, first, hop;
-    int channels;
+    int channels, slices;
+    const float *fresh;
+    long long fresh_stride, new_first, keep_from;
 };
 // src != nullptr needs a plan whose long FFT runs in two passes (can_fuse_slice_cut)
 cudaError_t launch_rfft_forward(const cqt_plan &p, const float *x, int64_t x_stride, int64_t batch, int64_t valid_len,

@@ -25,13 +25,16 @@ struct LongArgs {
     int planes;
     const int32_t *cover;
     int *dbg;
-    // sliced source (forward column pass of the streaming form): row r is slice r / channels of channel r % channels,
-    // its sample i is slice_win[i] * ring[channel][(slice_first + (r / channels) * hop + i) mod ring_len], zero
-    // before the start of the stream
-    const float *ring;
+    // sliced source (forward column pass of the streaming form, see SliceSource)
+    float *ring;
     const float *slice_win;
-    long long ring_len, slice_first, hop;
-    int channels;
+    int ring_len, ring_base;      // position of the first slice's sample 0 in the ring
+    int lead;                     // samples of the first slice before the start of the stream
+    int hop, channels, slices;
+    const float *fresh;
+    long long fresh_stride;
+    int fresh_at, keep_at;        // sample of the first slice / of the last slice where the fresh / the kept ones begin
+    int fresh_pairs;              // fresh samples can be read in pairs
 };
 
 __device__ __forceinline__ float2 load_packed(const float *row, int j, int valid_len, int aligned) {
@@ -54,46 +57,73 @@ __device__ __forceinline__ void store_packed(float *row, int j, float2 v, int va
     }
 }
 
-__device__ __forceinline__ void stage_table(float2 *dst, const float2 *__restrict__ src, int n, int tid, int nthr) {
-    for (int i = tid; i < n; i += nthr) dst[i] = __ldg(src + i);
+// copies N entries of a table into shared memory on T threads, the first `scaled` of them times `scale`: all loads of a
+// thread are issued before any is stored, one trip to the L2 instead of one per round
+template <int N, int T>
+__device__ __forceinline__ void stage_table(float2 *dst, const float2 *__restrict__ src, int tid, int scaled = 0, float scale = 1.f) {
+    constexpr int rounds = (N + T - 1) / T;
+    float2 v[rounds];
+#pragma unroll
+    for (int i = 0; i < rounds; ++i)
+        if (tid + i * T < N) v[i] = __ldg(src + tid + i * T);
+#pragma unroll
+    for (int i = 0; i < rounds; ++i) {
+        const int e = tid + i * T;
+        if (e < scaled) { v[i].x *= scale; v[i].y *= scale; }
+        if (e < N) dst[e] = v[i];
+    }
 }
 
+// log2 of the low part of a two-level table of n = 2^m entries (see append_twiddles in api.cu), and its entry count
+__host__ __device__ constexpr int low_bits(int64_t n) {
+    int l = 0;
+    while ((1ll << (2 * l)) < n) ++l;
+    return l;
+}
+__host__ __device__ constexpr int two_level_entries(int64_t n) { return (int)((1ll << low_bits(n)) + (n >> low_bits(n))); }
+
 // ---------------------------------------------------------------- inverse: overlap-add
-// Sum of the planes that hold bin k.  MASK (at most three planes): the cover word is a bit mask of them; else it is
+// Sum of the planes that hold bin k.  MASK (at most 31 planes): the cover word is a bit mask of them; else it is
 // (plane of the first covering band << 8) | number of covering bands, band i of the range in plane (first + i) mod
-// planes.  The order is fixed either way.  The first three loads are issued before any value is used.
+// planes.  The order is fixed either way.  plane_first: three of them (the lowest three planes), without a branch, so
+// that the loads of several bins are in flight together; plane_rest adds the others (bins of the lowest bands, where
+// the minimum width makes many overlap).
 template <bool MASK>
-__device__ __forceinline__ float2 plane_sum(const LongArgs &a, const float2 *__restrict__ Y, int k, int32_t cover) {
+__device__ __forceinline__ float2 plane_first(const LongArgs &a, const float2 *Y, int k, int32_t cover) {
     float2 v[3];
-    if constexpr (MASK) {
+    const int n = cover & 255;
+    int plane = cover >> 8;
 #pragma unroll
-        for (int i = 0; i < 3; ++i) v[i] = (cover >> i) & 1 ? ld_data(Y + i * a.y_plane + k) : make_float2(0.f, 0.f);
-        return make_float2(v[0].x + v[1].x + v[2].x, v[0].y + v[1].y + v[2].y);
-    } else {
-        const int plane_len = (int)a.y_plane, wrap = a.planes * plane_len;
-        int n = cover & 255, off = (cover >> 8) * plane_len + k;
-        if (!CQT_CHK(a.dbg, 206, n, a.planes + 1)) n = 0;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            v[i] = i < n ? ld_data(Y + off) : make_float2(0.f, 0.f);
-            off += plane_len;
-            if (off >= wrap) off -= wrap;
+    for (int i = 0; i < 3; ++i) {
+        if constexpr (MASK) v[i] = (cover >> i) & 1 ? ld_data(Y + i * a.y_plane + k) : make_float2(0.f, 0.f);
+        else {
+            v[i] = i < n && CQT_CHK(a.dbg, 206, n, a.planes + 1) ? ld_data(Y + plane * a.y_plane + k) : make_float2(0.f, 0.f);
+            if (++plane >= a.planes) plane -= a.planes;
         }
-        float2 acc = make_float2(v[0].x + v[1].x + v[2].x, v[0].y + v[1].y + v[2].y);
-        // bins of the lowest bands, where the minimum width makes many of them overlap: a second round of loads
-        for (int i = 3; i < n; i += 4) {
-            float2 w[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                w[j] = i + j < n ? ld_data(Y + off) : make_float2(0.f, 0.f);
-                off += plane_len;
-                if (off >= wrap) off -= wrap;
-            }
-            acc.x += (w[0].x + w[1].x) + (w[2].x + w[3].x);
-            acc.y += (w[0].y + w[1].y) + (w[2].y + w[3].y);
-        }
-        return acc;
     }
+    return make_float2(v[0].x + v[1].x + v[2].x, v[0].y + v[1].y + v[2].y);
+}
+template <bool MASK>
+__device__ __forceinline__ void plane_rest(const LongArgs &a, const float2 *Y, int k, int32_t cover, float2 &acc) {
+    int left = MASK ? cover >> 3 : (cover & 255) - 3, plane = MASK ? 3 : (cover >> 8) + 3;
+    while (left > 0) {
+        float2 w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (!MASK && plane >= a.planes) plane -= a.planes;
+            w[j] = (MASK ? left & 1 : left > 0) && CQT_CHK(a.dbg, 207, plane, a.planes) ? ld_data(Y + plane * a.y_plane + k) : make_float2(0.f, 0.f);
+            ++plane;
+            left = MASK ? left >> 1 : left - 1;
+        }
+        acc.x += (w[0].x + w[1].x) + (w[2].x + w[3].x);
+        acc.y += (w[0].y + w[1].y) + (w[2].y + w[3].y);
+    }
+}
+template <bool MASK>
+__device__ __forceinline__ float2 plane_sum(const LongArgs &a, const float2 *Y, int k, int32_t cover) {
+    float2 acc = plane_first<MASK>(a, Y, k, cover);
+    plane_rest<MASK>(a, Y, k, cover, acc);
+    return acc;
 }
 
 // One pair (q, m = Lp - q) of packed bins from the half-spectrum bins X_q, X_m (Eq. retangle, w_{Lp-q} = -conj w_q):
@@ -129,9 +159,6 @@ inline LongArgs base_args(const cqt_plan &p, int64_t valid_len, int64_t x_stride
     a.dbg = p.d.dbg;
     return a;
 }
-
-// the cover words of the plan are bit masks of planes (see plane_sum)
-inline bool cover_is_mask(const cqt_plan &p) { return p.y_planes <= 3; }
 
 // one-pass real FFTs of short signals (short_fft.cu)
 cudaError_t launch_short_rfft_forward(const cqt_plan &p, LongArgs &a, int64_t batch, cudaStream_t st);

@@ -11,6 +11,8 @@
 // Lengths, radices, tile widths and strides are compile-time (A and B follow from N), a thread keeps its 16 loads in
 // flight before the first butterfly, and there is one exchange through shared memory per stage and none for the fold.
 // 32 signals of N = 2^19 (A = B = 512) before, with run-time strides and the fold through shared memory: 45 us + 50 us.
+#include <algorithm>
+
 #include "long_passes.cuh"
 
 namespace cqt {
@@ -26,11 +28,20 @@ __global__ void __launch_bounds__(ColsForward<A>::T, 1024 / ColsForward<A>::T) r
     pdl_launch_dependents();
     const int tid = threadIdx.x, col = tid % S::NC, j2 = blockIdx.x * S::NC + col, ch = blockIdx.y;
     float2 *buf = smem_long, *tws = buf + S::ELEMS, *wl = tws + A;
-    stage_table(tws, a.tw + a.tw_full_A, A, tid, S::T);
-    stage_table(wl, a.tw + a.tw_lp, a.n_lp, tid, S::T);
-    pdl_wait();   // the tables above belong to the plan; what follows reads the predecessor's output
+    stage_table<A, S::T>(tws, a.tw + a.tw_full_A, tid);
+    stage_table<two_level_entries(A * B), S::T>(wl, a.tw + a.tw_lp, tid);
     constexpr int R0 = S::R0, units = S::S0 * S::NC / S::T, step = S::T / S::NC;
     float re[units][R0], im[units][R0];
+    if constexpr (SLICED) {
+#pragma unroll
+        for (int u = 0; u < units; ++u)
+#pragma unroll
+            for (int q = 0; q < R0; ++q) {
+                const float2 w = __ldg(reinterpret_cast<const float2 *>(a.slice_win) + (tid / S::NC + u * step + q * S::S0) * B + j2);
+                re[u][q] = w.x; im[u][q] = w.y;
+            }
+    }
+    pdl_wait();   // the tables above belong to the plan; what follows reads the predecessor's output
     auto load_all = [&](auto load) {
 #pragma unroll
         for (int u = 0; u < units; ++u)
@@ -41,23 +52,39 @@ __global__ void __launch_bounds__(ColsForward<A>::T, 1024 / ColsForward<A>::T) r
             }
     };
     if constexpr (SLICED) {
-        const int s_rel = ch / a.channels, chan = ch - s_rel * a.channels;
-        const long long first = a.slice_first + (long long)s_rel * a.hop;   // stream index of the slice's sample 0
-        // position of sample 0 in the ring; the slice is no longer than the ring, so one conditional subtraction wraps.
-        // Hops and ring lengths are even: a pair of samples never straddles the end of the ring or the stream's start
-        const int R = (int)a.ring_len;
-        const int base = (int)(((first % a.ring_len) + a.ring_len) % a.ring_len);
-        const int lead = first < 0 ? (int)(-first) : 0;                      // samples before the start of the stream
-        const float *ring = a.ring + (long long)chan * a.ring_len;
-        load_all([&](int j1) -> float2 {
-            const int i = 2 * (j1 * B + j2);
-            if (i < lead) return make_float2(0.f, 0.f);
+        // re, im hold the window; it is constant for the stream's life and was fetched before the wait
+        const int s_rel = ch / a.channels, chan = ch - s_rel * a.channels, R = a.ring_len;
+        int base = a.ring_base + s_rel * a.hop;       // one wrap at most: the ring is longer than the slices of a call
+        if (base >= R) base -= R;
+        const int lead = a.lead - s_rel * a.hop, fresh_at = a.fresh_at - s_rel * a.hop;
+        const int keep = s_rel == a.slices - 1 ? max(a.keep_at, fresh_at) : 1 << 30;
+        float *ring = a.ring + (long long)chan * R;
+        const float *fresh = a.fresh + (long long)chan * a.fresh_stride - fresh_at;
+        auto sample = [&](int i) -> float {
+            if (i < lead || (i >= fresh_at && !a.fresh)) return 0.f;
             int p = base + i;
             if (p >= R) p -= R;
-            if (!CQT_CHK(a.dbg, 212, p + 1, R)) return make_float2(0.f, 0.f);
-            const float2 w = __ldg(reinterpret_cast<const float2 *>(a.slice_win + i)), x = ld_data(reinterpret_cast<const float2 *>(ring + p));
-            return make_float2(w.x * x.x, w.y * x.y);
-        });
+            if (!CQT_CHK(a.dbg, 212, p, R)) return 0.f;
+            return i >= fresh_at ? __ldcs(fresh + i) : __ldcs(ring + p);
+        };
+#pragma unroll
+        for (int u = 0; u < units; ++u)
+#pragma unroll
+            for (int q = 0; q < R0; ++q) {
+                const int i = 2 * ((tid / S::NC + u * step + q * S::S0) * B + j2);
+                int p = base + i;
+                if (p >= R) p -= R;
+                float2 v;
+                // hops, ring lengths and the start of the stream are even: only fresh samples may come unpaired
+                if (i >= lead && i + 1 < fresh_at && CQT_CHK(a.dbg, 213, p + 1, R)) v = ld_data(reinterpret_cast<const float2 *>(ring + p));
+                else if (i >= fresh_at && a.fresh_pairs) v = __ldcs(reinterpret_cast<const float2 *>(fresh + i));
+                else v = make_float2(sample(i), sample(i + 1));
+                if (i + 1 >= keep && CQT_CHK(a.dbg, 214, p + 1, R)) {
+                    if (i >= keep) ring[p] = v.x;
+                    ring[p + 1] = v.y;
+                }
+                re[u][q] *= v.x; im[u][q] *= v.y;
+            }
     } else {
         const float *row = a.x_in + (long long)ch * a.x_stride + 2 * j2;
         const int left = a.valid_len - 2 * j2;   // samples of this column pair's row run that exist
@@ -82,7 +109,7 @@ __global__ void __launch_bounds__(ColsForward<A>::T, 1024 / ColsForward<A>::T) r
     tile_middle<S, -1>(buf, tws, tid);
     float2 *T = a.T + (long long)ch * a.t_pitch + j2;
     constexpr int last = S::NL * S::NC / S::T;
-#pragma unroll
+#pragma unroll 1
     for (int u = 0; u < last; ++u) {
         const int b = tid / S::NC + u * step, low = S::low(b);
         float x[S::RL], y[S::RL];
@@ -113,13 +140,9 @@ __global__ void __launch_bounds__(RowsForward<B>::T, 1024 / RowsForward<B>::T) r
     pdl_launch_dependents();
     const int tid = threadIdx.x, ch = blockIdx.y, t = blockIdx.x;
     float2 *buf = smem_long, *tws = buf + S::ELEMS, *wn = tws + B;
-    stage_table(tws, a.tw + a.tw_full_B, B, tid, S::T);
+    stage_table<B, S::T>(tws, a.tw + a.tw_full_B, tid);
     // the low part of the table of W_N halved: the fold needs w / 2
-    for (int i = tid; i < a.n_n; i += S::T) {
-        float2 w = __ldg(a.tw + a.tw_n + i);
-        if (i < (1 << low_bits(N))) { w.x *= 0.5f; w.y *= 0.5f; }
-        wn[i] = w;
-    }
+    stage_table<two_level_entries(N), S::T>(wn, a.tw + a.tw_n, tid, 1 << low_bits(N), 0.5f);
     pdl_wait();   // the tables above belong to the plan; what follows reads the predecessor's output
     {
         const float2 *T = a.T + (long long)ch * a.t_pitch;
@@ -234,9 +257,19 @@ cudaError_t launch_rfft_forward(const cqt_plan &p, const float *x, int64_t x_str
         return e;
     }
     if (src) {
-        if (src->channels <= 0 || src->ring_len < p.N || (src->ring_len & 1) || (src->first & 1) || (src->hop & 1)) return cudaErrorInvalidValue;
+        const long long R = src->ring_len, last = src->first + (src->slices - 1) * src->hop;
+        if (src->channels <= 0 || R < p.N + (src->slices - 1) * src->hop || R > INT32_MAX / 2 || (R & 1) || (src->first & 1) || (src->hop & 1))
+            return cudaErrorInvalidValue;
+        auto clamp = [](long long v) { return (int)std::max<long long>(-(1 << 30), std::min<long long>(1 << 30, v)); };
         a.ring = src->ring; a.slice_win = src->win;
-        a.ring_len = src->ring_len; a.slice_first = src->first; a.hop = src->hop; a.channels = src->channels;
+        a.ring_len = (int)R;
+        a.ring_base = (int)(((src->first % R) + R) % R);
+        a.lead = clamp(-src->first);
+        a.hop = (int)src->hop; a.channels = src->channels; a.slices = src->slices;
+        a.fresh = src->fresh; a.fresh_stride = src->fresh_stride;
+        a.fresh_at = clamp(src->new_first - src->first);
+        a.keep_at = clamp(src->keep_from - last);
+        a.fresh_pairs = src->fresh && (a.fresh_at & 1) == 0 && (reinterpret_cast<uintptr_t>(src->fresh) & 7) == 0 && (src->fresh_stride & 1) == 0;
     }
     const ForwardKernels k = forward_kernels(p);
     cudaError_t e = launch_long(src ? k.cols_sliced : k.cols, k.cols_tiles, batch, k.cols_threads, k.cols_smem, a, st);

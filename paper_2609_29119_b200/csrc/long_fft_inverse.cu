@@ -29,15 +29,11 @@ __global__ void __launch_bounds__(RowsInverse<B>::T, 1024 / RowsInverse<B>::T) i
     constexpr float s = 0.5f / (float)Lp;    // a power of two
     pdl_launch_dependents();
     const int tid = threadIdx.x, ch = blockIdx.y, t = blockIdx.x;
-    float2 *buf = smem_long, *tws = buf + S::ELEMS, *wn = tws + B, *wl = wn + a.n_n;
-    stage_table(tws, a.tw + a.tw_full_B, B, tid, S::T);
+    float2 *buf = smem_long, *tws = buf + S::ELEMS, *wn = tws + B, *wl = wn + two_level_entries(N);
+    stage_table<B, S::T>(tws, a.tw + a.tw_full_B, tid);
     // the low part of the table of W_N times s
-    for (int i = tid; i < a.n_n; i += S::T) {
-        float2 w = __ldg(a.tw + a.tw_n + i);
-        if (i < (1 << C)) { w.x *= s; w.y *= s; }
-        wn[i] = w;
-    }
-    stage_table(wl, a.tw + a.tw_lp, a.n_lp, tid, S::T);
+    stage_table<two_level_entries(N), S::T>(wn, a.tw + a.tw_n, tid, 1 << C, s);
+    stage_table<two_level_entries(Lp), S::T>(wl, a.tw + a.tw_lp, tid);
     // thread: column r and its mirror r + TW; unit u: butterfly b = b0 + u step of the one, S0 - 1 - b of the other, whose
     // operands are the bins k = k0 + A (u step + q S0) and Lp - k
     const int r = tid % TW, b0 = tid / TW;
@@ -85,12 +81,20 @@ __global__ void __launch_bounds__(RowsInverse<B>::T, 1024 / RowsInverse<B>::T) i
             const int k = k0 + A * u * step;
             const float2 wlo = wn[k & ((1 << C) - 1)];
             const float2 *whi = wn + (1 << C) + (k >> C);
+            float2 vq[R0], vm[R0];
 #pragma unroll
             for (int q = 0; q < R0; ++q) {
                 const int kq = k + q * (A * S0);
-                const float2 vq = plane_sum<MASK>(a, Y, kq, cq[u][q]), vm = plane_sum<MASK>(a, Y, Lp - kq, cm[u][q]);
+                vq[q] = plane_first<MASK>(a, Y, kq, cq[u][q]);
+                vm[q] = plane_first<MASK>(a, Y, Lp - kq, cm[u][q]);
+            }
+#pragma unroll
+            for (int q = 0; q < R0; ++q) {
+                const int kq = k + q * (A * S0);
+                plane_rest<MASK>(a, Y, kq, cq[u][q], vq[q]);
+                plane_rest<MASK>(a, Y, Lp - kq, cm[u][q], vm[q]);
                 float2 zq, zm;
-                retangle(vq, vm, cmul(wlo, whi[q * ((A * S0) >> C)]), s, zq, zm);
+                retangle(vq[q], vm[q], cmul(wlo, whi[q * ((A * S0) >> C)]), s, zq, zm);
                 x[q] = zq.x; y[q] = zq.y;
                 xm[R0 - 1 - q] = zm.x; ym[R0 - 1 - q] = zm.y;
             }
@@ -104,7 +108,7 @@ __global__ void __launch_bounds__(RowsInverse<B>::T, 1024 / RowsInverse<B>::T) i
     const int col = tid % S::NC, q1 = row_of<A, TW>(t, col);
     float2 *T = a.T + (long long)ch * a.t_pitch + q1;
     constexpr int last = S::NL * S::NC / S::T;
-#pragma unroll
+#pragma unroll 1
     for (int u = 0; u < last; ++u) {
         const int b = tid / S::NC + u * (S::T / S::NC), low = S::low(b);
         float x[S::RL], y[S::RL];
@@ -124,7 +128,7 @@ __global__ void __launch_bounds__(ColsInverse<A>::T, 1024 / ColsInverse<A>::T) i
     pdl_launch_dependents();
     const int tid = threadIdx.x, j2_0 = blockIdx.x * S::NC, ch = blockIdx.y;
     float2 *buf = smem_long, *tws = buf + S::ELEMS;
-    stage_table(tws, a.tw + a.tw_full_A, A, tid, S::T);
+    stage_table<A, S::T>(tws, a.tw + a.tw_full_A, tid);
     pdl_wait();   // the table belongs to the plan; what follows reads the predecessor's output
     {
         // a column of Tinv[j2][q1] is a contiguous run: consecutive threads take consecutive q1
@@ -149,7 +153,7 @@ __global__ void __launch_bounds__(ColsInverse<A>::T, 1024 / ColsInverse<A>::T) i
     const int col = tid % S::NC, j2 = j2_0 + col, left = a.valid_len - 2 * j2;
     float *row = a.x_out + (long long)ch * a.x_stride + 2 * j2;
     constexpr int last = S::NL * S::NC / S::T;
-#pragma unroll
+#pragma unroll 1
     for (int u = 0; u < last; ++u) {
         const int b = tid / S::NC + u * (S::T / S::NC), low = S::low(b);
         float x[S::RL], y[S::RL];

@@ -98,8 +98,8 @@ __global__ void __launch_bounds__(S::T, S::T >= 512 ? 2 : 4) short_rfft_forward_
     pdl_launch_dependents();
     const int tid = threadIdx.x;
     float2 *buf = smem_short, *twf = buf + S::BUF, *wn = twf + S::Lp;
-    stage_table(twf, a.tw + a.tw_full_B, S::Lp, tid, S::T);
-    stage_table(wn, a.tw + a.tw_n, a.n_n, tid, S::T);
+    stage_table<S::Lp, S::T>(twf, a.tw + a.tw_full_B, tid);
+    stage_table<two_level_entries(2 * S::Lp), S::T>(wn, a.tw + a.tw_n, tid);
     pdl_wait();
     constexpr int NB = S::Lp / S::RL;
     for (int ch = blockIdx.x; ch < batch; ch += gridDim.x) {
@@ -132,13 +132,10 @@ __global__ void __launch_bounds__(S::T, S::T >= 512 ? 2 : 4) short_rfft_inverse_
     pdl_launch_dependents();
     const int tid = threadIdx.x;
     float2 *buf = smem_short, *twf = buf + S::BUF, *wn = twf + S::Lp, *nat = wn + a.n_n;
-    stage_table(twf, a.tw + a.tw_full_B, S::Lp, tid, S::T);
+    stage_table<S::Lp, S::T>(twf, a.tw + a.tw_full_B, tid);
     constexpr float s = 0.5f / (float)S::Lp;
-    for (int i = tid; i < a.n_n; i += S::T) {   // the low part of the table of W_N times s
-        float2 w = __ldg(a.tw + a.tw_n + i);
-        if (i < (1 << a.log_n_c)) { w.x *= s; w.y *= s; }
-        wn[i] = w;
-    }
+    // the low part of the table of W_N times s
+    stage_table<two_level_entries(2 * S::Lp), S::T>(wn, a.tw + a.tw_n, tid, 1 << low_bits(2 * S::Lp), s);
     // bin pairs (q, Lp - q): q = tid + u T for q <= Lp/2
     constexpr int NP = S::Lp / 2 / S::T > 0 ? S::Lp / 2 / S::T : 1;
     int32_t cq[NP], cm[NP];
@@ -153,13 +150,22 @@ __global__ void __launch_bounds__(S::T, S::T >= 512 ? 2 : 4) short_rfft_inverse_
     pdl_wait();
     for (int ch = blockIdx.x; ch < batch; ch += gridDim.x) {
         const float2 *Y = a.Y + (long long)ch * a.y_pitch;
+        float2 vq[NP], vm[NP];
+#pragma unroll
+        for (int u = 0; u < NP; ++u) {
+            const int q = min(tid + u * S::T, S::Lp / 2);
+            vq[u] = plane_first<MASK>(a, Y, q, cq[u]);
+            vm[u] = plane_first<MASK>(a, Y, S::Lp - q, cm[u]);
+        }
 #pragma unroll
         for (int u = 0; u < NP; ++u) {
             const int q = tid + u * S::T, m = S::Lp - q;
             if (q > S::Lp / 2) break;
-            float2 xq = plane_sum<MASK>(a, Y, q, cq[u]), xm = plane_sum<MASK>(a, Y, m, cm[u]), zq, zm;
-            if (q == 0) { xq.y = 0.f; xm.y = 0.f; }   // bins 0 and N/2 are made real
-            retangle(xq, xm, twiddle_s(wn, a.log_n_c, (uint32_t)q), s, zq, zm);
+            plane_rest<MASK>(a, Y, q, cq[u], vq[u]);
+            plane_rest<MASK>(a, Y, m, cm[u], vm[u]);
+            if (q == 0) { vq[u].y = 0.f; vm[u].y = 0.f; }   // bins 0 and N/2 are made real
+            float2 zq, zm;
+            retangle(vq[u], vm[u], twiddle_s(wn, a.log_n_c, (uint32_t)q), s, zq, zm);
             nat[q] = zq;
             if (q != 0 && m != q) nat[m] = zm;
         }

@@ -78,24 +78,35 @@ __global__ void slicq_cut_kernel(const float *ring, long long R, const float *w,
     }
 }
 
-// Overlap-add of reconstructed slices s0 .. s1 into the output ring, older slice first:
-// block b = [bH, (b+1)H) = second half of slice b (or what the ring already holds when b < s0)
-//                         + first half of slice b + 1 (when b + 1 <= s1).
-__global__ void slicq_ola_kernel(const float *stage, float *ring, long long R, long long sl, long long H, long long s0,
-                                 long long s1, int C) {
+// Overlap-add of reconstructed slices s0 .. s1, older slice first, and emission of finished frames, in one pass over the
+// frames first .. (s1 + 1) H - 1.  Block b = [bH, (b+1)H) = second half of slice b (or what the ring already holds when
+// b < s0) + first half of slice b + 1 (when b + 1 <= s1).  Frames emit_from .. emit_to - 1 are finished and go to y
+// (frame n at y[n - emit_from]); the others of blocks s0 - 1 .. s1 go to the ring; frames below block s0 - 1 are only
+// emitted (they waited in the ring).
+__global__ void slicq_ola_kernel(const float *stage, float *ring, long long R, long long sl, long long H, long long s0, long long s1, int C,
+                                 long long first, long long emit_from, long long emit_to, float *y, long long y_stride) {
     cqt::pdl_launch_dependents();
     cqt::pdl_wait();
     const int c = blockIdx.y;
-    const long long lo = (s0 - 1) * H, hi = (s1 + 1) * H;
-    for (long long n = lo + blockIdx.x * (long long)blockDim.x + threadIdx.x; n < hi; n += (long long)gridDim.x * blockDim.x) {
+    const long long hi = (s1 + 1) * H;
+    for (long long n = first + blockIdx.x * (long long)blockDim.x + threadIdx.x; n < hi; n += (long long)gridDim.x * blockDim.x) {
         if (n < 0) continue;
+        const bool emit = n >= emit_from && n < emit_to;
         const long long b = n / H, r = n - b * H;
-        float v = b >= s0 ? stage[((b - s0) * C + c) * sl + H + r] : ring[c * R + n % R];
-        if (b + 1 <= s1) v += stage[((b + 1 - s0) * C + c) * sl + r];
-        ring[c * R + n % R] = v;
+        float v;
+        if (b < s0 - 1) {
+            if (!emit) continue;
+            v = ring[c * R + n % R];
+        } else {
+            v = b >= s0 ? stage[((b - s0) * C + c) * sl + H + r] : ring[c * R + n % R];
+            if (b + 1 <= s1) v += stage[((b + 1 - s0) * C + c) * sl + r];
+        }
+        if (emit) y[c * y_stride + n - emit_from] = v;
+        else ring[c * R + n % R] = v;
     }
 }
 
+// Frames that were finished by an earlier call.
 __global__ void slicq_emit_kernel(const float *ring, long long R, long long pos, float *y, long long y_stride, long long n) {
     cqt::pdl_launch_dependents();
     cqt::pdl_wait();
@@ -136,20 +147,38 @@ __global__ void slicq_assemble_kernel(const cqt_c64 *coef, long long cc, long lo
 
 unsigned blocks_for(long long n) { return (unsigned)std::min<long long>(1024, std::max<long long>(1, (n + 255) / 256)); }
 
-cqt_status analyse_ready(cqt_slicq *s, cudaStream_t st) {
-    const int64_t ready = s->n_in / s->H;   // slices 0 .. ready - 1 are complete: (s + 1) H <= n_in
+cqt_status ingest(cqt_slicq *s, const float *x, int64_t x_stride, int64_t first, int64_t n, cudaStream_t st) {
+    if (n <= 0) return CQT_OK;
+    dim3 grid(blocks_for(n), (unsigned)s->C);
+    return cqt::launch_kernel_args(slicq_ingest_kernel, grid, dim3(256), 0, st, x, x_stride, s->d_in, s->ring_in, first, n, x ? 0 : 1) == cudaSuccess
+               ? CQT_OK : CQT_ERR_CUDA;
+}
+
+// Analyses every complete slice: 0 .. n_in / H - 1 ((s + 1) H <= n_in).  Samples from stream index new_first on are still
+// in the caller's buffer (fresh; null: zeros), the older ones in the ring.
+cqt_status analyse_ready(cqt_slicq *s, const float *fresh, int64_t fresh_stride, int64_t new_first, cudaStream_t st) {
+    const int64_t ready = s->n_in / s->H;
+    if (s->next_slice >= ready) return ingest(s, fresh, fresh_stride, new_first, s->n_in - new_first, st);
+    const bool fused = cqt::can_fuse_slice_cut(*s->plan) && s->ring_in >= s->sl;
+    // one-pass lengths cut the slices out of the ring in a kernel of their own
+    if (!fused) {
+        const cqt_status r = ingest(s, fresh, fresh_stride, new_first, s->n_in - new_first, st);
+        if (r != CQT_OK) return r;
+    }
     while (s->next_slice < ready) {
         // slices whose coefficient slots are consecutive in memory
         const int64_t slot = s->next_slice % s->K;
         const int64_t cnt = std::min<int64_t>(ready - s->next_slice, s->K - slot);
         cqt_c64 *coef = s->d_coef + slot * s->C * cqt_plan_coeff_count(s->plan);
         cqt_status r;
-        if (cqt::can_fuse_slice_cut(*s->plan) && s->ring_in >= s->sl) {
-            // the slice cut (window x ring samples) happens in the load of the long FFT's first pass
-            const cqt::SliceSource src{s->d_in, s->d_win, s->ring_in, s->next_slice * s->H - s->H, s->H, s->C};
+        if (fused) {
+            // the slice cut (window x stream samples) happens in the load of the long FFT's first pass, which also puts
+            // the fresh samples that the next slice needs into the ring
+            const int64_t keep = s->next_slice + cnt == ready ? (ready - 1) * s->H : INT64_MAX / 2;
+            const cqt::SliceSource src{s->d_in, s->d_win, s->ring_in, s->next_slice * s->H - s->H, s->H, s->C, (int)cnt,
+                                       fresh, fresh_stride, new_first, keep};
             r = cqt::analyse_slices(s->plan, src, cnt * s->C, coef, s->d_ws, s->ws_bytes, st);
         } else {
-            // short slices (one-pass long FFT): a kernel of its own writes the windowed slices to a staging buffer
             dim3 grid(blocks_for(s->sl), (unsigned)(cnt * s->C));
             if (cqt::launch_kernel_args(slicq_cut_kernel, grid, dim3(256), 0, st, s->d_in, s->ring_in, s->d_win, s->d_stage, s->sl,
                                         s->H, s->next_slice, s->C) != cudaSuccess)
@@ -159,10 +188,13 @@ cqt_status analyse_ready(cqt_slicq *s, cudaStream_t st) {
         if (r != CQT_OK) return r;
         s->next_slice += cnt;
     }
-    return CQT_OK;
+    if (!fused) return CQT_OK;
+    // what follows the last complete slice
+    const int64_t tail = std::max(new_first, ready * s->H);
+    return ingest(s, fresh ? fresh + (tail - new_first) : nullptr, fresh_stride, tail, s->n_in - tail, st);
 }
 
-cqt_status push_impl(cqt_slicq *s, const float *x, int64_t x_stride, int64_t n, int zero, cudaStream_t st) {
+cqt_status push_impl(cqt_slicq *s, const float *x, int64_t x_stride, int64_t n, cudaStream_t st) {
     // slices this push completes must fit the free coefficient slots
     const int64_t will_be_ready = (s->n_in + n) / s->H;
     if (will_be_ready - s->next_synth > s->K) return CQT_ERR_STATE;
@@ -173,14 +205,11 @@ cqt_status push_impl(cqt_slicq *s, const float *x, int64_t x_stride, int64_t n, 
         const int64_t room = s->ring_in - (s->n_in - oldest);
         const int64_t m = std::min<int64_t>(n - done, room);
         if (m <= 0) return CQT_ERR_STATE;
-        dim3 grid(blocks_for(m), (unsigned)s->C);
-        if (cqt::launch_kernel_args(slicq_ingest_kernel, grid, dim3(256), 0, st, zero ? (const float *)nullptr : x + done, x_stride, s->d_in,
-                               s->ring_in, s->n_in, m, zero) != cudaSuccess)
-            return CQT_ERR_CUDA;
+        const int64_t new_first = s->n_in;
         s->n_in += m;
-        done += m;
-        cqt_status r = analyse_ready(s, st);
+        const cqt_status r = analyse_ready(s, x ? x + done : nullptr, x_stride, new_first, st);
         if (r != CQT_OK) return r;
+        done += m;
     }
     return CQT_OK;
 }
@@ -249,7 +278,7 @@ cqt_status slicq_push(cqt_slicq *s, const float *x, int64_t x_stride, int64_t n,
     OnPlanDevice guard(s);
     if (!guard.ok) return CQT_ERR_CUDA;
     if (n > 0) { s->last_stream = reinterpret_cast<cudaStream_t>(stream); s->used = true; }
-    cqt_status r = n > 0 ? push_impl(s, x, x_stride, n, 0, reinterpret_cast<cudaStream_t>(stream)) : CQT_OK;
+    cqt_status r = n > 0 ? push_impl(s, x, x_stride, n, reinterpret_cast<cudaStream_t>(stream)) : CQT_OK;
     if (slices_completed) *slices_completed = s->next_slice;
     return r;
 }
@@ -262,7 +291,7 @@ cqt_status slicq_flush(cqt_slicq *s, void *stream) {
     s->used = true;
     // enough zeros that every frame pushed so far becomes final: n_in -> (ceil(n_in / H) + 1) H
     const int64_t target = ((s->n_in + s->H - 1) / s->H + 1) * s->H;
-    return push_impl(s, nullptr, 0, target - s->n_in, 1, reinterpret_cast<cudaStream_t>(stream));
+    return push_impl(s, nullptr, 0, target - s->n_in, reinterpret_cast<cudaStream_t>(stream));
 }
 
 cqt_status slicq_coeffs(cqt_slicq *s, int64_t slice_index, cqt_c64 **c) {
@@ -281,9 +310,10 @@ cqt_status slicq_pull(cqt_slicq *s, float *y, int64_t y_stride, int64_t n_max, v
     s->used = true;
     int64_t written = 0;
     for (;;) {
-        // synthesise as many pending slices as the output ring has room for
+        // synthesise as many pending slices as the output ring has room for: it holds frames n_out .. next_synth * H - 1,
+        // every slice adds H frames, and what this call emits need not stay
+        int64_t done = 0;
         while (s->next_synth < s->next_slice) {
-            // the ring holds frames n_out .. next_synth * H - 1; every slice adds H frames
             const int64_t room_slices = (s->ring_out - (s->next_synth * s->H - s->n_out)) / s->H;
             const int64_t slot = s->next_synth % s->K;
             const int64_t cnt = std::min<int64_t>({s->next_slice - s->next_synth, s->K - slot, room_slices});
@@ -291,13 +321,20 @@ cqt_status slicq_pull(cqt_slicq *s, float *y, int64_t y_stride, int64_t n_max, v
             cqt_status r = cqt_synthesise(s->plan, s->d_coef + slot * s->C * cqt_plan_coeff_count(s->plan), cnt * s->C, s->sl,
                                           s->d_stage, s->sl, s->d_ws, s->ws_bytes, st);
             if (r != CQT_OK) return r;
-            dim3 grid(blocks_for((cnt + 1) * s->H), (unsigned)s->C);
-            if (cqt::launch_kernel_args(slicq_ola_kernel, grid, dim3(256), 0, st, s->d_stage, s->d_out, s->ring_out, s->sl, s->H,
-                                   s->next_synth, s->next_synth + cnt - 1, s->C) != cudaSuccess)
+            // frames below (next_synth - 1) H are final once these slices are in
+            const int64_t s0 = s->next_synth, s1 = s0 + cnt - 1;
+            const int64_t m = std::max<int64_t>(0, std::min<int64_t>(n_max - written, s1 * s->H - s->n_out));
+            const int64_t first = m > 0 ? std::min<int64_t>(s->n_out, (s0 - 1) * s->H) : (s0 - 1) * s->H;
+            dim3 grid(blocks_for((s1 + 1) * s->H - first), (unsigned)s->C);
+            if (cqt::launch_kernel_args(slicq_ola_kernel, grid, dim3(256), 0, st, s->d_stage, s->d_out, s->ring_out, s->sl, s->H, s0, s1,
+                                   s->C, first, s->n_out, s->n_out + m, y + written, y_stride) != cudaSuccess)
                 return CQT_ERR_CUDA;
             s->next_synth += cnt;
+            s->n_out += m;
+            written += m;
+            done += cnt;
         }
-        // frames below (next_synth - 1) H are final
+        // frames that were final before and wait in the ring
         const int64_t final_to = std::max<int64_t>(0, (s->next_synth - 1) * s->H);
         const int64_t m = std::min<int64_t>(n_max - written, final_to - s->n_out);
         if (m > 0) {
@@ -308,7 +345,7 @@ cqt_status slicq_pull(cqt_slicq *s, float *y, int64_t y_stride, int64_t n_max, v
             s->n_out += m;
             written += m;
         }
-        if (m <= 0 || written >= n_max || s->next_synth >= s->next_slice) break;
+        if ((m <= 0 && done == 0) || written >= n_max || s->next_synth >= s->next_slice) break;
     }
     *n_written = written;
     return CQT_OK;

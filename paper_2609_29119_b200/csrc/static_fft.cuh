@@ -53,7 +53,7 @@ __device__ __forceinline__ void tile_middle(float2 *buf, const float2 *twf, int 
     if constexpr (S::R2 > 1) {
         constexpr int R1 = S::R1, R2 = S::R2, units = S::LEN / R1 * S::NC / S::T;
         static_assert(units * S::T * R1 == S::LEN * S::NC, "whole rounds");
-#pragma unroll
+#pragma unroll 1
         for (int u = 0; u < units; ++u) {
             const int w = tid + u * S::T, col = w % S::NC, b = w / S::NC, np = b % R2, p = (b / R2) * S::S0 + np;
             float re[R1], im[R1];
@@ -80,13 +80,6 @@ __device__ __forceinline__ void last_butterfly(const float2 *buf, int b, int col
         re[q] = v.x; im[q] = v.y;
     }
     dft<S::RL, SIGN>(re, im);
-}
-
-// log2 of the low part of a two-level table of n = 2^m entries (see append_twiddles in api.cu)
-__host__ __device__ constexpr int low_bits(int64_t n) {
-    int l = 0;
-    while ((1ll << (2 * l)) < n) ++l;
-    return l;
 }
 
 }  // namespace cqt
