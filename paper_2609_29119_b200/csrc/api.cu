@@ -174,6 +174,7 @@ void free_device(cqt_plan *p) {
     for (auto &c : p->cls) cudaFree(c.d_items);
     cudaFree(p->merged.d_items);
     cudaFree(p->chirp.d_recs);
+    cudaFree(p->split.d_items); cudaFree(p->split.d_recs);
     for (auto &g : p->two_pass) cudaFree(g.d_recs);
     for (cudaEvent_t e : p->ev) cudaEventDestroy(e);
     for (int i = 0; i < cqt_plan::kHelpers; ++i) {
@@ -493,6 +494,20 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
             if (mg.segs.empty() || mg.segs.back().lg_nthr != lg) mg.segs.push_back({(int)i, 0, lg, 0});
             mg.segs.back().n_bands++;
             mg.segs.back().elems = std::max(mg.segs.back().elems, (int)band_elems(mg.work[i]));
+            if (lg < 10) continue;
+            // the longest ones are split into four work items instead
+            BandItem item;
+            const int64_t M = p->bands[(size_t)mg.work[i]].M;
+            item.br = p->bands[(size_t)mg.work[i]];
+            item.fp = p->ffts[(size_t)plan_for(M / 4, kPlanBand, 16)];
+            SplitRec sr{};
+            int lc = 0;
+            sr.tw_m = append_twiddles(tw, M, lc);
+            sr.log_m_c = lc;
+            sr.n_m = (int32_t)tw.size() - sr.tw_m;
+            p->split.items.push_back(item);
+            p->split.recs.push_back(sr);
+            p->split.max_elems = std::max(p->split.max_elems, (int)(M / 4) + 16 + item.fp.tw_count + sr.n_m);
         }
     }
     // estimates for the per-call assignment of classes to streams (band.cu): total work, and the time one CTA
@@ -562,6 +577,8 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     for (auto &c : p->cls) upload_items(c.d_items, c.work);
     upload_items(p->merged.d_items, p->merged.work);
     chk(upload(p->chirp.d_recs, p->chirp.recs));
+    chk(upload(p->split.d_items, p->split.items));
+    chk(upload(p->split.d_recs, p->split.recs));
     cudaDeviceProp prop;
     chk(cudaGetDeviceProperties(&prop, p->device));
     p->sm_count = prop.multiProcessorCount;
@@ -577,6 +594,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     chk(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
     if (e == cudaSuccess) chk(configure_band_kernels(*p));
     if (e == cudaSuccess) chk(configure_chirp_kernels(*p));
+    if (e == cudaSuccess) chk(configure_split_kernels(*p));
     if (e == cudaSuccess) chk(p->lf.A == 1 ? configure_short_fft_kernels(*p) : configure_long_forward_kernels(*p));
     if (e == cudaSuccess && p->lf.A > 1) chk(configure_long_inverse_kernels(*p));
     for (auto &g : p->two_pass) chk(upload(g.d_recs, g.bands));

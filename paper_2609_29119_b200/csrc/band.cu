@@ -57,15 +57,16 @@ static cudaError_t launch_class(const cqt_plan &p, int cls, const char *name, Ba
 const void *band_analysis_merged_kernel();    // band_analysis.cu
 const void *band_synthesis_merged_kernel();   // band_synthesis.cu
 
-// Shape of the few-items form for a batch: the bands longer than class 0's in one launch (two when some of them take
-// 1024 threads each: those then do not set the CTA size of the others), class 0 in one.
+// Shape of the few-items form for a batch: the bands longer than class 0's in one launch, those of them that would take
+// 1024 threads each (the first segment) split into four work items in another, class 0 in one.
 struct FewLaunch {
     struct Part {
         BandSegments sg{};
         int threads = 0, grid = 0;
         size_t smem = 0;
     };
-    Part part[2];
+    Part part;
+    bool split = false;                 // bands on the split kernel
     bool chirp = false;                 // bands on the chirp-z kernel
     int short_threads = 0, short_grid = 0;
 };
@@ -105,8 +106,9 @@ static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
         bool spread = false;
         t.chirp = !p.chirp.recs.empty();
         long long sms = t.chirp ? (chirp_grid(p, batch, nullptr) + 1) / 2 : 0;   // two CTAs of it share an SM
-        sms += few_part(p, batch, 0, split, share, t.part[0], spread);
-        sms += few_part(p, batch, split, n, share, t.part[1], spread);
+        t.split = split > 0;
+        sms += 2 * (long long)p.split.recs.size() * batch;                  // and of the split kernel
+        sms += few_part(p, batch, split, n, share, t.part, spread);
         if (sms > p.sm_count) {
             if (share == 1) return false;
             break;
@@ -123,24 +125,27 @@ static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
 
 template <bool ANALYSIS>
 static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cudaStream_t st) {
-    static const char *names[2][3] = {{"bands_to_spectrum/1024_threads", "bands_to_spectrum/merged", "bands_to_spectrum/class0"},
-                                      {"bands_from_spectrum/1024_threads", "bands_from_spectrum/merged", "bands_from_spectrum/class0"}};
+    static const char *names[2][2] = {{"bands_to_spectrum/merged", "bands_to_spectrum/class0"},
+                                      {"bands_from_spectrum/merged", "bands_from_spectrum/class0"}};
     cudaError_t e = cudaSuccess;
-    const int launches = f.chirp + (f.part[0].grid > 0) + (f.part[1].grid > 0) + (f.short_grid > 0);
+    const int launches = f.chirp + f.split + (f.part.grid > 0) + (f.short_grid > 0);
     a.chain = launches > 1 ? kChainHead : kAlone;
     if (f.chirp) {
         e = launch_chirp(p, ANALYSIS, a, st);
-        a.chain = kChainMember;
+        a.chain = a.chain == kChainHead ? kChainMember : a.chain;
     }
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
-        FewLaunch::Part &t = f.part[i];
-        if (!t.grid) continue;
+    if (f.split && e == cudaSuccess) {
+        e = launch_split(p, ANALYSIS, a, st);
+        a.chain = a.chain == kChainHead ? kChainMember : a.chain;
+    }
+    if (f.part.grid && e == cudaSuccess) {
+        FewLaunch::Part &t = f.part;
         a.items = p.merged.d_items;
         void *args[] = {&a, &t.sg};
         const void *fn = ANALYSIS ? band_analysis_merged_kernel() : band_synthesis_merged_kernel();
         e = launch_kernel(fn, dim3((unsigned)t.grid), dim3((unsigned)t.threads), args, t.smem, st);
-        note_launch(p, names[ANALYSIS][i], st);
-        a.chain = kChainMember;
+        note_launch(p, names[ANALYSIS][0], st);
+        a.chain = a.chain == kChainHead ? kChainMember : a.chain;
     }
     if (f.short_grid && e == cudaSuccess) {
         const BandClass &c = p.cls[0];
@@ -148,7 +153,7 @@ static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cuda
         void *args[] = {&a};
         e = launch_kernel(class_kernel<ANALYSIS>(c, 32), dim3((unsigned)f.short_grid), dim3((unsigned)f.short_threads), args,
                           (size_t)c.max_elems * (f.short_threads / 32) * sizeof(float2), st);
-        note_launch(p, names[ANALYSIS][2], st);
+        note_launch(p, names[ANALYSIS][1], st);
     }
     return e;
 }

@@ -113,20 +113,15 @@ __device__ __forceinline__ void fetch_item(const BandItem &g, BandItem &s, int t
 
 // Analysis form, any band: slot m of the transform's input, i.e. tab[d] X[kc + d] with d = m or m - M, zero outside the
 // support; bins outside 0..N/2 are the conjugates of their mirror bins.
+// No branch around the loads, so that those of several slots are in flight together.
 __device__ __forceinline__ float2 slot_value(const BandRec &br, const float *__restrict__ tab,
                                              const float2 *__restrict__ X, int N, int m) {
-    const int last_pos = br.d0 + br.S - 1, first_neg = br.M + br.d0;
-    int d;
-    if (m <= last_pos) d = m;
-    else if (m >= first_neg) d = m - br.M;
-    else return make_float2(0.f, 0.f);
-    const float g = __ldg(tab + (d - br.d0));
-    const int k = br.kc + d;
-    float2 xv;
-    if (k < 0) xv = cconj(ld_data(X + (-k)));
-    else if (k > (N >> 1)) xv = cconj(ld_data(X + (N - k)));
-    else xv = ld_data(X + k);
-    return make_float2(g * xv.x, g * xv.y);
+    const bool lo = m <= br.d0 + br.S - 1, ok = lo || m >= br.M + br.d0;
+    const int d = ok ? (lo ? m : m - br.M) : 0, k = br.kc + d, half = N >> 1;
+    const bool mirrored = k < 0 || k > half;
+    const float g = ok ? __ldg(tab + (d - br.d0)) : 0.f;
+    const float2 x = ld_data(X + (k < 0 ? -k : (k > half ? N - k : k)));
+    return make_float2(g * x.x, mirrored ? -(g * x.y) : g * x.y);
 }
 
 // Synthesis form, any band: output u of slot m, times the window table, to bin kc + d of the band's plane Y (only bins
@@ -143,6 +138,9 @@ __device__ __forceinline__ void slot_store(const BandRec &br, const float *__res
     const float h = __ldg(tab + (d - br.d0));
     if (CQT_CHK(dbg, 404, k, limit)) Y[k] = make_float2(h * u.x, h * u.y);
 }
+
+// band_split.cu: long bands of calls with few items
+cudaError_t launch_split(const cqt_plan &p, bool analysis, const BandArgs &b, cudaStream_t st);
 
 // band_chirp.cu: bands of more than 128 coefficients whose length has a prime factor above 5
 constexpr int kChirpThreads = 256;

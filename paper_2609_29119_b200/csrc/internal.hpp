@@ -43,6 +43,14 @@ struct ChirpBands {
     ChirpRec *d_recs = nullptr;
 };
 
+struct SplitBands {
+    std::vector<BandItem> items;     // record of the band, radix plan of a quarter of its length
+    std::vector<SplitRec> recs;
+    BandItem *d_items = nullptr;
+    SplitRec *d_recs = nullptr;
+    int max_elems = 0;               // shared-memory elements (float2) of one item
+};
+
 struct LongFft {
     int64_t Lp = 0, A = 1, B = 0;
     int fft_A = -1, fft_B = -1;   // FftPlan indices
@@ -92,6 +100,7 @@ struct cqt_plan {
     cqt::BandClass cls[cqt::kNumClasses];
     cqt::MergedBands merged;
     cqt::ChirpBands chirp;
+    cqt::SplitBands split;             // the bands of the first segment of `merged` when that has 1024 threads per item
     std::vector<int8_t> band_class;    // length class of every band, -1: two-pass kernels
     cqt::TwoPassGroup two_pass[2];     // [0]: both factors <= 256, [1]: larger factors
     int64_t two_pass_pitch = 0;        // scratch elements per signal for the two-pass bands
@@ -201,6 +210,9 @@ cudaError_t configure_band_kernels(const cqt_plan &p);
 int chirp_length_index(int64_t m);     // which L serves m-point sub-transforms, -1: none
 int chirp_length(int index);
 cudaError_t configure_chirp_kernels(const cqt_plan &p);
+
+// band_split.cu
+cudaError_t configure_split_kernels(const cqt_plan &p);
 
 // band_two_pass.cu
 cudaError_t launch_two_pass_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, float2 *c,

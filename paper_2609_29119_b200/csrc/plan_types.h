@@ -67,6 +67,11 @@ struct ChirpRec {
 };
 constexpr int kChirpLengths = 7;   // L = 8192 ... 128
 
+// A band split into four work items (band_split.cu): two-level table of W_M
+struct SplitRec {
+    int32_t tw_m, log_m_c, n_m, pad_;
+};
+
 // A band transformed in two passes (M = A * B) through a scratch row.
 struct TwoPassRec {
     int32_t band;
