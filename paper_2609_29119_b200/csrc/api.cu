@@ -312,8 +312,24 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     }
     lf.fft_B = plan_for(lf.B, kPlanPow2, 16);
     lf.fft_A = lf.A > 1 ? plan_for(lf.A, kPlanPow2, 16) : lf.fft_B;
-    lf.tw_lp = append_twiddles(tw, lf.Lp, lf.log_lp_c);
-    lf.n_lp = (int)tw.size() - lf.tw_lp;
+    if (lf.A > 1) {
+        // twiddles between the passes, W_Lp^{i (low + q NL)} = U[low][i] V[q][i] for element q of the last-stage butterfly whose
+        // lowest frequency is low: both factors rounded once from their exact value
+        auto outer = [&](int64_t rows, int64_t cols, int64_t scale) {   // [row][col] = W_Lp^{scale row col}
+            const int off = (int)tw.size();
+            for (int64_t r = 0; r < rows; ++r)
+                for (int64_t c = 0; c < cols; ++c) {
+                    const double ang = -2.0 * kPi * (double)((scale * r * c) % lf.Lp) / (double)lf.Lp;
+                    tw.push_back(make_float2((float)std::cos(ang), (float)std::sin(ang)));
+                }
+            return off;
+        };
+        const int64_t nl_cols = lf.A / long_cols_last_radix(lf.A), nl_rows = lf.B / long_rows_inverse_last_radix(lf.B);
+        lf.tw_fwd_u = outer(nl_cols, lf.B, 1);
+        lf.tw_fwd_v = outer(lf.A / nl_cols, lf.B, nl_cols);
+        lf.tw_inv_u = outer(nl_rows, lf.A, 1);
+        lf.tw_inv_v = outer(lf.B / nl_rows, lf.A, nl_rows);
+    }
     lf.tw_n = append_twiddles(tw, N, lf.log_n_c);
     lf.n_n = (int)tw.size() - lf.tw_n;
     lf.x_pitch = (lf.Lp + 1 + 7) / 8 * 8;

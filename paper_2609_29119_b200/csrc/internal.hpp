@@ -54,9 +54,8 @@ struct SplitBands {
 struct LongFft {
     int64_t Lp = 0, A = 1, B = 0;
     int fft_A = -1, fft_B = -1;   // FftPlan indices
-    int tw_lp = 0, tw_n = 0;      // two-level tables of W_Lp and W_N inside the twiddle array
-    int log_lp_c = 0, log_n_c = 0;
-    int n_lp = 0, n_n = 0;        // entry counts of those tables
+    int tw_n = 0, log_n_c = 0, n_n = 0;           // two-level table of W_N inside the twiddle array, its entry count
+    int tw_fwd_u = 0, tw_fwd_v = 0, tw_inv_u = 0, tw_inv_v = 0;   // twiddles between the passes (api.cu)
     int64_t x_pitch = 0;          // elements per signal of the half-spectrum buffer (Lp + 1 rounded up)
 };
 
@@ -162,6 +161,9 @@ inline cudaError_t allow_dynamic_smem(const void *fn, size_t need, const cqt_pla
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
+// radix of the last stage of the passes that end with the twiddles between the passes
+int long_cols_last_radix(int64_t A);            // forward pass C
+int long_rows_inverse_last_radix(int64_t B);    // inverse pass R'
 cudaError_t configure_long_forward_kernels(const cqt_plan &p);
 cudaError_t configure_long_inverse_kernels(const cqt_plan &p);
 cudaError_t configure_short_fft_kernels(const cqt_plan &p);

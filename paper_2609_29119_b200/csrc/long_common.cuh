@@ -8,7 +8,7 @@ namespace cqt {
 struct LongArgs {
     const float2 *tw;
     int tw_full_A, tw_full_B;    // full tables of W_A, W_B
-    int tw_lp, n_lp;             // two-level table of W_Lp and its entry count
+    int tw_u, tw_v;              // twiddles between the passes: U[low][i], V[q][i] (long_fft_forward.cu)
     int tw_n, log_n_c, n_n;      // two-level table of W_N
     int valid_len;
     int aligned;           // signal rows allow float2 access
@@ -142,8 +142,6 @@ inline LongArgs base_args(const cqt_plan &p, int64_t valid_len, int64_t x_stride
     a.tw = p.d.tw;
     a.tw_full_A = p.ffts[(size_t)p.lf.fft_A].tw_full_off;
     a.tw_full_B = p.ffts[(size_t)p.lf.fft_B].tw_full_off;
-    a.tw_lp = p.lf.tw_lp;
-    a.n_lp = p.lf.n_lp;
     a.tw_n = p.lf.tw_n;
     a.log_n_c = p.lf.log_n_c;
     a.n_n = p.lf.n_n;

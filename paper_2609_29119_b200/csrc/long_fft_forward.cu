@@ -27,9 +27,8 @@ __global__ void __launch_bounds__(ColsForward<A>::T, 1024 / ColsForward<A>::T) r
     using S = ColsForward<A>;
     pdl_launch_dependents();
     const int tid = threadIdx.x, col = tid % S::NC, j2 = blockIdx.x * S::NC + col, ch = blockIdx.y;
-    float2 *buf = smem_long, *tws = buf + S::ELEMS, *wl = tws + A;
+    float2 *buf = smem_long, *tws = buf + S::ELEMS;
     stage_table<A, S::T>(tws, a.tw + a.tw_full_A, tid);
-    stage_table<two_level_entries(A * B), S::T>(wl, a.tw + a.tw_lp, tid);
     constexpr int R0 = S::R0, units = S::S0 * S::NC / S::T, step = S::T / S::NC;
     float re[units][R0], im[units][R0];
     if constexpr (SLICED) {
@@ -108,16 +107,20 @@ __global__ void __launch_bounds__(ColsForward<A>::T, 1024 / ColsForward<A>::T) r
     __syncthreads();
     tile_middle<S, -1>(buf, tws, tid);
     float2 *T = a.T + (long long)ch * a.t_pitch + j2;
+    // W_Lp^{j2 k1}, k1 = low + q NL, as U[low][j2] V[q][j2]: neighbouring columns read neighbouring entries (a two-level table
+    // indexed by the product j2 k1 cost two conflicting shared loads per element), a thread's U is one load
+    const float2 *U = a.tw + a.tw_u + j2, *V = a.tw + a.tw_v + j2;
     constexpr int last = S::NL * S::NC / S::T;
 #pragma unroll 1
     for (int u = 0; u < last; ++u) {
         const int b = tid / S::NC + u * step, low = S::low(b);
+        const float2 wu = __ldg(U + low * B);
         float x[S::RL], y[S::RL];
         last_butterfly<S, -1>(buf, b, col, x, y);
 #pragma unroll
         for (int q = 0; q < S::RL; ++q) {
             const int k1 = low + q * S::NL;
-            const float2 w = two_level<A * B>(wl, (uint32_t)j2 * (uint32_t)k1);
+            const float2 w = cmul(wu, __ldg(V + q * B));
             if (CQT_CHK(a.dbg, 201, k1 * B + j2, A * B)) T[k1 * B] = cmul(make_float2(x[q], y[q]), w);
         }
     }
@@ -236,7 +239,7 @@ static ForwardKernels forward_kernels(const cqt_plan &p) {
         k.cols = Forward<A_, B_>::cols(false); k.cols_sliced = Forward<A_, B_>::cols(true); k.rows = Forward<A_, B_>::rows(); \
         k.cols_threads = C::T; k.rows_threads = R::T;                                                \
         k.cols_tiles = B_ / C::NC; k.rows_tiles = A_ / R::NC;                                        \
-        k.cols_smem = sizeof(float2) * ((size_t)C::ELEMS + A_ + p.lf.n_lp);                          \
+        k.cols_smem = sizeof(float2) * ((size_t)C::ELEMS + A_);                                     \
         k.rows_smem = sizeof(float2) * ((size_t)R::ELEMS + B_ + p.lf.n_n);                           \
     }
     CQT_LONG_SPLITS(X)
@@ -250,6 +253,8 @@ cudaError_t launch_rfft_forward(const cqt_plan &p, const float *x, int64_t x_str
     a.x_in = x;
     a.T = T;
     a.X = X;
+    a.tw_u = p.lf.tw_fwd_u;
+    a.tw_v = p.lf.tw_fwd_v;
     if (p.lf.A == 1) {
         if (src) return cudaErrorInvalidValue;
         cudaError_t e = launch_short_rfft_forward(p, a, batch, st);
@@ -278,6 +283,13 @@ cudaError_t launch_rfft_forward(const cqt_plan &p, const float *x, int64_t x_str
     e = launch_long(k.rows, k.rows_tiles, batch, k.rows_threads, k.rows_smem, a, st);
     note_launch(p, "rfft_rows_fwd", st);
     return e;
+}
+
+int long_cols_last_radix(int64_t A) {
+#define X(A_, B_) if (A == A_) return ColsForward<A_>::RL;
+    CQT_LONG_SPLITS(X)
+#undef X
+    return 1;
 }
 
 cudaError_t configure_long_forward_kernels(const cqt_plan &p) {

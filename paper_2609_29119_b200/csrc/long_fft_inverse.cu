@@ -29,11 +29,10 @@ __global__ void __launch_bounds__(RowsInverse<B>::T, 1024 / RowsInverse<B>::T) i
     constexpr float s = 0.5f / (float)Lp;    // a power of two
     pdl_launch_dependents();
     const int tid = threadIdx.x, ch = blockIdx.y, t = blockIdx.x;
-    float2 *buf = smem_long, *tws = buf + S::ELEMS, *wn = tws + B, *wl = wn + two_level_entries(N);
+    float2 *buf = smem_long, *tws = buf + S::ELEMS, *wn = tws + B;
     stage_table<B, S::T>(tws, a.tw + a.tw_full_B, tid);
     // the low part of the table of W_N times s
     stage_table<two_level_entries(N), S::T>(wn, a.tw + a.tw_n, tid, 1 << C, s);
-    stage_table<two_level_entries(Lp), S::T>(wl, a.tw + a.tw_lp, tid);
     // thread: column r and its mirror r + TW; unit u: butterfly b = b0 + u step of the one, S0 - 1 - b of the other, whose
     // operands are the bins k = k0 + A (u step + q S0) and Lp - k
     const int r = tid % TW, b0 = tid / TW;
@@ -107,16 +106,18 @@ __global__ void __launch_bounds__(RowsInverse<B>::T, 1024 / RowsInverse<B>::T) i
     // transposed intermediate Tinv[j2][q1]: consecutive threads take consecutive columns, runs of TW rows
     const int col = tid % S::NC, q1 = row_of<A, TW>(t, col);
     float2 *T = a.T + (long long)ch * a.t_pitch + q1;
+    const float2 *U = a.tw + a.tw_u + q1, *V = a.tw + a.tw_v + q1;   // W_Lp^{j2 q1} = U[low][q1] V[q][q1], j2 = low + q NL
     constexpr int last = S::NL * S::NC / S::T;
 #pragma unroll 1
     for (int u = 0; u < last; ++u) {
         const int b = tid / S::NC + u * (S::T / S::NC), low = S::low(b);
+        const float2 wu = __ldg(U + low * A);
         float x[S::RL], y[S::RL];
         last_butterfly<S, +1>(buf, b, col, x, y);
 #pragma unroll
         for (int q = 0; q < S::RL; ++q) {
             const int j2 = low + q * S::NL;
-            const float2 w = two_level<Lp>(wl, (uint32_t)j2 * (uint32_t)q1);
+            const float2 w = cmul(wu, __ldg(V + q * A));
             if (CQT_CHK(a.dbg, 207, j2 * A + q1, Lp)) T[j2 * A] = cmul(make_float2(x[q], y[q]), cconj(w));
         }
     }
@@ -188,7 +189,7 @@ static InverseKernels inverse_kernels(const cqt_plan &p) {
         k.cols = (const void *)irfft_cols_kernel<A_, B_>;                                                          \
         k.rows_threads = R::T; k.cols_threads = C::T;                                                              \
         k.rows_tiles = A_ / R::NC; k.cols_tiles = B_ / C::NC;                                                      \
-        k.rows_smem = sizeof(float2) * ((size_t)R::ELEMS + B_ + p.lf.n_n + p.lf.n_lp);                             \
+        k.rows_smem = sizeof(float2) * ((size_t)R::ELEMS + B_ + p.lf.n_n);                                         \
         k.cols_smem = sizeof(float2) * ((size_t)C::ELEMS + A_);                                                    \
     }
     CQT_LONG_SPLITS(X)
@@ -202,6 +203,8 @@ cudaError_t launch_rfft_inverse(const cqt_plan &p, const float2 *Y, float2 *T, f
     a.x_out = x;
     a.T = T;
     a.Y = Y;
+    a.tw_u = p.lf.tw_inv_u;
+    a.tw_v = p.lf.tw_inv_v;
     if (p.lf.A == 1) {
         cudaError_t e = launch_short_rfft_inverse(p, a, batch, st);
         note_launch(p, "irfft_rows", st);
@@ -214,6 +217,13 @@ cudaError_t launch_rfft_inverse(const cqt_plan &p, const float2 *Y, float2 *T, f
     e = launch_long(k.cols, k.cols_tiles, batch, k.cols_threads, k.cols_smem, a, st);
     note_launch(p, "irfft_cols", st);
     return e;
+}
+
+int long_rows_inverse_last_radix(int64_t B) {
+#define X(A_, B_) if (B == B_) return RowsInverse<B_>::RL;
+    CQT_LONG_SPLITS(X)
+#undef X
+    return 1;
 }
 
 cudaError_t configure_long_inverse_kernels(const cqt_plan &p) {
