@@ -153,29 +153,49 @@ void make_chirp_tables(int64_t m, int64_t L, std::vector<float2> &tw, ChirpRec &
     for (const std::complex<double> &v : b) tw.push_back(make_float2((float)(v.real() / (double)L), (float)(v.imag() / (double)L)));
 }
 
-template <class T>
-cudaError_t upload(T *&dst, const std::vector<T> &src) {
-    dst = nullptr;
-    if (src.empty()) return cudaSuccess;
-    cudaError_t e = cudaMalloc((void **)&dst, src.size() * sizeof(T));
-    if (e != cudaSuccess) return e;
-    return cudaMemcpy(dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
-}
+// Device tables of a plan.  Small ones are collected into one allocation and one copy (twenty of each took most of the time
+// of creating a small plan), large ones go straight from their vector, which has to live until run().
+struct TableUpload {
+    static constexpr size_t kSmall = 1 << 20;
+    struct Piece { void **dst; const void *src; size_t offset, bytes; };
+    std::vector<char> small;
+    std::vector<Piece> pieces;      // src == nullptr: in `small`, offset there
+    template <class T>
+    void add(T *&dst, const std::vector<T> &src) {
+        dst = nullptr;
+        const size_t n = src.size() * sizeof(T);
+        if (n == 0) return;
+        if (n > kSmall) { pieces.push_back({reinterpret_cast<void **>(&dst), src.data(), 0, n}); return; }
+        const size_t off = (small.size() + 255) / 256 * 256;
+        small.resize(off + n);
+        std::memcpy(small.data() + off, src.data(), n);
+        pieces.push_back({reinterpret_cast<void **>(&dst), nullptr, off, n});
+    }
+    cudaError_t run(std::vector<void *> &allocations) {
+        auto copy = [&](const void *src, size_t n, char *&base) {
+            void *p = nullptr;
+            cudaError_t e = cudaMalloc(&p, n);
+            if (e != cudaSuccess) return e;
+            allocations.push_back(p);
+            base = static_cast<char *>(p);
+            return cudaMemcpy(p, src, n, cudaMemcpyHostToDevice);
+        };
+        char *base = nullptr, *own = nullptr;
+        cudaError_t e = copy(small.data(), small.size(), base);
+        for (const Piece &p : pieces) {
+            if (p.src && e == cudaSuccess) e = copy(p.src, p.bytes, own);
+            if (e == cudaSuccess) *p.dst = p.src ? own : base + p.offset;
+        }
+        return e;
+    }
+};
 
 void free_device(cqt_plan *p) {
     if (p->device < 0) return;
     int cur = 0;
     cudaGetDevice(&cur);
     cudaSetDevice(p->device);
-    cudaFree(p->d.bands); cudaFree(p->d.ffts); cudaFree(p->d.tw);
-    cudaFree(p->d.tab_analysis); cudaFree(p->d.tab_synthesis);
-    cudaFree(p->d.tab_analysis_adj); cudaFree(p->d.tab_synthesis_adj);
-    cudaFree(p->d.cover); cudaFree(p->d.dbg); cudaFree(p->d.zero_seg);
-    for (auto &c : p->cls) cudaFree(c.d_items);
-    cudaFree(p->merged.d_items);
-    cudaFree(p->chirp.d_recs);
-    cudaFree(p->split.d_items); cudaFree(p->split.d_recs);
-    for (auto &g : p->two_pass) cudaFree(g.d_recs);
+    for (void *a : p->d.allocations) cudaFree(a);
     for (cudaEvent_t e : p->ev) cudaEventDestroy(e);
     for (int i = 0; i < cqt_plan::kHelpers; ++i) {
         if (p->aux[i]) cudaStreamDestroy(p->aux[i]);
@@ -561,14 +581,15 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     }
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-    chk(upload(p->d.bands, p->bands));
-    chk(upload(p->d.ffts, p->ffts));
-    chk(upload(p->d.tw, tw));
-    chk(upload(p->d.tab_analysis, tA));
-    chk(upload(p->d.tab_synthesis, tS));
-    chk(upload(p->d.tab_analysis_adj, tTA));
-    chk(upload(p->d.tab_synthesis_adj, tSA));
-    chk(upload(p->d.cover, cover));
+    TableUpload up;
+    up.add(p->d.bands, p->bands);
+    up.add(p->d.ffts, p->ffts);
+    up.add(p->d.tw, tw);
+    up.add(p->d.tab_analysis, tA);
+    up.add(p->d.tab_synthesis, tS);
+    up.add(p->d.tab_analysis_adj, tTA);
+    up.add(p->d.tab_synthesis_adj, tSA);
+    up.add(p->d.cover, cover);
     // nested supports: the bins of a band's widened range outside its support hold zeros in the band's plane
     std::vector<int2> zero_seg;
     for (size_t i = 0; i < L.bands.size(); ++i) {
@@ -578,8 +599,8 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         if (hb.zr > 0) zero_seg.push_back(make_int2((int)(p->bands[i].y_off + en + 1), (int)hb.zr));
     }
     p->n_zero_seg = (int)zero_seg.size();
-    if (p->n_zero_seg) chk(upload(p->d.zero_seg, zero_seg));
-    chk(upload(p->d.dbg, std::vector<int>(8, 0)));
+    if (p->n_zero_seg) up.add(p->d.zero_seg, zero_seg);
+    up.add(p->d.dbg, std::vector<int>(8, 0));
     auto upload_items = [&](BandItem *&dst, const std::vector<int32_t> &work) {
         // record and radix plan of every band of the class, in launch order: what a work item fetches first
         std::vector<BandItem> items(work.size());
@@ -588,17 +609,17 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
             items[i].br = p->bands[(size_t)b];
             items[i].fp = p->ffts[(size_t)p->bands[(size_t)b].fft];
         }
-        chk(upload(dst, items));
+        up.add(dst, items);
     };
     for (auto &c : p->cls) upload_items(c.d_items, c.work);
     upload_items(p->merged.d_items, p->merged.work);
-    chk(upload(p->chirp.d_recs, p->chirp.recs));
-    chk(upload(p->split.d_items, p->split.items));
-    chk(upload(p->split.d_recs, p->split.recs));
-    cudaDeviceProp prop;
-    chk(cudaGetDeviceProperties(&prop, p->device));
-    p->sm_count = prop.multiProcessorCount;
-    p->max_smem_optin = (int)prop.sharedMemPerBlockOptin;
+    up.add(p->chirp.d_recs, p->chirp.recs);
+    up.add(p->split.d_items, p->split.items);
+    up.add(p->split.d_recs, p->split.recs);
+    for (auto &g : p->two_pass) up.add(g.d_recs, g.bands);
+    chk(up.run(p->d.allocations));
+    chk(cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device));
+    chk(cudaDeviceGetAttribute(&p->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
     // the helper streams carry the shorter classes: at the highest priority their CTAs are placed ahead of the
     // long class on the caller's stream, whatever order the launches (or the nodes of a captured graph) arrive in
     int prio_least = 0, prio_greatest = 0;
@@ -613,7 +634,6 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     if (e == cudaSuccess) chk(configure_split_kernels(*p));
     if (e == cudaSuccess) chk(p->lf.A == 1 ? configure_short_fft_kernels(*p) : configure_long_forward_kernels(*p));
     if (e == cudaSuccess && p->lf.A > 1) chk(configure_long_inverse_kernels(*p));
-    for (auto &g : p->two_pass) chk(upload(g.d_recs, g.bands));
     if (e == cudaSuccess) chk(configure_two_pass_kernels(*p));
     cudaSetDevice(cur);
     if (e != cudaSuccess) { cqt_plan_destroy(p); return CQT_ERR_CUDA; }

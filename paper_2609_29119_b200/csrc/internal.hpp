@@ -70,6 +70,7 @@ struct TwoPassGroup {
 };
 
 struct DevicePlan {
+    std::vector<void *> allocations;   // what the pointers below lie in
     BandRec *bands = nullptr;
     FftPlan *ffts = nullptr;
     float2 *tw = nullptr;
