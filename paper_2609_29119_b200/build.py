@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libcqt_b200.so")
 EXT = os.path.join(HERE, "_cqt_torch.so")        # Python side of the transform calls, linked to LIB and torch
-SOURCES = ["layout.cpp", "api.cu", "band.cu", "band_analysis.cu", "band_synthesis.cu", "band_two_pass.cu", "band_chirp.cu", "band_split.cu", "long_fft_forward.cu", "long_fft_inverse.cu", "short_fft.cu", "slicq.cu", "static_ws.cu"]
+SOURCES = ["layout.cpp", "api.cu", "band.cu", "band_analysis.cu", "band_synthesis.cu", "band_two_pass.cu", "band_chirp.cu", "band_split.cu", "band_pow2.cu", "long_fft_forward.cu", "long_fft_inverse.cu", "short_fft.cu", "slicq.cu", "static_ws.cu"]
 HEADERS = ["layout.hpp", "plan_types.h", "internal.hpp", "engine.cuh", "band_common.cuh", "long_common.cuh", "long_passes.cuh",
            "static_fft.cuh", "codelets_gen.cuh",
            os.path.join("..", "..", "include", "cqt.h")]

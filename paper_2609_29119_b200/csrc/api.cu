@@ -438,6 +438,11 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     };
     p->band_class.assign(L.bands.size(), -1);
     std::vector<int> chirp_bands[kChirpLengths];
+    // plans whose bands of more than 128 coefficients are all powers of two (those beyond one CTA's shared memory apart)
+    auto pow2_band = [&](int64_t M) { return pow2_length_index(M) >= 0 && M <= two_pass_min && M + M / 8 + 64 <= smem_cap_elems; };
+    bool all_pow2 = true;
+    for (const HostBand &hb : L.bands) all_pow2 = all_pow2 && (hb.M <= limits[0] || pow2_band(hb.M) || hb.M + 16 > smem_cap_elems);
+    std::vector<int> pow2_bands[kPow2Lengths];
     for (int i : order) {
         const int64_t M = L.bands[i].M;
         int c = 0;
@@ -446,6 +451,10 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         int64_t A2 = 0;
         if (!single) { A2 = split_two_pass(M); single = A2 == 0; }
         p->band_class[(size_t)i] = (int8_t)c;
+        if (c > 0 && all_pow2 && pow2_band(M)) {
+            pow2_bands[pow2_length_index(M)].push_back(i);
+            continue;
+        }
         if (c > 0 && !smooth(M)) {
             const int li = M % 4 == 0 ? chirp_length_index(M / 4) : -1;
             if (li < 0) { delete p; return CQT_ERR_UNSUPPORTED; }
@@ -491,6 +500,29 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
                 g.smem_cols[wi] = std::max(g.smem_cols[wi], two_pass_smem_cols(tb, tw_tile));
                 g.smem_rows[wi] = std::max(g.smem_rows[wi], two_pass_smem_rows(tb, tw_tile));
             }
+        }
+    }
+    for (int li = 0; li < kPow2Lengths; ++li) {
+        p->pow2.n_bands[li] = (int)pow2_bands[li].size();
+        if (pow2_bands[li].empty()) continue;
+        // per stage but the last (sub-transforms of n points, radix r): rows W_n^{p y}, y < n / r, p = 1, 2, 4, ... < r
+        int r[4];
+        pow2_radices(li, r);
+        const int off = (int)tw.size();
+        int64_t n = L.bands[(size_t)pow2_bands[li][0]].M;
+        for (int j = 0; j < 3 && r[j + 1] > 1; ++j) {
+            for (int64_t pw = 1; pw < r[j]; pw *= 2)
+                for (int64_t y = 0; y < n / r[j]; ++y) {
+                    const double ang = -2.0 * kPi * (double)((pw * y) % n) / (double)n;
+                    tw.push_back(make_float2((float)std::cos(ang), (float)std::sin(ang)));
+                }
+            n /= r[j];
+        }
+        for (int b : pow2_bands[li]) {
+            Pow2Rec rec{};
+            rec.br = p->bands[(size_t)b];
+            rec.tw_off = off;
+            p->pow2.recs.push_back(rec);
         }
     }
     // every length L that occurs: one full twiddle table; bands of equal length share their tables
@@ -614,6 +646,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     for (auto &c : p->cls) upload_items(c.d_items, c.work);
     upload_items(p->merged.d_items, p->merged.work);
     up.add(p->chirp.d_recs, p->chirp.recs);
+    up.add(p->pow2.d_recs, p->pow2.recs);
     up.add(p->split.d_items, p->split.items);
     up.add(p->split.d_recs, p->split.recs);
     for (auto &g : p->two_pass) up.add(g.d_recs, g.bands);
@@ -631,6 +664,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     chk(cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming));
     if (e == cudaSuccess) chk(configure_band_kernels(*p));
     if (e == cudaSuccess) chk(configure_chirp_kernels(*p));
+    if (e == cudaSuccess) chk(configure_pow2_kernels(*p));
     if (e == cudaSuccess) chk(configure_split_kernels(*p));
     if (e == cudaSuccess) chk(p->lf.A == 1 ? configure_short_fft_kernels(*p) : configure_long_forward_kernels(*p));
     if (e == cudaSuccess && p->lf.A > 1) chk(configure_long_inverse_kernels(*p));

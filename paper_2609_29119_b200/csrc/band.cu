@@ -158,6 +158,29 @@ static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cuda
     return e;
 }
 
+// Power-of-two plans: two or three launches, chained, at any batch.
+template <bool ANALYSIS>
+static cudaError_t launch_pow2_plan(const cqt_plan &p, BandArgs &a, cudaStream_t st) {
+    const BandClass &c = p.cls[0];
+    const bool longer = pow2_has(p, true), shorter = pow2_has(p, false);
+    cudaError_t e = cudaSuccess;
+    a.chain = longer + shorter + (c.n_bands > 0) > 1 ? kChainHead : kAlone;
+    for (bool long_ones : {true, false}) {
+        if (!(long_ones ? longer : shorter) || e != cudaSuccess) continue;
+        e = launch_pow2(p, ANALYSIS, long_ones, a, st);
+        a.chain = a.chain == kChainHead ? kChainMember : a.chain;
+    }
+    if (c.n_bands > 0 && e == cudaSuccess) {
+        const long long items = (long long)c.n_bands * a.batch;
+        const int lanes = lanes_for(p, c, items), threads = items > 4ll * p.sm_count ? c.threads : 64, per_cta = threads / lanes;
+        void *args[] = {&a};
+        e = launch_kernel(class_kernel<ANALYSIS>(c, lanes), dim3((unsigned)((items + per_cta - 1) / per_cta)), dim3((unsigned)threads), args,
+                          (size_t)c.max_elems * per_cta * sizeof(float2), st);
+        note_launch(p, ANALYSIS ? "bands_from_spectrum/class0" : "bands_to_spectrum/class0", st);
+    }
+    return e;
+}
+
 // The classes of one call are independent (disjoint outputs), and most of them alone leave SMs idle, so they run
 // side by side on the caller's stream and the plan's helper streams (one stream per class when all five classes
 // have bands): fork after the caller's stream, join back into it.
@@ -216,17 +239,26 @@ static bool has_two_pass(const cqt_plan &p) { return !p.two_pass[0].bands.empty(
 cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, float2 *c,
                                        float2 *scratch, int64_t batch, cudaStream_t st) {
     FewLaunch f;
-    if (!has_two_pass(p) && few_shape(p, batch, f)) {
+    if (!has_two_pass(p) && (!p.pow2.recs.empty() || few_shape(p, batch, f))) {
         BandArgs a = make_args(p, p.cls[0], table, batch);
         a.spec = X;
         a.spec_pitch = p.lf.x_pitch;
         a.coef = c;
-        return launch_few<true>(p, a, f, st);
+        return p.pow2.recs.empty() ? launch_few<true>(p, a, f, st) : launch_pow2_plan<true>(p, a, st);
     }
     ForkJoin fj(p, st, batch);
     if (has_two_pass(p)) {
         cudaError_t e = launch_two_pass_from_spectrum(p, table, X, c, scratch, batch, fj.two_pass_stream());
         if (e != cudaSuccess) { fj.join(); return e; }
+    }
+    if (!p.pow2.recs.empty()) {   // its other bands are class 0's and two-pass ones
+        BandArgs a = make_args(p, p.cls[0], table, batch);
+        a.spec = X;
+        a.spec_pitch = p.lf.x_pitch;
+        a.coef = c;
+        cudaError_t e = launch_pow2_plan<true>(p, a, st);
+        fj.join();
+        return e;
     }
     if (!p.chirp.recs.empty()) {
         BandArgs a = make_args(p, p.cls[0], table, batch);
@@ -267,17 +299,26 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
         if (e != cudaSuccess) return e;
     }
     FewLaunch f;
-    if (!has_two_pass(p) && few_shape(p, batch, f)) {
+    if (!has_two_pass(p) && (!p.pow2.recs.empty() || few_shape(p, batch, f))) {
         BandArgs a = make_args(p, p.cls[0], table, batch);
         a.coef = const_cast<float2 *>(c);
         a.Y = Y;
         a.fold = fold_sidebands ? 1 : 0;
-        return launch_few<false>(p, a, f, st);
+        return p.pow2.recs.empty() ? launch_few<false>(p, a, f, st) : launch_pow2_plan<false>(p, a, st);
     }
     ForkJoin fj(p, st, batch);
     if (has_two_pass(p)) {
         cudaError_t e = launch_two_pass_to_spectrum(p, table, fold_sidebands, c, Y, scratch, batch, fj.two_pass_stream());
         if (e != cudaSuccess) { fj.join(); return e; }
+    }
+    if (!p.pow2.recs.empty()) {   // its other bands are class 0's and two-pass ones
+        BandArgs a = make_args(p, p.cls[0], table, batch);
+        a.coef = const_cast<float2 *>(c);
+        a.Y = Y;
+        a.fold = fold_sidebands ? 1 : 0;
+        cudaError_t e = launch_pow2_plan<false>(p, a, st);
+        fj.join();
+        return e;
     }
     if (!p.chirp.recs.empty()) {
         BandArgs a = make_args(p, p.cls[0], table, batch);

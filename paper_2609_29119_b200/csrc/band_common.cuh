@@ -139,6 +139,11 @@ __device__ __forceinline__ void slot_store(const BandRec &br, const float *__res
     if (CQT_CHK(dbg, 404, k, limit)) Y[k] = make_float2(h * u.x, h * u.y);
 }
 
+// band_pow2.cu: every band of more than 128 coefficients of a plan where those are all powers of two, in two launches by
+// length (the first often empty)
+bool pow2_has(const cqt_plan &p, bool long_ones);
+cudaError_t launch_pow2(const cqt_plan &p, bool analysis, bool long_ones, const BandArgs &b, cudaStream_t st);
+
 // band_split.cu: long bands of calls with few items
 cudaError_t launch_split(const cqt_plan &p, bool analysis, const BandArgs &b, cudaStream_t st);
 

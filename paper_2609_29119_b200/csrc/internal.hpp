@@ -43,6 +43,12 @@ struct ChirpBands {
     ChirpRec *d_recs = nullptr;
 };
 
+struct Pow2Bands {
+    int n_bands[kPow2Lengths] = {};    // per length, longest first
+    std::vector<Pow2Rec> recs;         // in that order
+    Pow2Rec *d_recs = nullptr;
+};
+
 struct SplitBands {
     std::vector<BandItem> items;     // record of the band, radix plan of a quarter of its length
     std::vector<SplitRec> recs;
@@ -100,6 +106,7 @@ struct cqt_plan {
     cqt::BandClass cls[cqt::kNumClasses];
     cqt::MergedBands merged;
     cqt::ChirpBands chirp;
+    cqt::Pow2Bands pow2;
     cqt::SplitBands split;             // the bands of the first segment of `merged` when that has 1024 threads per item
     std::vector<int8_t> band_class;    // length class of every band, -1: two-pass kernels
     cqt::TwoPassGroup two_pass[2];     // [0]: both factors <= 256, [1]: larger factors
@@ -213,6 +220,11 @@ cudaError_t configure_band_kernels(const cqt_plan &p);
 int chirp_length_index(int64_t m);     // which L serves m-point sub-transforms, -1: none
 int chirp_length(int index);
 cudaError_t configure_chirp_kernels(const cqt_plan &p);
+
+// band_pow2.cu
+int pow2_length_index(int64_t M);                  // place of a length in Pow2Bands::n_bands, -1: not a length of that kernel
+void pow2_radices(int index, int (&r)[4]);         // its stages (1: none)
+cudaError_t configure_pow2_kernels(const cqt_plan &p);
 
 // band_split.cu
 cudaError_t configure_split_kernels(const cqt_plan &p);

@@ -67,6 +67,14 @@ struct ChirpRec {
 };
 constexpr int kChirpLengths = 7;   // L = 8192 ... 128
 
+// A band on the power-of-two kernel.
+struct Pow2Rec {
+    BandRec br;
+    int32_t tw_off;      // twiddle rows of its length in the twiddle array (Pow2Shape in band_pow2.cu)
+    int32_t pad_[3];
+};
+constexpr int kPow2Lengths = 7;   // 16,384 ... 256
+
 // A band split into four work items (band_split.cu): two-level table of W_M
 struct SplitRec {
     int32_t tw_m, log_m_c, n_m, pad_;

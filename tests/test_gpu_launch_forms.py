@@ -48,18 +48,16 @@ def test_band_launch_forms(kw, batch):
     check_rows(small_workload("forms", **{"fs": 44100.0, "fmin": 60.0, "fmax": 22050.0, "channels": batch, **kw}), batch)
 
 
-@pytest.mark.parametrize("m", [33, 64 - 3, 127, 257, 509, 1021, 2039, 2053, 3191])
-def test_lengths_with_a_large_prime_factor(m):
-    """Regular bands of 4 m coefficients, m prime or not 5-smooth, up to both sides of each convolution length: against
-    numpy's FFT of the windowed, slot-placed spectrum; the round trip covers the synthesis form."""
-    from paper_2609_29119_b200 import Plan, M_MULT4
-    N, M = 1 << 15, 4 * m
+def check_bands_of_length(M, width, policy, batch):
+    """Two overlapping regular bands of M coefficients against numpy's FFT of the windowed, slot-placed spectrum; the round
+    trip covers the synthesis form."""
+    from paper_2609_29119_b200 import Plan
+    N = 1 << 15
     centre = [N / 4.0 - 0.1 * M, N / 4.0 + 0.1 * M]
-    plan = Plan.from_bands(float(N), N, centre, [M - 1.5] * 2, m_policy=M_MULT4)
-    rng = np.random.default_rng(m)
-    x = rng.standard_normal((3, N)).astype(np.float32)
-    xd = torch.from_numpy(x).cuda()
-    c = plan.analyse(xd)
+    plan = Plan.from_bands(float(N), N, centre, [width] * 2, m_policy=policy)
+    rng = np.random.default_rng(M)
+    x = rng.standard_normal((batch, N)).astype(np.float32)
+    c = plan.analyse(torch.from_numpy(x).cuda())
     g, _ = plan.tables()
     X = np.fft.rfft(x.astype(np.float64))
     for bi in plan.bands():
@@ -67,7 +65,7 @@ def test_lengths_with_a_large_prime_factor(m):
             continue
         assert bi.M == M
         d = np.arange(bi.first_offset, bi.first_offset + bi.support)
-        slots = np.zeros((3, M), dtype=np.complex128)
+        slots = np.zeros((batch, M), dtype=np.complex128)
         slots[:, d % M] = g[bi.table_offset:bi.table_offset + bi.support] * X[:, bi.centre_bin + d]
         want = np.fft.ifft(slots)
         got = c[:, bi.coeff_offset:bi.coeff_offset + M].cpu().numpy()
@@ -75,3 +73,17 @@ def test_lengths_with_a_large_prime_factor(m):
     y = plan.synthesise(c).cpu().numpy().astype(np.float64)
     assert (np.sum((y - x) ** 2, axis=1) / np.sum(x.astype(np.float64) ** 2, axis=1)).max() <= 1e-12
     plan.close()
+
+
+@pytest.mark.parametrize("m", [33, 64 - 3, 127, 257, 509, 1021, 2039, 2053, 3191])
+def test_lengths_with_a_large_prime_factor(m):
+    """4 m coefficients, m prime or not 5-smooth, up to both sides of each convolution length."""
+    check_bands_of_length(4 * m, 4 * m - 1.5, wl.M_MULT4, 3)
+
+
+@pytest.mark.parametrize("batch", [1, 33])
+@pytest.mark.parametrize("fill", [1.0, 0.52])
+@pytest.mark.parametrize("M", [256, 512, 1024, 2048, 4096, 8192])
+def test_power_of_two_lengths(M, fill, batch):
+    """Full support and one that leaves nearly half of the slots empty; an odd number of items in CTAs that share several."""
+    check_bands_of_length(M, fill * M - 1.5, wl.M_POW2, batch)
