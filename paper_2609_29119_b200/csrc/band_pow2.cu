@@ -245,7 +245,7 @@ __device__ __forceinline__ void pow2_cta(const Pow2Args &a, const Pow2Segment &s
 }
 
 template <bool ANALYSIS, bool LONG>
-__global__ void __launch_bounds__(LONG ? 512 : 256, LONG ? 2 : 3) pow2_bands_kernel(Pow2Args a) {
+__global__ void __launch_bounds__(LONG ? 512 : 256, LONG ? 2 : 4) pow2_bands_kernel(Pow2Args a) {
     chain_enter(a.b);
     int i = 0;
 #define X(S)                                                                                                                        \
