@@ -103,11 +103,6 @@ bool make_fft_plan(int64_t M, bool pow2, std::vector<float2> &tw, FftPlan &fp, b
             const double ang = -2.0 * kPi * (double)y / (double)M;
             tw.push_back(make_float2((float)std::cos(ang), (float)std::sin(ang)));
         }
-        for (int j = 0; j < fp.nstages && pow2; ++j) {
-            int l = 0;
-            while ((1 << l) < fp.st[j].radix) ++l;
-            fp.st[j].lg = l;
-        }
     }
     return true;
 }
@@ -335,12 +330,16 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     if (lf.A > 1) {
         // twiddles between the passes, W_Lp^{i (low + q NL)} = U[low][i] V[q][i] for element q of the last-stage butterfly whose
         // lowest frequency is low: both factors rounded once from their exact value
+        std::vector<std::complex<double>> fine, coarse;   // W_Lp^y and W_Lp^{2048 y}
+        for (int64_t y = 0; y < 2048; ++y) fine.push_back(std::polar(1.0, -2.0 * kPi * (double)y / (double)lf.Lp));
+        for (int64_t y = 0; y < (lf.Lp + 2047) / 2048; ++y) coarse.push_back(std::polar(1.0, -2.0 * kPi * (double)(2048 * y) / (double)lf.Lp));
         auto outer = [&](int64_t rows, int64_t cols, int64_t scale) {   // [row][col] = W_Lp^{scale row col}
             const int off = (int)tw.size();
             for (int64_t r = 0; r < rows; ++r)
                 for (int64_t c = 0; c < cols; ++c) {
-                    const double ang = -2.0 * kPi * (double)((scale * r * c) % lf.Lp) / (double)lf.Lp;
-                    tw.push_back(make_float2((float)std::cos(ang), (float)std::sin(ang)));
+                    const int64_t y = (scale * r * c) % lf.Lp;   // product of two double factors: 1e-16, rounded once
+                    const std::complex<double> w = fine[(size_t)(y & 2047)] * coarse[(size_t)(y >> 11)];
+                    tw.push_back(make_float2((float)w.real(), (float)w.imag()));
                 }
             return off;
         };

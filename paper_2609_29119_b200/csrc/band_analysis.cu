@@ -36,7 +36,7 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
         float2 *alt = buf + M;
         for (int m = tid; m < M; m += nthr) buf[m] = load(m, 0);
         Sync::sync(nthr);
-        fft_dif<+1, Sync, false>(buf, alt, 1, 1, 0u, fp, a.tw, tid, nthr);
+        fft_dif<+1, Sync>(buf, alt, 1, 1, 0u, fp, a.tw, tid, nthr);
         for (int n = tid; n < M; n += nthr) out[n] = buf[dif_pos(fp, n)];
         return;
     }
@@ -59,10 +59,10 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
             const float2 xv = ld_data(Xs + j);
             return make_float2(g * xv.x, g * xv.y);
         };
-        fft_fused<+1, Sync, false, true, false, true, false, false, MAXR>(t, fp, tws, load_regular, store, tid, nthr);
+        fft_fused<+1, Sync, true, false, true, false, false, MAXR>(t, fp, tws, load_regular, store, tid, nthr);
         return;
     }
-    fft_fused<+1, Sync, false, true, false, true, false, false, MAXR>(t, fp, tws, load, store, tid, nthr);
+    fft_fused<+1, Sync, true, false, true, false, false, MAXR>(t, fp, tws, load, store, tid, nthr);
 }
 
 // One class: groups of LANES lanes (or the whole CTA) per item.

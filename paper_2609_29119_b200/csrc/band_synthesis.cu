@@ -62,7 +62,7 @@ __device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem
         float2 *alt = buf + M;
         for (int n = tid; n < M; n += nthr) buf[n] = load(n, 0);
         Sync::sync(nthr);
-        fft_dif<-1, Sync, false>(buf, alt, 1, 1, 0u, fp, a.tw, tid, nthr);
+        fft_dif<-1, Sync>(buf, alt, 1, 1, 0u, fp, a.tw, tid, nthr);
         for (int m = tid; m < M; m += nthr) store(m, 0, buf[dif_pos(fp, m)]);
         return;
     }
@@ -77,10 +77,10 @@ __device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem
         const RegularStore store_regular{tab, Ys, last_pos, first_neg, br.d0, shift_neg};
         // coefficients are read once: streaming loads keep the L2 for the weighted-bin planes
         auto load_regular = [&](int n, int) -> float2 { return __ldcs(in + n); };
-        fft_fused<-1, Sync, false, true, false, true, false, false, MAXR>(t, fp, tws, load_regular, store_regular, tid, nthr);
+        fft_fused<-1, Sync, true, false, true, false, false, MAXR>(t, fp, tws, load_regular, store_regular, tid, nthr);
         return;
     }
-    fft_fused<-1, Sync, false, true, false, true, false, false, MAXR>(t, fp, tws, load, store, tid, nthr);
+    fft_fused<-1, Sync, true, false, true, false, false, MAXR>(t, fp, tws, load, store, tid, nthr);
 }
 
 // One class: groups of LANES lanes (or the whole CTA) per item.

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(THREADS, MINB) band2p_cols_kernel(TwoPassArgs 
         if (ANALYSIS) w.y = -w.y;
         if (CQT_CHK(a.dbg, 401, (long long)r * rec.B + c0 + c, br.M)) T[(long long)r * rec.B + c0 + c] = cmul(v, w);
     };
-    fft_fused<ANALYSIS ? +1 : -1, BlockSync, false, false, true, false, true, true>(t, fp, twf, load, store, tid, nthr);
+    fft_fused<ANALYSIS ? +1 : -1, BlockSync, false, true, false, true, true>(t, fp, twf, load, store, tid, nthr);
     __syncthreads();   // the next signal's first stage overwrites the tile
     }
 }
@@ -119,14 +119,14 @@ __global__ void __launch_bounds__(THREADS, MINB) band2p_rows_kernel(TwoPassArgs 
             const long long n = (long long)(r0 + r) + (long long)rec.A * q;
             if (r < nrows && CQT_CHK(a.dbg, 403, n, br.M)) out[n] = v;
         };
-        fft_fused<+1, BlockSync, false, false, false, false, true, true>(t, fp, twf, load, store, tid, nthr);
+        fft_fused<+1, BlockSync, false, false, false, true, true>(t, fp, twf, load, store, tid, nthr);
     } else {
         const float *tab = a.table + br.tab_off;
         float2 *Y = a.Y + (long long)ch * a.y_pitch + br.y_off;
         auto store = [&](int q, int r, float2 u) {
             if (r < nrows) slot_store(br, tab, Y, a.N, (r0 + r) + rec.A * q, u, a.dbg, (long long)a.y_pitch - br.y_off);
         };
-        fft_fused<-1, BlockSync, false, false, false, false, true, true>(t, fp, twf, load, store, tid, nthr);
+        fft_fused<-1, BlockSync, false, false, false, true, true>(t, fp, twf, load, store, tid, nthr);
     }
     __syncthreads();   // the next signal's first stage overwrites the tile
     }

@@ -163,9 +163,8 @@ __device__ void dif_stage_generic(float2 *buf, float2 *alt, float2 *wp, int pitc
 }
 
 // SIGN = -1: forward DFT (exp(-...)), SIGN = +1: unnormalised inverse.
-// POW2 restricts the radix switch to powers of two (long-FFT kernels).
 // The caller must synchronise before (inputs visible); the routine ends with a sync.
-template <int SIGN, class Sync, bool POW2>
+template <int SIGN, class Sync>
 __device__ void fft_dif(float2 *buf, float2 *alt, int pitch, int ncols, uint32_t ncols_magic, const FftPlan &fp,
                         const float2 *__restrict__ tw_base, int tid, int nthr) {
     const float2 *tw = tw_base + fp.tw_off;
@@ -179,19 +178,12 @@ __device__ void fft_dif(float2 *buf, float2 *alt, int pitch, int ncols, uint32_t
     case RR:                                                                                               \
         dif_stage<RR, SIGN>(buf, pitch, ncols, ncols_magic, M, n_cur, s, sm, tmul, tw, logC, tid, nthr); \
         break;
-        if (POW2) {
-            switch (r) {
-                CQT_STAGE(2) CQT_STAGE(4) CQT_STAGE(8) CQT_STAGE(16)
-                default: break;
-            }
-        } else {
-            switch (r) {
-                CQT_STAGE(2) CQT_STAGE(3) CQT_STAGE(4) CQT_STAGE(5) CQT_STAGE(6) CQT_STAGE(8) CQT_STAGE(9)
-                CQT_STAGE(10) CQT_STAGE(12) CQT_STAGE(15) CQT_STAGE(16)
-                default:
-                    dif_stage_generic<SIGN, Sync>(buf, alt, alt + (size_t)M * pitch, pitch, ncols, M, r, tw, logC, tid, nthr);
-                    break;
-            }
+        switch (r) {
+            CQT_STAGE(2) CQT_STAGE(3) CQT_STAGE(4) CQT_STAGE(5) CQT_STAGE(6) CQT_STAGE(8) CQT_STAGE(9)
+            CQT_STAGE(10) CQT_STAGE(12) CQT_STAGE(15) CQT_STAGE(16)
+            default:
+                dif_stage_generic<SIGN, Sync>(buf, alt, alt + (size_t)M * pitch, pitch, ncols, M, r, tw, logC, tid, nthr);
+                break;
         }
 #undef CQT_STAGE
         Sync::sync(nthr);
@@ -258,18 +250,6 @@ __device__ __forceinline__ void apply_twiddle_direct(const float2 *twf, uint32_t
         re[q] = fmaf(x, w.x, -y * wi);
         im[q] = fmaf(x, wi, y * w.x);
     }
-}
-
-// position of frequency k for a power-of-two plan: digit reversal by shifts
-__device__ __forceinline__ uint32_t dif_pos_pow2(const FftPlan &fp, uint32_t k) {
-    uint32_t pos = 0, rem = k;
-#pragma unroll 1
-    for (int j = 0; j < fp.nstages; ++j) {
-        const int l = fp.st[j].lg;
-        pos = (pos << l) | (rem & ((1u << l) - 1));
-        rem >>= l;
-    }
-    return pos;
 }
 
 struct Tile {
@@ -487,7 +467,6 @@ __device__ __forceinline__ void only_stage(const Tile &t, Load load, Store store
 }
 
 #define CQT_RADIX_CASES_ALL(X) X(2) X(3) X(4) X(5) X(6) X(8) X(9) X(10) X(12) X(15) X(16)
-#define CQT_RADIX_CASES_POW2(X) X(2) X(4) X(8) X(16)
 
 // Runs the first `nrun` stages of the plan (nrun = nstages: the whole transform with the last stage fused
 // into `store`; nrun = nstages - 1... not offered: use fft_fused_keep for "results stay in shared memory").
@@ -496,69 +475,33 @@ __device__ __forceinline__ void only_stage(const Tile &t, Load load, Store store
 // Requires a non-generic plan.  tw = shared-memory copy of the plan's two-level table, written by the
 // caller (stage_twiddles) WITHOUT a barrier after it: the first stage synchronises once its operand loads
 // are issued.  The routine synchronises between stages, not at the end.
-template <int SIGN, class Sync, bool POW2, bool PAD, bool COLFAST_IN, bool REV, bool COLFAST_OUT, bool DIRECT, int MAXR = 16, class Load, class Store>
+template <int SIGN, class Sync, bool PAD, bool COLFAST_IN, bool REV, bool COLFAST_OUT, bool DIRECT, int MAXR = 16, class Load, class Store>
 __device__ __forceinline__ void fft_fused(const Tile &t, const FftPlan &fp, const float2 *tw, Load load, Store store, int tid, int nthr) {
     const int d = fp.nstages;
     if (d == 1) {
         Sync::sync(nthr);   // tables staged by the caller become visible to the functors
-#define X(RR) case RR: if constexpr (POW2 || RR <= MAXR) only_stage<RR, SIGN>(t, load, store, tid, nthr); break;
-        if (POW2) { switch (fp.st[0].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
-        else { switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
+#define X(RR) case RR: if constexpr (RR <= MAXR) only_stage<RR, SIGN>(t, load, store, tid, nthr); break;
+        switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; }
 #undef X
         return;
     }
-#define X(RR) case RR: if constexpr (POW2 || RR <= MAXR) first_stage<RR, SIGN, PAD, COLFAST_IN, DIRECT, Sync>(t, fp, tw, load, tid, nthr); break;
-    if (POW2) { switch (fp.st[0].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
-    else { switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
+#define X(RR) case RR: if constexpr (RR <= MAXR) first_stage<RR, SIGN, PAD, COLFAST_IN, DIRECT, Sync>(t, fp, tw, load, tid, nthr); break;
+    switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; }
 #undef X
     Sync::sync(nthr);
     int n_cur = fp.st[0].stride, tmul = fp.st[0].radix;
 #pragma unroll 1
     for (int j = 1; j < d - 1; ++j) {
-#define X(RR) case RR: if constexpr (POW2 || RR <= MAXR) middle_stage<RR, SIGN, PAD, DIRECT>(t, fp, tw, j, n_cur, tmul, tid, nthr); break;
-        if (POW2) { switch (fp.st[j].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
-        else { switch (fp.st[j].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
+#define X(RR) case RR: if constexpr (RR <= MAXR) middle_stage<RR, SIGN, PAD, DIRECT>(t, fp, tw, j, n_cur, tmul, tid, nthr); break;
+        switch (fp.st[j].radix) { CQT_RADIX_CASES_ALL(X) default: break; }
 #undef X
         Sync::sync(nthr);
         n_cur = fp.st[j].stride;
         tmul *= fp.st[j].radix;
     }
-#define X(RR) case RR: if constexpr (POW2 || RR <= MAXR) last_stage<RR, SIGN, PAD, REV, COLFAST_OUT>(t, fp, store, tid, nthr); break;
-    if (POW2) { switch (fp.st[d - 1].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
-    else { switch (fp.st[d - 1].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
+#define X(RR) case RR: if constexpr (RR <= MAXR) last_stage<RR, SIGN, PAD, REV, COLFAST_OUT>(t, fp, store, tid, nthr); break;
+    switch (fp.st[d - 1].radix) { CQT_RADIX_CASES_ALL(X) default: break; }
 #undef X
-}
-
-// Same, but every stage after the first runs in shared memory and the results stay there
-// (digit-reversed positions, see dif_pos); ends with a sync.
-template <int SIGN, class Sync, bool POW2, bool COLFAST_IN, bool DIRECT, class Load>
-__device__ __forceinline__ void fft_fused_keep(const Tile &t, const FftPlan &fp, const float2 *tw, Load load, int tid, int nthr) {
-    const int d = fp.nstages;
-    if (d == 1) {
-        auto keep = [&](int k, int col, float2 v) { t.buf[(size_t)k * t.pitch + col] = v; };
-#define X(RR) case RR: only_stage<RR, SIGN>(t, load, keep, tid, nthr); break;
-        if (POW2) { switch (fp.st[0].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
-        else { switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
-#undef X
-        Sync::sync(nthr);
-        return;
-    }
-#define X(RR) case RR: first_stage<RR, SIGN, false, COLFAST_IN, DIRECT, Sync>(t, fp, tw, load, tid, nthr); break;
-    if (POW2) { switch (fp.st[0].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
-    else { switch (fp.st[0].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
-#undef X
-    Sync::sync(nthr);
-    int n_cur = fp.st[0].stride, tmul = fp.st[0].radix;
-#pragma unroll 1
-    for (int j = 1; j < d; ++j) {
-#define X(RR) case RR: middle_stage<RR, SIGN, false, DIRECT>(t, fp, tw, j, n_cur, tmul, tid, nthr); break;
-        if (POW2) { switch (fp.st[j].radix) { CQT_RADIX_CASES_POW2(X) default: break; } }
-        else { switch (fp.st[j].radix) { CQT_RADIX_CASES_ALL(X) default: break; } }
-#undef X
-        Sync::sync(nthr);
-        n_cur = fp.st[j].stride;
-        tmul *= fp.st[j].radix;
-    }
 }
 
 }  // namespace cqt

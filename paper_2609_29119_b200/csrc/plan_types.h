@@ -20,8 +20,7 @@ struct alignas(16) StageRec {
     uint32_t smagic;    // ceil(2^32 / s_j)
     int32_t k1div;      // s_0 / n_j: butterfly blocks of stage j per first-stage output digit
     uint32_t k1magic;
-    int32_t lg;         // log2 r_j for power-of-two plans
-    int32_t pad_;
+    int32_t pad_[2];
 };
 
 struct FftPlan {
@@ -87,12 +86,6 @@ struct TwoPassRec {
     int32_t fft_A, fft_B;        // FftPlan indices (plans with full twiddle tables)
     int32_t tw_m, log_m_c, n_m;  // two-level table of W_M
     int64_t scratch_off;         // into one signal's two-pass scratch row
-};
-
-// Per-bin cover: bands cover_lo .. cover_lo + cover_n - 1 contain the bin (contiguous because
-// support starts and ends are monotone in the band index).
-struct BinCover {
-    int32_t lo_n;       // (cover_lo << 8) | cover_n
 };
 
 }  // namespace cqt

@@ -159,8 +159,9 @@ cqt_status ingest(cqt_slicq *s, const float *x, int64_t x_stride, int64_t first,
 cqt_status analyse_ready(cqt_slicq *s, const float *fresh, int64_t fresh_stride, int64_t new_first, cudaStream_t st) {
     const int64_t ready = s->n_in / s->H;
     if (s->next_slice >= ready) return ingest(s, fresh, fresh_stride, new_first, s->n_in - new_first, st);
-    const bool fused = cqt::can_fuse_slice_cut(*s->plan) && s->ring_in >= s->sl;
-    // one-pass lengths cut the slices out of the ring in a kernel of their own
+    // ring positions of the fused cut are 32-bit
+    const bool fused = cqt::can_fuse_slice_cut(*s->plan) && s->ring_in >= s->sl && s->ring_in <= INT32_MAX / 2;
+    // the others (one-pass lengths) cut the slices out of the ring in a kernel of their own
     if (!fused) {
         const cqt_status r = ingest(s, fresh, fresh_stride, new_first, s->n_in - new_first, st);
         if (r != CQT_OK) return r;
