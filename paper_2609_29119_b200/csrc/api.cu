@@ -387,17 +387,20 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         br.fft = -1;
     }
     // ---- launch classes by band length
-    // class 0: 8 lanes per item, 32 items per CTA; the others one CTA per item, sized so that several CTAs
-    // share an SM (64 registers per thread) except for the longest bands, which fill its shared memory
+    // class 0: 8 lanes per item, 32 items per CTA; class 1: a warp per item, 8 items per CTA (calls with few items take the
+    // merged form; with a CTA of 64 threads per item the class was bound by the rate at which CTAs start: 17 % of the warps
+    // active, 256 signals at 24 bands per octave 57 -> 52 us, and fewer warps leave more of the SMs to the classes beside
+    // it, the whole analysis 102 -> 88 us); the others one CTA per item, sized so that several CTAs share an SM (64 registers
+    // per thread) except for the longest bands, which fill its shared memory
     const int limits[kNumClasses] = {128, 1024, 4096, 13500, 1 << 30};
     {
-        const int threads[kNumClasses] = {256, 64, 256, 512, 1024};
-        const int minb[kNumClasses] = {4, 16, 4, 2, 1};
+        const int threads[kNumClasses] = {256, 256, 256, 512, 1024};
+        const int minb[kNumClasses] = {4, 4, 4, 2, 1};
         for (int c = 0; c < kNumClasses; ++c) {
             p->cls[c].threads = threads[c];
             p->cls[c].min_blocks = minb[c];
-            p->cls[c].lanes_few = c == 0 ? 32 : 0;
-            p->cls[c].lanes_many = c == 0 ? 8 : 0;
+            p->cls[c].lanes_few = c <= 1 ? 32 : 0;
+            p->cls[c].lanes_many = c == 0 ? 8 : (c == 1 ? 32 : 0);
             p->cls[c].max_radix = c <= 1 ? 8 : (c == 2 ? 12 : 16);
         }
     }

@@ -160,6 +160,6 @@ cudaError_t launch_chirp(const cqt_plan &p, bool analysis, const BandArgs &b, cu
 // compiled in), each with and without the prime-factor paths (GEN): code a class never runs is left out, which also
 // frees registers in the paths it does run.
 #define CQT_KERNEL_TABLE(X) \
-    X(256, 4, 8, 8) X(256, 4, 32, 8) X(64, 16, 0, 8) X(128, 8, 0, 12) X(256, 4, 0, 12) X(512, 2, 0, 16) X(1024, 1, 0, 16)
+    X(256, 4, 8, 8) X(256, 4, 32, 8) X(128, 8, 0, 12) X(256, 4, 0, 12) X(512, 2, 0, 16) X(1024, 1, 0, 16)
 
 }  // namespace cqt
