@@ -808,21 +808,21 @@ cqt_status end_call(const Call &c, cudaError_t e) {
 
 cqt_status run_analysis_form(const cqt_plan *p, const float *table, const float *x, int64_t x_stride, int64_t batch,
                              int64_t valid_len, cqt_c64 *c, void *ws, size_t ws_bytes, void *stream,
-                             const cqt::SliceSource *src = nullptr) {
+                             const cqt::SliceSource *src = nullptr, int row0 = 0, int rows = INT32_MAX) {
     Call k;
     cqt_status s = begin_call(p, x, x_stride, batch, valid_len, c, ws, ws_bytes, stream, k);
     if (s != CQT_OK) return s;
     cudaError_t e = launch_rfft_forward(*p, x, x_stride, batch, valid_len, k.T, k.second, k.st, src);
-    if (e == cudaSuccess) e = launch_bands_from_spectrum(*p, table, k.second, reinterpret_cast<float2 *>(c), k.huge, batch, k.st);
+    if (e == cudaSuccess) e = launch_bands_from_spectrum(*p, table, k.second, CoefRows{reinterpret_cast<float2 *>(c), row0, rows}, k.huge, batch, k.st);
     return end_call(k, e);
 }
 
 cqt_status run_synthesis_form(const cqt_plan *p, const float *table, bool fold, const cqt_c64 *c, int64_t batch,
-                              int64_t valid_len, float *x, int64_t x_stride, void *ws, size_t ws_bytes, void *stream) {
+                              int64_t valid_len, float *x, int64_t x_stride, void *ws, size_t ws_bytes, void *stream, int row0 = 0, int rows = INT32_MAX) {
     Call k;
     cqt_status s = begin_call(p, x, x_stride, batch, valid_len, c, ws, ws_bytes, stream, k);
     if (s != CQT_OK) return s;
-    cudaError_t e = launch_bands_to_spectrum(*p, table, fold, reinterpret_cast<const float2 *>(c), k.second, k.huge, batch, k.st);
+    cudaError_t e = launch_bands_to_spectrum(*p, table, fold, CoefRows{reinterpret_cast<float2 *>(const_cast<cqt_c64 *>(c)), row0, rows}, k.second, k.huge, batch, k.st);
     if (e == cudaSuccess) e = launch_rfft_inverse(*p, k.second, k.T, x, x_stride, batch, valid_len, k.st);
     return end_call(k, e);
 }
@@ -831,12 +831,17 @@ cqt_status run_synthesis_form(const cqt_plan *p, const float *table, bool fold, 
 
 namespace cqt {
 
-// Analysis of slices cut from a stream's ring buffer (slicq.cu): cqt_analyse with the slice cut fused into the load of
-// the long FFT's first pass.  batch = slices x channels rows of the plan's full length.
-cqt_status analyse_slices(const cqt_plan *p, const SliceSource &src, int64_t batch, cqt_c64 *c, void *ws, size_t ws_bytes,
-                          void *stream) {
-    if (!p || !src.ring || !src.win || !can_fuse_slice_cut(*p)) return CQT_ERR_INVALID_ARG;
-    return run_analysis_form(p, p->d.tab_analysis, src.ring, p->N, batch, p->N, c, ws, ws_bytes, stream, &src);
+// The sliced form (slicq.cu): transforms whose coefficient rows lie in a ring of `rows` rows at c, the first at row0.
+// src: the slice cut fused into the load of the long FFT's first pass; else the slices are the rows of x.
+cqt_status analyse_slices(const cqt_plan *p, const SliceSource *src, const float *x, int64_t batch, cqt_c64 *c, int row0, int rows, void *ws,
+                          size_t ws_bytes, void *stream) {
+    if (!p || (src && (!src->ring || !src->win || !can_fuse_slice_cut(*p)))) return CQT_ERR_INVALID_ARG;
+    return run_analysis_form(p, p->d.tab_analysis, src ? src->ring : x, p->N, batch, p->N, c, ws, ws_bytes, stream, src, row0, rows);
+}
+cqt_status synthesise_slices(const cqt_plan *p, const cqt_c64 *c, int row0, int rows, int64_t batch, float *x, void *ws, size_t ws_bytes,
+                             void *stream) {
+    if (!p) return CQT_ERR_INVALID_ARG;
+    return run_synthesis_form(p, p->d.tab_synthesis, false, c, batch, p->N, x, p->N, ws, ws_bytes, stream, row0, rows);
 }
 
 }  // namespace cqt

@@ -21,6 +21,12 @@ static BandArgs make_args(const cqt_plan &p, const BandClass &c, const float *ta
     return a;
 }
 
+static void set_rows(BandArgs &a, const CoefRows &c) {
+    a.coef = c.base;
+    a.row0 = c.row0;
+    a.rows = c.rows;
+}
+
 const void *band_analysis_kernel(const BandClass &c, int lanes);    // band_analysis.cu
 const void *band_synthesis_kernel(const BandClass &c, int lanes);   // band_synthesis.cu
 
@@ -236,14 +242,14 @@ struct ForkJoin {
 
 static bool has_two_pass(const cqt_plan &p) { return !p.two_pass[0].bands.empty() || !p.two_pass[1].bands.empty(); }
 
-cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, float2 *c,
+cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, const CoefRows &c,
                                        float2 *scratch, int64_t batch, cudaStream_t st) {
     FewLaunch f;
     if (!has_two_pass(p) && (!p.pow2.recs.empty() || few_shape(p, batch, f))) {
         BandArgs a = make_args(p, p.cls[0], table, batch);
         a.spec = X;
         a.spec_pitch = p.lf.x_pitch;
-        a.coef = c;
+        set_rows(a, c);
         return p.pow2.recs.empty() ? launch_few<true>(p, a, f, st) : launch_pow2_plan<true>(p, a, st);
     }
     ForkJoin fj(p, st, batch);
@@ -255,7 +261,7 @@ cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, co
         BandArgs a = make_args(p, p.cls[0], table, batch);
         a.spec = X;
         a.spec_pitch = p.lf.x_pitch;
-        a.coef = c;
+        set_rows(a, c);
         cudaError_t e = launch_pow2_plan<true>(p, a, st);
         fj.join();
         return e;
@@ -264,7 +270,7 @@ cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, co
         BandArgs a = make_args(p, p.cls[0], table, batch);
         a.spec = X;
         a.spec_pitch = p.lf.x_pitch;
-        a.coef = c;
+        set_rows(a, c);
         cudaError_t e = launch_chirp(p, true, a, fj.two_pass_stream());
         if (e != cudaSuccess) { fj.join(); return e; }
     }
@@ -275,7 +281,7 @@ cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, co
         BandArgs a = make_args(p, p.cls[i], table, batch);
         a.spec = X;
         a.spec_pitch = p.lf.x_pitch;
-        a.coef = c;
+        set_rows(a, c);
         cudaError_t e = launch_class<true>(p, i, names[i], a, fj.stream_for(i));
         if (e != cudaSuccess) { fj.join(); return e; }
     }
@@ -290,7 +296,7 @@ __global__ void __launch_bounds__(128) zero_fill_kernel(float2 *Y, long long y_p
     for (int i = threadIdx.x; i < sg.y; i += blockDim.x) y[i] = make_float2(0.f, 0.f);
 }
 
-cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool fold_sidebands, const float2 *c,
+cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool fold_sidebands, const CoefRows &c,
                                      float2 *Y, float2 *scratch, int64_t batch, cudaStream_t st) {
     if (p.n_zero_seg > 0) {
         zero_fill_kernel<<<dim3((unsigned)p.n_zero_seg, (unsigned)batch), 128, 0, st>>>(Y, p.y_pitch, p.d.zero_seg);
@@ -301,7 +307,7 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
     FewLaunch f;
     if (!has_two_pass(p) && (!p.pow2.recs.empty() || few_shape(p, batch, f))) {
         BandArgs a = make_args(p, p.cls[0], table, batch);
-        a.coef = const_cast<float2 *>(c);
+        set_rows(a, c);
         a.Y = Y;
         a.fold = fold_sidebands ? 1 : 0;
         return p.pow2.recs.empty() ? launch_few<false>(p, a, f, st) : launch_pow2_plan<false>(p, a, st);
@@ -313,7 +319,7 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
     }
     if (!p.pow2.recs.empty()) {   // its other bands are class 0's and two-pass ones
         BandArgs a = make_args(p, p.cls[0], table, batch);
-        a.coef = const_cast<float2 *>(c);
+        set_rows(a, c);
         a.Y = Y;
         a.fold = fold_sidebands ? 1 : 0;
         cudaError_t e = launch_pow2_plan<false>(p, a, st);
@@ -322,7 +328,7 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
     }
     if (!p.chirp.recs.empty()) {
         BandArgs a = make_args(p, p.cls[0], table, batch);
-        a.coef = const_cast<float2 *>(c);
+        set_rows(a, c);
         a.Y = Y;
         a.fold = fold_sidebands ? 1 : 0;
         cudaError_t e = launch_chirp(p, false, a, fj.two_pass_stream());
@@ -333,7 +339,7 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
                                               "bands_to_spectrum/class4"};
     for (int i = kNumClasses - 1; i >= 0; --i) {
         BandArgs a = make_args(p, p.cls[i], table, batch);
-        a.coef = const_cast<float2 *>(c);
+        set_rows(a, c);
         a.Y = Y;
         a.fold = fold_sidebands ? 1 : 0;
         cudaError_t e = launch_class<false>(p, i, names[i], a, fj.stream_for(i));

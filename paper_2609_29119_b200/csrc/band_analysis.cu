@@ -28,7 +28,7 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
         const float2 xv = ld_data(X + km);
         return make_float2(g * xv.x, mirrored ? -(g * xv.y) : g * xv.y);
     };
-    float2 *out = a.coef + (long long)ch * a.coeff_count + br.coeff_off;
+    float2 *out = a.coef + coef_row(a.row0, a.rows, ch) * a.coeff_count + br.coeff_off;
     // GEN: the class holds lengths with prime factors above 5 (only the multiple-of-4 length policy makes them, and the
     // longer ones run on the chirp-z kernel); the other instantiations leave the direct-sum code out
     if (GEN && fp.generic) {

@@ -26,7 +26,8 @@ struct BandArgs {
     int fold;                // synthesis form: add conj of the mirrored slot for sidebands
     const float2 *spec;      // analysis form: half spectrum rows; synthesis form: unused
     long long spec_pitch;
-    float2 *coef;            // coefficients (read or written)
+    float2 *coef;            // coefficients (read or written), see CoefRows
+    int row0, rows;
     long long coeff_count;
     float2 *Y;               // synthesis form: weighted-bin rows
     long long y_pitch;

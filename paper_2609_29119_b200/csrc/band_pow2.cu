@@ -169,7 +169,7 @@ __device__ __forceinline__ void pow2_cta(const Pow2Args &a, const Pow2Segment &s
     const float *tab = a.b.table + br.tab_off;
     constexpr int M = S::L;
     chain_begin(a.b);   // the record belongs to the plan; what follows touches the predecessor's output
-    float2 *c = a.b.coef + (long long)ch * a.b.coeff_count + br.coeff_off;
+    float2 *c = a.b.coef + coef_row(a.b.row0, a.b.rows, ch) * a.b.coeff_count + br.coeff_off;
     const int last_pos = br.d0 + br.S - 1, first_neg = M + br.d0;
     // support entry of slot m, -1: none
     auto entry = [&](int m) { return m <= last_pos ? m - br.d0 : (m >= first_neg ? m - first_neg : -1); };

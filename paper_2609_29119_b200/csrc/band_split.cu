@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) split_bands_kernel(BandArgs 
     __syncthreads();
     const float *tab = a.table + br.tab_off;
     const float2 *X = ANALYSIS ? a.spec + (long long)ch * a.spec_pitch : nullptr;
-    float2 *c = a.coef + (long long)ch * a.coeff_count + br.coeff_off;
+    float2 *c = a.coef + coef_row(a.row0, a.rows, ch) * a.coeff_count + br.coeff_off;
     float2 *Y = ANALYSIS ? nullptr : a.Y + (long long)ch * a.y_pitch + br.y_off;
     const bool fold = !ANALYSIS && a.fold && br.side != 0;
     auto in = [&](int n) -> float2 {

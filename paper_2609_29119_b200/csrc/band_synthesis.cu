@@ -30,7 +30,7 @@ __device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem
     const BandRec br = it.br;
     const FftPlan &fp = it.fp;
     const int M = br.M;
-    const float2 *in = a.coef + (long long)ch * a.coeff_count + br.coeff_off;
+    const float2 *in = a.coef + coef_row(a.row0, a.rows, ch) * a.coeff_count + br.coeff_off;
     // adjoint of analysis, sidebands: U[m] + conj U[-m] is the DFT of 2 Re c
     const bool fold = a.fold && br.side != 0;
     auto load = [&](int n, int) -> float2 {

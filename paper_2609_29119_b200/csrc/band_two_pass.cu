@@ -31,7 +31,8 @@ struct TwoPassArgs {
     int fold;                // synthesis form, adjoint: sideband input is replaced by 2 Re c
     const float2 *spec;      // analysis form: half-spectrum rows
     long long spec_pitch;
-    float2 *coef;
+    float2 *coef;            // see CoefRows
+    int row0, rows;
     long long coeff_count;
     float2 *Y;
     long long y_pitch;
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(THREADS, MINB) band2p_cols_kernel(TwoPassArgs 
     pdl_wait();   // tables and records belong to the plan; the loop touches the predecessor's output
     for (int ch = ch0; ch < ch1; ++ch) {
     const float2 *X = ANALYSIS ? a.spec + (long long)ch * a.spec_pitch : nullptr;
-    const float2 *cin = ANALYSIS ? nullptr : a.coef + (long long)ch * a.coeff_count + br.coeff_off;
+    const float2 *cin = ANALYSIS ? nullptr : a.coef + coef_row(a.row0, a.rows, ch) * a.coeff_count + br.coeff_off;
     float2 *T = a.scratch + (long long)ch * a.scratch_pitch + rec.scratch_off;
     auto load = [&](int r, int c) -> float2 {
         if (c >= ncols) return make_float2(0.f, 0.f);
@@ -114,7 +115,7 @@ __global__ void __launch_bounds__(THREADS, MINB) band2p_rows_kernel(TwoPassArgs 
         return CQT_CHK(a.dbg, 402, i, br.M) ? ld_data(T + i) : make_float2(0.f, 0.f);
     };
     if (ANALYSIS) {
-        float2 *out = a.coef + (long long)ch * a.coeff_count + br.coeff_off;
+        float2 *out = a.coef + coef_row(a.row0, a.rows, ch) * a.coeff_count + br.coeff_off;
         auto store = [&](int q, int r, float2 v) {
             const long long n = (long long)(r0 + r) + (long long)rec.A * q;
             if (r < nrows && CQT_CHK(a.dbg, 403, n, br.M)) out[n] = v;
@@ -158,7 +159,7 @@ static const void *rows_kernel(int g, int wi) {
 }
 
 template <bool ANALYSIS>
-static cudaError_t run_group(const cqt_plan &p, int g, const float *table, bool fold, const float2 *X, float2 *coef,
+static cudaError_t run_group(const cqt_plan &p, int g, const float *table, bool fold, const float2 *X, const CoefRows &coef,
                              float2 *Y, float2 *scratch, int64_t batch, cudaStream_t st) {
     const TwoPassGroup &grp = p.two_pass[g];
     if (grp.bands.empty()) return cudaSuccess;
@@ -172,7 +173,7 @@ static cudaError_t run_group(const cqt_plan &p, int g, const float *table, bool 
     a.N = (int)p.N;
     a.fold = fold ? 1 : 0;
     a.spec = X; a.spec_pitch = p.lf.x_pitch;
-    a.coef = coef; a.coeff_count = p.lay.coeff_count;
+    a.coef = coef.base; a.row0 = coef.row0; a.rows = coef.rows; a.coeff_count = p.lay.coeff_count;
     a.Y = Y; a.y_pitch = p.y_pitch;
     a.scratch = scratch; a.scratch_pitch = p.two_pass_pitch;
     a.dbg = p.d.dbg;
@@ -201,7 +202,7 @@ static cudaError_t run_group(const cqt_plan &p, int g, const float *table, bool 
     return e;
 }
 
-cudaError_t launch_two_pass_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, float2 *c,
+cudaError_t launch_two_pass_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, const CoefRows &c,
                                           float2 *scratch, int64_t batch, cudaStream_t st) {
     for (int g = 1; g >= 0; --g) {
         cudaError_t e = run_group<true>(p, g, table, false, X, c, nullptr, scratch, batch, st);
@@ -210,10 +211,10 @@ cudaError_t launch_two_pass_from_spectrum(const cqt_plan &p, const float *table,
     return cudaSuccess;
 }
 
-cudaError_t launch_two_pass_to_spectrum(const cqt_plan &p, const float *table, bool fold, const float2 *c, float2 *Y,
+cudaError_t launch_two_pass_to_spectrum(const cqt_plan &p, const float *table, bool fold, const CoefRows &c, float2 *Y,
                                         float2 *scratch, int64_t batch, cudaStream_t st) {
     for (int g = 1; g >= 0; --g) {
-        cudaError_t e = run_group<false>(p, g, table, fold, nullptr, const_cast<float2 *>(c), Y, scratch, batch, st);
+        cudaError_t e = run_group<false>(p, g, table, fold, nullptr, c, Y, scratch, batch, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -207,12 +207,20 @@ inline cudaError_t launch_kernel_args(void (*kernel)(KArgs...), dim3 grid, dim3 
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Coefficient rows of a call: row r at base + ((row0 + r) mod rows) * coeff_count.  Plain calls have row0 = 0 and no end;
+// the sliced form keeps its slices in a ring of rows, and slices that wrap around its end go through one call.
+struct CoefRows {
+    float2 *base;
+    int row0 = 0, rows = INT32_MAX;
+};
+__host__ __device__ inline long long coef_row(int row0, int rows, int r) { return r < rows - row0 ? row0 + r : row0 + r - rows; }
+
 // band.cu
 // every band of the plan: the single-CTA classes and, beside them on a stream of their own, the two-pass bands
 // (scratch: their rows in the workspace)
-cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, float2 *c,
+cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, const CoefRows &c,
                                        float2 *scratch, int64_t batch, cudaStream_t st);
-cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool fold_sidebands, const float2 *c,
+cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool fold_sidebands, const CoefRows &c,
                                      float2 *Y, float2 *scratch, int64_t batch, cudaStream_t st);
 cudaError_t configure_band_kernels(const cqt_plan &p);
 
@@ -230,9 +238,9 @@ cudaError_t configure_pow2_kernels(const cqt_plan &p);
 cudaError_t configure_split_kernels(const cqt_plan &p);
 
 // band_two_pass.cu
-cudaError_t launch_two_pass_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, float2 *c,
+cudaError_t launch_two_pass_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, const CoefRows &c,
                                           float2 *scratch, int64_t batch, cudaStream_t st);
-cudaError_t launch_two_pass_to_spectrum(const cqt_plan &p, const float *table, bool fold, const float2 *c, float2 *Y,
+cudaError_t launch_two_pass_to_spectrum(const cqt_plan &p, const float *table, bool fold, const CoefRows &c, float2 *Y,
                                         float2 *scratch, int64_t batch, cudaStream_t st);
 cudaError_t configure_two_pass_kernels(const cqt_plan &p);
 // tile widths (columns of pass 1 / rows of pass 2 per CTA) the kernels are compiled for, widest first

@@ -13,9 +13,11 @@
 #include "internal.hpp"
 
 namespace cqt {
-// api.cu: cqt_analyse on slices cut from a ring buffer, the cut fused into the load of the long FFT's first pass
-cqt_status analyse_slices(const cqt_plan *p, const SliceSource &src, int64_t batch, cqt_c64 *c, void *ws, size_t ws_bytes,
-                          void *stream);
+// api.cu: the transforms on coefficient rows that lie in a ring
+cqt_status analyse_slices(const cqt_plan *p, const SliceSource *src, const float *x, int64_t batch, cqt_c64 *c, int row0, int rows, void *ws,
+                          size_t ws_bytes, void *stream);
+cqt_status synthesise_slices(const cqt_plan *p, const cqt_c64 *c, int row0, int rows, int64_t batch, float *x, void *ws, size_t ws_bytes,
+                             void *stream);
 }  // namespace cqt
 
 struct cqt_slicq {
@@ -166,29 +168,25 @@ cqt_status analyse_ready(cqt_slicq *s, const float *fresh, int64_t fresh_stride,
         const cqt_status r = ingest(s, fresh, fresh_stride, new_first, s->n_in - new_first, st);
         if (r != CQT_OK) return r;
     }
-    while (s->next_slice < ready) {
-        // slices whose coefficient slots are consecutive in memory
-        const int64_t slot = s->next_slice % s->K;
-        const int64_t cnt = std::min<int64_t>(ready - s->next_slice, s->K - slot);
-        cqt_c64 *coef = s->d_coef + slot * s->C * cqt_plan_coeff_count(s->plan);
-        cqt_status r;
-        if (fused) {
-            // the slice cut (window x stream samples) happens in the load of the long FFT's first pass, which also puts
-            // the fresh samples that the next slice needs into the ring
-            const int64_t keep = s->next_slice + cnt == ready ? (ready - 1) * s->H : INT64_MAX / 2;
-            const cqt::SliceSource src{s->d_in, s->d_win, s->ring_in, s->next_slice * s->H - s->H, s->H, s->C, (int)cnt,
-                                       fresh, fresh_stride, new_first, keep};
-            r = cqt::analyse_slices(s->plan, src, cnt * s->C, coef, s->d_ws, s->ws_bytes, st);
-        } else {
-            dim3 grid(blocks_for(s->sl), (unsigned)(cnt * s->C));
-            if (cqt::launch_kernel_args(slicq_cut_kernel, grid, dim3(256), 0, st, s->d_in, s->ring_in, s->d_win, s->d_stage, s->sl,
-                                        s->H, s->next_slice, s->C) != cudaSuccess)
-                return CQT_ERR_CUDA;
-            r = cqt_analyse(s->plan, s->d_stage, s->sl, cnt * s->C, s->sl, coef, s->d_ws, s->ws_bytes, st);
-        }
-        if (r != CQT_OK) return r;
-        s->next_slice += cnt;
+    // all of them in one call (at most K wait for their synthesis); their coefficients lie in the ring of K slots
+    const int64_t cnt = ready - s->next_slice;
+    const int row0 = (int)(s->next_slice % s->K * s->C), rows = (int)(s->K * s->C);
+    cqt_status r;
+    if (fused) {
+        // the slice cut (window x stream samples) happens in the load of the long FFT's first pass, which also puts
+        // the fresh samples that the next slice needs into the ring
+        const cqt::SliceSource src{s->d_in, s->d_win, s->ring_in, s->next_slice * s->H - s->H, s->H, s->C, (int)cnt,
+                                   fresh, fresh_stride, new_first, (ready - 1) * s->H};
+        r = cqt::analyse_slices(s->plan, &src, nullptr, cnt * s->C, s->d_coef, row0, rows, s->d_ws, s->ws_bytes, st);
+    } else {
+        dim3 grid(blocks_for(s->sl), (unsigned)(cnt * s->C));
+        if (cqt::launch_kernel_args(slicq_cut_kernel, grid, dim3(256), 0, st, s->d_in, s->ring_in, s->d_win, s->d_stage, s->sl,
+                                    s->H, s->next_slice, s->C) != cudaSuccess)
+            return CQT_ERR_CUDA;
+        r = cqt::analyse_slices(s->plan, nullptr, s->d_stage, cnt * s->C, s->d_coef, row0, rows, s->d_ws, s->ws_bytes, st);
     }
+    if (r != CQT_OK) return r;
+    s->next_slice += cnt;
     if (!fused) return CQT_OK;
     // what follows the last complete slice
     const int64_t tail = std::max(new_first, ready * s->H);
@@ -316,11 +314,10 @@ cqt_status slicq_pull(cqt_slicq *s, float *y, int64_t y_stride, int64_t n_max, v
         int64_t done = 0;
         while (s->next_synth < s->next_slice) {
             const int64_t room_slices = (s->ring_out - (s->next_synth * s->H - s->n_out)) / s->H;
-            const int64_t slot = s->next_synth % s->K;
-            const int64_t cnt = std::min<int64_t>({s->next_slice - s->next_synth, s->K - slot, room_slices});
+            const int64_t cnt = std::min<int64_t>(s->next_slice - s->next_synth, room_slices);
             if (cnt <= 0) break;
-            cqt_status r = cqt_synthesise(s->plan, s->d_coef + slot * s->C * cqt_plan_coeff_count(s->plan), cnt * s->C, s->sl,
-                                          s->d_stage, s->sl, s->d_ws, s->ws_bytes, st);
+            cqt_status r = cqt::synthesise_slices(s->plan, s->d_coef, (int)(s->next_synth % s->K * s->C), (int)(s->K * s->C), cnt * s->C,
+                                                  s->d_stage, s->d_ws, s->ws_bytes, st);
             if (r != CQT_OK) return r;
             // frames below (next_synth - 1) H are final once these slices are in
             const int64_t s0 = s->next_synth, s1 = s0 + cnt - 1;
