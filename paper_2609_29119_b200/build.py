@@ -13,7 +13,7 @@ LIB = os.path.join(HERE, "libcqt_b200.so")
 EXT = os.path.join(HERE, "_cqt_torch.so")        # Python side of the transform calls, linked to LIB and torch
 SOURCES = ["layout.cpp", "api.cu", "band.cu", "band_analysis.cu", "band_synthesis.cu", "band_two_pass.cu", "band_chirp.cu", "band_split.cu", "band_pow2.cu", "long_fft_forward.cu", "long_fft_inverse.cu", "short_fft.cu", "slicq.cu", "static_ws.cu"]
 HEADERS = ["layout.hpp", "plan_types.h", "internal.hpp", "engine.cuh", "band_common.cuh", "long_common.cuh", "long_passes.cuh",
-           "static_fft.cuh", "codelets_gen.cuh",
+           "static_fft.cuh", "codelets_gen.cuh", "table_upload.hpp",
            os.path.join("..", "..", "include", "cqt.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]

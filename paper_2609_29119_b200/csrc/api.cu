@@ -10,6 +10,7 @@
 
 #include "../../include/cqt.h"
 #include "internal.hpp"
+#include "table_upload.hpp"
 
 using namespace cqt;
 
@@ -147,43 +148,6 @@ void make_chirp_tables(int64_t m, int64_t L, std::vector<float2> &tw, ChirpRec &
     cr.filter_off = (int32_t)tw.size();
     for (const std::complex<double> &v : b) tw.push_back(make_float2((float)(v.real() / (double)L), (float)(v.imag() / (double)L)));
 }
-
-// Device tables of a plan.  Small ones are collected into one allocation and one copy (twenty of each took most of the time
-// of creating a small plan), large ones go straight from their vector, which has to live until run().
-struct TableUpload {
-    static constexpr size_t kSmall = 1 << 20;
-    struct Piece { void **dst; const void *src; size_t offset, bytes; };
-    std::vector<char> small;
-    std::vector<Piece> pieces;      // src == nullptr: in `small`, offset there
-    template <class T>
-    void add(T *&dst, const std::vector<T> &src) {
-        dst = nullptr;
-        const size_t n = src.size() * sizeof(T);
-        if (n == 0) return;
-        if (n > kSmall) { pieces.push_back({reinterpret_cast<void **>(&dst), src.data(), 0, n}); return; }
-        const size_t off = (small.size() + 255) / 256 * 256;
-        small.resize(off + n);
-        std::memcpy(small.data() + off, src.data(), n);
-        pieces.push_back({reinterpret_cast<void **>(&dst), nullptr, off, n});
-    }
-    cudaError_t run(std::vector<void *> &allocations) {
-        auto copy = [&](const void *src, size_t n, char *&base) {
-            void *p = nullptr;
-            cudaError_t e = cudaMalloc(&p, n);
-            if (e != cudaSuccess) return e;
-            allocations.push_back(p);
-            base = static_cast<char *>(p);
-            return cudaMemcpy(p, src, n, cudaMemcpyHostToDevice);
-        };
-        char *base = nullptr, *own = nullptr;
-        cudaError_t e = copy(small.data(), small.size(), base);
-        for (const Piece &p : pieces) {
-            if (p.src && e == cudaSuccess) e = copy(p.src, p.bytes, own);
-            if (e == cudaSuccess) *p.dst = p.src ? own : base + p.offset;
-        }
-        return e;
-    }
-};
 
 void free_device(cqt_plan *p) {
     if (p->device < 0) return;
@@ -618,12 +582,12 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     TableUpload up;
     up.add(p->d.bands, p->bands);
     up.add(p->d.ffts, p->ffts);
-    up.add(p->d.tw, tw);
-    up.add(p->d.tab_analysis, tA);
-    up.add(p->d.tab_synthesis, tS);
-    up.add(p->d.tab_analysis_adj, tTA);
-    up.add(p->d.tab_synthesis_adj, tSA);
-    up.add(p->d.cover, cover);
+    up.add(p->d.tw, std::move(tw));
+    up.add(p->d.tab_analysis, std::move(tA));
+    up.add(p->d.tab_synthesis, std::move(tS));
+    up.add(p->d.tab_analysis_adj, std::move(tTA));
+    up.add(p->d.tab_synthesis_adj, std::move(tSA));
+    up.add(p->d.cover, std::move(cover));
     // nested supports: the bins of a band's widened range outside its support hold zeros in the band's plane
     std::vector<int2> zero_seg;
     for (size_t i = 0; i < L.bands.size(); ++i) {
@@ -633,7 +597,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         if (hb.zr > 0) zero_seg.push_back(make_int2((int)(p->bands[i].y_off + en + 1), (int)hb.zr));
     }
     p->n_zero_seg = (int)zero_seg.size();
-    if (p->n_zero_seg) up.add(p->d.zero_seg, zero_seg);
+    up.add(p->d.zero_seg, std::move(zero_seg));
     up.add(p->d.dbg, std::vector<int>(8, 0));
     auto upload_items = [&](BandItem *&dst, const std::vector<int32_t> &work) {
         // record and radix plan of every band of the class, in launch order: what a work item fetches first
@@ -643,7 +607,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
             items[i].br = p->bands[(size_t)b];
             items[i].fp = p->ffts[(size_t)p->bands[(size_t)b].fft];
         }
-        up.add(dst, items);
+        up.add(dst, std::move(items));
     };
     for (auto &c : p->cls) upload_items(c.d_items, c.work);
     upload_items(p->merged.d_items, p->merged.work);
@@ -652,7 +616,14 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     up.add(p->split.d_items, p->split.items);
     up.add(p->split.d_recs, p->split.recs);
     for (auto &g : p->two_pass) up.add(g.d_recs, g.bands);
-    chk(up.run(p->d.allocations));
+    up.run([&](const void *src, size_t n, void *&dev) {
+        chk(cudaMalloc(&dev, n));
+        if (e == cudaSuccess) {
+            p->d.allocations.push_back(dev);
+            chk(cudaMemcpy(dev, src, n, cudaMemcpyHostToDevice));
+        }
+        return e == cudaSuccess;
+    });
     chk(cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device));
     chk(cudaDeviceGetAttribute(&p->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
     // the helper streams carry the shorter classes: at the highest priority their CTAs are placed ahead of the

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import workloads as wl
-from helpers import band_rel_errors, library_plan, oracle_layout, small_workload, split_bands
+from helpers import band_rel_errors, library_plan, oracle_layout, small_workload, snr_db, split_bands
 from oracle import nsgt_oracle as orc
 
 torch = pytest.importorskip("torch")
@@ -87,3 +87,25 @@ def test_lengths_with_a_large_prime_factor(m):
 def test_power_of_two_lengths(M, fill, batch):
     """Full support and one that leaves nearly half of the slots empty; an odd number of items in CTAs that share several."""
     check_bands_of_length(M, fill * M - 1.5, wl.M_POW2, batch)
+
+
+# more than 3,120 bands of one class: the list of their records is a large table, uploaded by itself (class 0; class 1 and the
+# list of the one-launch form, on both sides of the batch where that form ends)
+@pytest.mark.parametrize("n_bands, width, spacing, log_n, batch", [(4000, 32.0, 16, 17, 2), (3300, 200.0, 36, 18, 1), (3300, 200.0, 36, 18, 2)])
+def test_plans_with_thousands_of_bands(n_bands, width, spacing, log_n, batch):
+    N = 1 << log_n
+    centres = [float(150 + spacing * i) for i in range(n_bands)]
+    w = small_workload("many_bands", N=N, fs=float(N), valid_len=N, channels=batch, m_policy=wl.M_SMOOTH,
+                       bands=tuple((c, width) for c in centres))
+    lay, plan = oracle_layout(w), library_plan(w)
+    assert plan.num_bands == n_bands + 2
+    x = wl.make_signal(w)
+    c = plan.analyse(torch.from_numpy(x).cuda())
+    got, X = c.cpu().numpy(), orc.long_dft(orc.pad_signal(x, N))
+    for i in (0, 1, 2, n_bands // 2, 3119, 3120, 3121, 3122, n_bands - 1, n_bands, n_bands + 1):
+        n = np.arange(lay.bands[i].M) if lay.bands[i].M < 1000 else np.arange(0, lay.bands[i].M, 97)
+        want = orc.analyse_band(lay, X, i, n)
+        err = np.linalg.norm(got[:, lay.coeff_offsets[i] + n] - want, axis=-1) / np.linalg.norm(want, axis=-1)
+        assert err.max() <= TOL, (i, err)
+    assert snr_db(x, plan.synthesise(c).cpu().numpy()).min() >= 120.0
+    plan.close()
