@@ -579,15 +579,21 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     }
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
-    TableUpload up;
+    TableUpload up([&](const void *src, size_t n, void *&dev) {
+        chk(cudaMalloc(&dev, n));
+        if (e != cudaSuccess) return false;
+        p->d.allocations.push_back(dev);
+        chk(cudaMemcpy(dev, src, n, cudaMemcpyHostToDevice));
+        return e == cudaSuccess;
+    });
     up.add(p->d.bands, p->bands);
     up.add(p->d.ffts, p->ffts);
-    up.add(p->d.tw, std::move(tw));
-    up.add(p->d.tab_analysis, std::move(tA));
-    up.add(p->d.tab_synthesis, std::move(tS));
-    up.add(p->d.tab_analysis_adj, std::move(tTA));
-    up.add(p->d.tab_synthesis_adj, std::move(tSA));
-    up.add(p->d.cover, std::move(cover));
+    up.add(p->d.tw, tw);
+    up.add(p->d.tab_analysis, tA);
+    up.add(p->d.tab_synthesis, tS);
+    up.add(p->d.tab_analysis_adj, tTA);
+    up.add(p->d.tab_synthesis_adj, tSA);
+    up.add(p->d.cover, cover);
     // nested supports: the bins of a band's widened range outside its support hold zeros in the band's plane
     std::vector<int2> zero_seg;
     for (size_t i = 0; i < L.bands.size(); ++i) {
@@ -597,7 +603,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         if (hb.zr > 0) zero_seg.push_back(make_int2((int)(p->bands[i].y_off + en + 1), (int)hb.zr));
     }
     p->n_zero_seg = (int)zero_seg.size();
-    up.add(p->d.zero_seg, std::move(zero_seg));
+    up.add(p->d.zero_seg, zero_seg);
     up.add(p->d.dbg, std::vector<int>(8, 0));
     auto upload_items = [&](BandItem *&dst, const std::vector<int32_t> &work) {
         // record and radix plan of every band of the class, in launch order: what a work item fetches first
@@ -607,7 +613,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
             items[i].br = p->bands[(size_t)b];
             items[i].fp = p->ffts[(size_t)p->bands[(size_t)b].fft];
         }
-        up.add(dst, std::move(items));
+        up.add(dst, items);
     };
     for (auto &c : p->cls) upload_items(c.d_items, c.work);
     upload_items(p->merged.d_items, p->merged.work);
@@ -616,14 +622,7 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     up.add(p->split.d_items, p->split.items);
     up.add(p->split.d_recs, p->split.recs);
     for (auto &g : p->two_pass) up.add(g.d_recs, g.bands);
-    up.run([&](const void *src, size_t n, void *&dev) {
-        chk(cudaMalloc(&dev, n));
-        if (e == cudaSuccess) {
-            p->d.allocations.push_back(dev);
-            chk(cudaMemcpy(dev, src, n, cudaMemcpyHostToDevice));
-        }
-        return e == cudaSuccess;
-    });
+    up.finish();
     chk(cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device));
     chk(cudaDeviceGetAttribute(&p->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
     // the helper streams carry the shorter classes: at the highest priority their CTAs are placed ahead of the
