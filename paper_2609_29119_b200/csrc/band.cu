@@ -27,12 +27,12 @@ static void set_rows(BandArgs &a, const CoefRows &c) {
     a.rows = c.rows;
 }
 
-const void *band_analysis_kernel(const BandClass &c, int lanes);    // band_analysis.cu
-const void *band_synthesis_kernel(const BandClass &c, int lanes);   // band_synthesis.cu
+const void *band_analysis_kernel(const BandClass &c, int lanes, bool chained);    // band_analysis.cu
+const void *band_synthesis_kernel(const BandClass &c, int lanes, bool chained);   // band_synthesis.cu
 
 template <bool ANALYSIS>
-static const void *class_kernel(const BandClass &c, int lanes) {
-    return ANALYSIS ? band_analysis_kernel(c, lanes) : band_synthesis_kernel(c, lanes);
+static const void *class_kernel(const BandClass &c, int lanes, bool chained) {
+    return ANALYSIS ? band_analysis_kernel(c, lanes, chained) : band_synthesis_kernel(c, lanes, chained);
 }
 
 // Lanes per work item of the class of the shortest bands (0: the class gives every item a whole CTA).  A band of at
@@ -53,7 +53,7 @@ static cudaError_t launch_class(const cqt_plan &p, int cls, const char *name, Ba
     const size_t smem = (size_t)c.max_elems * per_cta * sizeof(float2);
     const long long grid = (items + per_cta - 1) / per_cta;
     void *args[] = {&a};
-    const void *fn = class_kernel<ANALYSIS>(c, lanes);
+    const void *fn = class_kernel<ANALYSIS>(c, lanes, false);
     if (!fn) return cudaErrorInvalidDeviceFunction;
     cudaError_t e = launch_kernel(fn, dim3((unsigned)grid), dim3(c.threads), args, smem, st);
     note_launch(p, name, st);
@@ -157,7 +157,7 @@ static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cuda
         const BandClass &c = p.cls[0];
         a.items = c.d_items;
         void *args[] = {&a};
-        e = launch_kernel(class_kernel<ANALYSIS>(c, 32), dim3((unsigned)f.short_grid), dim3((unsigned)f.short_threads), args,
+        e = launch_kernel(class_kernel<ANALYSIS>(c, 32, true), dim3((unsigned)f.short_grid), dim3((unsigned)f.short_threads), args,
                           (size_t)c.max_elems * (f.short_threads / 32) * sizeof(float2), st);
         note_launch(p, names[ANALYSIS][1], st);
     }
@@ -180,7 +180,7 @@ static cudaError_t launch_pow2_plan(const cqt_plan &p, BandArgs &a, cudaStream_t
         const long long items = (long long)c.n_bands * a.batch;
         const int lanes = lanes_for(p, c, items), threads = items > 4ll * p.sm_count ? c.threads : 64, per_cta = threads / lanes;
         void *args[] = {&a};
-        e = launch_kernel(class_kernel<ANALYSIS>(c, lanes), dim3((unsigned)((items + per_cta - 1) / per_cta)), dim3((unsigned)threads), args,
+        e = launch_kernel(class_kernel<ANALYSIS>(c, lanes, true), dim3((unsigned)((items + per_cta - 1) / per_cta)), dim3((unsigned)threads), args,
                           (size_t)c.max_elems * per_cta * sizeof(float2), st);
         note_launch(p, ANALYSIS ? "bands_from_spectrum/class0" : "bands_to_spectrum/class0", st);
     }
@@ -356,14 +356,16 @@ cudaError_t configure_band_kernels(const cqt_plan &p) {
     }
     for (int i = 0; i < kNumClasses; ++i) {
         if (p.cls[i].n_bands == 0) continue;
-        for (int lanes : {p.cls[i].lanes_few, p.cls[i].lanes_many}) {
-            const size_t s = (size_t)p.cls[i].max_elems * (lanes ? p.cls[i].threads / lanes : 1) * sizeof(float2);
-            if (!class_kernel<true>(p.cls[i], lanes)) return cudaErrorInvalidDeviceFunction;
-            cudaError_t e = allow_dynamic_smem(class_kernel<true>(p.cls[i], lanes), s, p);
-            if (e != cudaSuccess) return e;
-            e = allow_dynamic_smem(class_kernel<false>(p.cls[i], lanes), s, p);
-            if (e != cudaSuccess) return e;
-        }
+        for (int lanes : {p.cls[i].lanes_few, p.cls[i].lanes_many})
+            for (bool chained : {false, true}) {
+                if (chained && i > 0) continue;   // chains contain class 0 only
+                const size_t s = (size_t)p.cls[i].max_elems * (lanes ? p.cls[i].threads / lanes : 1) * sizeof(float2);
+                if (!class_kernel<true>(p.cls[i], lanes, chained)) return cudaErrorInvalidDeviceFunction;
+                cudaError_t e = allow_dynamic_smem(class_kernel<true>(p.cls[i], lanes, chained), s, p);
+                if (e != cudaSuccess) return e;
+                e = allow_dynamic_smem(class_kernel<false>(p.cls[i], lanes, chained), s, p);
+                if (e != cudaSuccess) return e;
+            }
     }
     return cudaSuccess;
 }

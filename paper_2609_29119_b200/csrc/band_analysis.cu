@@ -4,7 +4,8 @@
 namespace cqt {
 
 // One work item (band record and radix plan `it`, signal ch) on nthr threads with `buf` as their shared memory.
-template <class Sync, int MAXR, bool GEN>
+// CHAINED: the launch may be a member of a chain (band_common.cuh).
+template <class Sync, int MAXR, bool GEN, bool CHAINED>
 __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem &it, int ch, float2 *buf, int tid, int nthr) {
     const BandRec br = it.br;
     const FftPlan &fp = it.fp;
@@ -25,7 +26,7 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
         const bool mirrored = k < 0 || k > half;
         const int km = k < 0 ? -k : (k > half ? a.N - k : k);
         if (!CQT_CHK(a.dbg, 302, km, half + 1)) return make_float2(0.f, 0.f);
-        const float2 xv = ld_data(X + km);
+        const float2 xv = ld_spectrum<CHAINED>(X + km);
         return make_float2(g * xv.x, mirrored ? -(g * xv.y) : g * xv.y);
     };
     float2 *out = a.coef + coef_row(a.row0, a.rows, ch) * a.coeff_count + br.coeff_off;
@@ -56,7 +57,7 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
             const int j = lo ? m - br.d0 : m - shift_neg;
             if (!CQT_CHK(a.dbg, 309, j, br.S)) return make_float2(0.f, 0.f);
             const float g = __ldg(tab + j);
-            const float2 xv = ld_data(Xs + j);
+            const float2 xv = ld_spectrum<CHAINED>(Xs + j);
             return make_float2(g * xv.x, g * xv.y);
         };
         fft_fused<+1, Sync, true, false, true, false, false, MAXR>(t, fp, tws, load_regular, store, tid, nthr);
@@ -66,7 +67,7 @@ __device__ __forceinline__ void analysis_item(const BandArgs &a, const BandItem 
 }
 
 // One class: groups of LANES lanes (or the whole CTA) per item.
-template <int THREADS, int MINB, int LANES, int MAXR, bool GEN>
+template <int THREADS, int MINB, int LANES, int MAXR, bool GEN, bool CHAINED>
 __global__ void __launch_bounds__(THREADS, MINB) bands_from_spectrum_kernel(BandArgs a) {
     chain_enter(a);
     using G = Group<LANES>;
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_from_spectrum_kernel(Band
     __shared__ BandItem item_s[LANES ? THREADS / (LANES ? LANES : 1) : 1];
     BandItem &it = item_s[G::slot()];
     fetch_item<Sync>(a.items[item / a.batch], it, tid, nthr);   // records in launch order of the class
-    analysis_item<Sync, MAXR, GEN>(a, it, item % a.batch, smem_band + (size_t)G::slot() * a.max_elems, tid, nthr);
+    analysis_item<Sync, MAXR, GEN, CHAINED>(a, it, item % a.batch, smem_band + (size_t)G::slot() * a.max_elems, tid, nthr);
     chain_end(a);
 }
 
@@ -89,16 +90,23 @@ __global__ void __launch_bounds__(1024, 1) all_bands_from_spectrum_kernel(BandAr
     __shared__ BandItem item_s[kMaxGroups];
     BandItem &it = item_s[m.slot];
     fetch_item<NamedSync>(a.items[m.band], it, m.tid, m.nthr);
-    analysis_item<NamedSync, 16, false>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
+    analysis_item<NamedSync, 16, false, true>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
     chain_end(a);
 }
 
 const void *band_analysis_merged_kernel() { return (const void *)all_bands_from_spectrum_kernel; }
 
-const void *band_analysis_kernel(const BandClass &c, int lanes) {
-#define X(T, B, W, R)                                                                          \
-    if (c.threads == T && c.min_blocks == B && lanes == W && c.max_radix <= R)  \
-        return W && c.has_generic ? (const void *)bands_from_spectrum_kernel<T, B, W, R, (W > 0)> : (const void *)bands_from_spectrum_kernel<T, B, W, R, false>;
+// whole-CTA kernels are in no chain and in no class with direct sums
+template <int T, int B, int W, int R>
+static const void *class_variant(bool generic, bool chained) {
+    if constexpr (W == 0) return generic || chained ? nullptr : (const void *)bands_from_spectrum_kernel<T, B, W, R, false, false>;
+    else if (chained) return generic ? (const void *)bands_from_spectrum_kernel<T, B, W, R, true, true> : (const void *)bands_from_spectrum_kernel<T, B, W, R, false, true>;
+    else return generic ? (const void *)bands_from_spectrum_kernel<T, B, W, R, true, false> : (const void *)bands_from_spectrum_kernel<T, B, W, R, false, false>;
+}
+
+const void *band_analysis_kernel(const BandClass &c, int lanes, bool chained) {
+#define X(T, B, W, R) \
+    if (c.threads == T && c.min_blocks == B && lanes == W && c.max_radix <= R) return class_variant<T, B, W, R>(W && c.has_generic, chained);
     CQT_KERNEL_TABLE(X)
 #undef X
     return nullptr;

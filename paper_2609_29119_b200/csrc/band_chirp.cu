@@ -185,7 +185,7 @@ __device__ __forceinline__ void chirp_cta(const ChirpArgs &a, const ChirpSegment
         float2 *Y = a.b.Y + (long long)ch * a.b.y_pitch + br.y_off;
         const bool fold = a.b.fold && br.side != 0;
         auto in = [&](int n) {
-            const float2 v = ld_data(c + n);
+            const float2 v = ld_chained(c + n);
             return fold ? make_float2(2.f * v.x, 0.f) : v;
         };
         chirp_convolve<S>(buf, twf, filter, m, active, t, [&](int n) { return combine(in(n), in(n + m), in(n + 2 * m), in(n + 3 * m), n); },

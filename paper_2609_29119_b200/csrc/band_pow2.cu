@@ -182,7 +182,7 @@ __device__ __forceinline__ void pow2_cta(const Pow2Args &a, const Pow2Segment &s
 #pragma unroll
                 for (int q = 0; q < S::R0; ++q) {
                     const int j = entry(b + q * S::S0);
-                    const float2 v = j >= 0 && CQT_CHK(a.b.dbg, 701, j, br.S) ? ld_data(Xs + j) : make_float2(0.f, 0.f);
+                    const float2 v = j >= 0 && CQT_CHK(a.b.dbg, 701, j, br.S) ? ld_chained(Xs + j) : make_float2(0.f, 0.f);
                     re[q] = v.x; im[q] = v.y;
                 }
 #pragma unroll
@@ -211,7 +211,7 @@ __device__ __forceinline__ void pow2_cta(const Pow2Args &a, const Pow2Segment &s
         auto load = [&](int b, float (&re)[S::R0], float (&im)[S::R0]) {
 #pragma unroll
             for (int q = 0; q < S::R0; ++q) {
-                const float2 v = __ldcs(c + b + q * S::S0);   // read once
+                const float2 v = ld_chained(c + b + q * S::S0);   // read once
                 re[q] = v.x; im[q] = v.y;
             }
             if (fold) {

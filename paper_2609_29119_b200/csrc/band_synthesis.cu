@@ -25,7 +25,8 @@ struct RegularStore {
 };
 
 // One work item (band record and radix plan `it`, signal ch) on nthr threads with `buf` as their shared memory.
-template <class Sync, int MAXR, bool GEN>
+// CHAINED: the launch may be a member of a chain (band_common.cuh).
+template <class Sync, int MAXR, bool GEN, bool CHAINED>
 __device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem &it, int ch, float2 *buf, int tid, int nthr) {
     const BandRec br = it.br;
     const FftPlan &fp = it.fp;
@@ -35,7 +36,7 @@ __device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem
     const bool fold = a.fold && br.side != 0;
     auto load = [&](int n, int) -> float2 {
         if (!CQT_CHK(a.dbg, 304, n, M)) return make_float2(0.f, 0.f);
-        float2 v = __ldcs(in + n);
+        float2 v = ld_coefficient<CHAINED>(in + n);
         if (fold) v = make_float2(2.f * v.x, 0.f);
         return v;
     };
@@ -76,7 +77,7 @@ __device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem
         const int shift_neg = M + br.d0;
         const RegularStore store_regular{tab, Ys, last_pos, first_neg, br.d0, shift_neg};
         // coefficients are read once: streaming loads keep the L2 for the weighted-bin planes
-        auto load_regular = [&](int n, int) -> float2 { return __ldcs(in + n); };
+        auto load_regular = [&](int n, int) -> float2 { return ld_coefficient<CHAINED>(in + n); };
         fft_fused<-1, Sync, true, false, true, false, false, MAXR>(t, fp, tws, load_regular, store_regular, tid, nthr);
         return;
     }
@@ -84,7 +85,7 @@ __device__ __forceinline__ void synthesis_item(const BandArgs &a, const BandItem
 }
 
 // One class: groups of LANES lanes (or the whole CTA) per item.
-template <int THREADS, int MINB, int LANES, int MAXR, bool GEN>
+template <int THREADS, int MINB, int LANES, int MAXR, bool GEN, bool CHAINED>
 __global__ void __launch_bounds__(THREADS, MINB) bands_to_spectrum_kernel(BandArgs a) {
     chain_enter(a);
     using G = Group<LANES>;
@@ -95,7 +96,7 @@ __global__ void __launch_bounds__(THREADS, MINB) bands_to_spectrum_kernel(BandAr
     __shared__ BandItem item_s[LANES ? THREADS / (LANES ? LANES : 1) : 1];
     BandItem &it = item_s[G::slot()];
     fetch_item<Sync>(a.items[item / a.batch], it, tid, nthr);   // records in launch order of the class
-    synthesis_item<Sync, MAXR, GEN>(a, it, item % a.batch, smem_band + (size_t)G::slot() * a.max_elems, tid, nthr);
+    synthesis_item<Sync, MAXR, GEN, CHAINED>(a, it, item % a.batch, smem_band + (size_t)G::slot() * a.max_elems, tid, nthr);
     chain_end(a);
 }
 
@@ -107,16 +108,23 @@ __global__ void __launch_bounds__(1024, 1) all_bands_to_spectrum_kernel(BandArgs
     __shared__ BandItem item_s[kMaxGroups];
     BandItem &it = item_s[m.slot];
     fetch_item<NamedSync>(a.items[m.band], it, m.tid, m.nthr);
-    synthesis_item<NamedSync, 16, false>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
+    synthesis_item<NamedSync, 16, false, true>(a, it, m.ch, smem_band + m.smem_off, m.tid, m.nthr);
     chain_end(a);
 }
 
 const void *band_synthesis_merged_kernel() { return (const void *)all_bands_to_spectrum_kernel; }
 
-const void *band_synthesis_kernel(const BandClass &c, int lanes) {
-#define X(T, B, W, R)                                                                          \
-    if (c.threads == T && c.min_blocks == B && lanes == W && c.max_radix <= R)  \
-        return W && c.has_generic ? (const void *)bands_to_spectrum_kernel<T, B, W, R, (W > 0)> : (const void *)bands_to_spectrum_kernel<T, B, W, R, false>;
+// whole-CTA kernels are in no chain and in no class with direct sums
+template <int T, int B, int W, int R>
+static const void *class_variant(bool generic, bool chained) {
+    if constexpr (W == 0) return generic || chained ? nullptr : (const void *)bands_to_spectrum_kernel<T, B, W, R, false, false>;
+    else if (chained) return generic ? (const void *)bands_to_spectrum_kernel<T, B, W, R, true, true> : (const void *)bands_to_spectrum_kernel<T, B, W, R, false, true>;
+    else return generic ? (const void *)bands_to_spectrum_kernel<T, B, W, R, true, false> : (const void *)bands_to_spectrum_kernel<T, B, W, R, false, false>;
+}
+
+const void *band_synthesis_kernel(const BandClass &c, int lanes, bool chained) {
+#define X(T, B, W, R) \
+    if (c.threads == T && c.min_blocks == B && lanes == W && c.max_radix <= R) return class_variant<T, B, W, R>(W && c.has_generic, chained);
     CQT_KERNEL_TABLE(X)
 #undef X
     return nullptr;

@@ -28,6 +28,14 @@ __device__ __forceinline__ float2 ld_data(const float2 *p) {
     return v;
 }
 
+// The same where the reading kernel has not waited itself (members of a chain of band kernels, see band_common.cuh): the
+// load is a strong one at device scope, which the L1 of the SM, where an older copy of the line could be, does not serve.
+__device__ __forceinline__ float2 ld_chained(const float2 *p) {
+    float2 v;
+    asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 // sync(nthr): barrier of the nthr threads that work on one item
 struct BlockSync {
     static __device__ __forceinline__ void sync(int) { __syncthreads(); }

@@ -109,3 +109,37 @@ def test_plans_with_thousands_of_bands(n_bands, width, spacing, log_n, batch):
         assert err.max() <= TOL, (i, err)
     assert snr_db(x, plan.synthesise(c).cpu().numpy()).min() >= 120.0
     plan.close()
+
+
+# chained band kernels read what the kernel before the chain wrote, in buffers that the calls before have used too
+@pytest.mark.parametrize("kw", [dict(N=1 << 14, valid_len=1 << 14, bins_per_octave=12, m_policy=wl.M_MULT4, channels=1),   # chirp-z, merged, short
+                                dict(N=1 << 17, valid_len=99225, bins_per_octave=36, fmax=18000.0, m_policy=wl.M_SMOOTH, channels=3),   # split first
+                                dict(N=1 << 16, valid_len=60001, bins_per_octave=24, m_policy=wl.M_POW2, channels=5)],
+                         ids=lambda k: f"n{k['N']}_p{k['m_policy']}")
+def test_chained_kernels_see_the_call_before(kw):
+    """Round trips of changing signals through the same buffers, enqueued without a pause, equal bit for bit those that are
+    waited for after every kernel."""
+    w = small_workload("chain", **{"fs": 44100.0, "fmin": 60.0, "fmax": 22050.0, **kw})
+    plan, steps = library_plan(w), 24
+    xs = torch.randn(steps, w.channels, w.valid_len, generator=torch.Generator().manual_seed(5)).cuda()
+    xs *= torch.logspace(-3, 3, steps, device="cuda")[:, None, None]
+    c = torch.empty((w.channels, plan.coeff_count), dtype=torch.complex64, device="cuda")
+    y, ws = torch.empty_like(xs[0]), plan.workspace(w.channels)
+    want = []
+    for x in xs:
+        plan.analyse(x, valid_len=w.valid_len, out=c, ws=ws)
+        torch.cuda.synchronize()
+        plan.synthesise(c, valid_len=w.valid_len, out=y, ws=ws)
+        torch.cuda.synchronize()
+        want.append((c.clone(), y.clone()))
+    got_c, got_y = torch.empty((steps,) + c.shape, dtype=c.dtype, device="cuda"), torch.empty_like(xs)
+    for _ in range(3):
+        for i in range(steps):
+            plan.analyse(xs[i], valid_len=w.valid_len, out=got_c[0], ws=ws)      # one buffer for all: rewritten by every call
+            plan.synthesise(got_c[0], valid_len=w.valid_len, out=got_y[i], ws=ws)
+        for i in range(1, steps):
+            plan.analyse(xs[i], valid_len=w.valid_len, out=got_c[i], ws=ws)
+        torch.cuda.synchronize()
+        assert all(torch.equal(got_y[i], want[i][1]) for i in range(steps))
+        assert all(torch.equal(torch.view_as_real(got_c[i]), torch.view_as_real(want[i][0])) for i in range(1, steps))
+    plan.close()
