@@ -7,6 +7,7 @@
 #include <Python.h>
 
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/custom_function.h>
 #include <torch/csrc/autograd/function.h>
@@ -73,6 +74,16 @@ void *stream_of(PyObject *stream) {
     return reinterpret_cast<void *>((intptr_t)int_attr(stream, s_cuda_stream));
 }
 
+// The library reads memory as it lies there, and a tensor may be a conjugate or a negative of it that is still to be
+// computed.  Such an input is computed on the stream of the call: its memory is then given back in that stream's order too.
+at::Tensor as_stored(const at::Tensor &t, void *stream) {
+    if (!t.is_conj() && !t.is_neg()) return t;
+    at::AutoDispatchBelowADInplaceOrView no_grad;
+    const c10::cuda::CUDAStreamGuard guard(c10::cuda::getStreamFromExternal(reinterpret_cast<cudaStream_t>(stream), t.device().index()));
+    return t.resolve_conj().resolve_neg();
+}
+void require_stored(const at::Tensor &t) { require(!t.is_conj() && !t.is_neg(), "the output is no conjugate or negative view"); }
+
 // Plan._ws, grown by Plan.workspace when it is too small
 at::Tensor workspace_of(PyObject *plan, const cqt_plan *p, int64_t batch) {
     PyObject *w = PyObject_GetAttr(plan, s_ws);
@@ -106,18 +117,20 @@ at::Tensor run(PyObject *plan, int which, const at::Tensor &in, int64_t valid_le
         if (valid_len == kAbsent) valid_len = int_attr(plan, s_N);
         if (!out.defined()) out = at::empty({batch, valid_len}, in.options().dtype(at::kFloat));
     }
+    require_stored(out);
     if (!ws.defined() && which != kAnalyseStatic && batch > 0) ws = workspace_of(plan, p, batch);
     void *stream = stream_of(stream_arg);
+    const at::Tensor src = as_stored(in, stream);
     void *wp = ws.defined() ? ws.data_ptr() : nullptr;
     const size_t wn = ws.defined() ? (size_t)ws.numel() : 0;
-    void *ip = in.data_ptr(), *op = out.data_ptr();
+    void *ip = src.data_ptr(), *op = out.data_ptr();
     cqt_status s;
     {
         GilRelease nogil;
         if (forward) {
             const float *x = (const float *)ip;
             cqt_c64 *c = (cqt_c64 *)op;
-            const int64_t stride = in.stride(0);
+            const int64_t stride = src.stride(0);
             s = which == kAnalyse             ? cqt_analyse(p, x, stride, batch, valid_len, c, wp, wn, stream)
                 : which == kSynthesiseAdjoint ? cqt_synthesise_adjoint(p, x, stride, batch, valid_len, c, wp, wn, stream)
                                               : cqt_analyse_static_ws(p, x, stride, batch, valid_len, c, stream);
@@ -178,7 +191,7 @@ struct AdjointNode final : torch::autograd::Node {
     torch::autograd::variable_list apply(torch::autograd::variable_list &&grads) override {
         if (!grads[0].defined()) return {at::Tensor()};
         at::AutoDispatchBelowADInplaceOrView no_grad;
-        const at::Tensor g = grads[0].resolve_conj().contiguous();
+        const at::Tensor g = grads[0].contiguous();
         at::Tensor out;
         // columns beyond valid_len were never read: zero gradient
         if (which == kAnalyseAdjoint && width != valid_len) out = at::zeros({g.size(0), width}, g.options().dtype(at::kFloat));
@@ -207,7 +220,7 @@ PyObject *differentiable(PyObject *, PyObject *const *a, Py_ssize_t n) {
         at::Tensor out;
         {
             at::AutoDispatchBelowADInplaceOrView no_grad;
-            out = run(a[0], which, x.resolve_conj().contiguous(), valid_len, at::Tensor(), at::Tensor(), Py_None);
+            out = run(a[0], which, x.contiguous(), valid_len, at::Tensor(), at::Tensor(), Py_None);
         }
         if (torch::autograd::compute_requires_grad(x)) {
             auto node = std::shared_ptr<AdjointNode>(
@@ -224,8 +237,8 @@ PyObject *push(PyObject *, PyObject *const *a, Py_ssize_t n) {
     return guarded([&]() -> PyObject * {
         require(n == 3, "three arguments");
         cqt_slicq *s = reinterpret_cast<cqt_slicq *>((intptr_t)PyLong_AsLongLong(a[0]));
-        const at::Tensor &x = tensor_of(a[1]);
         void *stream = stream_of(a[2]);
+        const at::Tensor x = as_stored(tensor_of(a[1]), stream);
         const int64_t frames = x.size(1);
         const float *p = frames ? (const float *)x.data_ptr() : nullptr;
         int64_t done = 0;
@@ -243,6 +256,7 @@ PyObject *pull(PyObject *, PyObject *const *a, Py_ssize_t n) {
         require(n == 3, "three arguments");
         cqt_slicq *s = reinterpret_cast<cqt_slicq *>((intptr_t)PyLong_AsLongLong(a[0]));
         const at::Tensor &y = tensor_of(a[1]);
+        require_stored(y);
         void *stream = stream_of(a[2]);
         int64_t wrote = 0;
         float *p = (float *)y.data_ptr();

@@ -66,3 +66,52 @@ def test_coefficient_loss_gradient_and_padding_columns():
     assert np.all(got[:, w.valid_len:] == 0)
     assert min(snr_db(want, got[:, :w.valid_len])) >= 100.0
     plan.close()
+
+
+def test_conjugate_and_negative_views_are_read_as_what_they_stand_for():
+    """Tensors whose conjugation or negation is still to be computed (torch's conj and neg bits), as inputs and cotangents."""
+    from paper_2609_29119_b200 import SliCQ
+    from paper_2609_29119_b200 import autograd as ad
+    w = CASES[0]
+    plan = library_plan(w)
+    x = torch.from_numpy(wl.make_signal(w)).cuda()
+    m = torch.from_numpy(wl.make_cotangent(w, plan.coeff_count)).cuda()
+
+    def same(a, b):
+        a, b = (t.resolve_conj().resolve_neg() for t in (a, b))
+        return torch.equal(torch.view_as_real(a), torch.view_as_real(b)) if a.is_complex() else torch.equal(a, b)
+    neg_x, conj_m, neg_m = torch._neg_view(x), m.conj(), torch._neg_view(m)
+    assert neg_x.is_neg() and conj_m.is_conj() and neg_m.is_neg() and torch._neg_view(conj_m).is_conj()
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    for stream in (None, side):
+        out_c, out_x = torch.empty_like(m), torch.empty_like(x)
+        plan.analyse(neg_x, out=out_c, stream=stream)
+        torch.cuda.synchronize()
+        assert same(out_c, plan.analyse(-x))
+        for view in (conj_m, neg_m, torch._neg_view(conj_m)):
+            stored = view.resolve_conj().resolve_neg().clone()
+            plan.synthesise(view, out=out_x, stream=stream)
+            torch.cuda.synchronize()
+            assert same(out_x, plan.synthesise(stored))
+            plan.analyse_adjoint(view, out=out_x, stream=stream)
+            torch.cuda.synchronize()
+            assert same(out_x, plan.analyse_adjoint(stored))
+    # cotangents and differentiable inputs
+    xg, cg = x.clone().requires_grad_(True), m.clone().requires_grad_(True)
+    c, y = ad.analyse(plan, xg), ad.synthesise(plan, cg)
+    for view in (conj_m, neg_m):
+        got, = torch.autograd.grad(c, xg, grad_outputs=view, retain_graph=True)
+        assert same(got, plan.analyse_adjoint(view.resolve_conj().resolve_neg()))
+    got, = torch.autograd.grad(y, cg, grad_outputs=neg_x, retain_graph=True)
+    assert same(got, plan.synthesise_adjoint(-x))
+    got, = torch.autograd.grad(ad.synthesise(plan, torch._neg_view(cg.conj())), cg, grad_outputs=x)
+    assert same(got, (-plan.synthesise_adjoint(x)).conj().resolve_conj())
+    # the sliced form, and outputs that are such views
+    a, b = SliCQ(plan, w.channels, 512, 2), SliCQ(plan, w.channels, 512, 2)
+    assert a.push(neg_x) == b.push(-x) == 2
+    assert same(a.coeffs(1).clone(), b.coeffs(1).clone())
+    for call in (lambda: plan.analyse(x, out=conj_m), lambda: plan.synthesise(m, out=neg_x), lambda: a.pull(neg_x)):
+        with pytest.raises(AssertionError):
+            call()
+    a.close(); b.close(); plan.close()
