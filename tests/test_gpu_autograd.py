@@ -115,3 +115,26 @@ def test_conjugate_and_negative_views_are_read_as_what_they_stand_for():
         with pytest.raises(AssertionError):
             call()
     a.close(); b.close(); plan.close()
+
+
+def test_backward_runs_on_the_stream_of_the_forward_pass():
+    """Forward passes on a side stream, backward calls from the default one, inputs that change from step to step: the same
+    gradients as on one stream."""
+    from paper_2609_29119_b200 import autograd as ad
+    w = CASES[2]
+    plan, one = library_plan(w), library_plan(w)
+    side = torch.cuda.Stream()
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    for _ in range(8):
+        x = torch.randn(w.channels, w.valid_len, generator=gen, device="cuda")
+        t = torch.randn(w.channels, w.valid_len, generator=gen, device="cuda")
+        a, b = x.clone().requires_grad_(True), x.clone().requires_grad_(True)
+        ((ad.synthesise(one, ad.analyse(one, a)) - t) ** 2).sum().backward()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            loss = ((ad.synthesise(plan, ad.analyse(plan, b)) - t) ** 2).sum()
+        torch.cuda.current_stream().wait_stream(side)
+        loss.backward()
+        assert torch.equal(a.grad, b.grad)
+        torch.cuda.synchronize()          # the next forward pass reuses the plan's workspace on the side stream
+    plan.close(); one.close()

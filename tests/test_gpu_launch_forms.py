@@ -48,11 +48,10 @@ def test_band_launch_forms(kw, batch):
     check_rows(small_workload("forms", **{"fs": 44100.0, "fmin": 60.0, "fmax": 22050.0, "channels": batch, **kw}), batch)
 
 
-def check_bands_of_length(M, width, policy, batch):
+def check_bands_of_length(M, width, policy, batch, N=1 << 15):
     """Two overlapping regular bands of M coefficients against numpy's FFT of the windowed, slot-placed spectrum; the round
     trip covers the synthesis form."""
     from paper_2609_29119_b200 import Plan
-    N = 1 << 15
     centre = [N / 4.0 - 0.1 * M, N / 4.0 + 0.1 * M]
     plan = Plan.from_bands(float(N), N, centre, [width] * 2, m_policy=policy)
     rng = np.random.default_rng(M)
@@ -87,6 +86,34 @@ def test_lengths_with_a_large_prime_factor(m):
 def test_power_of_two_lengths(M, fill, batch):
     """Full support and one that leaves nearly half of the slots empty; an odd number of items in CTAs that share several."""
     check_bands_of_length(M, fill * M - 1.5, wl.M_POW2, batch)
+
+
+@pytest.mark.parametrize("batch", [1, 33])
+@pytest.mark.parametrize("log_n, fill", [(15, 0.52), (17, 1.0)], ids=["alone", "beside_two_pass_bands"])
+def test_longest_power_of_two_length(log_n, fill, batch):
+    """16,384 coefficients, the longest that one CTA transforms; in the longer signal the sidebands take the two-pass kernels."""
+    check_bands_of_length(1 << 14, fill * (1 << 14) - 1.5, wl.M_POW2, batch, N=1 << log_n)
+
+
+# more bands over one bin than a word has bits for planes: another form of the cover words and of the inverse kernels
+@pytest.mark.parametrize("batch", [1, 9])
+@pytest.mark.parametrize("log_n", [12, 15])
+def test_more_than_31_planes(log_n, batch):
+    N = 1 << log_n
+    centres = [210 + 10 * i for i in range(80)] + list(range(1010, N // 2 - 210, 150))
+    w = small_workload("planes", N=N, fs=float(N), valid_len=N - 5, channels=batch, m_policy=wl.M_SMOOTH,
+                       bands=tuple((float(c), 400.0) for c in centres))
+    cover = np.zeros(N // 2 + 1, dtype=int)
+    for c in centres:
+        cover[c - 199:c + 200] += 1
+    assert cover.max() > 31
+    check_rows(w, batch)
+    lay, plan = oracle_layout(w), library_plan(w)
+    y = wl.make_cotangent(w, lay.coeff_count)[:1]
+    got = plan.analyse_adjoint(torch.from_numpy(y).cuda(), valid_len=w.valid_len).cpu().numpy()
+    want = orc.analyse_adjoint(lay, split_bands(lay, y.astype(np.complex128)))[..., :w.valid_len]
+    assert np.linalg.norm(got - want) <= TOL * np.linalg.norm(want)
+    plan.close()
 
 
 # more than 3,120 bands of one class: the list of their records is a large table, uploaded by itself (class 0; class 1 and the

@@ -215,3 +215,48 @@ def test_saved_state_resumes_the_stream_bit_for_bit():
     assert e.value.status == -6
     other.close(); c.close(); a.close()
     plan.close()
+
+
+# slices whose coefficient slots wrap around the ring go through one call: in every kernel that bands can run on
+@pytest.mark.parametrize("kw, tuning", [
+    (dict(m_policy=wl.M_POW2), {}),
+    (dict(m_policy=wl.M_MULT4), {}),                                     # chirp-z, merged launch
+    (dict(m_policy=wl.M_MULT4, channels=40), {}),                        # chirp-z beside the classes
+    (dict(m_policy=wl.M_SMOOTH), dict(max_cta_elems=600)),               # two-pass bands
+    (dict(m_policy=wl.M_SMOOTH, N=1 << 15, fmax=16000.0, channels=1), {}),   # a sideband that is split into four items
+], ids=["pow2", "mult4", "mult4_40ch", "two_pass", "split"])
+def test_slices_that_wrap_around_the_slots(kw, tuning):
+    from paper_2609_29119_b200 import SliCQ
+    kw = {"N": 1 << 14, "channels": 2, **kw}
+    sl = kw["N"]
+    H = sl // 2
+    w = small_workload("wrap", **{**dict(valid_len=sl, fs=44100.0, fmin=60.0, fmax=22050.0, bins_per_octave=12, kind="pink_notes",
+                                         slice_len=sl, transition=sl // 4, stream_len=9 * H), **kw})
+    lay, plan = oracle_layout(w), library_plan(w, **tuning)
+    if "max_cta_elems" in tuning:
+        assert any(b.launch_class == -1 for b in plan.bands())
+    if kw["m_policy"] == wl.M_MULT4:
+        assert any(b.M > 128 and 60 ** 12 % b.M for b in plan.bands())     # a prime factor above 5
+    x = wl.make_signal(w)
+    xd, check = torch.from_numpy(x).cuda(), [0, w.channels - 1]
+    sq = SliCQ(plan, w.channels, w.transition, 5)          # slots 0 1 2, 3 4 0, 1 2 3: the second and the third push wrap
+    out = torch.zeros((w.channels, 12 * H), device="cuda")
+    slices = orc.slicq_cut(x[check].astype(np.float64), sl, w.transition)
+    got, rec = 0, []
+    for push in range(3):
+        assert sq.push(xd[:, 3 * H * push:3 * H * (push + 1)]) == 3 * (push + 1)
+        for s in range(3 * push, 3 * push + 3):
+            want = orc.analyse(lay, slices[:, s, :])
+            errs = band_rel_errors(lay, sq.coeffs(s).cpu().numpy()[check], want)
+            assert errs.max() <= 1e-5, (s, int(errs.argmax()), errs.max())
+            rec.append(orc.synthesise(lay, want))
+        got += sq.pull(out[:, got:])
+    n = 8 * H
+    assert got == n                                          # the last block waits for the slice after it
+    want_y = orc.slicq_overlap_add(np.stack(rec, axis=1), 9 * H)[:, :n]
+    y = out[check, :n].cpu().numpy()
+    rel = np.linalg.norm(y - want_y, axis=-1) / np.linalg.norm(want_y, axis=-1)
+    assert rel.max() <= 1e-5, rel
+    assert snr_db(x[check][:, :n], y).min() >= 120.0
+    sq.close()
+    plan.close()
