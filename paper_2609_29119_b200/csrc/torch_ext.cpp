@@ -216,6 +216,10 @@ PyObject *differentiable(PyObject *, PyObject *const *a, Py_ssize_t n) {
         int64_t valid_len = optional_length(a[3]);
         require(which == kAnalyse || which == kSynthesise, "analyse or synthesise");
         require(x.dim() == 2, "a [batch, n] tensor");
+        if (x._fw_grad(0).defined()) {   // its tangent would be lost without a word
+            PyErr_SetString(PyExc_NotImplementedError, "the transforms have no forward-mode derivative: use the backward one, or transform the tangent");
+            throw PyFailure();
+        }
         if (valid_len == kAbsent) valid_len = which == kAnalyse ? x.size(1) : int_attr(a[0], s_N);
         at::Tensor out;
         {

@@ -138,3 +138,25 @@ def test_backward_runs_on_the_stream_of_the_forward_pass():
         assert torch.equal(a.grad, b.grad)
         torch.cuda.synchronize()          # the next forward pass reuses the plan's workspace on the side stream
     plan.close(); one.close()
+
+
+def test_what_the_wrappers_do_not_support_is_refused():
+    """Forward-mode derivatives and function transforms raise instead of dropping the tangent or reading a wrapper's memory."""
+    import torch.autograd.forward_ad as fwd
+    from paper_2609_29119_b200 import autograd as ad
+    w = CASES[0]
+    plan = library_plan(w)
+    x = torch.from_numpy(wl.make_signal(w)).cuda()
+    m = torch.from_numpy(wl.make_cotangent(w, plan.coeff_count)).cuda()
+    for f, t in ((lambda t: ad.analyse(plan, t), x), (lambda t: ad.synthesise(plan, t), m)):
+        with fwd.dual_level():
+            with pytest.raises(NotImplementedError):
+                f(fwd.make_dual(t, torch.ones_like(t)))
+            f(t)                                  # a tensor without a tangent is taken
+        with pytest.raises(RuntimeError):
+            torch.func.vmap(f)(t[None].repeat(2, 1, 1))
+        with pytest.raises(RuntimeError):
+            torch.func.jvp(f, (t,), (t,))
+        with pytest.raises(RuntimeError):
+            torch.func.grad(lambda t: f(t).abs().sum())(t)
+    plan.close()
