@@ -351,11 +351,14 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         br.fft = -1;
     }
     // ---- launch classes by band length
-    // class 0: 8 lanes per item, 32 items per CTA; class 1: a warp per item, 8 items per CTA (calls with few items take the
-    // merged form; with a CTA of 64 threads per item the class was bound by the rate at which CTAs start: 17 % of the warps
-    // active, 256 signals at 24 bands per octave 57 -> 52 us, and fewer warps leave more of the SMs to the classes beside
-    // it, the whole analysis 102 -> 88 us); the others one CTA per item, sized so that several CTAs share an SM (64 registers
-    // per thread) except for the longest bands, which fill its shared memory
+    // class 0: 8 lanes per item, 32 items per CTA, or a warp per item in a call with few items.
+    // class 1: a warp per item, 8 items per CTA, in every call.  With a CTA of 64 threads per item the class was bound by the
+    // rate at which CTAs start (17 % of the warps active): 256 signals at 24 bands per octave 57 -> 52 us, their whole
+    // analysis 102 -> 95.  Most calls with few items take the merged form instead; those with a two-pass band do not, and
+    // for them the two are alike: round trip of one 2^22-sample signal at 96 bands per octave 215.7 us, with 64 threads
+    // per item 215.0, of one 2^20-sample signal at 48 111.9 and 119.7, of four 2^18-sample ones at 24 88.4 and 83.7.
+    // The others: one CTA per item, sized so that several CTAs share an SM (64 registers per thread) except for the longest
+    // bands, which fill its shared memory.
     const int limits[kNumClasses] = {128, 1024, 4096, 13500, 1 << 30};
     {
         const int threads[kNumClasses] = {256, 256, 256, 512, 1024};

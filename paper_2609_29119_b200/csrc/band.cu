@@ -77,6 +77,11 @@ struct FewLaunch {
     int short_threads = 0, short_grid = 0;
 };
 
+// CTAs of a launch that share an SM, at most `most` (what its launch bounds allow): its shared memory decides the rest.
+static long long ctas_per_sm(const cqt_plan &p, size_t smem, int most) {
+    return std::min<long long>(most, (p.max_smem_optin + 1024ll) / ((long long)smem + 1024));
+}
+
 // Segments [first, last) in CTAs filled to 1 / share; returns the SMs the launch occupies, and whether CTAs hold more
 // than one item.
 static long long few_part(const cqt_plan &p, int64_t batch, int first, int last, int share, FewLaunch::Part &t, bool &spread) {
@@ -96,13 +101,24 @@ static long long few_part(const cqt_plan &p, int64_t batch, int first, int last,
         if (grid > (1 << 20)) return grid;
     }
     t.grid = (int)grid;
-    const long long cta_smem = (long long)t.smem + kMaxGroups * (long long)sizeof(BandItem) + 1024;
-    const long long per_sm = std::min<long long>(1024 / t.threads, (p.max_smem_optin + 1024) / cta_smem);
+    const long long per_sm = ctas_per_sm(p, t.smem + kMaxGroups * sizeof(BandItem), 1024 / t.threads);
     return per_sm > 0 ? (grid + per_sm - 1) / per_sm : 1 << 20;
 }
 
 // The few-items form is taken where every CTA of the longer bands is resident at once.  A call that small is a chain of
-// latencies, and side by side on streams each class adds a launch, an event and two cross-stream waits to it.
+// latencies, and side by side on streams each class adds a launch, an event and two cross-stream waits to it (round trips
+// at 48 bands per octave: 4 signals of 2^13 samples 35.8 us in this form, 43.5 in the other; 398 bands of 80 bins, 4
+// signals of 2^15: 37.8 and 45.3).
+//
+// The short class is chained behind them on a warp per item, up to 16 items per SM.  Above, neither form is the faster one
+// for every plan: at 17 - 22 items per SM the chained form took 39 us where the classes took 41 (8 signals of 2^13 samples
+// at 48 bands per octave) and 42 where they took 49 (398 bands of 80 bins), but 49 where they took 41 (8 signals of 2^15
+// samples at 48 bands per octave); from 80 items per SM on the classes' 8 lanes per item win (63 against 77 us at 129).
+//
+// Up to 4 items per SM its CTAs have 64 threads, so that they lie on all SMs, above that 256.  Where the class holds direct
+// sums, whose items take long, that pays (multiple-of-4 lengths, 2 signals of 2^16: 52.5 us, with 256 threads 55.8); for
+// 5-smooth lengths it is within the spread of runs or a little slower (2^13 samples, 24 bands per octave, 4 signals: 38.7
+// us, with 256 threads 37.2).
 static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
     const int n = (int)p.merged.segs.size();
     const int split = n && p.merged.segs[0].lg_nthr == 10 ? 1 : 0;
@@ -111,9 +127,14 @@ static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
         FewLaunch t;
         bool spread = false;
         t.chirp = !p.chirp.recs.empty();
-        long long sms = t.chirp ? (chirp_grid(p, batch, nullptr) + 1) / 2 : 0;   // two CTAs of it share an SM
         t.split = split > 0;
-        sms += 2 * (long long)p.split.recs.size() * batch;                  // and of the split kernel
+        // launch bounds of two CTAs per SM; one sub-transform of 8,192 points gives every CTA of its launch 139 KB
+        auto add = [&](long long ctas, size_t smem) {
+            const long long per_sm = std::max(1ll, ctas_per_sm(p, smem, 2));
+            return (ctas + per_sm - 1) / per_sm;
+        };
+        long long sms = t.chirp ? add(chirp_grid(p, batch, nullptr), chirp_smem(p)) : 0;
+        if (t.split) sms += add(4 * (long long)p.split.recs.size() * batch, split_smem(p));
         sms += few_part(p, batch, split, n, share, t.part, spread);
         if (sms > p.sm_count) {
             if (share == 1) return false;

@@ -162,6 +162,7 @@ bool pow2_has(const cqt_plan &p, bool long_ones);
 cudaError_t launch_pow2(const cqt_plan &p, bool analysis, bool long_ones, const BandArgs &b, cudaStream_t st);
 
 // band_split.cu: long bands of calls with few items
+size_t split_smem(const cqt_plan &p);
 cudaError_t launch_split(const cqt_plan &p, bool analysis, const BandArgs &b, cudaStream_t st);
 
 // band_chirp.cu: bands of more than 128 coefficients whose length has a prime factor above 5

@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) split_bands_kernel(BandArgs 
     chain_end(a);
 }
 
-static size_t split_smem(const cqt_plan &p) { return (size_t)p.split.max_elems * sizeof(float2); }
+size_t split_smem(const cqt_plan &p) { return (size_t)p.split.max_elems * sizeof(float2); }
 
 cudaError_t launch_split(const cqt_plan &p, bool analysis, const BandArgs &b, cudaStream_t st) {
     BandArgs a = b;

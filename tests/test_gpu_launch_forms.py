@@ -116,6 +116,25 @@ def test_more_than_31_planes(log_n, batch):
     plan.close()
 
 
+def test_few_items_form_ends_where_its_ctas_are_no_longer_resident():
+    """Two bands of 8,212 coefficients (convolution length 8,192: one CTA per SM, four per band and signal) and two sidebands
+    split into four items (two CTAs per SM): 12 SMs per signal."""
+    from paper_2609_29119_b200 import Plan
+    N, M = 1 << 15, 8212
+    plan = Plan.from_bands(float(N), N, [N / 4.0 - 0.1 * M, N / 4.0 + 0.1 * M], [M - 1.5] * 2, m_policy=wl.M_MULT4)
+    assert [b.M for b in plan.bands()][1:3] == [M, M] and min(plan.band_info(0).M, plan.band_info(3).M) > 13500
+    most = torch.cuda.get_device_properties(0).multi_processor_count // 12
+    for batch, few in ((1, True), (most, True), (most + 1, False)):
+        x = torch.zeros(batch, N, device="cuda")
+        plan.set_timing(True)
+        plan.synthesise(plan.analyse(x))
+        torch.cuda.synchronize()
+        names = {n.split("/")[1] for n, _ in plan.read_timing() if "/" in n}
+        plan.set_timing(False)
+        assert "chirp" in names and ("split" in names) == few and ("class4" in names) == (not few), (batch, names)
+    plan.close()
+
+
 # more than 3,120 bands of one class: the list of their records is a large table, uploaded by itself (class 0; class 1 and the
 # list of the one-launch form, on both sides of the batch where that form ends)
 @pytest.mark.parametrize("n_bands, width, spacing, log_n, batch", [(4000, 32.0, 16, 17, 2), (3300, 200.0, 36, 18, 1), (3300, 200.0, 36, 18, 2)])
