@@ -4,14 +4,15 @@
 //            conj W_Lp^{j2 q1}, written transposed to Tinv[j2][q1].
 //   pass C': inverse A-point DFT over q1, unpacked to x[2j], x[2j+1]; only valid_len samples are written.
 //
-// Weighted-bin scratch: P planes of Lp+1 bins per signal; band b writes plane b mod P, where P is the largest number of
-// bands covering one bin, so two bands of one plane never share a bin and the sum over the bands covering bin k reads
-// its planes at index k: coalesced, in fixed order, no atomics.
+// Weighted-bin scratch: P planes of Lp+1 bins per signal, P the largest number of bands covering one bin.  A band writes the
+// lowest plane that is free at its first bin (interval colouring at plan creation; with more than 31 planes band b writes plane
+// b mod P), so two bands of one plane never share a bin and the sum over the bands covering bin k reads their planes at
+// index k: coalesced, in fixed order, no atomics.
 //
 // Bounds: issue slots and, in pass R', the latency of a chain of loads (cover word, planes).  The two operands of every
 // fold feed two butterflies of one thread, so sums and fold stay in its registers and the tile is written once; cover
-// words belong to the plan and are fetched before the predecessor kernel is waited for; with at most three planes the
-// word is a bit mask of the planes that hold the bin.  The last stage stores straight to Tinv.  32 signals of
+// words belong to the plan and are fetched before the predecessor kernel is waited for; up to 31 planes the word is a
+// bit mask of the planes that hold the bin (MASK).  The last stage stores straight to Tinv.  32 signals of
 // N = 2^19 before (fold, transform and transposition through shared memory, run-time strides): 88 us + 35 us.
 #include "long_passes.cuh"
 
