@@ -52,7 +52,7 @@ typedef enum {
     CQT_ERR_UNSUPPORTED = -2,  /* N not a power of two in range, a band too long for the kernels */
     CQT_ERR_BAD_LAYOUT = -3,   /* windows do not cover every bin, first centre below bin 2, support > M */
     CQT_ERR_WORKSPACE = -4,    /* ws null, misaligned or smaller than cqt_plan_workspace_bytes */
-    CQT_ERR_CUDA = -5,         /* a CUDA runtime call or launch failed */
+    CQT_ERR_CUDA = -5,         /* a CUDA runtime call or launch failed, or host memory ran out */
     CQT_ERR_STATE = -6,        /* host-only plan used for a transform; slicq call out of order */
     CQT_ERR_DEVICE_CHECK = -7  /* reserved: a device-side self check reported a violation */
 } cqt_status;

@@ -6,6 +6,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <new>
 
 #include "../../include/cqt.h"
@@ -164,6 +165,16 @@ void free_device(cqt_plan *p) {
     cudaSetDevice(cur);
 }
 
+struct PlanDestroy {
+    void operator()(cqt_plan *p) const { cqt_plan_destroy(p); }
+};
+using OwnedPlan = std::unique_ptr<cqt_plan, PlanDestroy>;   // on every path out of a creating function, exceptions among them
+
+struct RestoreDevice {
+    int cur;
+    ~RestoreDevice() { cudaSetDevice(cur); }
+};
+
 bool is_pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
 
 }  // namespace
@@ -195,7 +206,7 @@ cqt_status cqt_plan_create(double fs, double fmin, double fmax, int bins_per_oct
     return cqt_plan_create_ex(&d, out);
 }
 
-static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan_tuning &tune, cqt_plan **out);
+static cqt_status finish_plan(OwnedPlan p, int64_t N, int device, const cqt_plan_tuning &tune, cqt_plan **out);
 
 static bool length_supported(int64_t N) { return is_pow2(N) && N >= 64 && N <= (1ll << 22); }
 
@@ -203,7 +214,7 @@ cqt_status cqt_plan_create_ex(const cqt_plan_desc *desc, cqt_plan **out) {
     return cqt_plan_create_tuned(desc, nullptr, out);
 }
 
-cqt_status cqt_plan_create_tuned(const cqt_plan_desc *desc, const cqt_plan_tuning *tuning, cqt_plan **out) {
+cqt_status cqt_plan_create_tuned(const cqt_plan_desc *desc, const cqt_plan_tuning *tuning, cqt_plan **out) try {
     if (!desc || !out) return CQT_ERR_INVALID_ARG;
     cqt_plan_tuning tune{};
     if (tuning) tune = *tuning;
@@ -211,17 +222,18 @@ cqt_status cqt_plan_create_tuned(const cqt_plan_desc *desc, const cqt_plan_tunin
     const int64_t N = desc->L;
     if (N < 0) return CQT_ERR_INVALID_ARG;
     if (!length_supported(N)) return CQT_ERR_UNSUPPORTED;
-    cqt_plan *p = new (std::nothrow) cqt_plan();
-    if (!p) return CQT_ERR_CUDA;
+    OwnedPlan p(new cqt_plan());
     LayoutDesc ld{desc->fs, desc->fmin, desc->fmax, desc->bins_per_octave, N, desc->window, desc->m_policy,
                   desc->min_win > 0 ? desc->min_win : 4.0};
     std::string why;
     int rc = build_layout(ld, p->lay, why);
-    if (rc != 0) { delete p; return (cqt_status)rc; }
-    return finish_plan(p, N, desc->device, tune, out);
+    if (rc != 0) return (cqt_status)rc;
+    return finish_plan(std::move(p), N, desc->device, tune, out);
+} catch (...) {   // host memory ran out
+    return CQT_ERR_CUDA;
 }
 
-cqt_status cqt_plan_create_bands(const cqt_band_list_desc *desc, cqt_plan **out) {
+cqt_status cqt_plan_create_bands(const cqt_band_list_desc *desc, cqt_plan **out) try {
     if (!desc || !out || !desc->centre_hz || !desc->width_bins || desc->n_bands < 1 || desc->L < 0) return CQT_ERR_INVALID_ARG;
     const int64_t N = desc->L;
     if (!length_supported(N)) return CQT_ERR_UNSUPPORTED;
@@ -229,18 +241,19 @@ cqt_status cqt_plan_create_bands(const cqt_band_list_desc *desc, cqt_plan **out)
     std::vector<BandSpec> specs((size_t)desc->n_bands);
     for (int64_t i = 0; i < desc->n_bands; ++i)
         specs[i] = BandSpec{desc->centre_hz[i], desc->width_bins[i], desc->group ? desc->group[i] : -1};
-    cqt_plan *p = new (std::nothrow) cqt_plan();
-    if (!p) return CQT_ERR_CUDA;
+    OwnedPlan p(new cqt_plan());
     LayoutDesc ld{desc->fs, 0.0, 0.0, 0, N, desc->window, desc->m_policy, 4.0};
     std::string why;
     int rc = build_layout_bands(ld, specs, p->lay, why);
-    if (rc != 0) { delete p; return (cqt_status)rc; }
-    return finish_plan(p, N, desc->device, cqt_plan_tuning{}, out);
+    if (rc != 0) return (cqt_status)rc;
+    return finish_plan(std::move(p), N, desc->device, cqt_plan_tuning{}, out);
+} catch (...) {
+    return CQT_ERR_CUDA;
 }
 
 cqt_status cqt_multires_bands(double fs, double fmin, int64_t L, const int *octaves, const int *bins_per_octave,
                               int n_sections, double min_win, int64_t capacity, double *centre_hz, double *width_bins,
-                              int32_t *group, int64_t *n_bands) {
+                              int32_t *group, int64_t *n_bands) try {
     if (!n_bands || capacity < 0) return CQT_ERR_INVALID_ARG;
     std::vector<BandSpec> specs;
     std::string why;
@@ -253,11 +266,12 @@ cqt_status cqt_multires_bands(double fs, double fmin, int64_t L, const int *octa
         if (group) group[i] = specs[i].group;
     }
     return CQT_OK;
+} catch (...) {
+    return CQT_ERR_CUDA;
 }
 
-static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan_tuning &tune, cqt_plan **out) {
+static cqt_status finish_plan(OwnedPlan p, int64_t N, int device, const cqt_plan_tuning &tune, cqt_plan **out) {
     p->N = N;
-    p->device = device;
     const HostLayout &L = p->lay;
     p->g32.resize(L.table_len);
     p->h32.resize(L.table_len);
@@ -426,18 +440,18 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
         }
         if (c > 0 && !smooth(M)) {
             const int li = M % 4 == 0 ? chirp_length_index(M / 4) : -1;
-            if (li < 0) { delete p; return CQT_ERR_UNSUPPORTED; }
+            if (li < 0) return CQT_ERR_UNSUPPORTED;
             chirp_bands[li].push_back(i);
             continue;
         }
         if (single) {
             // short bands: fewer registers, more CTAs per SM
             p->bands[i].fft = plan_for(M, kPlanBand, p->cls[c].max_radix);
-            if (p->bands[i].fft < 0) { delete p; return CQT_ERR_UNSUPPORTED; }
+            if (p->bands[i].fft < 0) return CQT_ERR_UNSUPPORTED;
             const int64_t elems = band_elems(i);
             if (elems > smem_cap_elems) {   // the cap is per work item; the classes with several items per CTA are far below it
                 A2 = split_two_pass(M);
-                if (!A2) { delete p; return CQT_ERR_UNSUPPORTED; }
+                if (!A2) return CQT_ERR_UNSUPPORTED;
                 single = false;
             } else {
                 p->cls[c].work.push_back(i);
@@ -562,11 +576,13 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
             bc.latency_us = bc.n_bands ? 5.0 + us_per_elem[c] * (double)longest : 0.0;
         }
     }
-    if (p->device < 0) { *out = p; return CQT_OK; }
+    if (device < 0) { *out = p.release(); return CQT_OK; }
 
     // ---- device tables
     int cur = 0;
-    if (cudaGetDevice(&cur) != cudaSuccess || cudaSetDevice(p->device) != cudaSuccess) { p->device = -1; delete p; return CQT_ERR_CUDA; }
+    if (cudaGetDevice(&cur) != cudaSuccess || cudaSetDevice(device) != cudaSuccess) return CQT_ERR_CUDA;
+    const RestoreDevice restore{cur};
+    p->device = device;   // from here on there may be something to free on it
     std::vector<float> tA(L.table_len), tS(L.table_len), tTA(L.table_len), tSA(L.table_len);
     for (size_t i = 0; i < L.bands.size(); ++i) {
         const HostBand &hb = L.bands[i];
@@ -644,9 +660,8 @@ static cqt_status finish_plan(cqt_plan *p, int64_t N, int device, const cqt_plan
     if (e == cudaSuccess) chk(p->lf.A == 1 ? configure_short_fft_kernels(*p) : configure_long_forward_kernels(*p));
     if (e == cudaSuccess && p->lf.A > 1) chk(configure_long_inverse_kernels(*p));
     if (e == cudaSuccess) chk(configure_two_pass_kernels(*p));
-    cudaSetDevice(cur);
-    if (e != cudaSuccess) { cqt_plan_destroy(p); return CQT_ERR_CUDA; }
-    *out = p;
+    if (e != cudaSuccess) return CQT_ERR_CUDA;
+    *out = p.release();
     return CQT_OK;
 }
 

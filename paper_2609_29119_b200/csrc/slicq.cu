@@ -5,7 +5,7 @@
 #include <cstring>
 #include <algorithm>
 #include <cmath>
-#include <new>
+#include <memory>
 #include <vector>
 
 #include "../../include/cqt.h"
@@ -218,14 +218,16 @@ cqt_status push_impl(cqt_slicq *s, const float *x, int64_t x_stride, int64_t n, 
 extern "C" {
 
 cqt_status slicq_create(const cqt_plan *plan, int channels, int64_t transition, int64_t max_slices_in_flight,
-                        cqt_slicq **out) {
+                        cqt_slicq **out) try {
     if (!plan || !out || channels < 1 || max_slices_in_flight < 1) return CQT_ERR_INVALID_ARG;
     if (plan->device < 0) return CQT_ERR_STATE;
     const int64_t sl = plan->N, H = sl / 2;
     if (transition <= 0 || transition > H) return CQT_ERR_INVALID_ARG;
     if (max_slices_in_flight * channels > 65535) return CQT_ERR_INVALID_ARG;
-    cqt_slicq *s = new (std::nothrow) cqt_slicq();
-    if (!s) return CQT_ERR_CUDA;
+    struct Destroy {
+        void operator()(cqt_slicq *p) const { slicq_destroy(p); }
+    };
+    std::unique_ptr<cqt_slicq, Destroy> s(new cqt_slicq());
     s->plan = plan; s->C = channels; s->sl = sl; s->H = H; s->tr = transition; s->K = max_slices_in_flight;
     s->ring_in = (s->K + 2) * H;
     s->ring_out = (s->K + 2) * H;
@@ -239,9 +241,8 @@ cqt_status slicq_create(const cqt_plan *plan, int channels, int64_t transition, 
         else if (t < hi) v = 0.5 * (1.0 + std::cos(3.14159265358979323846 * (t - lo) / (double)transition));
         w[i] = (float)v;
     }
-    int cur = 0;
-    cudaGetDevice(&cur);
-    if (cudaSetDevice(plan->device) != cudaSuccess) { delete s; return CQT_ERR_CUDA; }
+    const OnPlanDevice guard(s.get());
+    if (!guard.ok) return CQT_ERR_CUDA;
     const int64_t cc = cqt_plan_coeff_count(plan);
     s->ws_bytes = cqt_plan_workspace_bytes(plan, s->K * channels);
     const size_t b_win = sl * sizeof(float), b_in = (size_t)channels * s->ring_in * sizeof(float),
@@ -266,10 +267,11 @@ cqt_status slicq_create(const cqt_plan *plan, int channels, int64_t transition, 
     if (e == cudaSuccess) chk(cudaMemcpy(s->d_win, w.data(), b_win, cudaMemcpyHostToDevice));
     if (e == cudaSuccess) chk(cudaMemset(s->d_out, 0, b_out));
     s->total_bytes = b_win + b_in + b_stage + b_coef + b_out + s->ws_bytes;
-    cudaSetDevice(cur);
-    if (e != cudaSuccess) { slicq_destroy(s); return CQT_ERR_CUDA; }
-    *out = s;
+    if (e != cudaSuccess) return CQT_ERR_CUDA;
+    *out = s.release();
     return CQT_OK;
+} catch (...) {   // host memory ran out
+    return CQT_ERR_CUDA;
 }
 
 cqt_status slicq_push(cqt_slicq *s, const float *x, int64_t x_stride, int64_t n, void *stream, int64_t *slices_completed) {

@@ -176,3 +176,30 @@ def test_band_list_errors():
         assert e.value.status == status
     # a narrow band nested deep inside a wide neighbour is a legal frame
     cq.Plan.from_bands(1024.0, 1024, [100.0, 101.0, 200.0], [180.0, 8.0, 200.0], device=-1).close()
+
+
+def test_creating_a_plan_without_enough_host_memory_returns_a_status():
+    """Nothing throws across the C boundary: with the address space limited, creating a large host-only plan returns
+    CQT_ERR_CUDA; with the limit lifted it succeeds in the same process."""
+    import subprocess
+    import sys
+    code = """
+import resource
+from paper_2609_29119_b200 import binding as B
+B.load_library()
+now = int(open('/proc/self/statm').read().split()[0]) * resource.getpagesize()
+soft, hard = resource.getrlimit(resource.RLIMIT_AS)
+make = lambda: B.Plan(48000.0, 20.0, 20000.0, 96, 1 << 22, window=1, m_policy=1, device=-1)
+for megabytes in (2, 8, 20, 40, 60):
+    resource.setrlimit(resource.RLIMIT_AS, (now + (megabytes << 20), hard))
+    try:
+        make()
+        print('created')
+    except B.CqtError as e:
+        print(e.status)
+resource.setrlimit(resource.RLIMIT_AS, (soft, hard))
+print(make().num_bands)
+"""
+    res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT)
+    assert res.returncode == 0, res.stderr[-2000:]
+    assert res.stdout.split() == ["-5"] * 5 + ["959"]
