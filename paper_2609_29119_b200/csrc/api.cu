@@ -642,6 +642,9 @@ static cqt_status finish_plan(OwnedPlan p, int64_t N, int device, const cqt_plan
     up.add(p->split.d_recs, p->split.recs);
     for (auto &g : p->two_pass) up.add(g.d_recs, g.bands);
     up.finish();
+    // a copy from pageable memory may return when the data is staged; the first call may come on a stream that does not wait
+    // for the default one
+    chk(cudaStreamSynchronize(nullptr));
     chk(cudaDeviceGetAttribute(&p->sm_count, cudaDevAttrMultiProcessorCount, p->device));
     chk(cudaDeviceGetAttribute(&p->max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
     // the helper streams carry the shorter classes: at the highest priority their CTAs are placed ahead of the

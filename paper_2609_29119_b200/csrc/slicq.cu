@@ -266,6 +266,8 @@ cqt_status slicq_create(const cqt_plan *plan, int channels, int64_t transition, 
     }
     if (e == cudaSuccess) chk(cudaMemcpy(s->d_win, w.data(), b_win, cudaMemcpyHostToDevice));
     if (e == cudaSuccess) chk(cudaMemset(s->d_out, 0, b_out));
+    // copies and memset above may still be on their way; the first push may come on a stream that does not wait for the default one
+    if (e == cudaSuccess) chk(cudaStreamSynchronize(nullptr));
     s->total_bytes = b_win + b_in + b_stage + b_coef + b_out + s->ws_bytes;
     if (e != cudaSuccess) return CQT_ERR_CUDA;
     *out = s.release();

@@ -260,3 +260,23 @@ def test_slices_that_wrap_around_the_slots(kw, tuning):
     assert snr_db(x[check][:, :n], y).min() >= 120.0
     sq.close()
     plan.close()
+
+
+def test_objects_are_ready_for_any_stream_when_they_are_created():
+    """A plan and a stream object used at once on a stream that does not wait for the default one."""
+    from paper_2609_29119_b200 import SliCQ
+    x = torch.from_numpy(wl.make_signal(W16))[:, :4 * (W16.slice_len // 2)].cuda()
+    torch.cuda.synchronize()
+    results = []
+    for i in range(6):
+        side = torch.cuda.Stream() if i else torch.cuda.current_stream()
+        y = torch.zeros(x.shape, device="cuda")
+        torch.cuda.synchronize()
+        plan = library_plan(W16)
+        sq = SliCQ(plan, x.shape[0], W16.transition, 4)
+        assert sq.push(x, stream=side) == 4
+        frames = sq.pull(y, stream=side)
+        side.synchronize()
+        results.append(y[:, :frames].clone())
+        sq.close(); plan.close()
+    assert all(torch.equal(r, results[0]) for r in results)
