@@ -190,27 +190,56 @@ def job_throughput(samples_per_rank: float, world: int, ms_total: float, steps: 
     return samples_per_rank * world / (ms_total / steps / 1e3) / 1e6
 
 
-def kernel_algorithmic_bytes(plan, w, batch):
+def kernel_algorithmic_bytes(plan, w, batch, names):
     """Minimal HBM bytes each kernel is responsible for per launch: signal samples, coefficients and window
-    tables; the packed spectrum, the half spectrum and the weighted-bin rows are intermediates (0 bytes)."""
-    cls_m = {}
-    cls_s = {}
+    tables; the packed spectrum, the half spectrum and the weighted-bin rows are intermediates (0 bytes).
+    names: the kernels that ran, which tell the launch form and with it the kernel of every band."""
+    forms = {n.split("/", 1)[1] for n in names if n.startswith("bands_from_spectrum/")}
+
+    def kernel_of(bi):
+        smooth = 60 ** 23 % bi.M == 0
+        if "pow2" in forms and bi.M > 128 and bi.launch_class >= 0:
+            return "pow2_long" if bi.M > 4096 else "pow2"
+        if bi.M > 128 and not smooth:
+            return "chirp"
+        if "merged" in forms and bi.M > 128:
+            return "split" if "split" in forms and bi.M > 6144 else "merged"
+        return f"class{bi.launch_class}"
+    owned, two_pass_bands = {}, 0
     for bi in plan.bands():
-        cls_m[bi.launch_class] = cls_m.get(bi.launch_class, 0) + bi.M
-        cls_s[bi.launch_class] = cls_s.get(bi.launch_class, 0) + bi.support
+        b = 8 * bi.M * batch + 4 * bi.support
+        if bi.launch_class < 0:
+            two_pass_bands += b
+        else:
+            owned[kernel_of(bi)] = owned.get(kernel_of(bi), 0) + b
     sig = 4 * w.valid_len * batch
     two_pass = plan.N // 2 > 4096
     out = {"rfft_cols_fwd": sig if two_pass else 0, "rfft_rows_fwd": 0 if two_pass else sig,
            "irfft_cols": sig if two_pass else 0, "irfft_rows": 0 if two_pass else sig}
-    for c in cls_m:
-        b = 8 * cls_m[c] * batch + 4 * cls_s[c]
-        if c < 0:      # bands on the two-pass kernels: pass 2 writes (analysis) / pass 1 reads (synthesis) the coefficients
-            out["band2p_rows/analysis"] = b
-            out["band2p_cols/synthesis"] = b
-        else:
-            out[f"bands_from_spectrum/class{c}"] = b
-            out[f"bands_to_spectrum/class{c}"] = b
+    for k, b in owned.items():
+        out[f"bands_from_spectrum/{k}"] = out[f"bands_to_spectrum/{k}"] = b
+    # bands on the two-pass kernels: pass 2 writes (analysis), pass 1 reads (synthesis) the coefficients
+    for which in ("band2p_rows/analysis", "band2p_cols/synthesis"):
+        ran = [n for n in names if n.startswith(which)]
+        if len(ran) == 1:      # two of them: bands on either side of their size limit
+            out[ran[0]] = two_pass_bands
     return out
+
+
+def kernel_source_digest():
+    """Digest of the kernels' sources without comments and white space: counters captured from other kernels are not
+    printed as those of the present ones."""
+    import hashlib
+    import re
+    src = os.path.join(ROOT, "paper_2609_29119_b200", "csrc")
+    h = hashlib.sha256()
+    for name in sorted(os.listdir(src)):
+        if name.endswith((".cu", ".cuh", ".cpp", ".hpp", ".h", ".py")) and name not in ("codelets_gen.cuh", "torch_ext.cpp"):
+            text = open(os.path.join(src, name)).read()
+            if not name.endswith(".py"):
+                text = re.sub(r"/\*.*?\*/|//[^\n]*", "", text, flags=re.S)
+            h.update((name + re.sub(r"\s+", "", text)).encode())
+    return h.hexdigest()[:16]
 
 
 def path_algorithmic_bytes(plan, w, batch, second_is_adjoint=False):
@@ -453,7 +482,7 @@ def run_ours(args, w):
         return
 
     peak, peak_kind = measured_peaks()
-    alg = kernel_algorithmic_bytes(plan, w, batch)
+    alg = kernel_algorithmic_bytes(plan, w, batch, per)
     tot_ms = sum(v[1] for v in per.values())
     kernels = {n: {"launches": v[0], "avg_us": 1e3 * v[1] / v[0], "share": v[1] / tot_ms,
                    "alg_bytes": alg.get(n, 0),
@@ -469,7 +498,8 @@ def run_ours(args, w):
     prof = os.path.join(ROOT, "profiles", "dram_traffic_workload2.txt")
     if os.path.exists(prof):
         try:
-            table = json.load(open(prof)).get(w.name, {})
+            captured = json.load(open(prof))
+            table = captured.get(w.name, {}) if captured.get("kernel_sources") == kernel_source_digest() else {}
             traffic = table.get(dom)
             traffic_total = sum(table.values()) if table else None
         except Exception:
