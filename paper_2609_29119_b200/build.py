@@ -11,10 +11,13 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libcqt_b200.so")
 EXT = os.path.join(HERE, "_cqt_torch.so")        # Python side of the transform calls, linked to LIB and torch
-SOURCES = ["layout.cpp", "api.cu", "band.cu", "band_analysis.cu", "band_synthesis.cu", "band_two_pass.cu", "band_chirp.cu", "band_split.cu", "band_pow2.cu", "long_fft_forward.cu", "long_fft_inverse.cu", "short_fft.cu", "slicq.cu", "static_ws.cu"]
+SOURCES = ["band_two_pass.cu", "band_analysis.cu", "band_synthesis.cu", "layout.cpp", "api.cu", "band.cu", "band_chirp.cu", "band_split.cu", "band_pow2.cu", "band_smooth.cu", "long_fft_forward.cu", "long_fft_inverse.cu", "short_fft.cu", "slicq.cu", "static_ws.cu"]
+# compiled once per class and direction (CQT_SMOOTH_KERNELS in band_smooth.cuh)
+VARIANTS = [("band_smooth_kernel.cu", f"band_smooth_{c}{'sa'[a]}.o", [f"-DCQT_CLASS={c}", f"-DCQT_ANALYSIS={a}"]) for c, a in ((0, 0), (0, 1))]
 HEADERS = ["layout.hpp", "plan_types.h", "internal.hpp", "engine.cuh", "band_common.cuh", "long_common.cuh", "long_passes.cuh",
            "static_fft.cuh", "codelets_gen.cuh", "table_upload.hpp",
            os.path.join("..", "..", "include", "cqt.h")]
+SMOOTH_HEADERS = ["band_smooth.cuh", "band_shapes.cuh"]   # of the sources that start with band_smooth
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC"]
 
@@ -58,12 +61,13 @@ def build(force: bool = False, verbose: bool = False, debug_bounds: bool = False
     nvcc = _nvcc()
     jobs = []
     objs = []
-    for s in SOURCES:
+    for s, o, flags in [(s, os.path.splitext(s)[0] + ".o", []) for s in SOURCES] + VARIANTS:
         src = os.path.join(CSRC, s)
-        obj = os.path.join(OBJ, os.path.splitext(s)[0] + ".o")
+        obj = os.path.join(OBJ, o)
         objs.append(obj)
-        if force or _stale(obj, [src] + hdrs):
-            cmd = [nvcc] + NVCC_FLAGS + flags_extra + (["-Xptxas", "-v"] if verbose else []) + ["-x", "cu", "-c", src, "-o", obj]
+        own = [os.path.join(CSRC, h) for h in SMOOTH_HEADERS] if s.startswith("band_smooth") else []
+        if force or _stale(obj, [src] + hdrs + own):
+            cmd = [nvcc] + NVCC_FLAGS + flags + flags_extra + (["-Xptxas", "-v"] if verbose else []) + ["-x", "cu", "-c", src, "-o", obj]
             jobs.append(cmd)
     if jobs:
         with cf.ThreadPoolExecutor(max_workers=min(8, len(jobs))) as ex:

@@ -39,6 +39,28 @@ int append_twiddles(std::vector<float2> &tw, int64_t n, int &logC) {
     return off;
 }
 
+// Twiddle rows of the stages before the last (radices r, trailing ones: fewer stages), appended to tw: on sub-transforms of n
+// points rows W_n^{p y}, y < n / r, p = 1, 2, 4, ... < r.  Returns the offset.  W_n^y is a product of two double factors
+// (1e-16), rounded once: sqrt(n) sines and cosines instead of n.
+int append_twiddle_rows(std::vector<float2> &tw, int64_t M, const int (&r)[5]) {
+    const int off = (int)tw.size();
+    int64_t n = M;
+    std::vector<std::complex<double>> fine(64), coarse;
+    for (int j = 0; j < 4 && r[j + 1] > 1; ++j) {
+        coarse.resize((size_t)((n + 63) / 64));
+        for (size_t i = 0; i < fine.size(); ++i) fine[i] = std::polar(1.0, -2.0 * kPi * (double)i / (double)n);
+        for (size_t i = 0; i < coarse.size(); ++i) coarse[i] = std::polar(1.0, -2.0 * kPi * (double)(64 * i) / (double)n);
+        for (int64_t pw = 1; pw < r[j]; pw *= 2)
+            for (int64_t i = 0; i < n / r[j]; ++i) {
+                const int64_t y = pw * i;   // below n
+                const std::complex<double> u = fine[(size_t)(y & 63)], v = coarse[(size_t)(y >> 6)];
+                tw.push_back(make_float2((float)(u.real() * v.real() - u.imag() * v.imag()), (float)(u.real() * v.imag() + u.imag() * v.real())));
+            }
+        n /= r[j];
+    }
+    return off;
+}
+
 const int kBandRadices[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
 const int kPow2Radices[] = {16, 8, 4, 2};
 
@@ -508,6 +530,27 @@ static cqt_status finish_plan(OwnedPlan p, int64_t N, int device, const cqt_plan
             p->pow2.recs.push_back(rec);
         }
     }
+    // classes whose lengths all have a shape of their own: records by length, longest first, and the lengths' twiddle rows
+    for (int c = 0; c < kNumClasses; ++c) {
+        const std::vector<int32_t> &work = p->cls[c].work;
+        int r[5];
+        if (!std::all_of(work.begin(), work.end(), [&](int32_t b) { return smooth_radices(L.bands[(size_t)b].M, r); })) continue;
+        SmoothBands &sb = p->smooth[c];
+        int off = 0;
+        for (int32_t b : work) {
+            const int64_t M = L.bands[(size_t)b].M;
+            if (sb.lengths.empty() || sb.lengths.back().M != M) {
+                smooth_radices(M, r);
+                off = append_twiddle_rows(tw, M, r);
+                sb.lengths.push_back({(int)M, (int)sb.recs.size(), 0});
+            }
+            sb.lengths.back().n_bands++;
+            SmoothRec rec{};
+            rec.br = p->bands[(size_t)b];
+            rec.tw_off = off;
+            sb.recs.push_back(rec);
+        }
+    }
     // every length L that occurs: one full twiddle table; bands of equal length share their tables
     for (int li = 0; li < kChirpLengths; ++li) {
         p->chirp.n_bands[li] = (int)chirp_bands[li].size();
@@ -638,6 +681,7 @@ static cqt_status finish_plan(OwnedPlan p, int64_t N, int device, const cqt_plan
     upload_items(p->merged.d_items, p->merged.work);
     up.add(p->chirp.d_recs, p->chirp.recs);
     up.add(p->pow2.d_recs, p->pow2.recs);
+    for (auto &sb : p->smooth) up.add(sb.d_recs, sb.recs);
     up.add(p->split.d_items, p->split.items);
     up.add(p->split.d_recs, p->split.recs);
     for (auto &g : p->two_pass) up.add(g.d_recs, g.bands);
@@ -659,6 +703,7 @@ static cqt_status finish_plan(OwnedPlan p, int64_t N, int device, const cqt_plan
     if (e == cudaSuccess) chk(configure_band_kernels(*p));
     if (e == cudaSuccess) chk(configure_chirp_kernels(*p));
     if (e == cudaSuccess) chk(configure_pow2_kernels(*p));
+    if (e == cudaSuccess) chk(configure_smooth_kernels(*p));
     if (e == cudaSuccess) chk(configure_split_kernels(*p));
     if (e == cudaSuccess) chk(p->lf.A == 1 ? configure_short_fft_kernels(*p) : configure_long_forward_kernels(*p));
     if (e == cudaSuccess && p->lf.A > 1) chk(configure_long_inverse_kernels(*p));

@@ -75,6 +75,7 @@ struct FewLaunch {
     bool split = false;                 // bands on the split kernel
     bool chirp = false;                 // bands on the chirp-z kernel
     int short_threads = 0, short_grid = 0;
+    bool short_smooth = false;          // class 0 on the kernel of 5-smooth lengths
 };
 
 // CTAs of a launch that share an SM, at most `most` (what its launch bounds allow): its shared memory decides the rest.
@@ -118,7 +119,9 @@ static long long few_part(const cqt_plan &p, int64_t batch, int first, int last,
 // Up to 4 items per SM its CTAs have 64 threads, so that they lie on all SMs, above that 256.  Where the class holds direct
 // sums, whose items take long, that pays (multiple-of-4 lengths, 2 signals of 2^16: 52.5 us, with 256 threads 55.8); for
 // 5-smooth lengths it is within the spread of runs or a little slower (2^13 samples, 24 bands per octave, 4 signals: 38.7
-// us, with 256 threads 37.2).
+// us, with 256 threads 37.2).  5-smooth lengths run on their own kernel, 8 lanes per item, up to 6 items per SM (3 clips of 8,000
+// samples 38.6 -> 36.6 us, one hop of a stereo stream 42.1 -> 40.5); above, a warp per item is as fast or faster (7.5 items per
+// SM: seven signals of 99,225 samples 69.6 and 70.6).
 static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
     const int n = (int)p.merged.segs.size();
     const int split = n && p.merged.segs[0].lg_nthr == 10 ? 1 : 0;
@@ -146,6 +149,7 @@ static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
     const long long items = (long long)p.cls[0].n_bands * batch;
     if (items > 16ll * p.sm_count) return false;
     f.short_threads = items > 4ll * p.sm_count ? 256 : 64;
+    f.short_smooth = has_smooth(p, true, 0) && items <= 6ll * p.sm_count;
     f.short_grid = (int)((items * 32 + f.short_threads - 1) / f.short_threads);
     return true;
 }
@@ -176,6 +180,7 @@ static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cuda
     }
     if (f.short_grid && e == cudaSuccess) {
         const BandClass &c = p.cls[0];
+        if (f.short_smooth) return launch_smooth(p, ANALYSIS, 0, names[ANALYSIS][1], a, st);
         a.items = c.d_items;
         void *args[] = {&a};
         e = launch_kernel(class_kernel<ANALYSIS>(c, 32, true), dim3((unsigned)f.short_grid), dim3((unsigned)f.short_threads), args,
@@ -200,6 +205,8 @@ static cudaError_t launch_pow2_plan(const cqt_plan &p, BandArgs &a, cudaStream_t
     if (c.n_bands > 0 && e == cudaSuccess) {
         const long long items = (long long)c.n_bands * a.batch;
         const int lanes = lanes_for(p, c, items), threads = items > 4ll * p.sm_count ? c.threads : 64, per_cta = threads / lanes;
+        if (has_smooth(p, ANALYSIS, 0))
+            return launch_smooth(p, ANALYSIS, 0, ANALYSIS ? "bands_from_spectrum/class0" : "bands_to_spectrum/class0", a, st, threads);
         void *args[] = {&a};
         e = launch_kernel(class_kernel<ANALYSIS>(c, lanes, true), dim3((unsigned)((items + per_cta - 1) / per_cta)), dim3((unsigned)threads), args,
                           (size_t)c.max_elems * per_cta * sizeof(float2), st);
@@ -261,6 +268,14 @@ struct ForkJoin {
     }
 };
 
+// Classes of the side-by-side form that run on the kernels of 5-smooth lengths.
+// Class 0, 8 lanes per item either way, two stages instead of three: beside class 1 alone 136 -> 127 us (64 hops of a stereo
+// stream, both directions).  Beside classes of longer bands its narrower shared memory lets more of its CTAs in ahead of their long
+// items: front end of 64 clips, analysis 188 -> 190, synthesis 187 -> 192.
+static bool class_is_smooth(const cqt_plan &p, bool analysis, int cls) {
+    return has_smooth(p, analysis, cls) && !p.cls[2].n_bands && !p.cls[3].n_bands && !p.cls[4].n_bands;
+}
+
 static bool has_two_pass(const cqt_plan &p) { return !p.two_pass[0].bands.empty() || !p.two_pass[1].bands.empty(); }
 
 cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, const CoefRows &c,
@@ -303,7 +318,8 @@ cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, co
         a.spec = X;
         a.spec_pitch = p.lf.x_pitch;
         set_rows(a, c);
-        cudaError_t e = launch_class<true>(p, i, names[i], a, fj.stream_for(i));
+        if (p.cls[i].n_bands == 0) continue;
+        cudaError_t e = class_is_smooth(p, true, i) ? launch_smooth(p, true, i, names[i], a, fj.stream_for(i)) : launch_class<true>(p, i, names[i], a, fj.stream_for(i));
         if (e != cudaSuccess) { fj.join(); return e; }
     }
     fj.join();
@@ -363,7 +379,8 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
         set_rows(a, c);
         a.Y = Y;
         a.fold = fold_sidebands ? 1 : 0;
-        cudaError_t e = launch_class<false>(p, i, names[i], a, fj.stream_for(i));
+        if (p.cls[i].n_bands == 0) continue;
+        cudaError_t e = class_is_smooth(p, false, i) ? launch_smooth(p, false, i, names[i], a, fj.stream_for(i)) : launch_class<false>(p, i, names[i], a, fj.stream_for(i));
         if (e != cudaSuccess) { fj.join(); return e; }
     }
     fj.join();

@@ -49,6 +49,14 @@ struct Pow2Bands {
     Pow2Rec *d_recs = nullptr;
 };
 
+// Bands of one class on the kernels of 5-smooth lengths: equal lengths adjacent, longest first
+struct SmoothBands {
+    struct Length { int M, first_band, n_bands; };
+    std::vector<Length> lengths;
+    std::vector<SmoothRec> recs;
+    SmoothRec *d_recs = nullptr;
+};
+
 struct SplitBands {
     std::vector<BandItem> items;     // record of the band, radix plan of a quarter of its length
     std::vector<SplitRec> recs;
@@ -107,6 +115,7 @@ struct cqt_plan {
     cqt::MergedBands merged;
     cqt::ChirpBands chirp;
     cqt::Pow2Bands pow2;
+    cqt::SmoothBands smooth[cqt::kNumClasses];   // by class
     cqt::SplitBands split;             // the bands of the first segment of `merged` when that has 1024 threads per item
     std::vector<int8_t> band_class;    // length class of every band, -1: two-pass kernels
     cqt::TwoPassGroup two_pass[2];     // [0]: both factors <= 256, [1]: larger factors
@@ -233,6 +242,10 @@ cudaError_t configure_chirp_kernels(const cqt_plan &p);
 int pow2_length_index(int64_t M);                  // place of a length in Pow2Bands::n_bands, -1: not a length of that kernel
 void pow2_radices(int index, int (&r)[4]);         // its stages (1: none)
 cudaError_t configure_pow2_kernels(const cqt_plan &p);
+
+// band_smooth.cu
+bool smooth_radices(int64_t M, int (&r)[5]);       // stages of a length (1: none); false: no shape for it
+cudaError_t configure_smooth_kernels(const cqt_plan &p);
 
 // band_split.cu
 cudaError_t configure_split_kernels(const cqt_plan &p);

@@ -74,6 +74,14 @@ struct Pow2Rec {
 };
 constexpr int kPow2Lengths = 7;   // 16,384 ... 256
 
+// A band on the kernels of 5-smooth lengths.
+struct SmoothRec {
+    BandRec br;
+    int32_t tw_off;      // twiddle rows of its length in the twiddle array (SmoothShape in band_smooth.cuh)
+    int32_t pad_[3];
+};
+constexpr int kSmoothLengths = 60;   // lengths of a launch, at most
+
 // A band split into four work items (band_split.cu): two-level table of W_M
 struct SplitRec {
     int32_t tw_m, log_m_c, n_m, pad_;

@@ -1,0 +1,77 @@
+"""Every 5-smooth band length with a kernel of its own, in the forms that reach it, against numpy's FFT of the windowed, slot-placed
+spectrum; the round trip covers the synthesis form."""
+import numpy as np
+import pytest
+
+import workloads as wl
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5
+
+
+def smooth(m):
+    for f in (2, 3, 5):
+        while m % f == 0:
+            m //= f
+    return m == 1
+
+
+def lengths(lo, hi, limit=None):
+    """5-smooth multiples of 4 above lo up to hi: all, or about `limit` of them with the first and the last."""
+    every = [m for m in range(lo // 4 * 4 + 4, hi + 1, 4) if smooth(m)]
+    return every if limit is None else [every[i] for i in sorted({round(j * (len(every) - 1) / (limit - 1)) for j in range(limit)})]
+
+
+def check_lengths(wanted, fill, N, batch, policy=wl.M_SMOOTH, forms=None):
+    """Bands of the wanted lengths between bands of the longest one, which keep the frame complete.  fill: part of the slots used."""
+    from paper_2609_29119_b200 import Plan
+    longest = max(wanted)
+    step = max(1.0, longest / 8.0)
+    widths, centres = [], []
+    for m in sorted(wanted, reverse=True):
+        widths += [longest - 1.5, max(m - 1.5 if m == longest else fill * (m - 1.5), 2.5)]
+    centres = [N / 4.0 + step * i for i in range(len(widths))]
+    assert centres[-1] + longest < N / 2
+    plan = Plan.from_bands(float(N), N, centres, widths, m_policy=policy)
+    have = {b.M for b in plan.bands()}
+    assert fill < 1.0 or set(wanted) <= have
+    rng = np.random.default_rng(longest)
+    x = rng.standard_normal((batch, N)).astype(np.float32)
+    xg = torch.from_numpy(x).cuda()
+    if forms is not None:
+        plan.set_timing(True)
+        plan.synthesise(plan.analyse(xg))
+        torch.cuda.synchronize()
+        names = {n.split("/")[1] for n, _ in plan.read_timing() if "/" in n}
+        plan.set_timing(False)
+        assert forms <= names, names
+    c = plan.analyse(xg)
+    got, (g, _) = c.cpu().numpy(), plan.tables()
+    rows = sorted({0, 1, batch // 2, batch - 1} & set(range(batch)))
+    X = np.fft.rfft(x[rows].astype(np.float64))
+    for bi in plan.bands():
+        if bi.is_sideband:
+            continue
+        d = np.arange(bi.first_offset, bi.first_offset + bi.support)
+        slots = np.zeros((len(rows), bi.M), dtype=np.complex128)
+        slots[:, d % bi.M] = g[bi.table_offset:bi.table_offset + bi.support] * X[:, bi.centre_bin + d]
+        want = np.fft.ifft(slots)
+        err = np.linalg.norm(got[rows, bi.coeff_offset:bi.coeff_offset + bi.M] - want, axis=1) / np.linalg.norm(want, axis=1)
+        assert err.max() <= TOL, (bi.M, err.max())
+    y = plan.synthesise(c).cpu().numpy().astype(np.float64)
+    assert (np.sum((y - x) ** 2, axis=1) / np.sum(x.astype(np.float64) ** 2, axis=1)).max() <= 1e-12
+    plan.close()
+
+
+# 1 and 3 signals: the few-items form; 401: class kernels side by side, several units per CTA, the last one ragged
+@pytest.mark.parametrize("batch", [1, 3, 401])
+@pytest.mark.parametrize("fill", [1.0, 0.6])
+def test_short_lengths(fill, batch):
+    check_lengths(lengths(0, 128), fill, 1 << 12, batch)
+
+
+@pytest.mark.parametrize("batch", [1, 37, 701])
+def test_short_lengths_of_power_of_two_plans(batch):
+    check_lengths([4, 8, 16, 32, 64, 128], 1.0, 1 << 12, batch, policy=wl.M_POW2, forms={"class0"})
