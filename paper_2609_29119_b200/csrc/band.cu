@@ -268,15 +268,22 @@ struct ForkJoin {
     }
 };
 
-// Classes of the side-by-side form that run on the kernels of 5-smooth lengths.
-// Class 0, 8 lanes per item either way, two stages instead of three: beside class 1 alone 136 -> 127 us (64 hops of a stereo
-// stream, both directions).  Beside classes of longer bands its narrower shared memory lets more of its CTAs in ahead of their long
-// items: front end of 64 clips, analysis 188 -> 190, synthesis 187 -> 192.
-static bool class_is_smooth(const cqt_plan &p, bool analysis, int cls) {
-    return has_smooth(p, analysis, cls) && !p.cls[2].n_bands && !p.cls[3].n_bands && !p.cls[4].n_bands;
-}
-
 static bool has_two_pass(const cqt_plan &p) { return !p.two_pass[0].bands.empty() || !p.two_pass[1].bands.empty(); }
+
+// Classes of the side-by-side form that run on the kernels of 5-smooth lengths.
+// Analysis: class 1 alone 51 -> 44 us (256 signals of 2^15 samples at 24 bands per octave, whole call 90 -> 78), class 2 35 -> 31
+// (32 signals of 2^19).  The two stay on the run-time planned engine in calls with two-pass bands, which have few items (one
+// 2^22-sample signal 214 us, on these kernels 220), and in synthesis, where their last stage (window value, predicated store per
+// slot) holds the items longer: class 1 37 -> 39, class 2 35 -> 39.  Nor class 1 beside class 0 alone, whose items then come
+// late: 64 hops of a stereo stream 126.7 -> 131.6 us.
+// Class 0, 8 lanes per item either way, two stages instead of three: synthesis beside class 1 alone 132 -> 127 us (64 hops of a
+// stereo stream).  Beside classes of longer bands its narrower shared memory lets more of its CTAs in ahead of their long items:
+// synthesis of the front end of 64 clips 187 -> 192, its analysis 185.6 -> 187, but 256 signals at 24 bands per octave 82 -> 78.
+static bool class_is_smooth(const cqt_plan &p, bool analysis, int cls) {
+    if (!has_smooth(p, analysis, cls) || has_two_pass(p)) return false;
+    const bool longer = p.cls[2].n_bands || p.cls[3].n_bands || p.cls[4].n_bands;
+    return cls == 0 ? analysis || !longer : analysis && longer;
+}
 
 cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, const CoefRows &c,
                                        float2 *scratch, int64_t batch, cudaStream_t st) {

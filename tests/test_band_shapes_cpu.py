@@ -6,8 +6,8 @@ import re
 import numpy as np
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_29119_b200", "csrc")
-LIMITS = {0: (0, 128)}
-THREADS = {0: 256}
+LIMITS = {0: (0, 128), 1: (128, 1024), 2: (1024, 4096)}
+THREADS = {0: 256, 1: 256, 2: 256}
 SMEM_ELEMS = 227 * 1024 // 8       # of an SM
 
 

@@ -28,11 +28,11 @@ def check_lengths(wanted, fill, N, batch, policy=wl.M_SMOOTH, forms=None):
     """Bands of the wanted lengths between bands of the longest one, which keep the frame complete.  fill: part of the slots used."""
     from paper_2609_29119_b200 import Plan
     longest = max(wanted)
-    step = max(1.0, longest / 8.0)
+    step = longest / 12.0
     widths, centres = [], []
     for m in sorted(wanted, reverse=True):
         widths += [longest - 1.5, max(m - 1.5 if m == longest else fill * (m - 1.5), 2.5)]
-    centres = [N / 4.0 + step * i for i in range(len(widths))]
+    centres = [1.1 * longest + step * i for i in range(len(widths))]
     assert centres[-1] + longest < N / 2
     plan = Plan.from_bands(float(N), N, centres, widths, m_policy=policy)
     have = {b.M for b in plan.bands()}
@@ -69,9 +69,16 @@ def check_lengths(wanted, fill, N, batch, policy=wl.M_SMOOTH, forms=None):
 @pytest.mark.parametrize("batch", [1, 3, 401])
 @pytest.mark.parametrize("fill", [1.0, 0.6])
 def test_short_lengths(fill, batch):
-    check_lengths(lengths(0, 128), fill, 1 << 12, batch)
+    check_lengths(lengths(0, 128), fill, 1 << 11, batch)
 
 
 @pytest.mark.parametrize("batch", [1, 37, 701])
 def test_short_lengths_of_power_of_two_plans(batch):
-    check_lengths([4, 8, 16, 32, 64, 128], 1.0, 1 << 12, batch, policy=wl.M_POW2, forms={"class0"})
+    check_lengths([4, 8, 16, 32, 64, 128], 1.0, 1 << 11, batch, policy=wl.M_POW2, forms={"class0"})
+
+
+# enough items for the side-by-side form: a CTA has one or several units, the last one ragged
+@pytest.mark.parametrize("lo, hi, log_n, batch", [(128, 1024, 14, 151), (128, 1024, 14, 403), (1024, 4096, 16, 41), (1024, 4096, 16, 83)])
+@pytest.mark.parametrize("fill", [1.0, 0.6])
+def test_middle_lengths(fill, lo, hi, log_n, batch):
+    check_lengths(lengths(lo, hi), fill, 1 << log_n, batch, forms={"class1" if hi == 1024 else "class2"})
