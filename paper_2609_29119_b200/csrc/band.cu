@@ -276,13 +276,15 @@ static bool has_two_pass(const cqt_plan &p) { return !p.two_pass[0].bands.empty(
 // 2^22-sample signal 214 us, on these kernels 220), and in synthesis, where their last stage (window value, predicated store per
 // slot) holds the items longer: class 1 37 -> 39, class 2 35 -> 39.  Nor class 1 beside class 0 alone, whose items then come
 // late: 64 hops of a stereo stream 126.7 -> 131.6 us.
+// Class 4, both directions: the items of one call fill one round of the SMs, and what counts is the time of one of them: 42 -> 33 us
+// analysis, 39 -> 33 synthesis (128 items of up to 23,040 coefficients).
 // Class 0, 8 lanes per item either way, two stages instead of three: synthesis beside class 1 alone 132 -> 127 us (64 hops of a
 // stereo stream).  Beside classes of longer bands its narrower shared memory lets more of its CTAs in ahead of their long items:
 // synthesis of the front end of 64 clips 187 -> 192, its analysis 185.6 -> 187, but 256 signals at 24 bands per octave 82 -> 78.
 static bool class_is_smooth(const cqt_plan &p, bool analysis, int cls) {
     if (!has_smooth(p, analysis, cls) || has_two_pass(p)) return false;
     const bool longer = p.cls[2].n_bands || p.cls[3].n_bands || p.cls[4].n_bands;
-    return cls == 0 ? analysis || !longer : analysis && longer;
+    return cls == 0 ? analysis || !longer : (analysis && longer) || cls == 4;
 }
 
 cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, const CoefRows &c,

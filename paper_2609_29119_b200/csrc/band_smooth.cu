@@ -12,7 +12,7 @@ struct ShapeInfo {
 };
 const ShapeInfo kShapes[] = {   // longest first
 #define X(M, R0, R1, R2, R3, R4, T, PER, THREADS, PAD, CHUNK, ...) {M, PER, R0 * CHUNK, {R0, R1, R2, R3, R4}},
-    CQT_SHAPES_2(X) CQT_SHAPES_1(X) CQT_SHAPES_0(X)
+    CQT_SHAPES_4(X) CQT_SHAPES_2(X) CQT_SHAPES_1(X) CQT_SHAPES_0(X)
 #undef X
 };
 

@@ -303,6 +303,6 @@ template <bool ANALYSIS, int CLASS>
 struct SmoothKernel {
     static const void *get();
 };
-#define CQT_SMOOTH_KERNELS(X) X(0, false) X(0, true) X(1, true) X(2, true)
+#define CQT_SMOOTH_KERNELS(X) X(0, false) X(0, true) X(1, true) X(2, true) X(4, false) X(4, true)
 
 }  // namespace cqt

@@ -20,7 +20,7 @@ import gen_codelets as gc
 RADICES = (2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16)
 # class: lengths above, up to, threads per CTA, largest radix, threads of an item
 GROUPS = {0: (0, 128, 256, 16, lambda m: 8), 1: (128, 1024, 256, 10, lambda m: 32),
-          2: (1024, 4096, 256, 12, lambda m: 128 if m <= 2304 else 256)}
+          2: (1024, 4096, 256, 12, lambda m: 128 if m <= 2304 else 256), 4: (13500, 27648, 1024, 16, lambda m: 1024)}
 SMEM_ELEMS = 227 * 1024 // 8
 
 

@@ -6,8 +6,8 @@ import re
 import numpy as np
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2609_29119_b200", "csrc")
-LIMITS = {0: (0, 128), 1: (128, 1024), 2: (1024, 4096)}
-THREADS = {0: 256, 1: 256, 2: 256}
+LIMITS = {0: (0, 128), 1: (128, 1024), 2: (1024, 4096), 4: (13500, 27648)}
+THREADS = {0: 256, 1: 256, 2: 256, 4: 1024}
 SMEM_ELEMS = 227 * 1024 // 8       # of an SM
 
 
@@ -31,7 +31,7 @@ def smooth(m):
 
 def test_every_length_has_a_shape():
     rows = shapes()
-    assert sorted(r[1] for r in rows) == [m for m in range(4, max(upto for _, upto in LIMITS.values()) + 1, 4) if smooth(m)]
+    assert sorted(r[1] for r in rows) == [m for above, upto in LIMITS.values() for m in range(above // 4 * 4 + 4, upto + 1, 4) if smooth(m)]
     for group, (above, upto) in LIMITS.items():
         own = [r[1] for r in rows if r[0] == group]
         assert own == sorted(own, reverse=True) and len(own) <= 60

@@ -24,16 +24,23 @@ def lengths(lo, hi, limit=None):
     return every if limit is None else [every[i] for i in sorted({round(j * (len(every) - 1) / (limit - 1)) for j in range(limit)})]
 
 
+def band_list(wanted, fill, N):
+    """Bands of the wanted lengths between bands of the longest one, which keep the frame complete; long ones twice each, from
+    one end of the spectrum to the other.  fill: part of the slots used."""
+    longest, used = max(wanted), [max(m - 1.5 if m == max(wanted) else fill * (m - 1.5), 2.5) for m in wanted]
+    if longest > 4096:
+        widths = [w for w in used[::2] + used[1::2][::-1] for _ in range(2)]   # the longest in the middle
+        return [float(c) for c in np.linspace(0.6 * widths[0], N / 2 - 0.6 * widths[-1], len(widths))], widths
+    widths = [w for u in reversed(used) for w in (longest - 1.5, u)]
+    centres = [1.1 * longest + longest / 12.0 * i for i in range(len(widths))]
+    assert centres[-1] + longest < N / 2
+    return centres, widths
+
+
 def check_lengths(wanted, fill, N, batch, policy=wl.M_SMOOTH, forms=None):
-    """Bands of the wanted lengths between bands of the longest one, which keep the frame complete.  fill: part of the slots used."""
     from paper_2609_29119_b200 import Plan
     longest = max(wanted)
-    step = longest / 12.0
-    widths, centres = [], []
-    for m in sorted(wanted, reverse=True):
-        widths += [longest - 1.5, max(m - 1.5 if m == longest else fill * (m - 1.5), 2.5)]
-    centres = [1.1 * longest + step * i for i in range(len(widths))]
-    assert centres[-1] + longest < N / 2
+    centres, widths = band_list(wanted, fill, N)
     plan = Plan.from_bands(float(N), N, centres, widths, m_policy=policy)
     have = {b.M for b in plan.bands()}
     assert fill < 1.0 or set(wanted) <= have
@@ -82,3 +89,10 @@ def test_short_lengths_of_power_of_two_plans(batch):
 @pytest.mark.parametrize("fill", [1.0, 0.6])
 def test_middle_lengths(fill, lo, hi, log_n, batch):
     check_lengths(lengths(lo, hi), fill, 1 << log_n, batch, forms={"class1" if hi == 1024 else "class2"})
+
+
+# a CTA and nearly all of an SM's shared memory per item
+@pytest.mark.parametrize("fill", [1.0, 0.9])
+@pytest.mark.parametrize("part", range(3))
+def test_long_lengths(part, fill):
+    check_lengths(lengths(13500, 27648)[part::3], fill, 1 << 17, 8, forms={"class4"})
