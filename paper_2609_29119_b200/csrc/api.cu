@@ -45,15 +45,19 @@ int append_twiddles(std::vector<float2> &tw, int64_t n, int &logC) {
 int append_twiddle_rows(std::vector<float2> &tw, int64_t M, const int (&r)[5]) {
     const int off = (int)tw.size();
     int64_t n = M;
-    std::vector<std::complex<double>> fine(64), coarse;
+    std::vector<std::complex<double>> fine, coarse;
     for (int j = 0; j < 4 && r[j + 1] > 1; ++j) {
-        coarse.resize((size_t)((n + 63) / 64));
+        int lg = 2;
+        while ((1ll << (2 * lg)) < n) ++lg;
+        const int64_t low = (1ll << lg) - 1;
+        fine.resize((size_t)low + 1);
+        coarse.resize((size_t)((n + low) >> lg));
         for (size_t i = 0; i < fine.size(); ++i) fine[i] = std::polar(1.0, -2.0 * kPi * (double)i / (double)n);
-        for (size_t i = 0; i < coarse.size(); ++i) coarse[i] = std::polar(1.0, -2.0 * kPi * (double)(64 * i) / (double)n);
+        for (size_t i = 0; i < coarse.size(); ++i) coarse[i] = std::polar(1.0, -2.0 * kPi * (double)(i << lg) / (double)n);
         for (int64_t pw = 1; pw < r[j]; pw *= 2)
             for (int64_t i = 0; i < n / r[j]; ++i) {
                 const int64_t y = pw * i;   // below n
-                const std::complex<double> u = fine[(size_t)(y & 63)], v = coarse[(size_t)(y >> 6)];
+                const std::complex<double> u = fine[(size_t)(y & low)], v = coarse[(size_t)(y >> lg)];
                 tw.push_back(make_float2((float)(u.real() * v.real() - u.imag() * v.imag()), (float)(u.real() * v.imag() + u.imag() * v.real())));
             }
         n /= r[j];
@@ -533,16 +537,17 @@ static cqt_status finish_plan(OwnedPlan p, int64_t N, int device, const cqt_plan
     // classes whose lengths all have a shape of their own: records by length, longest first, and the lengths' twiddle rows
     for (int c = 0; c < kNumClasses; ++c) {
         const std::vector<int32_t> &work = p->cls[c].work;
-        int r[5];
-        if (!std::all_of(work.begin(), work.end(), [&](int32_t b) { return smooth_radices(L.bands[(size_t)b].M, r); })) continue;
+        if (c > 0 && !smooth_form(*p, true, c) && !smooth_form(*p, false, c)) continue;
+        if (!std::all_of(work.begin(), work.end(), [&](int32_t b) { return smooth_info(L.bands[(size_t)b].M) != nullptr; })) continue;
         SmoothBands &sb = p->smooth[c];
         int off = 0;
         for (int32_t b : work) {
             const int64_t M = L.bands[(size_t)b].M;
             if (sb.lengths.empty() || sb.lengths.back().M != M) {
-                smooth_radices(M, r);
-                off = append_twiddle_rows(tw, M, r);
-                sb.lengths.push_back({(int)M, (int)sb.recs.size(), 0});
+                const SmoothInfo &si = *smooth_info(M);
+                off = append_twiddle_rows(tw, M, si.r);
+                sb.lengths.push_back({(int)M, (int)sb.recs.size(), 0, si.per});
+                sb.smem = std::max(sb.smem, sizeof(float2) * (size_t)(si.per * si.buf));
             }
             sb.lengths.back().n_bands++;
             SmoothRec rec{};

@@ -281,11 +281,12 @@ static bool has_two_pass(const cqt_plan &p) { return !p.two_pass[0].bands.empty(
 // Class 0, 8 lanes per item either way, two stages instead of three: synthesis beside class 1 alone 132 -> 127 us (64 hops of a
 // stereo stream).  Beside classes of longer bands its narrower shared memory lets more of its CTAs in ahead of their long items:
 // synthesis of the front end of 64 clips 187 -> 192, its analysis 185.6 -> 187, but 256 signals at 24 bands per octave 82 -> 78.
-static bool class_is_smooth(const cqt_plan &p, bool analysis, int cls) {
-    if (!has_smooth(p, analysis, cls) || has_two_pass(p)) return false;
+bool smooth_form(const cqt_plan &p, bool analysis, int cls) {
+    if (has_two_pass(p)) return false;
     const bool longer = p.cls[2].n_bands || p.cls[3].n_bands || p.cls[4].n_bands;
     return cls == 0 ? analysis || !longer : (analysis && longer) || cls == 4;
 }
+static bool class_is_smooth(const cqt_plan &p, bool analysis, int cls) { return has_smooth(p, analysis, cls) && smooth_form(p, analysis, cls); }
 
 cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, const float2 *X, const CoefRows &c,
                                        float2 *scratch, int64_t batch, cudaStream_t st) {

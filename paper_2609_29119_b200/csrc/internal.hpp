@@ -51,8 +51,9 @@ struct Pow2Bands {
 
 // Bands of one class on the kernels of 5-smooth lengths: equal lengths adjacent, longest first
 struct SmoothBands {
-    struct Length { int M, first_band, n_bands; };
+    struct Length { int M, first_band, n_bands, per; };   // per: work items of a CTA (SmoothShape::PER)
     std::vector<Length> lengths;
+    size_t smem = 0;                   // of a CTA, the largest of the lengths
     std::vector<SmoothRec> recs;
     SmoothRec *d_recs = nullptr;
 };
@@ -244,7 +245,9 @@ void pow2_radices(int index, int (&r)[4]);         // its stages (1: none)
 cudaError_t configure_pow2_kernels(const cqt_plan &p);
 
 // band_smooth.cu
-bool smooth_radices(int64_t M, int (&r)[5]);       // stages of a length (1: none); false: no shape for it
+struct SmoothInfo { int M, per, buf, r[5]; };        // r: stages (1: none); buf: shared-memory elements (float2) of an item
+bool smooth_form(const cqt_plan &p, bool analysis, int cls);   // band.cu: the side-by-side form runs the class on them
+const SmoothInfo *smooth_info(int64_t M);          // null: no shape for that length
 cudaError_t configure_smooth_kernels(const cqt_plan &p);
 
 // band_split.cu

@@ -80,7 +80,7 @@ struct SmoothRec {
     int32_t tw_off;      // twiddle rows of its length in the twiddle array (SmoothShape in band_smooth.cuh)
     int32_t pad_[3];
 };
-constexpr int kSmoothLengths = 60;   // lengths of a launch, at most
+constexpr int kSmoothLengths = 40;   // lengths of a launch, at most
 
 // A band split into four work items (band_split.cu): two-level table of W_M
 struct SplitRec {

@@ -34,7 +34,7 @@ def test_every_length_has_a_shape():
     assert sorted(r[1] for r in rows) == [m for above, upto in LIMITS.values() for m in range(above // 4 * 4 + 4, upto + 1, 4) if smooth(m)]
     for group, (above, upto) in LIMITS.items():
         own = [r[1] for r in rows if r[0] == group]
-        assert own == sorted(own, reverse=True) and len(own) <= 60
+        assert own == sorted(own, reverse=True) and len(own) <= 40
         assert all(above < m <= upto for m in own)
 
 
