@@ -12,8 +12,9 @@ OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libcqt_b200.so")
 EXT = os.path.join(HERE, "_cqt_torch.so")        # Python side of the transform calls, linked to LIB and torch
 SOURCES = ["band_two_pass.cu", "band_analysis.cu", "band_synthesis.cu", "layout.cpp", "api.cu", "band.cu", "band_chirp.cu", "band_split.cu", "band_pow2.cu", "band_smooth.cu", "long_fft_forward.cu", "long_fft_inverse.cu", "short_fft.cu", "slicq.cu", "static_ws.cu"]
-# compiled once per class and direction (CQT_SMOOTH_KERNELS in band_smooth.cuh)
-VARIANTS = [("band_smooth_kernel.cu", f"band_smooth_{c}{'sa'[a]}.o", [f"-DCQT_CLASS={c}", f"-DCQT_ANALYSIS={a}"]) for c, a in ((0, 0), (0, 1), (1, 1), (2, 1), (4, 0), (4, 1))]
+# compiled once per class, direction and kind of launch (CQT_SMOOTH_KERNELS in band_smooth.cuh)
+VARIANTS = [("band_smooth_kernel.cu", f"band_smooth_{c}{'sa'[a]}{'_chained' * h}.o", [f"-DCQT_CLASS={c}", f"-DCQT_ANALYSIS={a}", f"-DCQT_CHAINED={h}"])
+            for c, a, h in ((0, 0, 0), (0, 0, 1), (0, 1, 0), (0, 1, 1), (1, 1, 0), (2, 1, 0), (4, 0, 0), (4, 1, 0))]
 HEADERS = ["layout.hpp", "plan_types.h", "internal.hpp", "engine.cuh", "band_common.cuh", "long_common.cuh", "long_passes.cuh",
            "static_fft.cuh", "codelets_gen.cuh", "table_upload.hpp",
            os.path.join("..", "..", "include", "cqt.h")]

@@ -13,8 +13,8 @@ const SmoothInfo kShapes[] = {   // longest first
 #undef X
 };
 
-const void *kernel_of(bool analysis, int cls) {
-#define X(C, A) if (cls == C && analysis == A) return SmoothKernel<A, C>::get();
+const void *kernel_of(bool analysis, int cls, bool chained) {
+#define X(C, A, H) if (cls == C && analysis == A && chained == H) return SmoothKernel<A, C, H>::get();
     CQT_SMOOTH_KERNELS(X)
 #undef X
     return nullptr;
@@ -28,7 +28,7 @@ const SmoothInfo *smooth_info(int64_t M) {
     return s != end && s->M == M ? s : nullptr;
 }
 
-bool has_smooth(const cqt_plan &p, bool analysis, int cls) { return !p.smooth[cls].recs.empty() && kernel_of(analysis, cls); }
+bool has_smooth(const cqt_plan &p, bool analysis, int cls) { return !p.smooth[cls].recs.empty() && kernel_of(analysis, cls, false); }
 
 // A CTA takes `repeat` units of one length one after another: the code of the length is fetched once for them, and warps that
 // are done with one are on with the loads of the next.  More of them leave fewer CTAs to even out the end of the launch:
@@ -54,7 +54,9 @@ cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const char 
         grid += ((int64_t)l.n_bands * b.batch + per_cta - 1) / per_cta;
     }
     void *args[] = {&a};
-    cudaError_t e = launch_kernel(kernel_of(analysis, cls), dim3((unsigned)grid), dim3((unsigned)threads), args, smem, st);
+    const void *fn = kernel_of(analysis, cls, b.chain == kChainMember);   // the head of a chain waits for itself
+    if (!fn) return cudaErrorInvalidDeviceFunction;
+    cudaError_t e = launch_kernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args, smem, st);
     note_launch(p, name, st);
     return e;
 }
@@ -63,8 +65,12 @@ cudaError_t configure_smooth_kernels(const cqt_plan &p) {
     for (int c = 0; c < kNumClasses; ++c)
         for (bool analysis : {false, true}) {
             if (!has_smooth(p, analysis, c)) continue;
-            cudaError_t e = allow_dynamic_smem(kernel_of(analysis, c), p.smooth[c].smem, p);
-            if (e != cudaSuccess) return e;
+            for (bool chained : {false, true}) {
+                const void *fn = kernel_of(analysis, c, chained);
+                if (!fn) continue;
+                cudaError_t e = allow_dynamic_smem(fn, p.smooth[c].smem, p);
+                if (e != cudaSuccess) return e;
+            }
         }
     return cudaSuccess;
 }

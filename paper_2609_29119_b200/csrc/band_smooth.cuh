@@ -188,7 +188,8 @@ struct SmoothArgs {
 
 extern __shared__ float2 smem_smooth[];
 
-template <bool ANALYSIS, class S>
+// CHAINED: the launch may be a member of a chain (band_common.cuh); only class 0 is ever in one.
+template <bool ANALYSIS, bool CHAINED, class S>
 __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
     const SmoothSegment sg = a.seg[seg];
     const int per = S::M <= 128 ? (int)blockDim.x / S::T : S::PER;   // class 0 also runs in narrower CTAs
@@ -222,7 +223,7 @@ __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
 #pragma unroll
                     for (int q = 0; q < S::R0; ++q) {
                         const int j = entry(b + q * S::S0);
-                        const float2 v = j >= 0 && CQT_CHK(a.b.dbg, 801, j, br.S) ? ld_chained(Xs + j) : make_float2(0.f, 0.f);
+                        const float2 v = j >= 0 && CQT_CHK(a.b.dbg, 801, j, br.S) ? ld_spectrum<CHAINED>(Xs + j) : make_float2(0.f, 0.f);
                         re[q] = v.x; im[q] = v.y;
                     }
 #pragma unroll
@@ -234,7 +235,7 @@ __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
                 } else {
 #pragma unroll
                     for (int q = 0; q < S::R0; ++q) {
-                        const float2 v = slot_value(br, tab, X, a.b.N, b + q * S::S0);
+                        const float2 v = slot_value<CHAINED>(br, tab, X, a.b.N, b + q * S::S0);
                         re[q] = v.x; im[q] = v.y;
                     }
                 }
@@ -253,7 +254,7 @@ __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
             auto load = [&](int b, float (&re)[S::R0], float (&im)[S::R0]) {
 #pragma unroll
                 for (int q = 0; q < S::R0; ++q) {
-                    const float2 v = ld_chained(c + b + q * S::S0);   // read once
+                    const float2 v = ld_coefficient<CHAINED>(c + b + q * S::S0);   // read once
                     re[q] = v.x; im[q] = v.y;
                 }
                 if (fold) {
@@ -298,11 +299,12 @@ __device__ __forceinline__ int smooth_segment(const SmoothArgs &a) {
     return lo;
 }
 
-// One kernel per class and direction, each compiled by itself (band_smooth_kernel.cu; the list is that of build.py)
-template <bool ANALYSIS, int CLASS>
+// One kernel per class, direction and kind of launch, each compiled by itself (band_smooth_kernel.cu; the list is that of build.py)
+template <bool ANALYSIS, int CLASS, bool CHAINED>
 struct SmoothKernel {
     static const void *get();
 };
-#define CQT_SMOOTH_KERNELS(X) X(0, false) X(0, true) X(1, true) X(2, true) X(4, false) X(4, true)
+#define CQT_SMOOTH_KERNELS(X) \
+    X(0, false, false) X(0, false, true) X(0, true, false) X(0, true, true) X(1, true, false) X(2, true, false) X(4, false, false) X(4, true, false)
 
 }  // namespace cqt

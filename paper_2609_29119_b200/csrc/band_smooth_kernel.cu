@@ -1,5 +1,5 @@
-// The kernel of one class of 5-smooth lengths and one direction (band_smooth.cuh); compiled once per pair, with CQT_CLASS and
-// CQT_ANALYSIS from the command line.
+// The kernel of one class of 5-smooth lengths, one direction and one kind of launch (band_smooth.cuh); compiled once for each, with
+// CQT_CLASS, CQT_ANALYSIS and CQT_CHAINED from the command line.
 #include "band_smooth.cuh"
 
 namespace cqt {
@@ -15,7 +15,7 @@ static __global__ void __launch_bounds__(kThreads, 1024 / kThreads) smooth_bands
     const int seg = smooth_segment(a);
     chain_begin(a.b);   // records and tables belong to the plan; what follows touches the predecessor's output
     switch (a.seg[seg].shape) {
-#define X(M, ...) case M: smooth_units<CQT_ANALYSIS != 0, SmoothShape<M, __VA_ARGS__>>(a, seg); break;
+#define X(M, ...) case M: smooth_units<CQT_ANALYSIS != 0, CQT_CHAINED != 0, SmoothShape<M, __VA_ARGS__>>(a, seg); break;
         CQT_SHAPES(X)
 #undef X
         default: break;
@@ -24,6 +24,6 @@ static __global__ void __launch_bounds__(kThreads, 1024 / kThreads) smooth_bands
 }
 
 template <>
-const void *SmoothKernel<CQT_ANALYSIS != 0, CQT_CLASS>::get() { return (const void *)smooth_bands_kernel; }
+const void *SmoothKernel<CQT_ANALYSIS != 0, CQT_CLASS, CQT_CHAINED != 0>::get() { return (const void *)smooth_bands_kernel; }
 
 }  // namespace cqt

@@ -95,12 +95,3 @@ def test_stages_stay_in_the_buffer_and_give_the_dft():
         out[w[None, :] + np.arange(RL)[:, None] * NL] = dft[RL] @ buf[where]
         want = np.fft.fft(x)
         assert np.linalg.norm(out - want) <= 1e-11 * np.linalg.norm(want), M
-
-
-def test_chained_kernels_load_past_the_l1():
-    """The kernels run as members of a chain of band kernels too (band_common.cuh)."""
-    code = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "band_smooth.cuh")).read())
-    assert not re.search(r"\bld_data\s*\(|__ldc[sgav]\s*\(|__ldlu\s*\(", code)
-    assert not re.search(r"__ldg\s*\(\s*(Xs?|c|in|Ys?|out)\b", code)
-    assert not re.search(r"=\s*\*?\b(Xs?|c|in|Ys)\s*\[", code)
-    assert len(re.findall(r"\bld_chained\s*\(", code)) == 2
