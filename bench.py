@@ -194,7 +194,9 @@ def kernel_algorithmic_bytes(plan, w, batch, names):
     """Minimal HBM bytes each kernel is responsible for per launch: signal samples, coefficients and window
     tables; the packed spectrum, the half spectrum and the weighted-bin rows are intermediates (0 bytes).
     names: the kernels that ran, which tell the launch form and with it the kernel of every band."""
-    forms = {n.split("/", 1)[1] for n in names if n.startswith("bands_from_spectrum/")}
+    # a class's kernel is named after the class, with a mark where it is the one of 5-smooth lengths
+    ran = {n.removesuffix("/smooth"): n for n in names}
+    forms = {n.split("/", 1)[1] for n in ran if n.startswith("bands_from_spectrum/")}
 
     def kernel_of(bi):
         smooth = 60 ** 23 % bi.M == 0
@@ -217,12 +219,13 @@ def kernel_algorithmic_bytes(plan, w, batch, names):
     out = {"rfft_cols_fwd": sig if two_pass else 0, "rfft_rows_fwd": 0 if two_pass else sig,
            "irfft_cols": sig if two_pass else 0, "irfft_rows": 0 if two_pass else sig}
     for k, b in owned.items():
-        out[f"bands_from_spectrum/{k}"] = out[f"bands_to_spectrum/{k}"] = b
+        for which in ("bands_from_spectrum", "bands_to_spectrum"):
+            out[ran.get(f"{which}/{k}", f"{which}/{k}")] = b
     # bands on the two-pass kernels: pass 2 writes (analysis), pass 1 reads (synthesis) the coefficients
     for which in ("band2p_rows/analysis", "band2p_cols/synthesis"):
-        ran = [n for n in names if n.startswith(which)]
-        if len(ran) == 1:      # two of them: bands on either side of their size limit
-            out[ran[0]] = two_pass_bands
+        passes = [n for n in names if n.startswith(which)]
+        if len(passes) == 1:      # two of them: bands on either side of their size limit
+            out[passes[0]] = two_pass_bands
     return out
 
 
@@ -500,7 +503,7 @@ def run_ours(args, w):
         try:
             captured = json.load(open(prof))
             table = captured.get(w.name, {}) if captured.get("kernel_sources") == kernel_source_digest() else {}
-            traffic = table.get(dom)
+            traffic = table.get(dom.removesuffix("/smooth"))
             traffic_total = sum(table.values()) if table else None
         except Exception:
             traffic = traffic_total = None

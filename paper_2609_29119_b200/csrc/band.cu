@@ -180,7 +180,7 @@ static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cuda
     }
     if (f.short_grid && e == cudaSuccess) {
         const BandClass &c = p.cls[0];
-        if (f.short_smooth) return launch_smooth(p, ANALYSIS, 0, names[ANALYSIS][1], a, st);
+        if (f.short_smooth) return launch_smooth(p, ANALYSIS, 0, a, st);
         a.items = c.d_items;
         void *args[] = {&a};
         e = launch_kernel(class_kernel<ANALYSIS>(c, 32, true), dim3((unsigned)f.short_grid), dim3((unsigned)f.short_threads), args,
@@ -205,8 +205,7 @@ static cudaError_t launch_pow2_plan(const cqt_plan &p, BandArgs &a, cudaStream_t
     if (c.n_bands > 0 && e == cudaSuccess) {
         const long long items = (long long)c.n_bands * a.batch;
         const int lanes = lanes_for(p, c, items), threads = items > 4ll * p.sm_count ? c.threads : 64, per_cta = threads / lanes;
-        if (has_smooth(p, ANALYSIS, 0))
-            return launch_smooth(p, ANALYSIS, 0, ANALYSIS ? "bands_from_spectrum/class0" : "bands_to_spectrum/class0", a, st, threads);
+        if (has_smooth(p, ANALYSIS, 0)) return launch_smooth(p, ANALYSIS, 0, a, st, threads);
         void *args[] = {&a};
         e = launch_kernel(class_kernel<ANALYSIS>(c, lanes, true), dim3((unsigned)((items + per_cta - 1) / per_cta)), dim3((unsigned)threads), args,
                           (size_t)c.max_elems * per_cta * sizeof(float2), st);
@@ -329,7 +328,7 @@ cudaError_t launch_bands_from_spectrum(const cqt_plan &p, const float *table, co
         a.spec_pitch = p.lf.x_pitch;
         set_rows(a, c);
         if (p.cls[i].n_bands == 0) continue;
-        cudaError_t e = class_is_smooth(p, true, i) ? launch_smooth(p, true, i, names[i], a, fj.stream_for(i)) : launch_class<true>(p, i, names[i], a, fj.stream_for(i));
+        cudaError_t e = class_is_smooth(p, true, i) ? launch_smooth(p, true, i, a, fj.stream_for(i)) : launch_class<true>(p, i, names[i], a, fj.stream_for(i));
         if (e != cudaSuccess) { fj.join(); return e; }
     }
     fj.join();
@@ -390,7 +389,7 @@ cudaError_t launch_bands_to_spectrum(const cqt_plan &p, const float *table, bool
         a.Y = Y;
         a.fold = fold_sidebands ? 1 : 0;
         if (p.cls[i].n_bands == 0) continue;
-        cudaError_t e = class_is_smooth(p, false, i) ? launch_smooth(p, false, i, names[i], a, fj.stream_for(i)) : launch_class<false>(p, i, names[i], a, fj.stream_for(i));
+        cudaError_t e = class_is_smooth(p, false, i) ? launch_smooth(p, false, i, a, fj.stream_for(i)) : launch_class<false>(p, i, names[i], a, fj.stream_for(i));
         if (e != cudaSuccess) { fj.join(); return e; }
     }
     fj.join();

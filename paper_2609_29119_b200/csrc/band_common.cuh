@@ -164,7 +164,7 @@ cudaError_t launch_pow2(const cqt_plan &p, bool analysis, bool long_ones, const 
 
 // band_smooth.cu: every band of class cls, where the plan and the direction have that form; threads: of a CTA, 0: the class's (only class 0 has a choice)
 bool has_smooth(const cqt_plan &p, bool analysis, int cls);
-cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const char *name, const BandArgs &b, cudaStream_t st, int threads = 0);
+cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const BandArgs &b, cudaStream_t st, int threads = 0);
 
 // band_split.cu: long bands of calls with few items
 size_t split_smem(const cqt_plan &p);

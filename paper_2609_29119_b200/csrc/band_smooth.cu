@@ -28,12 +28,17 @@ const SmoothInfo *smooth_info(int64_t M) {
     return s != end && s->M == M ? s : nullptr;
 }
 
+// names of the launches: the class's, as in the other kernels of the class, and this kernel's mark
+const char *const kNames[2][kNumClasses] = {
+    {"bands_to_spectrum/class0/smooth", "bands_to_spectrum/class1/smooth", "bands_to_spectrum/class2/smooth", "bands_to_spectrum/class3/smooth", "bands_to_spectrum/class4/smooth"},
+    {"bands_from_spectrum/class0/smooth", "bands_from_spectrum/class1/smooth", "bands_from_spectrum/class2/smooth", "bands_from_spectrum/class3/smooth", "bands_from_spectrum/class4/smooth"}};
+
 bool has_smooth(const cqt_plan &p, bool analysis, int cls) { return !p.smooth[cls].recs.empty() && kernel_of(analysis, cls, false); }
 
 // A CTA takes `repeat` units of one length one after another: the code of the length is fetched once for them, and warps that
 // are done with one are on with the loads of the next.  More of them leave fewer CTAs to even out the end of the launch:
 // twice where the launch is at least 1.5 rounds of the resident CTAs, four times from 8 rounds on.
-cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const char *name, const BandArgs &b, cudaStream_t st, int threads) {
+cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const BandArgs &b, cudaStream_t st, int threads) {
     if (threads == 0) threads = kSmoothThreads[cls];
     const SmoothBands &s = p.smooth[cls];
     SmoothArgs a;
@@ -57,7 +62,7 @@ cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const char 
     const void *fn = kernel_of(analysis, cls, b.chain == kChainMember);   // the head of a chain waits for itself
     if (!fn) return cudaErrorInvalidDeviceFunction;
     cudaError_t e = launch_kernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args, smem, st);
-    note_launch(p, name, st);
+    note_launch(p, kNames[analysis][cls], st);
     return e;
 }
 

@@ -18,6 +18,8 @@ FROM = "bands_from_spectrum/"
     ("config2", ["split", "merged", "class0"]),
     ("table1", ["pow2", "class0"]),
     ("config4", ["class0", "class1", "class2", "class3", "class4"]),
+    ("config2", ["class0/smooth", "class1/smooth", "class2/smooth", "class3", "class4/smooth"]),
+    ("table1", ["pow2", "class0/smooth"]),
 ])
 def test_every_band_belongs_to_one_kernel(name, forms):
     w = wl.CONFIGS[name]
@@ -27,6 +29,16 @@ def test_every_band_belongs_to_one_kernel(name, forms):
     owned = bench.kernel_algorithmic_bytes(plan, w, 3, names)
     assert set(n for n in owned if "bands_" in n) <= set(names)
     assert all(owned.get(n, 0) > 0 for n in names if "bands_" in n)
+    assert sum(owned.values()) == bench.path_algorithmic_bytes(plan, w, 3)
+    plan.close()
+
+
+def test_directions_may_differ_in_the_kernel_of_a_class():
+    w = wl.CONFIGS["config2"]
+    plan = library_plan(w, device=-1)
+    names = [FROM + f"class{c}/smooth" for c in (0, 1, 2, 4)] + [FROM + "class3"] + [f"bands_to_spectrum/class{c}" for c in range(4)] + ["bands_to_spectrum/class4/smooth"]
+    owned = bench.kernel_algorithmic_bytes(plan, w, 3, names)
+    assert {n for n in owned if "bands_" in n} == set(names)
     assert sum(owned.values()) == bench.path_algorithmic_bytes(plan, w, 3)
     plan.close()
 
