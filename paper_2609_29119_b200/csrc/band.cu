@@ -119,9 +119,17 @@ static long long few_part(const cqt_plan &p, int64_t batch, int first, int last,
 // Up to 4 items per SM its CTAs have 64 threads, so that they lie on all SMs, above that 256.  Where the class holds direct
 // sums, whose items take long, that pays (multiple-of-4 lengths, 2 signals of 2^16: 52.5 us, with 256 threads 55.8); for
 // 5-smooth lengths it is within the spread of runs or a little slower (2^13 samples, 24 bands per octave, 4 signals: 38.7
-// us, with 256 threads 37.2).  5-smooth lengths run on their own kernel, 8 lanes per item, up to 6 items per SM (3 clips of 8,000
-// samples 38.6 -> 36.6 us, one hop of a stereo stream 42.1 -> 40.5); above, a warp per item is as fast or faster (7.5 items per
-// SM: seven signals of 99,225 samples 69.6 and 70.6).
+// us, with 256 threads 37.2).
+//
+// 5-smooth lengths run on their own kernel, 8 lanes per item, up to 6 items per SM, unless bands are split (above 6144
+// coefficients).  Round trips of 1 - 12 signals in 16 layouts, a warp per item on the run-time planned kernel against this one: without
+// split bands 3.7 % less on average up to 4 items per SM (4 signals of 2^13 samples at 24 bands per octave 39.9 -> 34.0 us, one of 2^16
+// at 24 42.6 -> 41.1, one of 2^18 at 96 50.2 -> 47.0; four of 40 calls 2 - 4.5 % slower); above 6 items per SM the two alternate.
+// With split bands it costs more than it gives (36 bands per octave: one signal of 2^17 60.1 -> 69.3 us, two 61.0 -> 71.8; one of
+// 2^18 at 24 55.6 -> 65.3; 2^16 at 12: one 36.8 -> 38.2, two 44.9 -> 40.1, three 43.7 -> 48.5, six 46.4 -> 46.1): probably the code,
+// since the split and the merged kernel wait for instructions more than for anything else and up to 19 lengths' code then passes
+// through the same caches.  256 threads per CTA at any number of items: with 64 or 128 the same layouts gain 2.9 and 3.4 % where
+// 256 gain 3.7.
 static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
     const int n = (int)p.merged.segs.size();
     const int split = n && p.merged.segs[0].lg_nthr == 10 ? 1 : 0;
@@ -149,7 +157,7 @@ static bool few_shape(const cqt_plan &p, int64_t batch, FewLaunch &f) {
     const long long items = (long long)p.cls[0].n_bands * batch;
     if (items > 16ll * p.sm_count) return false;
     f.short_threads = items > 4ll * p.sm_count ? 256 : 64;
-    f.short_smooth = has_smooth(p, true, 0) && items <= 6ll * p.sm_count;
+    f.short_smooth = has_smooth(p, true, 0) && !f.split && items <= 6ll * p.sm_count;
     f.short_grid = (int)((items * 32 + f.short_threads - 1) / f.short_threads);
     return true;
 }

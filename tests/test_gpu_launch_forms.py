@@ -135,6 +135,24 @@ def test_few_items_form_ends_where_its_ctas_are_no_longer_resident():
     plan.close()
 
 
+# one signal: bands of 23,328 coefficients are split, and class 0 stays on the run-time planned kernel beside them
+@pytest.mark.parametrize("log_n, fmax, split", [(17, 18000.0, True), (15, 22050.0, False)])
+def test_short_class_beside_split_bands(log_n, fmax, split):
+    w = small_workload("short_class", N=1 << log_n, valid_len=99225 if split else 1 << log_n, fs=44100.0, fmin=55.0, fmax=fmax, bins_per_octave=36, channels=1, m_policy=wl.M_SMOOTH)
+    plan = library_plan(w)
+    x = torch.from_numpy(wl.make_signal(w)).cuda()
+    plan.set_timing(True)
+    y = plan.synthesise(plan.analyse(x, valid_len=w.valid_len), valid_len=w.valid_len)
+    torch.cuda.synchronize()
+    names = {n for n, _ in plan.read_timing()}
+    plan.set_timing(False)
+    for d in ("bands_from_spectrum", "bands_to_spectrum"):
+        assert (f"{d}/split" in names) == split and f"{d}/merged" in names
+        assert (f"{d}/class0" if split else f"{d}/class0/smooth") in names
+    assert snr_db(x.cpu().numpy(), y.cpu().numpy()).min() >= 120.0
+    plan.close()
+
+
 # more than 3,120 bands of one class: the list of their records is a large table, uploaded by itself (class 0; class 1 and the
 # list of the one-launch form, on both sides of the batch where that form ends)
 @pytest.mark.parametrize("n_bands, width, spacing, log_n, batch", [(4000, 32.0, 16, 17, 2), (3300, 200.0, 36, 18, 1), (3300, 200.0, 36, 18, 2)])
