@@ -198,7 +198,10 @@ static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cuda
     return e;
 }
 
-// Power-of-two plans: two or three launches, chained, at any batch.
+// Power-of-two plans: two or three launches, chained, at any batch.  Class 0 on the kernel of 5-smooth lengths: 60 calls drawn from 2^12 ...
+// 2^18 samples, 12 - 96 bands per octave, 3 - 120 items per SM, against the run-time planned one: round trips from 20 % less to 4 % more, 4 %
+// less on average; analysis alone from 31 % less to, at 2^12 and 2^14 samples, 31 % more (27 signals of 2^12 at 48 12.9 -> 16.9 us, 9 of 2^14 at 36
+// 14.1 -> 17.9, but 2 of 2^14 11.8 -> 11.5), 4 % less on average; neither items per SM nor share of the coefficients tells the two apart.
 template <bool ANALYSIS>
 static cudaError_t launch_pow2_plan(const cqt_plan &p, BandArgs &a, cudaStream_t st) {
     const BandClass &c = p.cls[0];
@@ -284,10 +287,14 @@ static bool has_two_pass(const cqt_plan &p) { return !p.two_pass[0].bands.empty(
 // slot) holds the items longer: class 1 37 -> 39, class 2 35 -> 39.  Nor class 1 beside class 0 alone, whose items then come
 // late: 64 hops of a stereo stream 126.7 -> 131.6 us.
 // Class 4, both directions: the items of one call fill one round of the SMs, and what counts is the time of one of them: 42 -> 33 us
-// analysis, 39 -> 33 synthesis (128 items of up to 23,040 coefficients).
-// Class 0, 8 lanes per item either way, two stages instead of three: synthesis beside class 1 alone 132 -> 127 us (64 hops of a
-// stereo stream).  Beside classes of longer bands its narrower shared memory lets more of its CTAs in ahead of their long items:
-// synthesis of the front end of 64 clips 187 -> 192, its analysis 185.6 -> 187, but 256 signals at 24 bands per octave 82 -> 78.
+// analysis, 39 -> 33 synthesis (128 items of up to 23,040 coefficients).  Not beside two-pass bands, where every SM has a length of
+// its own and all their code passes through the caches at once (86 items of 27 lengths, one 2^22-sample signal at 96 bands per octave:
+// analysis 85.0 -> 87.2, synthesis 113.8 -> 119.8; 49 items of 28 lengths, two 2^21-sample signals at 48: 99.6 -> 104.0, 121.8 -> 137.5).
+// Class 0, 8 lanes per item either way, two stages instead of three.  Analysis, 12 layouts with 2 - 512 signals: from 43 % less to 1.4 %
+// more (2^14 samples, 96 bands per octave: 512 signals 152 -> 86, 32 signals 21.4 -> 21.7); where it has 7 % of the coefficients or less,
+// between 4 % less and 0.6 % more, whatever the items per SM (front end of 16, 64, 128 signals: 32.9 -> 33.1, 85.9 -> 86.3, 161.8 -> 160.7).
+// Synthesis where class 1 is the longest: 33 % less to 0.9 % more in five layouts; beside longer classes its narrower shared memory lets
+// more of its CTAs in ahead of their long items (front end of 32 signals 55.6 -> 57.4, 64 signals of 2^16 samples 62.6 -> 63.6).
 bool smooth_form(const cqt_plan &p, bool analysis, int cls) {
     if (has_two_pass(p)) return false;
     const bool longer = p.cls[2].n_bands || p.cls[3].n_bands || p.cls[4].n_bands;

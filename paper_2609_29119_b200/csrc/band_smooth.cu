@@ -36,8 +36,15 @@ const char *const kNames[2][kNumClasses] = {
 bool has_smooth(const cqt_plan &p, bool analysis, int cls) { return !p.smooth[cls].recs.empty() && kernel_of(analysis, cls, false); }
 
 // A CTA takes `repeat` units of one length one after another: the code of the length is fetched once for them, and warps that
-// are done with one are on with the loads of the next.  More of them leave fewer CTAs to even out the end of the launch:
-// twice where the launch is at least 1.5 rounds of the resident CTAs, four times from 8 rounds on.
+// are done with one are on with the loads of the next.  More of them leave fewer CTAs to even out the end of the launch.
+// Two from 1.5 rounds of the resident CTAs on and four from 8, but two only from 3 rounds (class 0) or 2 (the others) where the class has at
+// least half of the coefficients: nothing beside it then fills the SMs that its last round leaves idle.  Whole transform with one / two:
+//   class 0, 56 % or more: 1.9 rounds 36.3 / 41.8 us, 2.5 47.9 / 51.3, 4 65.8 / 63.6 (2^13 samples, 24 bands per octave, synthesis); 2.5 26.9 / 28.7,
+//   3 29.0 / 29.1, 4 33.0 / 31.7 (2^14, 96); round trips: 1.2 43.6 / 57.7, 2.5 50.3 / 60.5 (2^13, 48), the other way 2.5 78.4 / 76.2 (2^12, 12)
+//   class 0, 28 %: 1.75 40.6 / 40.9, 2 43.4 / 43.0 (2^15, 48, analysis); 14 %: 1.8 81.9 / 79.8 (2^15, 24)
+//   class 1, 82 %: 1.75 44.9 / 49.7, 2 48.8 / 52.3, 2.5 59.4 / 58.0 (2^15, 24); 47 %: 1.5 72.2 / 70.7, 2 89.7 / 87.3 (2^17, 48)
+//   class 2, 46 %: 1.5 58.0 / 58.9, 2 76.7 / 73.6 (2^17, 48); 40 %: 1.25 72.3 / 70.9, 2 109.2 / 105.0 (2^18, 24)
+// and with two / four: class 0 at 8 rounds 174 / 169 (2^15, 48), class 1 at 6 126 / 122.
 cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const BandArgs &b, cudaStream_t st, int threads) {
     if (threads == 0) threads = kSmoothThreads[cls];
     const SmoothBands &s = p.smooth[cls];
@@ -50,7 +57,10 @@ cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const BandA
     const int64_t resident = p.sm_count * std::min<int64_t>(1024 / threads, (p.max_smem_optin + 1024) / ((int64_t)smem + 1024));
     int64_t units = 0;
     for (const SmoothBands::Length &l : s.lengths) units += ((int64_t)l.n_bands * b.batch + l.per / part - 1) / (l.per / part);
-    a.repeat = 2 * units < 3 * resident ? 1 : (units < 8 * resident ? 2 : 4);
+    int64_t coefficients = 0;
+    for (const SmoothBands::Length &l : s.lengths) coefficients += (int64_t)l.M * l.n_bands;
+    const int64_t halves = 2 * coefficients < p.lay.coeff_count ? 3 : (cls == 0 ? 6 : 4);   // half rounds
+    a.repeat = 2 * units < halves * resident ? 1 : (units < 8 * resident ? 2 : 4);
     int64_t grid = 0;
     for (int i = 0; i < a.n; ++i) {
         const SmoothBands::Length &l = s.lengths[(size_t)i];

@@ -83,8 +83,8 @@ def both(cls):
     return {("from", cls), ("to", cls)}
 
 
-# 1 and 3 signals: the few-items form; 401: class kernels side by side, several units per CTA, the last one ragged
-@pytest.mark.parametrize("batch", [1, 3, 401])
+# 1 and 3 signals: the few-items form; 401, 1601, 4501: class kernels side by side, one, two and four units per CTA, the last one ragged
+@pytest.mark.parametrize("batch", [1, 3, 401, 1601, 4501])
 @pytest.mark.parametrize("fill", [1.0, 0.6])
 def test_short_lengths(fill, batch):
     check_lengths(lengths(0, 128), fill, 1 << 11, batch, both("class0"))
@@ -95,8 +95,8 @@ def test_short_lengths_of_power_of_two_plans(batch):
     check_lengths([4, 8, 16, 32, 64, 128], 1.0, 1 << 11, batch, both("class0"), policy=wl.M_POW2)
 
 
-# enough items for the side-by-side form: a CTA has one or several units, the last one ragged
-@pytest.mark.parametrize("lo, hi, log_n, batch", [(128, 1024, 14, 151), (128, 1024, 14, 403), (1024, 4096, 16, 41), (1024, 4096, 16, 83)])
+# enough items for the side-by-side form: a CTA has one, two or four units, the last one ragged
+@pytest.mark.parametrize("lo, hi, log_n, batch", [(128, 1024, 14, 101), (128, 1024, 14, 403), (128, 1024, 14, 701), (1024, 4096, 16, 17), (1024, 4096, 16, 53), (1024, 4096, 16, 113)])
 @pytest.mark.parametrize("fill", [1.0, 0.6])
 def test_middle_lengths(fill, lo, hi, log_n, batch):
     check_lengths(lengths(lo, hi), fill, 1 << log_n, batch, {("from", "class1" if hi == 1024 else "class2")})
