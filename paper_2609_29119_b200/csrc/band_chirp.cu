@@ -177,7 +177,7 @@ __device__ __forceinline__ void chirp_cta(const ChirpArgs &a, const ChirpSegment
     if constexpr (ANALYSIS) {
         const float2 *X = a.b.spec + (long long)ch * a.b.spec_pitch;
         float2 *out = a.b.coef + coef_row(a.b.row0, a.b.rows, ch) * a.b.coeff_count + br.coeff_off;
-        auto in = [&](int n) { return cconj(slot_value<true>(br, tab, X, a.b.N, n)); };
+        auto in = [&](int n) { return cconj(slot_value<true>(br, tab, X, a.b.N, n, a.b.dbg)); };
         chirp_convolve<S>(buf, twf, filter, m, active, t, [&](int n) { return combine(in(n), in(n + m), in(n + 2 * m), in(n + 3 * m), n); },
                           [&](int n, float2 v) { out[k0 + 4 * n] = cconj(cmul(v, __ldg(post + n))); });
     } else {

@@ -133,12 +133,14 @@ __device__ __forceinline__ void fetch_item(const BandItem &g, BandItem &s, int t
 // No branch around the loads, so that those of several slots are in flight together.
 template <bool CHAINED>
 __device__ __forceinline__ float2 slot_value(const BandRec &br, const float *__restrict__ tab,
-                                             const float2 *__restrict__ X, int N, int m) {
+                                             const float2 *__restrict__ X, int N, int m, int *dbg) {
     const bool lo = m <= br.d0 + br.S - 1, ok = lo || m >= br.M + br.d0;
     const int d = ok ? (lo ? m : m - br.M) : 0, k = br.kc + d, half = N >> 1;
     const bool mirrored = k < 0 || k > half;
+    const int km = k < 0 ? -k : (k > half ? N - k : k);
+    if (!CQT_CHK(dbg, 405, d - br.d0, br.S) || !CQT_CHK(dbg, 406, km, half + 1)) return make_float2(0.f, 0.f);
     const float g = ok ? __ldg(tab + (d - br.d0)) : 0.f;
-    const float2 x = ld_spectrum<CHAINED>(X + (k < 0 ? -k : (k > half ? N - k : k)));
+    const float2 x = ld_spectrum<CHAINED>(X + km);
     return make_float2(g * x.x, mirrored ? -(g * x.y) : g * x.y);
 }
 

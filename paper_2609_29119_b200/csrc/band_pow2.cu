@@ -194,7 +194,7 @@ __device__ __forceinline__ void pow2_cta(const Pow2Args &a, const Pow2Segment &s
             } else {
 #pragma unroll
                 for (int q = 0; q < S::R0; ++q) {
-                    const float2 v = slot_value<true>(br, tab, X, a.b.N, b + q * S::S0);
+                    const float2 v = slot_value<true>(br, tab, X, a.b.N, b + q * S::S0, a.b.dbg);
                     re[q] = v.x; im[q] = v.y;
                 }
             }

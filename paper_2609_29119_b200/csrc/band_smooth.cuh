@@ -78,7 +78,7 @@ __device__ __forceinline__ void smooth_dft(float (&re)[R], float (&im)[R]) {
 // Stage of radix R on sub-transforms of length R * STRIDE, each inside one first-stage chunk.  Starts with the barrier that
 // ends the stage before; the first round's twiddles are fetched ahead of it.
 template <class S, int R, int STRIDE, int MAP, int SIGN>
-__device__ __forceinline__ void smooth_middle(float2 *buf, const float2 *rows, int t) {
+__device__ __forceinline__ void smooth_middle(float2 *buf, const float2 *rows, int t, int *dbg) {
     constexpr int blocks = S::S0 / (R * STRIDE), units = S::M / R;
     auto place = [](int w, int &np) {
         if constexpr (MAP) {   // short strides: neighbouring threads on neighbouring chunks, which lie in different banks
@@ -103,13 +103,14 @@ __device__ __forceinline__ void smooth_middle(float2 *buf, const float2 *rows, i
         float re[R], im[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-            const float2 v = d[q * S::at(STRIDE)];
+            const float2 v = CQT_CHK(dbg, 808, at + q * S::at(STRIDE), S::BUF) ? d[q * S::at(STRIDE)] : make_float2(0.f, 0.f);
             re[q] = v.x; im[q] = v.y;
         }
         smooth_dft<R, SIGN>(re, im);
         tw.template apply<SIGN>(re, im);
 #pragma unroll
-        for (int q = 0; q < R; ++q) d[q * S::at(STRIDE)] = make_float2(re[q], im[q]);
+        for (int q = 0; q < R; ++q)
+            if (CQT_CHK(dbg, 808, at + q * S::at(STRIDE), S::BUF)) d[q * S::at(STRIDE)] = make_float2(re[q], im[q]);
         w += S::T;
         if (w < units) {
             at = place(w, np);
@@ -122,7 +123,7 @@ __device__ __forceinline__ void smooth_middle(float2 *buf, const float2 *rows, i
 // store(w, re, im, pre): results w + q NL.  again: the buffer holds the item before, whose last stage some threads may still read;
 // the others are on with this item's loads and first butterflies meanwhile.
 template <class S, int SIGN, class Load, class Pre, class Store>
-__device__ __forceinline__ void smooth_fft(float2 *buf, const float2 *rows, int t, bool again, Load load, Pre pre, Store store) {
+__device__ __forceinline__ void smooth_fft(float2 *buf, const float2 *rows, int t, bool again, int *dbg, Load load, Pre pre, Store store) {
     constexpr int R0 = S::R0, RL = S::RL;
     constexpr int rounds = (S::S0 + S::T - 1) / S::T;
 #pragma unroll 1
@@ -140,12 +141,13 @@ __device__ __forceinline__ void smooth_fft(float2 *buf, const float2 *rows, int 
         if (b < S::S0) {
             float2 *d = buf + S::at(b);
 #pragma unroll
-            for (int q = 0; q < R0; ++q) d[q * S::CHUNK] = make_float2(re[q], im[q]);
+            for (int q = 0; q < R0; ++q)
+                if (CQT_CHK(dbg, 807, S::at(b) + q * S::CHUNK, S::BUF)) d[q * S::CHUNK] = make_float2(re[q], im[q]);
         }
     }
-    if constexpr (S::STAGES > 2) smooth_middle<S, S::R1, S::S1, S::MAP1, SIGN>(buf, rows + S::TW1, t);
-    if constexpr (S::STAGES > 3) smooth_middle<S, S::R2, S::S2, S::MAP2, SIGN>(buf, rows + S::TW2, t);
-    if constexpr (S::STAGES > 4) smooth_middle<S, S::R3, S::S3, S::MAP3, SIGN>(buf, rows + S::TW3, t);
+    if constexpr (S::STAGES > 2) smooth_middle<S, S::R1, S::S1, S::MAP1, SIGN>(buf, rows + S::TW1, t, dbg);
+    if constexpr (S::STAGES > 3) smooth_middle<S, S::R2, S::S2, S::MAP2, SIGN>(buf, rows + S::TW2, t, dbg);
+    if constexpr (S::STAGES > 4) smooth_middle<S, S::R3, S::S3, S::MAP3, SIGN>(buf, rows + S::TW3, t, dbg);
     int w = t;
     decltype(pre(0)) fetched{};
     if (w < S::NL) fetched = pre(w);
@@ -157,11 +159,12 @@ __device__ __forceinline__ void smooth_fft(float2 *buf, const float2 *rows, int 
         if constexpr (S::STAGES == 3) in = (w / R0) * S::S1;
         if constexpr (S::STAGES == 4) in = ((w / R0) % S::R1) * S::S1 + (w / (R0 * S::R1)) * S::S2;
         if constexpr (S::STAGES == 5) in = ((w / R0) % S::R1) * S::S1 + ((w / (R0 * S::R1)) % S::R2) * S::S2 + (w / (R0 * S::R1 * S::R2)) * S::S3;
-        const float2 *d = buf + (w % R0) * S::CHUNK + S::at(in);
+        const int at = (w % R0) * S::CHUNK + S::at(in);
+        const float2 *d = buf + at;
         float re[RL], im[RL];
 #pragma unroll
         for (int q = 0; q < RL; ++q) {
-            const float2 v = d[q];
+            const float2 v = CQT_CHK(dbg, 809, at + q, S::BUF) ? d[q] : make_float2(0.f, 0.f);
             re[q] = v.x; im[q] = v.y;
         }
         smooth_dft<RL, SIGN>(re, im);
@@ -223,19 +226,20 @@ __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
 #pragma unroll
                     for (int q = 0; q < S::R0; ++q) {
                         const int j = entry(b + q * S::S0);
-                        const float2 v = j >= 0 && CQT_CHK(a.b.dbg, 801, j, br.S) ? ld_spectrum<CHAINED>(Xs + j) : make_float2(0.f, 0.f);
+                        const bool in = j >= 0 && CQT_CHK(a.b.dbg, 801, j, br.S) && CQT_CHK(a.b.dbg, 802, br.kc + br.d0 + j, (a.b.N >> 1) + 1);
+                        const float2 v = in ? ld_spectrum<CHAINED>(Xs + j) : make_float2(0.f, 0.f);
                         re[q] = v.x; im[q] = v.y;
                     }
 #pragma unroll
                     for (int q = 0; q < S::R0; ++q) {
                         const int j = entry(b + q * S::S0);
-                        const float h = j >= 0 ? __ldg(tab + j) : 0.f;
+                        const float h = j >= 0 && CQT_CHK(a.b.dbg, 803, br.tab_off + j, a.b.table_len) ? __ldg(tab + j) : 0.f;
                         re[q] *= h; im[q] *= h;
                     }
                 } else {
 #pragma unroll
                     for (int q = 0; q < S::R0; ++q) {
-                        const float2 v = slot_value<CHAINED>(br, tab, X, a.b.N, b + q * S::S0);
+                        const float2 v = slot_value<CHAINED>(br, tab, X, a.b.N, b + q * S::S0, a.b.dbg);
                         re[q] = v.x; im[q] = v.y;
                     }
                 }
@@ -244,17 +248,16 @@ __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
             auto store = [&](int w, float (&re)[S::RL], float (&im)[S::RL], int) {
                 if (!active) return;
 #pragma unroll
-                for (int q = 0; q < S::RL; ++q) {
-                    __stcs(c + w + q * S::NL, make_float2(re[q], im[q]));
-                }
+                for (int q = 0; q < S::RL; ++q)
+                    if (CQT_CHK(a.b.dbg, 804, w + q * S::NL, M)) __stcs(c + w + q * S::NL, make_float2(re[q], im[q]));
             };
-            smooth_fft<S, +1>(buf, rows, t, u > u0, load, [](int) { return 0; }, store);
+            smooth_fft<S, +1>(buf, rows, t, u > u0, a.b.dbg, load, [](int) { return 0; }, store);
         } else {
             const bool fold = a.b.fold && br.side != 0;
             auto load = [&](int b, float (&re)[S::R0], float (&im)[S::R0]) {
 #pragma unroll
                 for (int q = 0; q < S::R0; ++q) {
-                    const float2 v = ld_coefficient<CHAINED>(c + b + q * S::S0);   // read once
+                    const float2 v = CQT_CHK(a.b.dbg, 805, b + q * S::S0, M) ? ld_coefficient<CHAINED>(c + b + q * S::S0) : make_float2(0.f, 0.f);   // read once
                     re[q] = v.x; im[q] = v.y;
                 }
                 if (fold) {
@@ -272,7 +275,7 @@ __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
 #pragma unroll
                 for (int q = 0; q < S::RL; ++q) {
                     const int j = kept(w + q * S::NL);
-                    f.h[q] = j >= 0 ? __ldg(tab + j) : 0.f;
+                    f.h[q] = j >= 0 && CQT_CHK(a.b.dbg, 803, br.tab_off + j, a.b.table_len) ? __ldg(tab + j) : 0.f;
                 }
                 return f;
             };
@@ -281,10 +284,10 @@ __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
 #pragma unroll
                 for (int q = 0; q < S::RL; ++q) {
                     const int j = kept(w + q * S::NL);
-                    if (j >= 0 && CQT_CHK(a.b.dbg, 802, (long long)br.y_off + k0 + j, a.b.y_pitch)) Ys[j] = make_float2(f.h[q] * re[q], f.h[q] * im[q]);
+                    if (j >= 0 && CQT_CHK(a.b.dbg, 806, (long long)br.y_off + k0 + j, a.b.y_pitch)) Ys[j] = make_float2(f.h[q] * re[q], f.h[q] * im[q]);
                 }
             };
-            smooth_fft<S, -1>(buf, rows, t, u > u0, load, pre, store);
+            smooth_fft<S, -1>(buf, rows, t, u > u0, a.b.dbg, load, pre, store);
         }
     }
 }

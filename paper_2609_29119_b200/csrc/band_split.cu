@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) split_bands_kernel(BandArgs 
     float2 *Y = ANALYSIS ? nullptr : a.Y + (long long)ch * a.y_pitch + br.y_off;
     const bool fold = !ANALYSIS && a.fold && br.side != 0;
     auto in = [&](int n) -> float2 {
-        if constexpr (ANALYSIS) return slot_value<true>(br, tab, X, a.N, n);
+        if constexpr (ANALYSIS) return slot_value<true>(br, tab, X, a.N, n, a.dbg);
         const float2 v = CQT_CHK(a.dbg, 601, n, br.M) ? ld_chained(c + n) : make_float2(0.f, 0.f);
         return fold ? make_float2(2.f * v.x, 0.f) : v;
     };

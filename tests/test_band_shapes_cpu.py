@@ -95,3 +95,20 @@ def test_stages_stay_in_the_buffer_and_give_the_dft():
         out[w[None, :] + np.arange(RL)[:, None] * NL] = dft[RL] @ buf[where]
         want = np.fft.fft(x)
         assert np.linalg.norm(out - want) <= 1e-11 * np.linalg.norm(want), M
+
+
+def test_debug_build_checks_every_access():
+    """-DCQT_DEBUG_BOUNDS: loads and stores of the spectrum, the window table, the coefficients, the planes and the buffer are behind
+    a check of their index; slot_value has its own."""
+    code = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "band_smooth.cuh")).read())
+    body = code[code.index("void smooth_middle("):]
+    access = re.compile(r"ld_spectrum<|ld_coefficient<|__ldg\(tab|__stcs\(|\bYs\[|\bd\[")
+    lines = body.split("\n")
+    found = [i for i, line in enumerate(lines) if access.search(line)]
+    assert len(found) == 10
+    for i in found:
+        assert "CQT_CHK(" in lines[i] or ("in ? ld_spectrum" in lines[i] and "CQT_CHK(" in lines[i - 1]), lines[i]
+    assert re.search(r"slot_value<CHAINED>\([^;]*a\.b\.dbg\)", body)
+    common = open(os.path.join(CSRC, "band_common.cuh")).read()
+    slot = re.search(r"float2 slot_value\(.*?\n}", common, re.S).group(0)
+    assert slot.index("CQT_CHK(dbg, 405") < slot.index("__ldg(") and slot.index("CQT_CHK(dbg, 406") < slot.index("ld_spectrum")
