@@ -46,13 +46,13 @@ bool has_smooth(const cqt_plan &p, bool analysis, int cls) { return !p.smooth[cl
 //   class 2, 46 %: 1.5 58.0 / 58.9, 2 76.7 / 73.6 (2^17, 48); 40 %: 1.25 72.3 / 70.9, 2 109.2 / 105.0 (2^18, 24)
 // and with two / four: class 0 at 8 rounds 174 / 169 (2^15, 48), class 1 at 6 126 / 122.
 cudaError_t launch_smooth(const cqt_plan &p, bool analysis, int cls, const BandArgs &b, cudaStream_t st, int threads) {
-    if (threads == 0) threads = kSmoothThreads[cls];
+    if (threads == 0) threads = smooth_threads(cls);
     const SmoothBands &s = p.smooth[cls];
     SmoothArgs a;
     a.b = b;
     a.recs = s.d_recs;
     a.n = (int)s.lengths.size();
-    const int part = kSmoothThreads[cls] / threads;   // narrower CTAs have so much fewer items and shared memory
+    const int part = smooth_threads(cls) / threads;   // narrower CTAs have so much fewer items and shared memory
     const size_t smem = s.smem / part;
     const int64_t resident = p.sm_count * std::min<int64_t>(1024 / threads, (p.max_smem_optin + 1024) / ((int64_t)smem + 1024));
     int64_t units = 0;

@@ -25,11 +25,12 @@ struct SmoothShape {
     // one element skipped per PAD positions of a first-stage chunk
     static __host__ __device__ constexpr int at(int p) { return PAD_ ? p + p / (PAD_ ? PAD_ : 1) : p; }
     static constexpr int BUF = R0 * CHUNK;
-    // barrier of the T threads of an item: a warp's, the CTA's, or a named one
-    static constexpr bool WARP_SYNC = T <= 32 && 32 % T == 0, CTA_SYNC = !WARP_SYNC && (PER == 1 || T % 32 != 0), NAMED_SYNC = !WARP_SYNC && !CTA_SYNC;
+    // barrier of the T threads of an item: a warp's, the CTA's, or a named one (1 ... PER)
+    static constexpr bool WARP_SYNC = T <= 32, CTA_SYNC = !WARP_SYNC && PER == 1;
     // twiddle rows of the stages before the last, one after another
     static constexpr int TW1 = twiddle_rows(R0) * S0, TW2 = TW1 + twiddle_rows(R1) * S1, TW3 = TW2 + twiddle_rows(R2) * S2;
-    static_assert(R0 * R1 * R2 * R3 * R4 == M && at(S0 - 1) < CHUNK && T * PER <= THREADS && (!NAMED_SYNC || PER < 16), "shape");
+    static_assert(R0 * R1 * R2 * R3 * R4 == M && at(S0 - 1) < CHUNK, "shape");
+    static_assert(T * PER == THREADS && (WARP_SYNC ? 32 % T == 0 : T % 32 == 0 && PER < 16), "every thread of a barrier belongs to the item");
     static_assert(PAD_ == 0 || PAD_ == RL, "the skipped elements lie at multiples of every stride");
 };
 
@@ -174,7 +175,7 @@ __device__ __forceinline__ void smooth_fft(float2 *buf, const float2 *rows, int 
     }
 }
 
-constexpr int kSmoothThreads[kNumClasses] = {256, 256, 256, 512, 1024};   // by class; 1024 threads of 64 registers share an SM
+constexpr int smooth_threads(int cls) { return cls == 4 ? 1024 : 256; }   // of a CTA; 1024 threads of 64 registers share an SM
 
 // Bands of one length, from CTA cta0 of the launch on.  A unit is PER work items of them, one per group of T threads; a CTA takes
 // `repeat` units one after another.
@@ -197,19 +198,17 @@ __device__ __noinline__ void smooth_units(const SmoothArgs &a, int seg) {
     const SmoothSegment sg = a.seg[seg];
     const int per = S::M <= 128 ? (int)blockDim.x / S::T : S::PER;   // class 0 also runs in narrower CTAs
     const int g = S::PER > 1 ? (int)threadIdx.x / S::T : 0;
-    const bool idle = S::PER * S::T < S::THREADS && (int)threadIdx.x >= S::PER * S::T;
-    if (S::NAMED_SYNC && idle) return;                         // whole warps that belong to no item's barrier
-    const int t = idle ? S::M : (int)threadIdx.x - g * S::T;   // no butterfly has that index
+    const int t = (int)threadIdx.x - g * S::T;
     const int batch = a.b.batch, last = sg.n_bands * batch - 1;
     const int u0 = ((int)blockIdx.x - sg.cta0) * a.repeat, u1 = min(u0 + a.repeat, last / per + 1);
     const SmoothRec *recs = a.recs + sg.first_band;
     const float2 *rows = a.b.tw + recs->tw_off;
-    float2 *buf = smem_smooth + (idle ? 0 : g * S::BUF);
+    float2 *buf = smem_smooth + g * S::BUF;
     constexpr int M = S::M;
 #pragma unroll 1
     for (int u = u0; u < u1; ++u) {
         const int idx = u * per + g;
-        const bool active = !idle && idx <= last;                  // groups beyond the last item repeat it and store nothing
+        const bool active = idx <= last;   // groups beyond the last item repeat it and store nothing
         const int item = active ? idx : last, band = item / batch, ch = item - band * batch;
         const BandRec br = recs[band].br;
         const float *tab = a.b.table + br.tab_off;

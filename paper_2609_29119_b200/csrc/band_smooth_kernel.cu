@@ -8,7 +8,7 @@ namespace cqt {
 #define CQT_CAT(a, b) CQT_CAT_(a, b)
 #define CQT_SHAPES CQT_CAT(CQT_SHAPES_, CQT_CLASS)
 
-constexpr int kThreads = kSmoothThreads[CQT_CLASS];
+constexpr int kThreads = smooth_threads(CQT_CLASS);
 
 static __global__ void __launch_bounds__(kThreads, 1024 / kThreads) smooth_bands_kernel(const __grid_constant__ SmoothArgs a) {
     chain_enter(a.b);

@@ -141,12 +141,12 @@ class Shape:
     def layout(s):
         """CHUNK, PAD and the maps with the fewest shared-memory cycles"""
         best = None
-        room = SMEM_ELEMS // (s.per * (3 if s.per >= 8 else 1024 // s.threads))
+        room = SMEM_ELEMS // (s.per * (1 if s.threads == 1024 else 3 if s.per >= 8 else 4))
         for pad in ([0, s.rl] if len(s.r) > 2 else [0]):
             s.pad = pad
             for extra in range(0, 17):
                 s.chunk = s.chunk_min() + extra
-                if s.buf() > room and (s.threads < 1024 or s.buf() > SMEM_ELEMS):
+                if s.buf() > room:
                     continue
                 cost = s.r[0] * s.conflicts(s.stride[0], lambda b: s.at(b)) * (s.M / s.r[0])
                 for j in range(1, len(s.r) - 1):
@@ -179,8 +179,6 @@ def choose(m, group):
     _, _, threads, cap, t_of = GROUPS[group]
     T = t_of(m)
     sets = {tuple(sorted(f)) for f in factorisations(m, 5) if len(f) >= 2 and max(f) <= cap}
-    if not sets:
-        sets = {tuple(sorted(f)) for f in factorisations(m, 5) if len(f) >= 2}
     fewest = min(len(f) for f in sets)
     smallest = min(max(f) for f in sets if len(f) == fewest)
     best = None

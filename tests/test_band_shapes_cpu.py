@@ -39,15 +39,12 @@ def test_every_length_has_a_shape():
 
 
 def test_barriers_are_met_by_all_their_threads():
-    """T threads per item and PER items: the barrier of an item counts T threads, so it has to be one of whole warps, or of the
-    whole CTA, or of the lanes of one warp."""
+    """T threads per item and PER items fill the CTA: the barrier of an item counts T threads, so it has to be one of whole warps, or of
+    the whole CTA, or of the lanes of one warp."""
     for group, M, *rest in shapes():
         T, per, threads = rest[5], rest[6], rest[7]
-        assert threads == THREADS[group] and 1 <= per * T <= threads
-        warp = T <= 32 and 32 % T == 0
-        whole = not warp and (per == 1 or T % 32 != 0)
-        if not warp and not whole:
-            assert T % 32 == 0 and per < 16, M     # named barriers 1 ... per
+        assert threads == THREADS[group] and per * T == threads
+        assert 32 % T == 0 if T <= 32 else T % 32 == 0 and per < 16, M     # named barriers 1 ... per
 
 
 def test_stages_stay_in_the_buffer_and_give_the_dft():
@@ -61,7 +58,7 @@ def test_stages_stay_in_the_buffer_and_give_the_dft():
             n //= r
             stride.append(n)
         buf_len = R0 * chunk
-        assert per * buf_len <= SMEM_ELEMS // (1 if threads == 1024 else 2 if threads == 512 else 3)
+        assert per * buf_len <= SMEM_ELEMS // (1 if threads == 1024 else 3)
         x = rng.standard_normal(M) + 1j * rng.standard_normal(M)
         buf = np.full(buf_len, np.nan, dtype=complex)
         dft = {r: np.exp(-2j * np.pi * np.outer(np.arange(r), np.arange(r)) / r) for r in radices}
