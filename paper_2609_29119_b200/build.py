@@ -16,7 +16,7 @@ SOURCES = ["band_two_pass.cu", "band_analysis.cu", "band_synthesis.cu", "layout.
 VARIANTS = [("band_smooth_kernel.cu", f"band_smooth_{c}{'sa'[a]}{'_chained' * h}.o", [f"-DCQT_CLASS={c}", f"-DCQT_ANALYSIS={a}", f"-DCQT_CHAINED={h}"])
             for c, a, h in ((0, 0, 0), (0, 0, 1), (0, 1, 0), (0, 1, 1), (1, 1, 0), (2, 1, 0), (4, 0, 0), (4, 1, 0))]
 HEADERS = ["layout.hpp", "plan_types.h", "internal.hpp", "engine.cuh", "band_common.cuh", "long_common.cuh", "long_passes.cuh",
-           "static_fft.cuh", "codelets_gen.cuh", "table_upload.hpp",
+           "static_fft.cuh", "twiddle_rows.cuh", "codelets_gen.cuh", "table_upload.hpp",
            os.path.join("..", "..", "include", "cqt.h")]
 SMOOTH_HEADERS = ["band_smooth.cuh", "band_shapes.cuh"]   # of the sources that start with band_smooth
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",

@@ -514,19 +514,9 @@ static cqt_status finish_plan(OwnedPlan p, int64_t N, int device, const cqt_plan
     for (int li = 0; li < kPow2Lengths; ++li) {
         p->pow2.n_bands[li] = (int)pow2_bands[li].size();
         if (pow2_bands[li].empty()) continue;
-        // per stage but the last (sub-transforms of n points, radix r): rows W_n^{p y}, y < n / r, p = 1, 2, 4, ... < r
-        int r[4];
+        int r[5];
         pow2_radices(li, r);
-        const int off = (int)tw.size();
-        int64_t n = L.bands[(size_t)pow2_bands[li][0]].M;
-        for (int j = 0; j < 3 && r[j + 1] > 1; ++j) {
-            for (int64_t pw = 1; pw < r[j]; pw *= 2)
-                for (int64_t y = 0; y < n / r[j]; ++y) {
-                    const double ang = -2.0 * kPi * (double)((pw * y) % n) / (double)n;
-                    tw.push_back(make_float2((float)std::cos(ang), (float)std::sin(ang)));
-                }
-            n /= r[j];
-        }
+        const int off = append_twiddle_rows(tw, L.bands[(size_t)pow2_bands[li][0]].M, r);
         for (int b : pow2_bands[li]) {
             Pow2Rec rec{};
             rec.br = p->bands[(size_t)b];

@@ -11,10 +11,9 @@
 #include <algorithm>
 
 #include "band_common.cuh"
+#include "twiddle_rows.cuh"
 
 namespace cqt {
-
-__host__ __device__ constexpr int lg2(int r) { return r <= 1 ? 0 : 1 + lg2(r / 2); }
 
 // L = R0 R1 R2 R3 (trailing ones: fewer stages) on T threads of a CTA of THREADS
 template <int R0_, int R1_, int R2_, int R3_, int THREADS_>
@@ -27,7 +26,7 @@ struct Pow2Shape {
     static __host__ __device__ constexpr int at(int p) { return R2 > 1 ? p + p / RL : p; }
     static constexpr int CHUNK = (at(S0 - 1) + 1) | 1, BUF = R0 * CHUNK;
     // twiddle rows of the stages before the last, one after another
-    static constexpr int TW1 = lg2(R0) * S0, TW2 = TW1 + (R2 > 1 ? lg2(R1) * S1 : 0), TW_COUNT = TW2 + (R3 > 1 ? lg2(R2) * S2 : 0);
+    static constexpr int TW1 = twiddle_rows(R0) * S0, TW2 = TW1 + (R2 > 1 ? twiddle_rows(R1) * S1 : 0), TW_COUNT = TW2 + (R3 > 1 ? twiddle_rows(R2) * S2 : 0);
 };
 using P256 = Pow2Shape<16, 16, 1, 1, 256>;
 using P512 = Pow2Shape<8, 8, 8, 1, 256>;
@@ -47,42 +46,6 @@ __device__ __forceinline__ void group_sync() {
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / T), "n"(T) : "memory");
 }
 
-// twiddles w, w^2, w^4, w^8 of one butterfly: rows of s entries
-template <int R>
-struct TwiddleRows {
-    float2 w[lg2(R)];
-    __device__ __forceinline__ TwiddleRows(const float2 *__restrict__ rows, int s, int np) {
-#pragma unroll
-        for (int i = 0; i < lg2(R); ++i) w[i] = __ldg(rows + i * s + np);
-    }
-    template <int SIGN>
-    __device__ __forceinline__ void apply(float (&re)[R], float (&im)[R]) const {
-        float wr[R], wi[R];
-#pragma unroll
-        for (int q = 1; q < R; ++q) {
-            const int hb = q >= 8 ? 8 : (q >= 4 ? 4 : (q >= 2 ? 2 : 1)), lo = q - hb;
-            if (lo == 0) {
-                wr[q] = w[lg2(hb)].x;
-                wi[q] = SIGN > 0 ? -w[lg2(hb)].y : w[lg2(hb)].y;
-            } else {
-                wr[q] = fmaf(wr[hb], wr[lo], -wi[hb] * wi[lo]);
-                wi[q] = fmaf(wr[hb], wi[lo], wi[hb] * wr[lo]);
-            }
-        }
-#pragma unroll
-        for (int q = 1; q < R; ++q) {
-            const float x = re[q], y = im[q];
-            re[q] = fmaf(x, wr[q], -y * wi[q]);
-            im[q] = fmaf(x, wi[q], y * wr[q]);
-        }
-    }
-};
-
-template <int R, int SIGN>
-__device__ __forceinline__ void pow2_dft(float (&re)[R], float (&im)[R]) {
-    if (SIGN < 0) Codelet<R>::run(re, im); else Codelet<R>::run(im, re);
-}
-
 // stage of radix R on sub-transforms of length R * STRIDE, each inside one first-stage chunk
 template <class S, int R, int STRIDE, int SIGN>
 __device__ __forceinline__ void pow2_middle(float2 *buf, const float2 *rows, int t) {
@@ -92,14 +55,15 @@ __device__ __forceinline__ void pow2_middle(float2 *buf, const float2 *rows, int
     for (int w = t; w < S::L / R; w += S::T) {
         const int np = w % STRIDE, blk = w / STRIDE, k0 = blk / blocks;
         float2 *d = buf + k0 * S::CHUNK + S::at((blk % blocks) * (R * STRIDE) + np);
-        const TwiddleRows<R> tw(rows, STRIDE, np);
+        TwiddleRows<R> tw;
+        tw.load(rows, STRIDE, np);
         float re[R], im[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) {
             const float2 v = d[q * S::at(STRIDE)];
             re[q] = v.x; im[q] = v.y;
         }
-        pow2_dft<R, SIGN>(re, im);
+        dft<R, SIGN>(re, im);
         tw.template apply<SIGN>(re, im);
 #pragma unroll
         for (int q = 0; q < R; ++q) d[q * S::at(STRIDE)] = make_float2(re[q], im[q]);
@@ -115,9 +79,10 @@ __device__ __forceinline__ void pow2_fft(float2 *buf, const float2 *rows, int t,
 #pragma unroll 1
     for (int b = t; b < S::S0; b += S::T) {
         float re[R0], im[R0];
-        const TwiddleRows<R0> tw(rows, S::S0, b);
+        TwiddleRows<R0> tw;
+        tw.load(rows, S::S0, b);
         load(b, re, im);
-        pow2_dft<R0, SIGN>(re, im);
+        dft<R0, SIGN>(re, im);
         tw.template apply<SIGN>(re, im);
         float2 *d = buf + S::at(b);
 #pragma unroll
@@ -140,7 +105,7 @@ __device__ __forceinline__ void pow2_fft(float2 *buf, const float2 *rows, int t,
             const float2 v = d[q];
             re[q] = v.x; im[q] = v.y;
         }
-        pow2_dft<RL, SIGN>(re, im);
+        dft<RL, SIGN>(re, im);
         store(w, re, im, fetched);
     }
 }
@@ -266,10 +231,9 @@ int pow2_length_index(int64_t M) {
     return -1;
 }
 
-// twiddle rows of a length in the order of Pow2Shape
-void pow2_radices(int index, int (&r)[4]) {
+void pow2_radices(int index, int (&r)[5]) {
     int i = 0;
-#define X(S) if (i++ == index) { r[0] = S::R0; r[1] = S::R1; r[2] = S::R2; r[3] = S::R3; }
+#define X(S) if (i++ == index) { r[0] = S::R0; r[1] = S::R1; r[2] = S::R2; r[3] = S::R3; r[4] = 1; }
     CQT_POW2_LONG(X) CQT_POW2_SHORT(X)
 #undef X
 }

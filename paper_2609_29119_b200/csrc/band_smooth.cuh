@@ -10,10 +10,9 @@
 #pragma once
 #include "band_common.cuh"
 #include "band_shapes.cuh"
+#include "twiddle_rows.cuh"
 
 namespace cqt {
-
-__host__ __device__ constexpr int twiddle_rows(int r) { return r <= 1 ? 0 : 1 + twiddle_rows((r + 1) / 2); }   // powers 1, 2, 4 ... below r
 
 template <int M_, int R0_, int R1_, int R2_, int R3_, int R4_, int T_, int PER_, int THREADS_, int PAD_, int CHUNK_, int MAP1_, int MAP2_, int MAP3_>
 struct SmoothShape {
@@ -41,41 +40,6 @@ __device__ __forceinline__ void smooth_sync() {
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / S::T), "n"(S::T) : "memory");
 }
 
-// Twiddles w, w^2, w^4, w^8 of one butterfly: rows of s entries, in the order in which consecutive butterflies read them; the
-// other powers are products of at most three of those (raising one rounded w to the q-th power would multiply its error by q).
-template <int R>
-struct SmoothTwiddles {
-    static constexpr int N = twiddle_rows(R);
-    float2 w[N];
-    __device__ __forceinline__ void load(const float2 *__restrict__ rows, int s, int np) {
-#pragma unroll
-        for (int i = 0; i < N; ++i) w[i] = __ldg(rows + i * s + np);
-    }
-    template <int SIGN>
-    __device__ __forceinline__ void apply(float (&re)[R], float (&im)[R]) const {
-        float wr[R], wi[R];
-#pragma unroll
-        for (int q = 1; q < R; ++q) {
-            const int hi = q >= 8 ? 3 : (q >= 4 ? 2 : (q >= 2 ? 1 : 0)), hb = 1 << hi, lo = q - hb;
-            if (lo == 0) {
-                wr[q] = w[hi].x;
-                wi[q] = SIGN > 0 ? -w[hi].y : w[hi].y;
-            } else {
-                wr[q] = fmaf(wr[hb], wr[lo], -wi[hb] * wi[lo]);
-                wi[q] = fmaf(wr[hb], wi[lo], wi[hb] * wr[lo]);
-            }
-            const float x = re[q], y = im[q];
-            re[q] = fmaf(x, wr[q], -y * wi[q]);
-            im[q] = fmaf(x, wi[q], y * wr[q]);
-        }
-    }
-};
-
-template <int R, int SIGN>
-__device__ __forceinline__ void smooth_dft(float (&re)[R], float (&im)[R]) {
-    if (SIGN < 0) Codelet<R>::run(re, im); else Codelet<R>::run(im, re);
-}
-
 // Stage of radix R on sub-transforms of length R * STRIDE, each inside one first-stage chunk.  Starts with the barrier that
 // ends the stage before; the first round's twiddles are fetched ahead of it.
 template <class S, int R, int STRIDE, int MAP, int SIGN>
@@ -93,7 +57,7 @@ __device__ __forceinline__ void smooth_middle(float2 *buf, const float2 *rows, i
         }
     };
     int w = t, np = 0, at = 0;
-    SmoothTwiddles<R> tw;
+    TwiddleRows<R> tw;
     if (w < units) {
         at = place(w, np);
         tw.load(rows, STRIDE, np);
@@ -107,7 +71,7 @@ __device__ __forceinline__ void smooth_middle(float2 *buf, const float2 *rows, i
             const float2 v = CQT_CHK(dbg, 808, at + q * S::at(STRIDE), S::BUF) ? d[q * S::at(STRIDE)] : make_float2(0.f, 0.f);
             re[q] = v.x; im[q] = v.y;
         }
-        smooth_dft<R, SIGN>(re, im);
+        dft<R, SIGN>(re, im);
         tw.template apply<SIGN>(re, im);
 #pragma unroll
         for (int q = 0; q < R; ++q)
@@ -132,10 +96,10 @@ __device__ __forceinline__ void smooth_fft(float2 *buf, const float2 *rows, int 
         const int b = t + r * S::T;
         float re[R0], im[R0];
         if (b < S::S0) {
-            SmoothTwiddles<R0> tw;
+            TwiddleRows<R0> tw;
             tw.load(rows, S::S0, b);
             load(b, re, im);
-            smooth_dft<R0, SIGN>(re, im);
+            dft<R0, SIGN>(re, im);
             tw.template apply<SIGN>(re, im);
         }
         if (again && r == 0) smooth_sync<S>();
@@ -168,7 +132,7 @@ __device__ __forceinline__ void smooth_fft(float2 *buf, const float2 *rows, int 
             const float2 v = CQT_CHK(dbg, 809, at + q, S::BUF) ? d[q] : make_float2(0.f, 0.f);
             re[q] = v.x; im[q] = v.y;
         }
-        smooth_dft<RL, SIGN>(re, im);
+        dft<RL, SIGN>(re, im);
         store(w, re, im, fetched);
         w += S::T;
         if (w < S::NL) fetched = pre(w);

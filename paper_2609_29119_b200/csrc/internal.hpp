@@ -241,7 +241,7 @@ cudaError_t configure_chirp_kernels(const cqt_plan &p);
 
 // band_pow2.cu
 int pow2_length_index(int64_t M);                  // place of a length in Pow2Bands::n_bands, -1: not a length of that kernel
-void pow2_radices(int index, int (&r)[4]);         // its stages (1: none)
+void pow2_radices(int index, int (&r)[5]);         // its stages (1: none)
 cudaError_t configure_pow2_kernels(const cqt_plan &p);
 
 // band_smooth.cu
