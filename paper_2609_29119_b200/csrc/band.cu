@@ -125,6 +125,10 @@ static long long few_part(const cqt_plan &p, int64_t batch, int first, int last,
 // coefficients).  Round trips of 1 - 12 signals in 16 layouts, a warp per item on the run-time planned kernel against this one: without
 // split bands 3.7 % less on average up to 4 items per SM (4 signals of 2^13 samples at 24 bands per octave 39.9 -> 34.0 us, one of 2^16
 // at 24 42.6 -> 41.1, one of 2^18 at 96 50.2 -> 47.0; four of 40 calls 2 - 4.5 % slower); above 6 items per SM the two alternate.
+// Single calls scatter, since launches that run at the same time share SMs as they happen to fall (2^12 samples at 24, analysis of one, two,
+// three signals on the run-time planned kernel: 11.3, 12.2, 10.3 us): over 76 calls of 2^12 ... 2^17 samples round trips differ from 17 % less
+// to 12 % more, 3.6 % less on average, analysis alone from 30 % less to 18 % more, 5.7 % less, synthesis alone from 25 % less to 19 % more,
+// 5.7 % less (64 threads per CTA: 2.9, 4.5 and 4.9 % less).
 // With split bands it costs more than it gives (36 bands per octave: one signal of 2^17 60.1 -> 69.3 us, two 61.0 -> 71.8; one of
 // 2^18 at 24 55.6 -> 65.3; 2^16 at 12: one 36.8 -> 38.2, two 44.9 -> 40.1, three 43.7 -> 48.5, six 46.4 -> 46.1): probably the code,
 // since the split and the merged kernel wait for instructions more than for anything else and up to 19 lengths' code then passes
@@ -198,10 +202,13 @@ static cudaError_t launch_few(const cqt_plan &p, BandArgs &a, FewLaunch &f, cuda
     return e;
 }
 
-// Power-of-two plans: two or three launches, chained, at any batch.  Class 0 on the kernel of 5-smooth lengths: 60 calls drawn from 2^12 ...
-// 2^18 samples, 12 - 96 bands per octave, 3 - 120 items per SM, against the run-time planned one: round trips from 20 % less to 4 % more, 4 %
-// less on average; analysis alone from 31 % less to, at 2^12 and 2^14 samples, 31 % more (27 signals of 2^12 at 48 12.9 -> 16.9 us, 9 of 2^14 at 36
-// 14.1 -> 17.9, but 2 of 2^14 11.8 -> 11.5), 4 % less on average; neither items per SM nor share of the coefficients tells the two apart.
+// Power-of-two plans: two or three launches, chained, at any batch.  Class 0 on the kernel of 5-smooth lengths, against the run-time planned
+// one, 38 calls of 2^12 ... 2^17 samples, 12 - 96 bands per octave and the multi-resolution layout, 1 - 415 signals: round trips from 24 % less to
+// 6 % more, 9 % less on average; analysis alone from 35 % less to 23 % more, 11 % less; synthesis alone from 37 % less to 17 % more, 7 % less.
+// A call that loses in one gains elsewhere (analysis, synthesis, round trip: 9 signals of 2^14 at 36 13.6 -> 16.7, 18.3 -> 16.5, 35.0 -> 34.5
+// us; 115 of 2^12 at 12 16.2 -> 11.9, 17.9 -> 20.1, 32.5 -> 34.5); neither items per SM nor share of the coefficients tells them apart.
+// CTAs of 64 or 128 threads instead of 256 above 4 items per SM: round trips 4 and 1 % slower on average (from 3 % less to 23 % more, 5 %
+// less to 12 % more).
 template <bool ANALYSIS>
 static cudaError_t launch_pow2_plan(const cqt_plan &p, BandArgs &a, cudaStream_t st) {
     const BandClass &c = p.cls[0];

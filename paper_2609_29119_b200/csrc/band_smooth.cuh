@@ -1,12 +1,16 @@
 // Bands whose length has no prime factor above 5, every length a transform of its own: radices, strides, threads and the layout
 // of the buffer are known at compile time (band_shapes.cuh, chosen by choose_shapes.py).
 //
-// Bounds: instructions, their fetch included.  On the run-time planned engine an element costs 34 instructions per radix stage,
-// here 26, and a band of at most 128 coefficients takes two stages instead of up to three.  The code of one length (4 - 20 KB)
+// Bounds: instructions, their fetch included.  Thread instructions per coefficient, on the run-time planned kernels and here: analysis
+// of class 1 151 and 106, of class 2 153 and 114 (3.2 and 3.9 stages on average), of class 4 143 and 119, its synthesis 141 and 125 (16
+// signals of 2^19 samples); a band of at most 128 coefficients takes two stages instead of up to three.  The code of one length (4 - 20 KB)
 // does not stay in an SM's instruction cache from one length to the next: a CTA's first pass over it waits for the cache that
 // the SMs of a GPC share (first stage of a 960-coefficient item 13,000 cycles, the same stage again 4,900).  Hence the order of
 // the grid, equal lengths adjacent, so that all SMs fetch the same code at about the same time (persistent CTAs that each walk a
 // length of their own: 51 us where this order takes 37), and several units per CTA where a call has many (launch_smooth).
+// All kernels have 64 registers per thread, so that 1024 threads share an SM, and most lengths spill (bytes of spill stores per thread,
+// the lengths that do, the most): analysis of class 0 11 of 19, 52; class 1 30 of 33, 32; class 2 33 of 35, 176; class 4 31 of 31, 184;
+// synthesis of class 0 9 of 19, 220; class 4 31 of 31, 392 (16,000 = 10 10 10 16, whose last butterflies hold 16 values and 16 window entries).
 #pragma once
 #include "band_common.cuh"
 #include "band_shapes.cuh"
